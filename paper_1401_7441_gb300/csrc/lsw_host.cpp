@@ -204,9 +204,8 @@ struct lsw_system_s {
     // the pattern, work matrices and the dense row scratch of the triple products
     DeviceBuf d_tpos, d_diag, d_ident, d_foe, d_foe_scratch;
     // confinement and preconditioning: per-atom tables of the 1D operators X_d^2, X_d^4,
-    // the batch boxes, and the conjugate-gradient vectors and scalars
+    // the boxes, tables and maps of a batch, and the conjugate-gradient vectors and scalars
     DeviceBuf d_qtab, d_qtab_off, d_cbox, d_cg, d_cgs;
-    int conf_batch = 0;
     std::vector<PanelSlab> slabs;
     DeviceBuf d_shift, d_fn_all;   // reformat: per-atom shifts, records of every function
     // density: real-space store, block records, tile lists (built for one grid)
@@ -1396,6 +1395,7 @@ lsw_status lsw_ctx_create(int device, void* stream, lsw_ctx* out) {
     CUDA_TRY(configure_kernels(c->max_smem));
     CUDA_TRY(configure_panel_kernels(c->max_smem));
     CUDA_TRY(configure_foe_kernels(c->max_smem));
+    CUDA_TRY(configure_confine_kernels(c->max_smem));
     *out = c.release();
     return LSW_OK;
 }
@@ -1871,9 +1871,14 @@ void conf_row(const FilterSet& F, const std::vector<double>& G, int m, int b, in
     }
 }
 
+// The tables of every atom, computed on the device from G and the filters.
 lsw_status build_conf_tables(lsw_system_s* s) {
     const FilterSet& F = s->ctx->filters;
-    const std::vector<double> G = conf_G(F);
+    std::vector<double> in = conf_G(F);                // then h, g, the positions
+    const size_t nG = in.size();
+    in.insert(in.end(), F.h, F.h + D16);
+    in.insert(in.end(), F.g, F.g + D16);
+    in.insert(in.end(), s->pos.begin(), s->pos.end());
     const int na = s->n_atoms;
     std::vector<int64_t> off(na + 1, 0);
     for (int a = 0; a < na; ++a) {
@@ -1881,35 +1886,36 @@ lsw_status build_conf_tables(lsw_system_s* s) {
         for (int d = 0; d < 3; ++d) n += 2LL * 4 * (s->L[a].n[d] + 2 * KIN_HALF) * KIN_TAPS;
         off[a + 1] = off[a] + n;
     }
-    std::vector<double> tab(std::max<int64_t>(off[na], 1), 0.0);
-    const double h = s->h;
-    parallel_for(na, [&](int a) {
-        int64_t base = off[a];
-        for (int d = 0; d < 3; ++d) {
-            const int E = s->L[a].n[d] + 2 * KIN_HALF;
-            const double c = s->pos[3 * a + d] / h;
-            for (int mi = 0; mi < 2; ++mi)
-                for (int b = 0; b < 2; ++b)
-                    for (int bp = 0; bp < 2; ++bp)
-                        for (int i = 0; i < E; ++i)
-                            conf_row(F, G, mi == 0 ? 2 : 4, b, bp, static_cast<double>(s->L[a].lo[d] - KIN_HALF + i), c, h,
-                                     &tab[base + ((static_cast<int64_t>(mi) * 4 + (b * 2 + bp)) * E + i) * KIN_TAPS]);
-            base += 2LL * 4 * E * KIN_TAPS;
-        }
-    });
     cudaStream_t st = s->stream;
-    CUDA_TRY(s->d_qtab.upload(tab, st));
+    DeviceBuf d_in;
+    CUDA_TRY(d_in.upload(in, st));
     CUDA_TRY(s->d_qtab_off.upload(off, st));
+    CUDA_TRY(s->d_qtab.alloc(static_cast<size_t>(std::max<int64_t>(off[na], 1)) * sizeof(double)));
+    const double* p = static_cast<const double*>(d_in.p);
+    cudaError_t e = conf_tables(na, static_cast<const AtomRec*>(s->d_atoms.p), p + nG + 2 * D16, p, p + nG, s->h,
+                                static_cast<const int64_t*>(s->d_qtab_off.p), static_cast<double*>(s->d_qtab.p), st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);       // d_in is freed on return
+    if (e != cudaSuccess) {
+        (void)s->d_qtab.alloc(0);
+        return cuda_fail(e, "confinement tables");
+    }
     return LSW_OK;
 }
 
-// Launch arguments of one batch [f0, f0 + nfn) of the confinement kernels.
-ConfLaunch conf_launch(lsw_system_s* s, int64_t f0, int nfn, const double* acoef, const double* eps, int64_t box_stride) {
-    ConfLaunch c;
+// Launch arguments of the confinement kernels for a region: box and map strides over every
+// function's atom, the tables (first call), the batch buffer (a budget of 2 GiB) and the
+// functions per batch.
+lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double* acoef, const double* eps, ConfLaunch* out,
+                        int* batch) {
+    if (s->d_qtab.bytes == 0) {
+        lsw_status e = build_conf_tables(s);
+        if (e != LSW_OK) return e;
+    }
+    ConfLaunch& c = *out;
     std::memset(&c, 0, sizeof(c));
     c.prec = s->prec;
-    c.f0 = f0;
-    c.nfn = nfn;
+    c.region = region;
+    c.precond = precond ? 1 : 0;
     c.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
     c.atoms = static_cast<const AtomRec*>(s->d_atoms.p);
     c.seg = static_cast<const Seg*>(s->d_seg.p);
@@ -1923,47 +1929,66 @@ ConfLaunch conf_launch(lsw_system_s* s, int64_t f0, int nfn, const double* acoef
     for (int b = 0; b < 4; ++b)
         for (int l = 0; l < KIN_TAPS; ++l) c.kin[b][l] = s->ctx->filters.kin[b][l];
     c.kin_scale = -1.0 / (2.0 * s->h * s->h);
-    c.box_stride = box_stride;
-    for (int64_t f = f0; f < f0 + nfn; ++f) {
-        const int a = s->sf_atom[f];
-        c.max_rows_L = std::max(c.max_rows_L, s->L[a].n[1] * s->L[a].n[2]);
+    for (int a = 0; a < s->n_atoms; ++a) {
+        if (s->nsf[a] == 0) continue;
+        const LocregHost& L = s->L[a];
+        const LocregHost& R = region ? s->Lp[a] : L;
+        int64_t n[3], m[3];
+        for (int d = 0; d < 3; ++d) {
+            n[d] = L.n[d];
+            m[d] = std::min(R.lo[d] + R.n[d], L.lo[d] + L.n[d] + KIN_HALF) - std::max(R.lo[d], L.lo[d] - KIN_HALF);
+            c.max_n = std::max(c.max_n, static_cast<int>(n[d]));
+            c.max_m = std::max(c.max_m, static_cast<int>(m[d]));
+        }
+        c.s_P = std::max(c.s_P, align64(8 * n[0] * n[1] * n[2]));
+        c.s_A = std::max(c.s_A, align64(8 * n[0] * n[1] * m[2]));
+        c.s_B = std::max(c.s_B, align64(8 * n[0] * m[1] * m[2]));
+        c.s_F = std::max(c.s_F, align64(8 * m[0] * m[1] * m[2]));
+        c.s_mem = std::max(c.s_mem, align64(m[0] * m[1] * m[2]));
+        c.s_xy = std::max(c.s_xy, align64(2 * n[0] * n[1]));
+        c.s_xz = std::max(c.s_xz, align64(2 * n[0] * n[2]));
+        c.s_x = std::max(c.s_x, align64(2 * n[0]));
+        c.s_row = std::max(c.s_row, align64(2 * m[1] * m[2]));
+        c.s_oxz = std::max(c.s_oxz, align64(2 * m[0] * m[2]));
+        c.max_lines[0] = std::max(c.max_lines[0], static_cast<int>(m[1] * m[2]));
+        c.max_lines[1] = std::max(c.max_lines[1], static_cast<int>(n[0] * m[2]));
+        c.max_lines[2] = std::max(c.max_lines[2], static_cast<int>(n[0] * n[1]));
+        c.max_rows_L = std::max(c.max_rows_L, L.n[1] * L.n[2]);
         c.max_rows_P = std::max(c.max_rows_P, s->Lp[a].n[1] * s->Lp[a].n[2]);
-        int64_t v = 1;
-        for (int d = 0; d < 3; ++d) v *= s->L[a].n[d] + 2 * KIN_HALF;
-        c.max_vol = std::max(c.max_vol, v);
     }
+    c.s_comb = align64(3LL * 4 * c.max_m * KIN_TAPS);
+    c.s_maps = c.s_mem + c.s_xy + c.s_xz + c.s_x + c.s_row + c.s_oxz;
+    const int64_t doubles = c.s_P + 2 * c.s_A + 2 * c.s_B + c.s_F + c.s_comb;
+    const size_t per = static_cast<size_t>(doubles) * sizeof(double) + static_cast<size_t>(c.s_maps);
+    const int64_t nf = static_cast<int64_t>(s->sf_atom.size());
+    const int b = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, nf, static_cast<int64_t>((size_t(2) << 30) / per)})));
+    if (s->d_cbox.bytes < per * b) {
+        CUDA_TRY(cudaStreamSynchronize(s->stream));
+        CUDA_TRY(s->d_cbox.alloc(per * b));
+    }
+    double* p = static_cast<double*>(s->d_cbox.p);
+    auto take = [&](int64_t stride) {
+        double* q = p;
+        p += stride * b;
+        return q;
+    };
+    c.P = take(c.s_P);
+    c.A = take(c.s_A);
+    c.OZ = take(c.s_A);
+    c.B = take(c.s_B);
+    c.OY = take(c.s_B);
+    c.F = take(c.s_F);
+    c.comb = take(c.s_comb);
+    c.maps = reinterpret_cast<unsigned char*>(p);
+    c.max_smem = s->ctx->max_smem - CONF_STATIC_SMEM;
     c.status = static_cast<int*>(s->d_status.p);
     c.qtab_n = static_cast<int64_t>(s->d_qtab.bytes / sizeof(double));
     c.seg_n = static_cast<int64_t>(s->d_seg.bytes / sizeof(Seg));
     c.rowptr_n = static_cast<int64_t>(s->d_rowptr.bytes / sizeof(int32_t));
     c.vec_n = s->off_L.back();
     c.dst_n = s->off_Lp.back();
-    c.n_sf = static_cast<int>(s->sf_atom.size());
+    c.n_sf = static_cast<int>(nf);
     c.n_atoms = s->n_atoms;
-    return c;
-}
-
-// Tables (first call) and batch boxes: three boxes per function of a batch, the batch
-// sized to a budget of 2 GiB.  Returns the box stride (elements) and the batch size.
-lsw_status conf_prepare(lsw_system_s* s, int64_t* box_stride, int* batch) {
-    if (s->d_qtab.bytes == 0) {
-        lsw_status e = build_conf_tables(s);
-        if (e != LSW_OK) return e;
-    }
-    int64_t vmax = 0;
-    for (int a = 0; a < s->n_atoms; ++a) {
-        int64_t v = 1;
-        for (int d = 0; d < 3; ++d) v *= s->L[a].n[d] + 2 * KIN_HALF;
-        vmax = std::max(vmax, v);
-    }
-    *box_stride = align64(8 * vmax);
-    const int64_t nf = static_cast<int64_t>(s->sf_atom.size());
-    const size_t per = 3 * static_cast<size_t>(*box_stride) * s->esize;
-    const int b = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({64, nf, static_cast<int64_t>((size_t(2) << 30) / per)})));
-    if (s->d_cbox.bytes < per * b) {
-        CUDA_TRY(cudaStreamSynchronize(s->stream));
-        CUDA_TRY(s->d_cbox.alloc(per * b));
-    }
     *batch = b;
     return LSW_OK;
 }
@@ -1986,17 +2011,15 @@ lsw_status lsw_add_confinement(lsw_system sys, const double* a_dev, const void* 
     if (!sys || !a_dev || !phi || !hphi) return fail(LSW_ERR_ARG, "lsw_add_confinement: NULL buffer");
     CUDA_TRY(cudaSetDevice(sys->ctx->device));
     (void)cudaGetLastError();   // an earlier call's error is not this call's
-    int64_t stride = 0;
+    ConfLaunch c;
     int batch = 0;
-    lsw_status e = conf_prepare(sys, &stride, &batch);
+    lsw_status e = conf_prepare(sys, 1, false, a_dev, nullptr, &c, &batch);
     if (e != LSW_OK) return e;
     const int64_t nf = static_cast<int64_t>(sys->sf_atom.size());
-    unsigned char* box = static_cast<unsigned char*>(sys->d_cbox.p);
-    const size_t bb = static_cast<size_t>(batch) * stride * sys->esize;
-    for (int64_t f0 = 0; f0 < nf; f0 += batch) {
-        const int nb = static_cast<int>(std::min<int64_t>(batch, nf - f0));
-        ConfLaunch c = conf_launch(sys, f0, nb, a_dev, nullptr, stride);
-        CUDA_TRY(conf_apply(c, phi, box, box + bb, box + 2 * bb, hphi, 1, 1, false, e_conf, sys->stream));
+    for (c.f0 = 0; c.f0 < nf; c.f0 += batch) {
+        c.nfn = static_cast<int>(std::min<int64_t>(batch, nf - c.f0));
+        CUDA_TRY(conf_setup(c, sys->stream));
+        CUDA_TRY(conf_apply(c, phi, hphi, 1, e_conf, sys->stream));
     }
     return LSW_OK;
 }
@@ -2010,41 +2033,32 @@ lsw_status lsw_precondition(lsw_system sys, const double* a_dev, const double* e
     if (iters < 1) return fail(LSW_ERR_ARG, "lsw_precondition: iters %d", iters);
     CUDA_TRY(cudaSetDevice(sys->ctx->device));
     (void)cudaGetLastError();   // an earlier call's error is not this call's
-    int64_t stride = 0;
+    ConfLaunch c;
     int batch = 0;
-    lsw_status e = conf_prepare(sys, &stride, &batch);
+    lsw_status e = conf_prepare(sys, 0, true, a_dev, eps_dev, &c, &batch);
     if (e != LSW_OK) return e;
     const int64_t nf = static_cast<int64_t>(sys->sf_atom.size());
     const int64_t nv = sys->off_L.back();
     const size_t vb = static_cast<size_t>(std::max<int64_t>(nv, 1)) * sys->esize;
-    if (sys->d_cg.bytes < 3 * vb || sys->d_cgs.bytes < 4 * nf * sizeof(double)) {
+    if (sys->d_cg.bytes < 3 * vb || sys->d_cgs.bytes < nf * sizeof(double)) {
         CUDA_TRY(cudaStreamSynchronize(sys->stream));
         CUDA_TRY(sys->d_cg.alloc(3 * vb));
-        CUDA_TRY(sys->d_cgs.alloc(static_cast<size_t>(4 * std::max<int64_t>(nf, 1)) * sizeof(double)));
+        CUDA_TRY(sys->d_cgs.alloc(static_cast<size_t>(std::max<int64_t>(nf, 1)) * sizeof(double)));
     }
     unsigned char* V = static_cast<unsigned char*>(sys->d_cg.p);
     void* r = V;
     void* p = V + vb;
     void* Ap = V + 2 * vb;
-    double* sc = static_cast<double*>(sys->d_cgs.p);
-    double* rr = sc;
-    double* rr_new = sc + nf;
-    double* pAp = sc + 2 * nf;
-    unsigned char* box = static_cast<unsigned char*>(sys->d_cbox.p);
-    const size_t bb = static_cast<size_t>(batch) * stride * sys->esize;
+    double* rr = static_cast<double*>(sys->d_cgs.p);
     cudaStream_t st = sys->stream;
-    for (int64_t f0 = 0; f0 < nf; f0 += batch) {
-        const int nb = static_cast<int>(std::min<int64_t>(batch, nf - f0));
-        ConfLaunch c = conf_launch(sys, f0, nb, a_dev, eps_dev, stride);
-        CUDA_TRY(conf_cg_init(c, g, gprec, r, p, st));
-        CUDA_TRY(conf_dot(c, r, r, rr, st));
+    for (c.f0 = 0; c.f0 < nf; c.f0 += batch) {
+        c.nfn = static_cast<int>(std::min<int64_t>(batch, nf - c.f0));
+        CUDA_TRY(conf_setup(c, st));
+        CUDA_TRY(conf_cg_init(c, g, gprec, r, p, rr, st));
         for (int it = 0; it < iters; ++it) {
             // Ap = P_L (T + Q - eps) P_L p
-            CUDA_TRY(conf_apply(c, p, box, box + bb, box + 2 * bb, Ap, 0, 0, true, nullptr, st));
-            CUDA_TRY(conf_dot(c, p, Ap, pAp, st));
-            CUDA_TRY(conf_cg_step1(c, rr, pAp, p, Ap, gprec, r, st));
-            CUDA_TRY(conf_dot(c, r, r, rr_new, st));
-            CUDA_TRY(conf_cg_step2(c, rr, rr_new, r, p, res ? res + static_cast<int64_t>(it) * nf : nullptr, st));
+            CUDA_TRY(conf_apply(c, p, Ap, 0, nullptr, st));
+            CUDA_TRY(conf_cg_step(c, rr, Ap, gprec, r, p, res ? res + static_cast<int64_t>(it) * nf : nullptr, st));
         }
     }
     return LSW_OK;

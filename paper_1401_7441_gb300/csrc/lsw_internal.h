@@ -24,6 +24,7 @@ constexpr int ZCOLS_F32 = 128;   // (FP32)
 constexpr size_t BWD_STATIC_SMEM = 16 * 1024 + 512;   // upper bound of k_bwd_xy's static shared memory
 constexpr size_t BWD_TC_STATIC_SMEM = 8 * 1024 + 512; // ... of its tensor-core versions (checked at set-up)
 constexpr size_t FWD_STATIC_SMEM = 4 * 1024;          // ... of k_fwd_xy
+constexpr size_t CONF_STATIC_SMEM = 2 * 1024;         // ... of k_conf_pass
 
 // Filter tables, FP64 (rounded once from double-double).
 struct FilterSet {
@@ -293,9 +294,13 @@ cudaError_t foe_ebs(const FoeLaunch& a, const double* K, const double* Ht, const
                     double* out, cudaStream_t s);
 
 // Quartic confinement and preconditioning (lsw_confine.cu): one batch of functions
-// f0 .. f0 + nfn - 1, each on its dense box E = L box widened by 14 (8 types).
+// f0 .. f0 + nfn - 1.  Boxes (FP64, strides s_* in elements per function, x fastest, 8 types
+// each): P on the L box n; A, OZ on [z: output box][y, x: L box]; B, OY on [z, y: output box]
+// [x: L box]; F on the output box m (region 0: the L box; 1: the L' box within the band's reach).
 struct ConfLaunch {
     int prec;
+    int region;                  // output region: 0 L, 1 L'
+    int precond;                 // 1: + T - eps (Eq. precond)
     int64_t f0;
     int nfn;
     const int32_t* sf_atom;
@@ -304,27 +309,49 @@ struct ConfLaunch {
     const int32_t* rowptr;
     const int64_t* off_L;
     const int64_t* off_Lp;
-    const double* qtab;          // per atom: [dim][m = 2, 4][b b'][i over E][l + 14] of X_d^m
+    const double* qtab;          // per atom: [dim][m = 2, 4][b b'][i over the L box widened by 14][l + 14] of X_d^m
     const int64_t* qtab_off;     // first table entry of each atom (n_atoms + 1)
     const double* acoef;         // a_f, the confinement prefactor of each function
     const double* eps;           // eps_f of the preconditioning equation (NULL otherwise)
     double kin[4][KIN_TAPS];     // kinetic blocks hh, hg, gh, gg
     double kin_scale;            // -1 / (2 h^2)
-    int64_t box_stride;          // elements of one function's box (8 types)
+    double *P, *A, *OZ, *B, *OY, *F;
+    double* comb;                // per function [dim][b b'][max_m][29]: a_f X_d^4 (+ kinetic)
+    unsigned char* maps;         // member maps of a batch (ConfMaps)
+    int64_t s_P, s_A, s_B, s_F, s_comb, s_maps;
+    int64_t s_mem, s_xy, s_xz, s_x, s_row, s_oxz;   // bytes of one function's maps
+    int max_n, max_m;            // largest extents of the L and the output boxes
+    int max_lines[3];            // largest number of lines of the passes along x, y, z
     int max_rows_L, max_rows_P;  // largest ny * nz of L and of L' boxes in the batch
-    int64_t max_vol;             // largest E volume in the batch
+    size_t max_smem;             // dynamic shared memory the pass kernels may use
     int* status;
     int64_t qtab_n, seg_n, rowptr_n, vec_n, dst_n;
     int n_sf, n_atoms;
 };
-cudaError_t conf_apply(const ConfLaunch& a, const void* vin, void* box_in, void* box_out, void* box_tmp, void* dst,
-                       int region, int accumulate, bool precond, double* energy, cudaStream_t s);
-cudaError_t conf_cg_init(const ConfLaunch& a, const void* g, void* x, void* r, void* p, cudaStream_t s);
-cudaError_t conf_dot(const ConfLaunch& a, const void* x, const void* y, double* out, cudaStream_t s);
-cudaError_t conf_cg_step1(const ConfLaunch& a, const double* rr, const double* pAp, const void* p, const void* Ap, void* x,
-                          void* r, cudaStream_t s);
-cudaError_t conf_cg_step2(const ConfLaunch& a, double* rr, const double* rr_new, const void* r, void* p, double* res,
-                          cudaStream_t s);
+// Maps of one function of a batch; the two halves of act_* and out_*: coarse, fine members.
+struct ConfMaps {
+    unsigned char *mem, *act_xy, *act_xz, *act_x, *out_row, *out_xz;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ ConfMaps conf_maps(const ConfLaunch& a, int k) {
+    ConfMaps m;
+    m.mem = a.maps + k * a.s_maps;
+    m.act_xy = m.mem + a.s_mem;
+    m.act_xz = m.act_xy + a.s_xy;
+    m.act_x = m.act_xz + a.s_xz;
+    m.out_row = m.act_x + a.s_x;
+    m.out_xz = m.out_row + a.s_row;
+    return m;
+}
+#endif
+cudaError_t configure_confine_kernels(size_t max_smem);
+cudaError_t conf_tables(int n_atoms, const AtomRec* atoms, const double* pos, const double* G, const double* XY, double h,
+                        const int64_t* off, double* tab, cudaStream_t s);
+cudaError_t conf_setup(const ConfLaunch& a, cudaStream_t s);
+cudaError_t conf_apply(const ConfLaunch& a, const void* vin, void* dst, int accumulate, double* energy, cudaStream_t s);
+cudaError_t conf_cg_init(const ConfLaunch& a, const void* g, void* x, void* r, void* p, double* rr, cudaStream_t s);
+cudaError_t conf_cg_step(const ConfLaunch& a, double* rr, const void* Ap, void* x, void* r, void* p, double* res,
+                         cudaStream_t s);
 
 // Fixed device scratch of the allocation-free Hamiltonian entry point (lsw_kernels.cu).
 constexpr size_t NOALLOC_SCRATCH_BYTES = static_cast<size_t>(32) << 20;   // 32 MiB
