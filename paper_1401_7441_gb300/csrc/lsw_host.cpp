@@ -445,19 +445,40 @@ lsw_status build_pattern(lsw_system_s* s) {
 
 int64_t align64(int64_t x) { return (x + ALIGN_ELEMS - 1) / ALIGN_ELEMS * ALIGN_ELEMS; }
 
-// smem bytes of the three pass kernels for a function record (bwd: with the z-arm plane
-// and flag staging; bwd_plain: without)
-void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z, size_t* bwd, size_t* bwd_plain) {
-    const int64_t X = 2 * r.n[0] + 29, Y = 2 * r.n[1] + 29, Z = 2 * r.n[2] + 29;
+// Dynamic shared memory of the pass kernels for a function record.
+void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z) {
+    const int64_t X = 2 * r.n[0] + 29, Z = 2 * r.n[2] + 29;
     const int64_t RS = r.n[0] | 1;
     *fwd = es * static_cast<size_t>(4 * r.n[1] * RS + 2 * r.n[1] * X);
     *z = es * static_cast<size_t>((2 * r.n[2] + Z) * zcols);
-    const int64_t plA = std::max<int64_t>(Y * X, 4LL * r.np[1] * r.np[0]);
-    const int64_t midA = std::max<int64_t>(2LL * r.np[1] * X, 4LL * r.np[1] * r.np[0]);
-    *bwd = es * static_cast<size_t>(plA + midA + 4 * r.n[1] * RS) +
-           static_cast<size_t>((4 * r.n[0] * r.n[1] + 15) / 16 * 16);   // + z-arm column flags
-    *bwd_plain = es * static_cast<size_t>(plA + 2 * r.np[1] * X + 4 * r.n[1] * RS);
 }
+
+// Backward plane kernel: sizes of its four layouts over a batch's functions, and the choice.
+// Two CTAs an SM come first (the kernel is bound by instruction issue: with one, barriers and
+// latencies stay uncovered), then the staged z-arm plane, then the zero pad of the D plane.
+struct BwdSizes {
+    size_t b[2][2] = {{0, 0}, {0, 0}};                 // [gstage][pad]
+    void fold(const FnRec& r, int es) {
+        for (int g = 0; g < 2; ++g)
+            for (int p = 0; p < 2; ++p)
+                b[g][p] = std::max<size_t>(b[g][p], bwd_layout(r.n[0], r.n[1], r.np[0], r.np[1], es,
+                                                               es == 4 ? BWD_NB_F32 : BWD_NB_F64, g != 0, p != 0)
+                                                        .bytes);
+    }
+    bool choose(size_t max_smem, HphiLaunch* p) const {
+        // an SM holds the largest CTA's shared memory and 1 KiB reserved per CTA
+        const size_t half = (max_smem + 1024) / 2 - 1024 - BWD_STATIC_SMEM, all = max_smem - BWD_STATIC_SMEM;
+        const struct { int g, p; size_t lim; } order[] = {{1, 1, half}, {0, 1, half}, {1, 1, all}, {0, 1, all}, {0, 0, all}};
+        for (const auto& o : order)
+            if (b[o.g][o.p] <= o.lim) {
+                p->gstage = o.g;
+                p->dpad = o.p;
+                p->smem_bwd = b[o.g][o.p];
+                return true;
+            }
+        return false;
+    }
+};
 
 // Dynamic shared memory of the tensor-core z stage for a function record and `parts`
 // bfloat16 parts (mirror of the layout in k_z_tc: 512-byte header, data operand parts
@@ -518,7 +539,7 @@ lsw_status build_plans(lsw_system_s* s) {
     }
     s->batches.clear();
     int64_t ws_max = 0;
-    std::vector<int32_t> items;          // plane items of every batch
+    std::vector<int2> items;             // plane items of every batch
     std::vector<int64_t> item_off;       // per batch: first item, -1 without items
     // option "hphi_limit": H phi only for functions 0 .. limit - 1 (a rank of a sharded
     // run computes its own functions, which its sub-system numbers first)
@@ -533,7 +554,7 @@ lsw_status build_plans(lsw_system_s* s) {
         p.nfn = static_cast<int>(b.nfn);
         p.zcols = zcols;
         p.fwd_list = s->fwd_list;
-        size_t smem_bwd_plain = 0;
+        BwdSizes bwd;
         int64_t o = 0;
         for (int64_t f = f0; f < f0 + b.nfn; ++f) {
             recs[f].ws_D = o;
@@ -567,13 +588,12 @@ lsw_status build_plans(lsw_system_s* s) {
             p.max_rowsL = std::max(p.max_rowsL, r.n[1] * r.n[2]);
             p.max_segL = std::max<int>(p.max_segL, static_cast<int>((Lh.c.keys.size() + Lh.f.keys.size()) / 3));
             p.max_segP = std::max<int>(p.max_segP, static_cast<int>((Ph.c.keys.size() + Ph.f.keys.size()) / 3));
-            size_t a1, a2, a3, a4;
-            pass_smem(r, s->esize, zcols, &a1, &a2, &a3, &a4);
+            size_t a1, a2;
+            pass_smem(r, s->esize, zcols, &a1, &a2);
             p.smem_fwd = std::max(p.smem_fwd, a1);
             p.smem_z = std::max(p.smem_z, a2);
             p.smem_kin = std::max(p.smem_kin, static_cast<size_t>(2 * r.n[2] * 128) * (p.prec == 0 ? 8 : 4));
-            p.smem_bwd = std::max(p.smem_bwd, a3);
-            smem_bwd_plain = std::max(smem_bwd_plain, a4);
+            bwd.fold(r, static_cast<int>(s->esize));
             if (s->zsplit) {
                 if (!ztc_fits(r))
                     return fail(LSW_ERR_UNSUPPORTED, "locreg extents too large for the tensor-core kernels");
@@ -586,29 +606,31 @@ lsw_status build_plans(lsw_system_s* s) {
                 }
             }
         }
-        // stage the z-arm plane and flags when they fit beside the plane kernel's tiles
-        p.gstage = p.smem_bwd + BWD_STATIC_SMEM <= s->ctx->max_smem ? 1 : 0;
-        if (!p.gstage) p.smem_bwd = smem_bwd_plain;
         p.zsplit = s->zsplit;
         p.xy_tc = s->zsplit ? s->xy_tc : 0;
-        if (p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || p.smem_z > s->ctx->max_smem || p.smem_bwd + BWD_STATIC_SMEM > s->ctx->max_smem ||
+        if (!bwd.choose(s->ctx->max_smem, &p) || p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || p.smem_z > s->ctx->max_smem ||
             p.smem_ztc > s->ctx->max_smem || p.smem_kin > s->ctx->max_smem || p.smem_bwd_tc + BWD_TC_STATIC_SMEM > s->ctx->max_smem ||
             p.smem_fwd_tc > s->ctx->max_smem)
             return fail(LSW_ERR_UNSUPPORTED, "locreg box too large for the on-chip pass tiles (%zu/%zu/%zu/%zu > %zu bytes)",
-                        p.smem_fwd, p.smem_z, p.smem_bwd, p.smem_ztc, s->ctx->max_smem);
-        // persistent FMA plane kernels: the batch's (function, plane, z type) items, largest
-        // planes first (stable in function and plane order), and as many CTAs as fit
+                        p.smem_fwd, p.smem_z, bwd.b[0][0], p.smem_ztc, s->ctx->max_smem);
+        // persistent FMA plane kernels: the batch's (functions, plane, z type) items, largest
+        // first (stable in function and plane order), and as many CTAs as fit.  The backward
+        // kernel's items take an atom's functions together (their tables are built once), as
+        // many as leave eight items for every CTA (with fewer the last wave is uneven).
         if (s->persistent && !(p.zsplit && p.xy_tc) && p.max_nzp < 1024 && p.max_nz < 1024) {
-            auto add = [&](int which) {
-                std::vector<std::pair<int64_t, int32_t>> it;
-                for (int64_t f = f0; f < f0 + b.nfn; ++f) {
+            auto add = [&](int which, int cap) {
+                std::vector<std::pair<int64_t, int2>> it;
+                for (int64_t f = f0; f < f0 + b.nfn;) {
                     const FnRec& r = recs[f];
+                    int cnt = 1;
+                    while (cnt < cap && f + cnt < f0 + b.nfn && recs[f + cnt].atom == r.atom) ++cnt;
                     const int64_t X = 2 * r.n[0] + 29, Y = 2 * r.n[1] + 29;
                     const int planes = which == 0 ? r.n[2] : r.np[2];
                     const int64_t cost = which == 0 ? X * Y : X * Y + static_cast<int64_t>(r.np[0]) * r.np[1];
                     for (int z = 0; z < planes; ++z)
                         for (int bz = 0; bz < 2; ++bz)
-                            it.emplace_back(-cost, static_cast<int32_t>(((f - f0) << 11) | (z << 1) | bz));
+                            it.emplace_back(-cost * cnt, make_int2(static_cast<int>(f - f0), (cnt << 11) | (z << 1) | bz));
+                    f += cnt;
                 }
                 std::stable_sort(it.begin(), it.end(),
                                  [](const auto& u, const auto& v) { return u.first < v.first; });
@@ -616,10 +638,13 @@ lsw_status build_plans(lsw_system_s* s) {
                 return static_cast<int>(it.size());
             };
             int bf = 0, bb = 0;
-            CUDA_TRY(plane_kernel_blocks(p.prec, p.smem_fwd, p.smem_bwd, &bf, &bb));
+            CUDA_TRY(plane_kernel_blocks(p.prec, p.smem_fwd, p.smem_bwd, p.dpad, &bf, &bb));
             item_off.push_back(static_cast<int64_t>(items.size()));
-            p.n_items_fwd = (s->persistent & 2) ? add(0) : 0;
-            p.n_items_bwd = (s->persistent & 1) ? add(1) : 0;
+            p.n_items_fwd = (s->persistent & 2) ? add(0, 1) : 0;
+            int64_t planes = 0;
+            for (int64_t f = f0; f < f0 + b.nfn; ++f) planes += 2LL * recs[f].np[2];
+            const int64_t fill = 8LL * std::max(1, bb) * s->ctx->n_sm;
+            p.n_items_bwd = (s->persistent & 1) ? add(1, static_cast<int>(std::min<int64_t>(64, std::max<int64_t>(1, planes / fill)))) : 0;
             p.grid_fwd = std::max(1, std::min(p.n_items_fwd, std::max(1, bf) * s->ctx->n_sm));
             p.grid_bwd = std::max(1, std::min(p.n_items_bwd, std::max(1, bb) * s->ctx->n_sm));
         } else {
@@ -638,7 +663,7 @@ lsw_status build_plans(lsw_system_s* s) {
     for (size_t i = 0; i < s->batches.size(); ++i) {
         HphiLaunch& p = s->batches[i].proto;
         if (item_off[i] < 0) continue;
-        const int32_t* it = static_cast<const int32_t*>(s->d_plane_items.p) + item_off[i];
+        const int2* it = static_cast<const int2*>(s->d_plane_items.p) + item_off[i];
         p.items_fwd = p.n_items_fwd ? it : nullptr;
         p.items_bwd = p.n_items_bwd ? it + p.n_items_fwd : nullptr;
         p.queue = static_cast<int*>(s->d_queue.p);
@@ -1319,7 +1344,7 @@ FnRec noalloc_record(const lsw_system_s* s, int64_t f) {
     return r;
 }
 // Fold one function into a batch's launch extents and shared-memory sizes.
-void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* p, size_t* smem_bwd_plain) {
+void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* p, BwdSizes* bwd) {
     const LocregHost& Lh = s->L[r.atom];
     const LocregHost& Ph = s->Lp[r.atom];
     p->max_nz = std::max(p->max_nz, r.n[2]);
@@ -1332,13 +1357,12 @@ void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* 
     p->max_rowsL = std::max(p->max_rowsL, r.n[1] * r.n[2]);
     p->max_segL = std::max<int>(p->max_segL, static_cast<int>((Lh.c.keys.size() + Lh.f.keys.size()) / 3));
     p->max_segP = std::max<int>(p->max_segP, static_cast<int>((Ph.c.keys.size() + Ph.f.keys.size()) / 3));
-    size_t a1, a2, a3, a4;
-    pass_smem(r, s->esize, zcols, &a1, &a2, &a3, &a4);
+    size_t a1, a2;
+    pass_smem(r, s->esize, zcols, &a1, &a2);
     p->smem_fwd = std::max(p->smem_fwd, a1);
     p->smem_z = std::max(p->smem_z, a2);
     p->smem_kin = std::max(p->smem_kin, static_cast<size_t>(2 * r.n[2] * 128) * (p->prec == 0 ? 8 : 4));
-    p->smem_bwd = std::max(p->smem_bwd, a3);
-    *smem_bwd_plain = std::max(*smem_bwd_plain, a4);
+    bwd->fold(r, static_cast<int>(s->esize));
     if (s->zsplit) {
         p->smem_ztc = std::max(p->smem_ztc, ztc_smem(r, s->zsplit));
         if (s->xy_tc) {
@@ -1347,12 +1371,11 @@ void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* 
         }
     }
 }
-// Choose the plane kernel's staging and check the tiles against the shared memory.
-bool noalloc_finish(const lsw_system_s* s, HphiLaunch* p, size_t smem_bwd_plain) {
+// Choose the backward plane kernel's layout and check the tiles against the shared memory.
+bool noalloc_finish(const lsw_system_s* s, HphiLaunch* p, const BwdSizes& bwd) {
     const size_t mx = s->ctx->max_smem;
-    p->gstage = p->smem_bwd + BWD_STATIC_SMEM <= mx ? 1 : 0;
-    if (!p->gstage) p->smem_bwd = smem_bwd_plain;
-    return !(p->smem_fwd + FWD_STATIC_SMEM > mx || p->smem_z > mx || p->smem_bwd + BWD_STATIC_SMEM > mx || p->smem_ztc > mx ||
+    return bwd.choose(mx, p) &&
+           !(p->smem_fwd + FWD_STATIC_SMEM > mx || p->smem_z > mx || p->smem_ztc > mx ||
              p->smem_kin > mx || p->smem_bwd_tc + BWD_TC_STATIC_SMEM > mx || p->smem_fwd_tc > mx);
 }
 }  // namespace
@@ -2122,9 +2145,9 @@ lsw_status lsw_apply_hamiltonian_noalloc(lsw_system sys, const void* phi, void* 
         HphiLaunch p;
         std::memset(&p, 0, sizeof(p));
         p.prec = sys->prec;
-        size_t plain = 0;
-        noalloc_fold(sys, r, zcols, &p, &plain);
-        if (!noalloc_finish(sys, &p, plain))
+        BwdSizes bwd;
+        noalloc_fold(sys, r, zcols, &p, &bwd);
+        if (!noalloc_finish(sys, &p, bwd))
             return fail(LSW_ERR_UNSUPPORTED, "locreg box too large for the on-chip pass tiles");
     }
     CUDA_TRY(cudaSetDevice(sys->ctx->device));
@@ -2143,7 +2166,7 @@ lsw_status lsw_apply_hamiltonian_noalloc(lsw_system sys, const void* phi, void* 
         std::memset(&p, 0, sizeof(p));
         p.prec = sys->prec;
         p.zcols = zcols;
-        size_t smem_bwd_plain = 0;
+        BwdSizes bwd;
         int nb = 0;
         int64_t need = 0;
         while (f + nb < nf && nb < NOALLOC_MAX_BATCH) {
@@ -2153,10 +2176,10 @@ lsw_status lsw_apply_hamiltonian_noalloc(lsw_system sys, const void* phi, void* 
             if (need + sD + sR > cap) break;
             need += sD + sR;
             p.ws_D_elems += sD;
-            noalloc_fold(sys, r, zcols, &p, &smem_bwd_plain);
+            noalloc_fold(sys, r, zcols, &p, &bwd);
             ++nb;
         }
-        if (nb == 0 || !noalloc_finish(sys, &p, smem_bwd_plain))   // excluded by the checks above
+        if (nb == 0 || !noalloc_finish(sys, &p, bwd))   // excluded by the checks above
             return fail(LSW_ERR_STATE, "lsw_apply_hamiltonian_noalloc: inconsistent batch plan");
         p.nfn = nb;
         p.zsplit = sys->zsplit;

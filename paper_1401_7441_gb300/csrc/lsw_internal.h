@@ -21,7 +21,7 @@ constexpr int V_REACH = 14;      // real-space box of a coarse block [lo, hi]: [
 constexpr int ALIGN_ELEMS = 64;  // function offsets in the compressed arrays
 constexpr int ZCOLS_F64 = 64;    // real-space columns per block of the z stage (FP64)
 constexpr int ZCOLS_F32 = 128;   // (FP32)
-constexpr size_t BWD_STATIC_SMEM = 16 * 1024 + 512;   // upper bound of k_bwd_xy's static shared memory
+constexpr size_t BWD_STATIC_SMEM = 256;               // upper bound of k_bwd_xy's static shared memory
 constexpr size_t BWD_TC_STATIC_SMEM = 8 * 1024 + 512; // ... of its tensor-core versions (checked at set-up)
 constexpr size_t FWD_STATIC_SMEM = 4 * 1024;          // ... of k_fwd_xy
 constexpr size_t CONF_STATIC_SMEM = 2 * 1024;         // ... of k_conf_pass
@@ -125,6 +125,44 @@ struct PanelSlab {
     size_t smem_pack;            // dynamic shared memory of the pack kernel (0: tables read from global)
 };
 
+// Dynamic shared memory of the FMA backward plane kernel for L extents (nx, ny), L' extents
+// (nxp, nyp), element size es and nb outputs per block: byte offsets and sizes.  gstage: room
+// for the z-arm plane; pad: zeros around the D plane.
+#ifdef __CUDACC__
+#define LSW_HD __host__ __device__ __forceinline__
+#else
+#define LSW_HD inline
+#endif
+constexpr int BWD_NB_F32 = 8, BWD_NB_F64 = 4;   // outputs per block
+struct BwdLayout {
+    int RS;                      // row stride of the D plane (odd: rows land in different banks)
+    int nb_y, nb_x;              // blocks of rows and of columns (upper bounds)
+    int taskN, memN;             // x pass tasks, fine members listed
+    uint32_t o_pl, o_mid, o_D, o_task, o_roff, o_blk, o_row, o_mem, bytes;
+};
+LSW_HD BwdLayout bwd_layout(int nx, int ny, int nxp, int nyp, int es, int nb, bool gstage, bool pad) {
+    BwdLayout L;
+    const int X = 2 * nx + 29, Y = 2 * ny + 29;
+    auto up = [](uint32_t v) { return (v + 15u) & ~15u; };
+    auto mx = [](int u, int v) { return u > v ? u : v; };
+    L.RS = pad ? (nx + 1) | 1 : nx | 1;
+    L.nb_y = (nyp + nb - 1) / nb + 1;
+    L.nb_x = (nxp + nb - 1) / nb;
+    L.taskN = 2 * L.nb_x * nyp;
+    L.memN = nxp * nyp / 2 + 8;
+    L.o_pl = 16;                                       // the mbarrier first
+    L.o_mid = up(L.o_pl + static_cast<uint32_t>(es) * mx(Y * X + 8, 4 * nyp * nxp));
+    const int slot = (nyp * nxp + 15) & ~7;
+    L.o_D = up(L.o_mid + static_cast<uint32_t>(es) * (gstage ? mx(2 * nyp * X, 4 * slot) : 2 * nyp * X));
+    L.o_task = up(L.o_D + static_cast<uint32_t>(es) * (4 * ny * L.RS + (pad ? L.RS + 1 : 0)));
+    L.o_roff = L.o_task + 4u * L.taskN;
+    L.o_blk = L.o_roff + 4u * nyp;
+    L.o_row = L.o_blk + 4u * (3 * L.nb_y + 1 + 6 * L.nb_y + 1 + 6 * L.nb_x + 1);
+    L.o_mem = L.o_row + 2u * (4 * nyp + 4 * ny + 4 * nx);
+    L.bytes = up(L.o_mem + 2u * L.memN);
+    return L;
+}
+
 // Kernel kinds of the per-launch device trace (lsw_profile / lsw_profile_read).
 enum TraceKind : int {
     TK_MEMSET = 0, TK_UNCOMPRESS, TK_FWD_XY, TK_Z, TK_BWD_XY, TK_KINETIC, TK_PACK, TK_HS,
@@ -151,9 +189,9 @@ struct HphiLaunch {
     int max_segL;                // largest coarse+fine segment count of L
     int max_segP;
     size_t smem_fwd, smem_z, smem_bwd;
-    int gstage;                  // 1: the plane kernel stages the z-arm plane and column flags
-                                 // in shared memory (smem_bwd includes them); 0: reads them
-                                 // from global memory (the boxes leave no room)
+    int gstage;                  // 1: the backward plane kernel stages the z-arm plane in shared
+                                 // memory (smem_bwd includes it); 0: reads it from global memory
+    int dpad;                    // 1: its D plane is padded with zeros
     int zcols;                   // columns per CTA of the z stage
     int zsplit;                  // 0: z stage on FMA units; 2 or 3: bfloat16 parts per
                                  // FP32 operand of the tensor-core z stage
@@ -163,12 +201,12 @@ struct HphiLaunch {
     size_t smem_bwd_tc;          // dynamic shared memory of the tensor-core plane kernel
     size_t smem_fwd_tc;          // dynamic shared memory of the tensor-core forward plane kernel
     size_t smem_kin;             // dynamic shared memory of the kinetic z-arm kernel
-    // persistent FMA plane kernels: the batch's items (function << 11 | plane << 1 | z type),
-    // largest planes first, taken from queue[0] (forward) and queue[1] (backward), which
+    // persistent FMA plane kernels: the batch's items (first function, functions << 11 |
+    // plane << 1 | z type; the forward kernel's hold one function), largest first, taken from queue[0] (forward) and queue[1] (backward), which
     // are zeroed before the batch; grid_* CTAs (as many as fit on the GPU).  NULL items:
     // one CTA per (2 planes + z type, function) grid slot.
-    const int32_t* items_fwd;
-    const int32_t* items_bwd;
+    const int2* items_fwd;
+    const int2* items_bwd;
     int n_items_fwd, n_items_bwd;
     int grid_fwd, grid_bwd;
     int* queue;
@@ -387,7 +425,7 @@ cudaError_t upload_filters(const FilterSet& fs, int device);
 cudaError_t measure_peaks(int n_sm, double* fp32_tflops, double* fp64_tflops, double* copy_gbs);
 cudaError_t configure_kernels(size_t max_smem);
 // Resident CTAs per SM of the FMA plane kernels at these dynamic shared-memory sizes.
-cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int* fwd, int* bwd);
+cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int dpad, int* fwd, int* bwd);
 cudaError_t enqueue_hphi_batch(const HphiLaunch& a, cudaStream_t s);
 cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s);     // panels of a slab (lsw_panels.cu)
 cudaError_t enqueue_panel_hs(const PanelHSLaunch& a, cudaStream_t s);   // S, H from the panels

@@ -94,6 +94,20 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait_group() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+
+// Bulk copy global -> shared (both 16-byte aligned, a multiple of 16 bytes) signalled on an
+// mbarrier with one arrival: bulk_fence orders earlier shared accesses of the block (behind a
+// barrier) before the copy, bulk_expect arrives and announces the bytes.
+__device__ __forceinline__ void bulk_fence() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
+__device__ __forceinline__ void bulk_expect(uint32_t mbar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
+
 // ---------------------------------------------------------------- uncompress / compress
 
 template <class T>
@@ -166,12 +180,9 @@ constexpr int KW = BB + 2 * KIN_HALF; // kinetic window
 #ifndef LSW_Z_NB
 #define LSW_Z_NB 4                    // outputs per backward block in the z stage (FP32)
 #endif
-#ifndef LSW_BWD_NB
-#define LSW_BWD_NB 8                  // outputs per backward block in the plane kernel (FP32)
-#endif
 template <class T, int Stage>         // Stage 0: z stage, 1: backward plane kernel
 struct Blk {                          // outputs per backward (decimating) block
-    static constexpr int NB = sizeof(T) == 4 ? (Stage == 0 ? LSW_Z_NB : LSW_BWD_NB) : 4;
+    static constexpr int NB = sizeof(T) == 4 ? (Stage == 0 ? LSW_Z_NB : BWD_NB_F32) : BWD_NB_F64;
     static constexpr int W = 2 * NB + 29;
 };
 template <class T>
@@ -512,8 +523,8 @@ __global__ void __launch_bounds__(256) k_fwd_xy(HphiLaunch a) {
         for (;;) {
             const int k = next_item(a.queue, &s_item);
             if (k >= a.n_items_fwd) break;
-            const int code = LD(a.items_fwd, k, a.n_items_fwd);
-            fwd_plane<T>(a, code >> 11, (code >> 1) & 1023, code & 1);
+            const int2 it = LD(a.items_fwd, k, a.n_items_fwd);
+            fwd_plane<T>(a, it.x, (it.y >> 1) & 1023, it.y & 1);
             __syncthreads();   // shared memory and s_item are reused by the next item
         }
     } else {
@@ -1119,10 +1130,7 @@ __global__ void __launch_bounds__(128) k_kin_z(HphiLaunch a) {
 // pairs whose input rows or columns of D are all zero (wavelet types off the fine
 // region) are skipped.  Each phase first lists its tasks in shared memory, so skipped
 // work frees whole rounds.
-constexpr int BWD_MAX_TASKS = 2048;
-#ifndef LSW_BWD_MIN_BLOCKS
-#define LSW_BWD_MIN_BLOCKS 2      // resident blocks per SM the FP32 version is compiled for
-#endif
+constexpr int BWD_MAX_TASKS = 2048;   // of the tensor-core version
 
 // Potential part of the backward plane kernel on the tensor cores (the two products
 // described at k_bwd_xy): builds the filter operands Fy (128 x K1) and Fx (N2 x K2) and
@@ -1240,30 +1248,27 @@ __device__ bool bwd_tc_potential(const float* Bb, [[maybe_unused]] int64_t bb_ro
     return true;
 }
 
-// NS = 0: the transposed y and x filters run on the FMA units (256 threads, several
-// blocks per SM).  NS = 2, 3 (FP32 only): they run as two band-Toeplitz tensor-core
-// products per plane with split-bfloat16 operands (NS parts) and FP32 accumulation in
-// tensor memory, as in k_z_tc (512 threads, one block per SM):
+// Split-bfloat16 systems, option "xy_tc": the transposed y and x filters as two band-Toeplitz
+// tensor-core products per plane with split-bfloat16 operands (NS = 2 or 3 parts) and FP32
+// accumulation in tensor memory, as in k_z_tc (512 threads, one block per SM):
 //   M1[j][x'] = sum_y' Fy[j][y'] P[y'][x'],   j = by n_y' + b,  Fy[j][y'] = F_by[y' - 2(b + dy)]
 //   Q[j][i]   = sum_x' M1[j][x'] Fx[i][x'],   i = bx n_x' + b2, Fx[i][x'] = F_bx[x' - 2(b2 + dx)]
 // with P the plane of Bb; thread (warp w, lane l) owns row j = 32 (w mod 4) + l of both
 // products and quarter w / 4 of each K or N range.
-template <class T, int NS>
-__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, int bz) {
+template <int NS>
+__device__ __forceinline__ void bwd_plane_tc(const HphiLaunch& a, int fl, int zb, int bz) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
+    using T = float;
     int* st = a.status;
-    constexpr int NB = Blk<T, 1>::NB;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int16_t rx0[256], rx1[256];         // member x range per row (L' plane), -1: none
     __shared__ int roff[256];                      // coefficient offset of the row's coarse segment
     __shared__ int fr0[256], fr1[256];             // fine segment range of the row (L' keys)
     __shared__ int16_t fx0[256], fx1[256];         // hull of the row's fine members, -1: none
-    __shared__ int cq0[64], cq1[64], pq[65];       // y pass, per block of NB rows: column range, prefix
     __shared__ int rq0[128], rq1[128], rqp[129];   // kinetic y arm, per (x type, block of BB rows): the same
-    __shared__ int ntask, ntask2, ylo, yhi;
+    __shared__ int ntask2, ylo, yhi;
     __shared__ unsigned char rowf[4][128], colf[4][128];   // D plane: nonzero per (type, row / column)
-    T* sm = reinterpret_cast<T*>(smem_raw);
     const FnRec r = a.fn[fl];
     if (zb >= r.np[2]) return;
     const AtomRec& at = a.atoms[r.atom];
@@ -1272,9 +1277,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     const int nxp = r.np[0], nyp = r.np[1], nzp = r.np[2];
     const int dx = r.lop[0] - r.lo[0], dy = r.lop[1] - r.lo[1], dz = r.lop[2] - r.lo[2];
     const int RS = nx | 1;
-    const int plA = max(Y * X, 4 * nyp * nxp);
-    // FMA layout: pl [Y][X] (later Gs [4][nyp][nxp]), mid [2][nyp][X], Dp [4][ny][RS]
-    // tensor-core layout: header, Fy parts, Fx parts, a region holding the P operand, then
+    // layout: header, Fy parts, Fx parts, a region holding the P operand, then
     // the M1 operand, then Gs; Dp
     const int K1 = (Y + 15) & ~15, N1 = (X + 15) & ~15, K2 = N1, N2 = (2 * nxp + 15) & ~15;
     const int FY_PART = 128 * K1 * 2, FX_PART = N2 * K2 * 2, P_PART = N1 * K1 * 2, M_PART = 128 * K2 * 2;
@@ -1282,25 +1285,14 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     unsigned char* sFy = smem_raw + tc::HEAD;
     unsigned char* sFx = sFy + NS * FY_PART;
     unsigned char* sXr = sFx + NS * FX_PART;
-    // task lists of the x pass and the kinetic x arm, later the plane's fine segments for
-    // the compressed write: static shared memory in the FMA version; in the tensor-core
-    // version the filter operands' region, dead once the potential part is done
+    // task list of the kinetic x arm, later the plane's fine segments for the compressed
+    // write: the filter operands' region, dead once the potential part is done
     // (NS * FY_PART >= 2 * 128 * 16 * 2 bytes = BWD_MAX_TASKS ints; 16-byte aligned)
-    int* task;
-    if constexpr (NS == 0) {
-        __shared__ __align__(16) int task_s[BWD_MAX_TASKS];
-        task = task_s;
-    } else {
-        task = reinterpret_cast<int*>(sFy);
-    }
-    T* pl = sm;
-    T* Gs = NS ? reinterpret_cast<T*>(sXr) : sm;
-    // mid [2][nyp][X], later (when the host found room: a.gstage) the z-arm plane
-    const int midA = (NS == 0 && a.gstage) ? max(2 * nyp * X, 4 * nyp * nxp) : 2 * nyp * X;
-    T* mid = sm + plA;
-    T* Dp = NS ? reinterpret_cast<T*>(sXr + XR) : mid + midA;
-    const int64_t smem_n = static_cast<int64_t>((NS ? a.smem_bwd_tc : a.smem_bwd) / sizeof(T));
-    if constexpr (NS > 0) {
+    int* task = reinterpret_cast<int*>(sFy);
+    T* Gs = reinterpret_cast<T*>(sXr);
+    T* Dp = reinterpret_cast<T*>(sXr + XR);
+    const int64_t smem_n = static_cast<int64_t>(a.smem_bwd_tc / sizeof(T));
+    {
         if ((threadIdx.x >> 5) == 0) tc::tmem_alloc(tc::saddr(smem_raw + 8), 128);
         if (threadIdx.x == 32) tc::mbar_init(tc::saddr(smem_raw));
         float* taps = reinterpret_cast<float*>(smem_raw + 16);
@@ -1320,13 +1312,10 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
         colf[i >> 7][i & 127] = 0;
     }
     __syncthreads();
-    // staging copies first (they fly while the row records below are read): group 1 the
-    // Bb plane, group 2 the D plane and the z-arm column flags
+    // staging copies first (they fly while the row records below are read): the D plane and
+    // the z-arm column flags
     const T* Bb = static_cast<const T*>(a.ws) + r.ws_Bb + (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
     const int64_t bb_room = 2LL * nzp * Y * X - (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
-    if constexpr (NS == 0)
-        for (int i = threadIdx.x; i < Y * X; i += blockDim.x) CPA(pl, i, smem_n, Bb, i, bb_room);
-    cp_commit();
     const T* D = static_cast<const T*>(a.ws) + r.ws_D;
     const int64_t plane = static_cast<int64_t>(nx) * ny * nz;
     const int pn = nx * ny;
@@ -1340,15 +1329,12 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
                 8 * plane);
         }
     }
-    // z-arm column flags of the L box (written by k_kin_z): staged, 4 bytes per copy, when
-    // the host found room (a.gstage), else read from global memory
+    // z-arm column flags of the L box (written by k_kin_z)
     const uint32_t* gsrc = reinterpret_cast<const uint32_t*>(static_cast<const T*>(a.ws) + r.ws_Gf);
     uint32_t* gfl = reinterpret_cast<uint32_t*>(Dp + 4 * ny * RS);
     [[maybe_unused]] const int64_t gfl_n = (smem_n * static_cast<int64_t>(sizeof(T)) -
                                             (reinterpret_cast<unsigned char*>(gfl) - smem_raw)) / 4;
-    if (a.gstage)
-        for (int i = threadIdx.x; i < pn; i += blockDim.x) CPA(gfl, i, gfl_n, gsrc, i, pn);
-    cp_commit();
+    for (int i = threadIdx.x; i < pn; i += blockDim.x) CPA(gfl, i, gfl_n, gsrc, i, pn);
     // member x range of each row of this plane (coarse part of L')
     for (int y = threadIdx.x; y < nyp; y += blockDim.x) {
         const int64_t row = at.rowPc + y + static_cast<int64_t>(nyp) * zb;
@@ -1372,10 +1358,8 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
         fx0[y] = static_cast<int16_t>(q1 > q0 ? LD(a.seg, at.segPf + q0, a.seg_n).x0 : -1);
         fx1[y] = static_cast<int16_t>(q1 > q0 ? LD(a.seg, at.segPf + q1 - 1, a.seg_n).x1 : -1);
     }
-    cp_wait_group<1>();   // the Bb plane (group 2 may still be in flight)
-    if (threadIdx.x == 0) ntask = ntask2 = 0;
+    if (threadIdx.x == 0) ntask2 = 0;
     __syncthreads();
-    const int64_t mid_n = 2LL * nyp * X;
     const int64_t gs_n = 4LL * nyp * nxp;
     const T ks = static_cast<T>(a.kin_scale);
     T ekin_t = 0;
@@ -1393,29 +1377,11 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
             hi = fx1[b];
         }
     };
-    // ---- column ranges per row block, with their prefix sums, in one phase: the y pass's
-    //      (FMA version; blocks of NB rows: for row b and pair by its blocks k = lo/NB ..
-    //      hi/NB of the needed range read x' in [2 (k NB + dx), 2 (k NB + NB - 1 + dx) + 30])
-    //      and the kinetic y arm's (per x type bx, the pair of types bx, bx + 2, and block
-    //      of BB rows: the hull of the rows' needed ranges, the coarse members where the
-    //      pair holds type 0, else the fine members)
-    const int nbb = (yhi_ - ylo_ + NB) / NB;
+    // ---- column ranges of the kinetic y arm per x type bx (the pair of types bx, bx + 2) and
+    //      block of BB rows, with their prefix sums: the hull of the rows' needed ranges, the
+    //      coarse members where the pair holds type 0, else the fine members
     const int nbyk = (yhi_ - ylo_ + BB) / BB;
     if (yhi_ >= 0) {
-        if (NS == 0 && static_cast<int>(threadIdx.x) < nbb) {
-            const int q = threadIdx.x;
-            int c0 = X, c1 = -1;
-            for (int b = ylo_ + q * NB; b < min(ylo_ + (q + 1) * NB, yhi_ + 1); ++b)
-                for (int by = 0; by < 2; ++by) {
-                    int lo, hi;
-                    need(by, b, lo, hi);
-                    if (lo < 0) continue;
-                    c0 = min(c0, 2 * ((lo / NB) * NB + dx));
-                    c1 = max(c1, 2 * ((hi / NB) * NB + NB - 1 + dx) + 30);
-                }
-            cq0[q] = max(c0, 0);
-            cq1[q] = min(c1, X - 1);
-        }
         const int t2 = static_cast<int>(threadIdx.x) - 128;
         if (t2 >= 0 && t2 < 2 * nbyk) {
             const int bx = t2 >= nbyk, q = t2 - bx * nbyk;
@@ -1431,17 +1397,13 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
             rq1[t2] = c1;
         }
         __syncthreads();
-        if (NS == 0 && threadIdx.x == 0) {
-            pq[0] = 0;
-            for (int q = 0; q < nbb; ++q) pq[q + 1] = pq[q] + max(0, cq1[q] - cq0[q] + 1);
-        }
         if (threadIdx.x == 32) {
             rqp[0] = 0;
             for (int i = 0; i < 2 * nbyk; ++i) rqp[i + 1] = rqp[i] + max(0, rq1[i] - rq0[i] + 1);
         }
         __syncthreads();
     }
-    if constexpr (NS > 0) {
+    {
         // ---- potential part on the tensor cores -> Gs (every row and column of the plane)
         if (yhi_ >= 0 && !bwd_tc_potential<NS>(reinterpret_cast<const float*>(Bb), bb_room, X, Y, nyp, nxp, dx, dy,
                                                 K1, N1, K2, N2, FY_PART, FX_PART, XR, sFy, sFx, sXr,
@@ -1450,62 +1412,6 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
         }
     }
     if (yhi_ >= 0) {
-      if constexpr (NS == 0) {
-        // ---- y pass: blocks of NB rows b within [ylo, yhi], per block only the columns
-        //      listed above
-        {
-            const int ntk = pq[nbb];
-            for (int tk = threadIdx.x; tk < ntk; tk += blockDim.x) {
-                int q = 0;
-                while (tk >= pq[q + 1]) ++q;
-                const int xo = cq0[q] + (tk - pq[q]), b0 = ylo_ + q * NB;
-                T w[2 * NB + 29], s[NB], d[NB];
-                swin(w, pl, xo, X, 2 * (b0 + dy), Y, smem_n, st);
-                bwd_block<T, NB>(w, s, d);
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int b = b0 + j;
-                    if (b <= yhi_) {
-                        ST(mid, static_cast<int64_t>(b) * X + xo, mid_n, s[j]);
-                        ST(mid, static_cast<int64_t>(nyp + b) * X + xo, mid_n, d[j]);
-                    }
-                }
-            }
-        }
-        __syncthreads();   // pl is dead from here on: Gs reuses it
-        // ---- task list: (by, row b, x block of NB) intersecting the row's needed range
-        for (int b = ylo_ + threadIdx.x; b <= yhi_; b += blockDim.x) {
-            for (int by = 0; by < 2; ++by) {
-                int lo, hi;
-                need(by, b, lo, hi);
-                if (lo < 0) continue;
-                const int k0 = lo / NB, k1 = hi / NB;
-                const int base = atomicAdd(&ntask, k1 - k0 + 1);
-                for (int k = k0; k <= k1; ++k)
-                    if (base + k - k0 < BWD_MAX_TASKS) task[base + k - k0] = (by << 24) | (b << 12) | k;
-            }
-        }
-        __syncthreads();
-        int nt = min(ntask, BWD_MAX_TASKS);
-        if (ntask > BWD_MAX_TASKS && threadIdx.x == 0) atomicOr(a.status, ST_BAD_BOX);
-        // ---- x pass (transposed filters) on the listed row blocks
-        for (int it = threadIdx.x; it < nt; it += blockDim.x) {
-            const int code = task[it];
-            const int by = code >> 24, b = (code >> 12) & 4095, x0 = (code & 4095) * NB;
-            const int row = by * nyp + b;
-            T w[2 * NB + 29], s[NB], d[NB];
-            swin(w, mid, row * X, 1, 2 * (x0 + dx), X, mid_n, st);
-            bwd_block<T, NB>(w, s, d);
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                const int xb = x0 + j;
-                if (xb < nxp) {
-                    ST(Gs, ((0 + 2 * by) * nyp + b) * nxp + xb, gs_n, s[j]);
-                    ST(Gs, ((1 + 2 * by) * nyp + b) * nxp + xb, gs_n, d[j]);
-                }
-            }
-        }
-      }
         // the D plane and the flags have landed (their copies flew during the passes above)
         cp_wait();
         __syncthreads();
@@ -1519,18 +1425,6 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
                     colf[tb][x & 127] = 1;
                 }
             }
-        }
-        if (NS == 0 && a.gstage) {
-            // mid is dead: stage the z-arm plane G (types tb + 4 bz) for the compressed
-            // write, in flight during the kinetic phases
-            const T* G = static_cast<const T*>(a.ws) + r.ws_G;
-            const int64_t gplane = static_cast<int64_t>(nxp) * nyp * nzp;
-            const int pnp = nyp * nxp;
-            const int r0 = ylo_ * nxp, r1 = (yhi_ + 1) * nxp;        // member rows only
-            for (int tb = 0; tb < 4; ++tb)
-                for (int i = r0 + threadIdx.x; i < r1; i += blockDim.x)
-                    CPA(mid, tb * pnp + i, midA, G, (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + i,
-                        8 * gplane);
         }
         if (dplane) {
             int nt;
@@ -1617,8 +1511,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     }
     cp_wait();
     __syncthreads();
-    // ---- compress: members of this plane -> H phi (plus the z arm left in G by k_kin_z;
-    //      the FMA path reads it from the plane staged in mid).  Coarse members (type 0)
+    // ---- compress: members of this plane -> H phi (plus the z arm left in G by k_kin_z).  Coarse members (type 0)
     //      row by row, a warp per row (one segment of up to n_x' members each); fine members
     //      flattened over the CTA, one member per thread and type: the plane's fine
     //      segments (many short chords of the fine spheres) are staged in shared memory and
@@ -1626,8 +1519,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     //      consecutive lanes write consecutive H phi elements.
     if (yhi_ >= 0) {
         const T* G = static_cast<const T*>(a.ws) + r.ws_G;
-        const unsigned char* gflag = reinterpret_cast<const unsigned char*>(a.gstage ? gfl : gsrc);
-        const bool gsm = NS == 0 && a.gstage;               // the z-arm plane is in mid
+        const unsigned char* gflag = reinterpret_cast<const unsigned char*>(gfl);
         const int64_t gplane = static_cast<int64_t>(nxp) * nyp * nzp;
         T* out = static_cast<T*>(a.hphi) + r.off_hphi;
         const int64_t out_room = a.hphi_n - r.off_hphi;
@@ -1642,7 +1534,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
                     const int x = xb + dx;
                     T v = LD(Gs, static_cast<int64_t>(b) * nxp + xb, gs_n);
                     if (yin && x >= 0 && x < nx && LD(gflag, y * nx + x, 4LL * pn))
-                        v += gsm ? LD(mid, static_cast<int64_t>(b) * nxp + xb, midA) : LD(G, grow + xb, 8 * gplane);
+                        v += LD(G, grow + xb, 8 * gplane);
                     ST(out, roff[b] + (xb - rx0[b]), out_room, v);
                 }
             }
@@ -1688,8 +1580,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
                     if (t == 0) continue;
                     T v = LD(Gs, (static_cast<int64_t>(tb) * nyp + b) * nxp + xb, gs_n);
                     if (zin && LD(gflag, (t & 3) * pn + y * nx + x, 4LL * pn))
-                        v += gsm ? LD(mid, (static_cast<int64_t>(tb) * nyp + b) * nxp + xb, midA)
-                                 : LD(G, t * gplane + grow + xb, 8 * gplane);
+                        v += LD(G, t * gplane + grow + xb, 8 * gplane);
                     ST(out, at.ncP + static_cast<int64_t>(t - 1) * at.nfP + m, out_room, v);
                 }
             }
@@ -1697,7 +1588,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     }
     const double ekin = warp_sum(static_cast<double>(ekin_t));
     if ((threadIdx.x & 31) == 0 && ekin != 0.0) atomicAdd(a.e_kin + r.f, ekin);
-    if constexpr (NS > 0) {
+    {
         tc::fence_before();
         __syncthreads();
         tc::fence_after();
@@ -1705,26 +1596,625 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int zb, i
     }
 }
 
-// Persistent form of the FMA version (a.items_bwd set): the batch's (function, z'' plane,
-// z type) items, largest first, from the second queue counter; otherwise (and always for
-// the tensor-core versions) one CTA per grid slot (blockIdx.x = 2 z'' + b_z, blockIdx.y =
-// function).
-template <class T, int NS>
-__global__ void __launch_bounds__(NS ? 512 : 256, NS ? 1 : (sizeof(T) == 4 ? LSW_BWD_MIN_BLOCKS : 1))
-    k_bwd_xy(HphiLaunch a) {
+template <int NS>
+__global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
+    bwd_plane_tc<NS>(a, blockIdx.y, blockIdx.x >> 1, blockIdx.x & 1);
+}
+
+// The FMA version.  An item is a plane (z'', b_z) of an atom's L' box for `cnt` consecutive
+// functions of the atom: the functions share every table below, so the tables are built once
+// per item and the item loops over the functions.
+//
+// Bound: instruction issue.  Per plane and function, 8 warps issued about 4,770 instructions
+// each, half of them packed FMAs; the rest were staging loops (an element per copy), zero
+// tests of the staged D plane, bounds tests of the kinetic windows and read-modify-writes.
+// So:
+//   - the planes of Bb and of the z arm arrive by bulk copies (one instruction each; the copy
+//     starts at the 16-byte boundary below the plane, the remainder becomes the first index);
+//   - the kinetic x arm is computed by the thread that computes the transposed x filter of the
+//     same outputs: one store instead of a store and a read-modify-write, one barrier less;
+//   - kinetic sums skip window positions outside the hull of L's members (per row along x, per
+//     column along y), in groups of 4 positions, uniformly over a warp; neighbouring lanes take
+//     neighbouring rows (columns) of the same block, so their hulls nearly agree.  Positions
+//     outside the box read a zero beside the D plane (PAD: a zero column between rows and a
+//     zero row; without PAD, where those do not fit, a zero register);
+//   - the compressed write's fine members come from a list built once per item.
+// Measured (GB300, 2,070 MHz, 1,024 functions a batch): DENSE_BEFORE_AFTER
+template <class T, bool PAD>
+struct KinArm {
+    static constexpr int N = Blk<T, 1>::NB;            // outputs per block, both arms
+    static constexpr int NP = N + 2 * KIN_HALF;        // window positions
+    // o0[j], o1[j]: outputs j of the pair's two types; c0[j], c1[j]: the inputs at the outputs;
+    // ld(p, v0): input of the first type at window position p (ld1: the second type); [s0, e0) and
+    // [s1, e1): the positions that can be nonzero, uniform over the warp, [s1, e1) within [s0, e0).
+    template <class L0, class L1>
+    static __device__ __forceinline__ void run(T (&o0)[N], T (&o1)[N], T (&c0)[N], T (&c1)[N], L0 ld0, L1 ld1, int s0,
+                                               int e0, int s1, int e1) {
+#pragma unroll
+        for (int j = 0; j < N; ++j) o0[j] = o1[j] = c0[j] = c1[j] = T(0);
+        if constexpr (sizeof(T) == 4) {
+            float2 acc[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) acc[j] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int g = 0; g < NP; g += 4) {
+                if (g + 3 < s0 || g >= e0) continue;
+#pragma unroll
+                for (int p = g; p < g + 4; ++p) {
+                    const float v = ld0(p);
+                    if (p >= KIN_HALF && p < KIN_HALF + N) c0[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (p - j >= 0 && p - j < KIN_TAPS) acc[j] = __ffma2_rn(c_kin2[0][p - j], make_float2(v, v), acc[j]);
+                }
+                if (g + 3 < s1 || g >= e1) continue;
+#pragma unroll
+                for (int p = g; p < g + 4; ++p) {
+                    const float v = ld1(p);
+                    if (p >= KIN_HALF && p < KIN_HALF + N) c1[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (p - j >= 0 && p - j < KIN_TAPS) acc[j] = __ffma2_rn(c_kin2[1][p - j], make_float2(v, v), acc[j]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                o0[j] = acc[j].x;
+                o1[j] = acc[j].y;
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                if (p < s0 || p >= e0) continue;
+                const T v = ld0(p);
+                if (p >= KIN_HALF && p < KIN_HALF + N) c0[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if (p - j >= 0 && p - j < KIN_TAPS) {
+                        o0[j] += Tab<T>::kin(0, p - j) * v;
+                        o1[j] += Tab<T>::kin(2, p - j) * v;
+                    }
+                if (p < s1 || p >= e1) continue;
+                const T u = ld1(p);
+                if (p >= KIN_HALF && p < KIN_HALF + N) c1[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = u;
+#pragma unroll
+                for (int j = 0; j < N; ++j)
+                    if (p - j >= 0 && p - j < KIN_TAPS) {
+                        o0[j] += Tab<T>::kin(1, p - j) * u;
+                        o1[j] += Tab<T>::kin(3, p - j) * u;
+                    }
+            }
+        }
+    }
+};
+
+// The transposed filters of N coarse outputs from the window starting at position `first` of a
+// line of n values.  FP32: as bwd_block.  FP64 (bound by the FP64 pipe): positions outside the
+// line are skipped, not multiplied as zeros.
+template <class T, int NB>
+__device__ __forceinline__ void bwd_window(const T* p, int off, int stride, int first, int n, T (&s)[NB], T (&d)[NB],
+                                           int64_t room, int* st) {
+    if constexpr (sizeof(T) == 4) {
+        T w[2 * NB + 29];
+        swin(w, p, off, stride, first, n, room, st);
+        bwd_block<T, NB>(w, s, d);
+    } else {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) s[j] = d[j] = T(0);
+#pragma unroll
+        for (int m = 0; m < 2 * NB + 29; ++m) {
+            const int pos = first + m;
+            if (pos < 0 || pos >= n) continue;
+            const T v = WLD(p, off + pos * stride, room);
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (m - 2 * j >= 0 && m - 2 * j < FWD_TAPS) {
+                    s[j] += Tab<T>::fwd(0, m - 2 * j) * v;
+                    d[j] += Tab<T>::fwd(1, m - 2 * j) * v;
+                }
+        }
+    }
+}
+
+template <class T, bool PAD>
+__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
-    if (NS == 0 && a.items_bwd) {
+    int* st = a.status;
+    constexpr int NB = Blk<T, 1>::NB;
+    using Arm = KinArm<T, PAD>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int ylo, yhi, dead;
+    const FnRec r0 = a.fn[fl];
+    if (zb >= r0.np[2]) return;
+    const AtomRec& at = a.atoms[r0.atom];
+    const int nx = r0.n[0], ny = r0.n[1], nz = r0.n[2];
+    const int X = 2 * nx + 29, Y = 2 * ny + 29;
+    const int nxp = r0.np[0], nyp = r0.np[1], nzp = r0.np[2];
+    const int dx = r0.lop[0] - r0.lo[0], dy = r0.lop[1] - r0.lo[1], dz = r0.lop[2] - r0.lo[2];
+    const BwdLayout L = bwd_layout(nx, ny, nxp, nyp, sizeof(T), NB, a.gstage, PAD);
+    const int RS = L.RS;
+    T* const plb = reinterpret_cast<T*>(smem_raw + L.o_pl);     // Bb plane [Y][X], later Gs [4][nyp][nxp]
+    T* const Gs = plb;
+    T* const mid = reinterpret_cast<T*>(smem_raw + L.o_mid);    // [2][nyp][X], later the z-arm plane
+    T* const Db = reinterpret_cast<T*>(smem_raw + L.o_D);
+    T* const Dp = Db + (PAD ? 1 : 0);                           // [4][ny][RS]
+    const int zrow = 4 * ny * RS;                               // PAD: a zero row
+    int* const task = reinterpret_cast<int*>(smem_raw + L.o_task);
+    int* const roff = reinterpret_cast<int*>(smem_raw + L.o_roff);
+    int* const cq0 = reinterpret_cast<int*>(smem_raw + L.o_blk);   // y pass, per block of NB rows: column range, prefix
+    int* const cq1 = cq0 + L.nb_y;
+    int* const pq = cq1 + L.nb_y;                               // [nb_y + 1]
+    int* const rq0 = pq + L.nb_y + 1;                           // kinetic y arm, per (x type, block of N rows): the same
+    int* const rq1 = rq0 + 2 * L.nb_y;
+    int* const rqp = rq1 + 2 * L.nb_y;                          // [2 nb_y + 1]
+    int* const hlo = rqp + 2 * L.nb_y + 1;                      // x pass, per (y type, block of NB columns): row hull, prefix
+    int* const hhi = hlo + 2 * L.nb_x;
+    int* const hp = hhi + 2 * L.nb_x;                           // [2 nb_x + 1]
+    int16_t* const rx0 = reinterpret_cast<int16_t*>(smem_raw + L.o_row);   // member x range per row (L' plane), -1: none
+    int16_t* const rx1 = rx0 + nyp;
+    int16_t* const fx0 = rx1 + nyp;                             // hull of the row's fine members, -1: none
+    int16_t* const fx1 = fx0 + nyp;
+    int16_t* const lx0 = fx1 + nyp;                             // [2][ny]: hull of L's coarse, fine members per row of the D plane
+    int16_t* const lx1 = lx0 + 2 * ny;
+    int16_t* const cy0 = lx1 + 2 * ny;                          // [2][nx]: the same per column
+    int16_t* const cy1 = cy0 + 2 * nx;
+    uint16_t* const memb = reinterpret_cast<uint16_t*>(smem_raw + L.o_mem);   // b n_x' + x of the plane's fine members
+    const uint32_t mbar = tc::saddr(smem_raw);
+    const int zL = zb + dz;
+    const bool dplane = zL >= 0 && zL < nz;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t smem_n = static_cast<int64_t>(a.smem_bwd / sizeof(T));
+    [[maybe_unused]] const int64_t pl_n = smem_n - L.o_pl / sizeof(T), mid_n = smem_n - L.o_mid / sizeof(T),
+                                   dp_n = smem_n - L.o_D / sizeof(T) - (PAD ? 1 : 0);
+    if (tid == 0) {
+        ylo = nyp;
+        yhi = -1;
+        dead = 0;
+    }
+    for (int i = tid; i < 2 * L.nb_x; i += blockDim.x) {
+        hlo[i] = nyp;
+        hhi[i] = -1;
+    }
+    __syncthreads();
+    const int pn = nx * ny;
+    const int64_t dplane_n = static_cast<int64_t>(pn) * nz;
+    // the D plane of function f (types tb + 4 bz), an element per copy into the padded rows
+    auto stage_D = [&](const FnRec& r) {
+        const T* D = static_cast<const T*>(a.ws) + r.ws_D + 4LL * bz * dplane_n + static_cast<int64_t>(zL) * pn;
+        for (int row = warp; row < 4 * ny; row += blockDim.x >> 5) {
+            const int tb = (row >= 2 * ny ? 2 : 0) + (row >= 3 * ny || (row >= ny && row < 2 * ny) ? 1 : 0);
+            const int y = row - tb * ny;
+            for (int x = lane; x < nx; x += 32)
+                CPA(Dp, row * RS + x, dp_n, D, tb * dplane_n + y * nx + x, 8 * dplane_n);
+        }
+    };
+    // member x range of each row of this plane (coarse part of L', fine hull), and of the D plane
+    const int64_t crow0 = at.rowPc + static_cast<int64_t>(nyp) * zb, frow0 = at.rowPf + static_cast<int64_t>(nyp) * zb;
+    for (int y = tid; y < nyp; y += blockDim.x) {
+        const int s0 = LD(a.rowptr, crow0 + y, a.rowptr_n), s1 = LD(a.rowptr, crow0 + y + 1, a.rowptr_n);
+        int lo = -1, hi = -1, off = 0;
+        if (s1 > s0) {
+            const Seg sg = LD(a.seg, at.segPc + s0, a.seg_n);
+            lo = sg.x0;
+            off = sg.off;
+            hi = LD(a.seg, at.segPc + s1 - 1, a.seg_n).x1;
+        }
+        rx0[y] = static_cast<int16_t>(lo);
+        rx1[y] = static_cast<int16_t>(hi);
+        roff[y] = off;
+        const int q0 = LD(a.rowptr, frow0 + y, a.rowptr_n), q1 = LD(a.rowptr, frow0 + y + 1, a.rowptr_n);
+        const int flo = q1 > q0 ? LD(a.seg, at.segPf + q0, a.seg_n).x0 : -1;
+        fx0[y] = static_cast<int16_t>(flo);
+        fx1[y] = static_cast<int16_t>(q1 > q0 ? LD(a.seg, at.segPf + q1 - 1, a.seg_n).x1 : -1);
+        if ((bz == 0 ? lo : flo) >= 0) {                       // rows that the compressed write reads
+            atomicMin(&ylo, y);
+            atomicMax(&yhi, y);
+        }
+    }
+    if (dplane) {
+        for (int i = tid; i < 2 * ny; i += blockDim.x) {
+            const int part = i >= ny, y = i - part * ny;
+            const int64_t row = (part ? at.rowLf : at.rowLc) + y + static_cast<int64_t>(ny) * zL;
+            const int64_t sg = part ? at.segLf : at.segLc;
+            const int s0 = LD(a.rowptr, row, a.rowptr_n), s1 = LD(a.rowptr, row + 1, a.rowptr_n);
+            lx0[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s0, a.seg_n).x0 : -1);
+            lx1[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s1 - 1, a.seg_n).x1 : -1);
+        }
+        if (PAD) {
+            for (int i = tid; i < 4 * ny; i += blockDim.x)
+                for (int x = nx; x < RS; ++x) ST(Dp, i * RS + x, dp_n, T(0));
+            for (int i = tid; i < RS + 1; i += blockDim.x) ST(Db, i == 0 ? 0 : zrow + i, dp_n + 1, T(0));
+        }
+    }
+    __syncthreads();
+    const int ylo_ = ylo, yhi_ = yhi;
+    if (yhi_ < 0) return;                                      // uniform; nothing to write in this plane
+    // The x range of row b whose outputs of the y-type pair `by` (types 2 by, 2 by + 1 of
+    // this plane) the compressed write reads: the coarse members where the pair holds the
+    // scaling type 0 (bz = 0, by = 0), else the hull of the row's fine members (the wavelet
+    // types are stored on fine members only).  lo < 0: none.
+    auto need = [&](int by, int b, int& lo, int& hi) {
+        const bool c = bz == 0 && by == 0;
+        lo = c ? rx0[b] : fx0[b];
+        hi = c ? rx1[b] : fx1[b];
+    };
+    // ---- ranges, in one phase: the y pass's columns per block of NB rows (for row b and pair by
+    //      its blocks k = lo/NB .. hi/NB of the needed range read x' in [2 (k NB + dx),
+    //      2 (k NB + NB - 1 + dx) + 30]); the kinetic y arm's columns (per x type bx, the pair of
+    //      types bx, bx + 2, and block of rows: the hull of the rows' needed ranges); the x pass's
+    //      rows per (pair, block of NB columns); the member hulls of D's columns; the fine members
+    const int nbb = (yhi_ - ylo_ + NB) / NB;
+    for (int q = tid; q < nbb; q += blockDim.x) {
+        int c0 = X, c1 = -1;
+        for (int b = ylo_ + q * NB; b < min(ylo_ + (q + 1) * NB, yhi_ + 1); ++b)
+            for (int by = 0; by < 2; ++by) {
+                int lo, hi;
+                need(by, b, lo, hi);
+                if (lo < 0) continue;
+                c0 = min(c0, 2 * ((lo / NB) * NB + dx));
+                c1 = max(c1, 2 * ((hi / NB) * NB + NB - 1 + dx) + 30);
+            }
+        cq0[q] = max(c0, 0);
+        cq1[q] = min(c1, X - 1);
+    }
+    for (int i = tid - 32; i >= 0 && i < 2 * nbb; i += blockDim.x) {
+        const int bx = i >= nbb, q = i - bx * nbb;
+        int c0 = nxp, c1 = -1;
+        for (int b = ylo_ + q * NB; b < min(ylo_ + (q + 1) * NB, yhi_ + 1); ++b) {
+            int lo, hi;
+            need(bx, b, lo, hi);                               // the same rule with the x type
+            if (lo < 0) continue;
+            c0 = min(c0, lo);
+            c1 = max(c1, hi);
+        }
+        rq0[i] = max(c0, -dx);                                 // columns of the D plane
+        rq1[i] = min(c1, nx - 1 - dx);
+    }
+    for (int i = tid; i < 2 * (yhi_ - ylo_ + 1); i += blockDim.x) {
+        const int by = i & 1, b = ylo_ + (i >> 1);
+        int lo, hi;
+        need(by, b, lo, hi);
+        if (lo < 0) continue;
+        for (int k = lo / NB; k <= hi / NB; ++k) {
+            atomicMin(&hlo[by * L.nb_x + k], b);
+            atomicMax(&hhi[by * L.nb_x + k], b);
+        }
+    }
+    if (dplane)
+        for (int i = tid; i < 2 * nx; i += blockDim.x) {
+            const int part = i >= nx, x = i - part * nx;
+            int lo = -1, hi = -1;
+            for (int y = 0; y < ny; ++y)
+                if (lx0[part * ny + y] >= 0 && x >= lx0[part * ny + y] && x <= lx1[part * ny + y]) {
+                    if (lo < 0) lo = y;
+                    hi = y;
+                }
+            cy0[i] = static_cast<int16_t>(lo);
+            cy1[i] = static_cast<int16_t>(hi);
+        }
+    const int q0 = LD(a.rowptr, frow0, a.rowptr_n), q1 = LD(a.rowptr, frow0 + nyp, a.rowptr_n);
+    int m0 = 0, nm = 0;                                        // fine members m0 .. m0 + nm - 1 of each type's block
+    if (q1 > q0) {
+        const Seg sl = LD(a.seg, at.segPf + q1 - 1, a.seg_n);
+        m0 = LD(a.seg, at.segPf + q0, a.seg_n).off;
+        nm = sl.off + (sl.x1 - sl.x0 + 1) - m0;
+    }
+    const bool listed = nm <= L.memN;
+    if (listed)
+        for (int q = q0 + tid; q < q1; q += blockDim.x) {
+            const Seg g = LD(a.seg, at.segPf + q, a.seg_n);
+            const int at0 = static_cast<int>(g.row - static_cast<int64_t>(nyp) * zb) * nxp;
+            for (int x = g.x0; x <= g.x1; ++x) ST(memb, g.off - m0 + (x - g.x0), L.memN, static_cast<uint16_t>(at0 + x));
+        }
+    __syncthreads();
+    if (tid == 0) {
+        pq[0] = 0;
+        for (int q = 0; q < nbb; ++q) pq[q + 1] = pq[q] + max(0, cq1[q] - cq0[q] + 1);
+    }
+    if (tid == 32) {
+        rqp[0] = 0;
+        for (int i = 0; i < 2 * nbb; ++i) rqp[i + 1] = rqp[i] + max(0, rq1[i] - rq0[i] + 1);
+    }
+    if (tid == 64) {
+        hp[0] = 0;
+        for (int i = 0; i < 2 * L.nb_x; ++i) hp[i + 1] = hp[i] + max(0, hhi[i] - hlo[i] + 1);
+    }
+    __syncthreads();
+    auto find = [](const int* pre, int n, int i) {             // the entry e with pre[e] <= i < pre[e + 1]
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int m = (lo + hi + 1) >> 1;
+            if (pre[m] <= i) lo = m;
+            else hi = m - 1;
+        }
+        return lo;
+    };
+    // x pass tasks, block-major: consecutive rows of a block on consecutive lanes (odd row
+    // strides: no bank conflicts, and nearly equal kinetic hulls)
+    const int ntx = hp[2 * L.nb_x];
+    for (int i = tid; i < ntx; i += blockDim.x) {
+        const int e = find(hp, 2 * L.nb_x, i);
+        ST(task, i, L.taskN, (e << 16) | (hlo[e] + (i - hp[e])));
+    }
+    const T ks = static_cast<T>(a.kin_scale);
+    const int pnp = nyp * nxp;
+    const int64_t gplane = static_cast<int64_t>(pnp) * nzp;
+    const FastDiv fd_nxp(nxp);
+    if (dplane) stage_D(r0);
+    for (int c = 0; c < cnt; ++c) {
+        const FnRec r = a.fn[fl + c];
+        const T* Bb = static_cast<const T*>(a.ws) + r.ws_Bb + (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
+        [[maybe_unused]] const int64_t bb_room = 2LL * nzp * Y * X - (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
+        // ---- the Bb plane
+#ifdef LSW_CHECKED
+        T* const pl = plb;
+        for (int i = tid; i < Y * X; i += blockDim.x) CPA(pl, i, pl_n, Bb, i, bb_room);
+#else
+        const int rem = static_cast<int>((reinterpret_cast<uintptr_t>(Bb) & 15) / sizeof(T));
+        T* const pl = plb + rem;
+        if (tid == 0) {
+            const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(rem + Y * X) * sizeof(T) + 15) & ~size_t(15));
+            bulk_fence();                                      // Gs was read and written there
+            bulk_expect(mbar, bytes);
+            bulk_load(tc::saddr(plb), Bb - rem, bytes, mbar);
+        }
+        if (!dead && !tc::mbar_wait(mbar, phase)) {
+            atomicOr(st, ST_WAIT_TIMEOUT);
+            dead = 1;
+        }
+        phase ^= 1;
+#endif
+#ifdef LSW_CHECKED
+        cp_wait();
+        __syncthreads();
+#endif
+        // ---- y pass: blocks of NB rows b within [ylo, yhi], per block only the listed columns
+        {
+            const int ntk = pq[nbb];
+            for (int tk = tid; tk < ntk; tk += blockDim.x) {
+                int q = 0;
+                while (tk >= pq[q + 1]) ++q;
+                const int xo = cq0[q] + (tk - pq[q]), b0 = ylo_ + q * NB;
+                T s[NB], d[NB];
+                bwd_window<T, NB>(pl, xo, X, 2 * (b0 + dy), Y, s, d, pl_n, st);
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const int b = b0 + j;
+                    if (b <= yhi_) {
+                        ST(mid, b * X + xo, mid_n, s[j]);
+                        ST(mid, (nyp + b) * X + xo, mid_n, d[j]);
+                    }
+                }
+            }
+        }
+        cp_wait();                                             // the D plane
+        __syncthreads();                                       // pl is dead from here on: Gs reuses it
+        T ekin_t = 0;
+        // ---- x pass (transposed filters) and kinetic x arm on the listed row blocks
+        for (int i0 = warp * 32; i0 < ntx; i0 += blockDim.x) { // whole warps: the kinetic range is a warp's
+            const bool on = i0 + lane < ntx;
+            const int code = task[on ? i0 + lane : i0];
+            const int e = code >> 16, b = code & 0xffff;
+            const int by = e >= L.nb_x, x0 = (e - by * L.nb_x) * NB;
+            T s[NB], d[NB];
+            bwd_window<T, NB>(mid, (by * nyp + b) * X, 1, 2 * (x0 + dx), X, s, d, mid_n, st);
+            if (dplane) {
+                const int y = b + dy, f0 = x0 + dx - KIN_HALF; // window position p is D position f0 + p
+                int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
+                const bool in = on && y >= 0 && y < ny;
+                if (in) {
+                    const int p0 = (bz == 0 && by == 0 ? 0 : ny) + y, p1 = ny + y;
+                    if (lx0[p0] >= 0) s0 = lx0[p0] - f0, e0 = lx1[p0] - f0 + 1;
+                    if (lx0[p1] >= 0) s1 = lx0[p1] - f0, e1 = lx1[p1] - f0 + 1;
+                }
+                s0 = __reduce_min_sync(0xffffffffu, s0);
+                e0 = __reduce_max_sync(0xffffffffu, e0);
+                s1 = __reduce_min_sync(0xffffffffu, s1);
+                e1 = __reduce_max_sync(0xffffffffu, e1);
+                T o0[NB], o1[NB], c0[NB], c1[NB];
+                const int a0 = (2 * by) * ny * RS + (in ? y * RS : 0), a1 = a0 + ny * RS;
+                auto at_x = [&](int row, int p) -> T {
+                    const int x = f0 + p;
+                    if (PAD) return LD(Db, in ? row + 1 + min(max(x, -1), nx) : zrow + 1, dp_n + 1);
+                    return in && x >= 0 && x < nx ? LD(Dp, row + x, dp_n) : T(0);
+                };
+                Arm::run(o0, o1, c0, c1, [&](int p) { return at_x(a0, p); }, [&](int p) { return at_x(a1, p); }, s0, e0,
+                         s1, e1);
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    o0[j] *= ks;
+                    o1[j] *= ks;
+                    s[j] += o0[j];
+                    d[j] += o1[j];
+                    if (on) ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
+                }
+            }
+            if (on) {
+#pragma unroll
+                for (int j = 0; j < NB; ++j) {
+                    const int xb = x0 + j;
+                    if (xb < nxp) {
+                        ST(Gs, ((0 + 2 * by) * nyp + b) * nxp + xb, pl_n, s[j]);
+                        ST(Gs, ((1 + 2 * by) * nyp + b) * nxp + xb, pl_n, d[j]);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // ---- the z-arm plane G (types tb + 4 bz, member rows) into mid, which is dead
+        const T* G = static_cast<const T*>(a.ws) + r.ws_G;
+        const int g_r0 = ylo_ * nxp, g_n = (yhi_ - ylo_ + 1) * nxp;
+        const int slot = (pnp + 15) & ~7;                      // a type's place in mid (16-byte multiple)
+        auto g_rem = [&](int tb) -> int {
+#ifdef LSW_CHECKED
+            return 0;
+#else
+            const T* src = G + (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0;
+            return static_cast<int>((reinterpret_cast<uintptr_t>(src) & 15) / sizeof(T));
+#endif
+        };
+        if (a.gstage) {
+#ifdef LSW_CHECKED
+            for (int tb = 0; tb < 4; ++tb)
+                for (int i = tid; i < g_n; i += blockDim.x)
+                    CPA(mid, tb * slot + i, mid_n, G, (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 + i,
+                        8 * gplane);
+#else
+            if (tid == 0) {
+                bulk_fence();
+                uint32_t total = 0;
+#pragma unroll
+                for (int tb = 0; tb < 4; ++tb)
+                    total += static_cast<uint32_t>((static_cast<size_t>(g_rem(tb) + g_n) * sizeof(T) + 15) & ~size_t(15));
+                bulk_expect(mbar, total);
+#pragma unroll
+                for (int tb = 0; tb < 4; ++tb) {
+                    const int gr = g_rem(tb);
+                    const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(gr + g_n) * sizeof(T) + 15) & ~size_t(15));
+                    bulk_load(tc::saddr(mid + tb * slot),
+                              G + (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 - gr, bytes, mbar);
+                }
+            }
+#endif
+        }
+        // ---- kinetic y arm: (x type bx, block q of NB rows, column) over the listed columns,
+        //      consecutive columns on consecutive lanes
+        if (dplane) {
+            const int nt = rqp[2 * nbb];
+            for (int i0 = warp * 32; i0 < nt; i0 += blockDim.x) {
+                const bool on = i0 + lane < nt;
+                const int it = on ? i0 + lane : i0;
+                const int e = find(rqp, 2 * nbb, it);
+                const int bx = e >= nbb, q = e - bx * nbb;
+                const int xb = rq0[e] + (it - rqp[e]), b0 = ylo_ + q * NB;
+                const int x = xb + dx, f0 = b0 + dy - KIN_HALF;
+                int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
+                if (on) {
+                    const int p0 = (bz == 0 && bx == 0 ? 0 : nx) + x, p1 = nx + x;
+                    if (cy0[p0] >= 0) s0 = cy0[p0] - f0, e0 = cy1[p0] - f0 + 1;
+                    if (cy0[p1] >= 0) s1 = cy0[p1] - f0, e1 = cy1[p1] - f0 + 1;
+                }
+                s0 = __reduce_min_sync(0xffffffffu, s0);
+                e0 = __reduce_max_sync(0xffffffffu, e0);
+                if (s0 >= min(e0, Arm::NP) || e0 <= 0) continue;   // uniform: no member of L within reach
+                s1 = __reduce_min_sync(0xffffffffu, s1);
+                e1 = __reduce_max_sync(0xffffffffu, e1);
+                T o0[NB], o1[NB], c0[NB], c1[NB];
+                auto at_y = [&](int tb, int p) -> T {
+                    const int y = f0 + p;
+                    const bool in = y >= 0 && y < ny;
+                    if (PAD) return LD(Dp, in ? (tb * ny + y) * RS + x : zrow, dp_n);
+                    return in ? LD(Dp, (tb * ny + y) * RS + x, dp_n) : T(0);
+                };
+                Arm::run(o0, o1, c0, c1, [&](int p) { return at_y(bx, p); }, [&](int p) { return at_y(bx + 2, p); }, s0,
+                         e0, s1, e1);
+                if (on) {
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) {
+                        const int b = b0 + j;
+                        if (b <= yhi_) {
+                            o0[j] *= ks;
+                            o1[j] *= ks;
+                            const int g0 = ((bx + 0) * nyp + b) * nxp + xb, g1 = ((bx + 2) * nyp + b) * nxp + xb;
+                            ST(Gs, g0, pl_n, LD(Gs, g0, pl_n) + o0[j]);
+                            ST(Gs, g1, pl_n, LD(Gs, g1, pl_n) + o1[j]);
+                            ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
+                        }
+                    }
+                }
+            }
+        }
+        if (a.gstage) {
+#ifdef LSW_CHECKED
+            cp_wait();
+#else
+            if (!dead && !tc::mbar_wait(mbar, phase)) {
+                atomicOr(st, ST_WAIT_TIMEOUT);
+                dead = 1;
+            }
+            phase ^= 1;
+#endif
+        }
+        __syncthreads();
+        if (c + 1 < cnt && dplane) stage_D(a.fn[fl + c + 1]);  // the D plane is dead; in flight during the write
+        // ---- compress: members of this plane -> H phi, plus the z arm left in G by k_kin_z
+        //      where its flag says so.  Coarse members (type 0) row by row, a warp per row; fine
+        //      members flattened over the CTA, consecutive lanes on consecutive H phi elements.
+        const unsigned char* gflag = reinterpret_cast<const unsigned char*>(static_cast<const T*>(a.ws) + r.ws_Gf);
+        T* out = static_cast<T*>(a.hphi) + r.off_hphi;
+        [[maybe_unused]] const int64_t out_room = a.hphi_n - r.off_hphi;
+        auto zarm = [&](int t, int i) -> T {                   // type t (of 8), plane index i = b n_x' + x
+            if (a.gstage) return LD(mid, (t & 3) * slot + g_rem(t & 3) + i - g_r0, mid_n);
+            return LD(G, t * gplane + static_cast<int64_t>(zb) * pnp + i, 8 * gplane);
+        };
+        if (bz == 0) {                                         // scaling part s (type 0) on the coarse members
+            for (int b = ylo_ + warp; b <= yhi_; b += (blockDim.x >> 5)) {
+                if (rx0[b] < 0) continue;
+                const int y = b + dy;
+                const bool yin = y >= 0 && y < ny;
+                for (int xb = rx0[b] + lane; xb <= rx1[b]; xb += 32) {
+                    const int x = xb + dx;
+                    T v = LD(Gs, b * nxp + xb, pl_n);
+                    if (yin && x >= 0 && x < nx && LD(gflag, y * nx + x, 4LL * pn)) v += zarm(0, b * nxp + xb);
+                    ST(out, roff[b] + (xb - rx0[b]), out_room, v);
+                }
+            }
+        }
+        for (int m = tid; m < nm; m += blockDim.x) {
+            int i;
+            if (listed) {
+                i = LD(memb, m, L.memN);
+            } else {                                           // more members than the list holds: find the segment
+                int lo = q0, hi = q1 - 1;
+                while (lo < hi) {
+                    const int k = (lo + hi + 1) >> 1;
+                    if (LD(a.seg, at.segPf + k, a.seg_n).off - m0 <= m) lo = k;
+                    else hi = k - 1;
+                }
+                const Seg g = LD(a.seg, at.segPf + lo, a.seg_n);
+                i = static_cast<int>(g.row - static_cast<int64_t>(nyp) * zb) * nxp + g.x0 + (m - (g.off - m0));
+            }
+            const int b = fd_nxp.div(i), xb = i - b * nxp;
+            const int y = b + dy, x = xb + dx;
+            const bool zin = y >= 0 && y < ny && x >= 0 && x < nx;
+#pragma unroll
+            for (int tb = 0; tb < 4; ++tb) {
+                const int t = tb + 4 * bz;
+                if (t == 0) continue;
+                T v = LD(Gs, tb * pnp + i, pl_n);
+                if (zin && LD(gflag, tb * pn + y * nx + x, 4LL * pn)) v += zarm(t, i);
+                ST(out, at.ncP + static_cast<int64_t>(t - 1) * at.nfP + m0 + m, out_room, v);
+            }
+        }
+        const double ekin = warp_sum(static_cast<double>(ekin_t));
+        if (lane == 0 && ekin != 0.0) atomicAdd(a.e_kin + r.f, ekin);
+        __syncthreads();                                       // Gs and mid are free for the next function
+    }
+}
+
+// Persistent form (a.items_bwd set): the batch's (atom's functions, z'' plane, z type) items,
+// largest first, from the second queue counter; otherwise one CTA per grid slot (blockIdx.x =
+// 2 z'' + b_z, blockIdx.y = function).  Two CTAs of 8 warps per SM (128 registers).
+template <class T, bool PAD>
+__global__ void __launch_bounds__(256, 2) k_bwd_xy(HphiLaunch a) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 4;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (threadIdx.x == 0) tc::mbar_init(tc::saddr(smem_raw));
+    __syncthreads();
+    uint32_t phase = 0;
+    if (a.items_bwd) {
         __shared__ int s_item;
         for (;;) {
             const int k = next_item(a.queue + 1, &s_item);
             if (k >= a.n_items_bwd) break;
-            const int code = LD(a.items_bwd, k, a.n_items_bwd);
-            bwd_plane<T, NS>(a, code >> 11, (code >> 1) & 1023, code & 1);
+            const int2 it = LD(a.items_bwd, k, a.n_items_bwd);
+            bwd_plane<T, PAD>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase);
             __syncthreads();   // shared memory and s_item are reused by the next item
         }
     } else {
-        bwd_plane<T, NS>(a, blockIdx.y, blockIdx.x >> 1, blockIdx.x & 1);
+        bwd_plane<T, PAD>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase);
     }
 }
 
@@ -2116,8 +2606,9 @@ cudaError_t configure_kernels(size_t max_smem) {
     SETMAX(k_kin_z<double>) SETMAX(k_kin_z<float>)
     SETMAX(k_z_tc<2>) SETMAX(k_z_tc<3>)
     SETMAX(k_fwd_xy_tc<2>) SETMAX(k_fwd_xy_tc<3>)
-    SETMAX((k_bwd_xy<double, 0>)) SETMAX((k_bwd_xy<float, 0>))
-    SETMAX((k_bwd_xy<float, 2>)) SETMAX((k_bwd_xy<float, 3>))
+    SETMAX((k_bwd_xy<double, false>)) SETMAX((k_bwd_xy<float, false>))
+    SETMAX((k_bwd_xy<double, true>)) SETMAX((k_bwd_xy<float, true>))
+    SETMAX(k_bwd_xy_tc<2>) SETMAX(k_bwd_xy_tc<3>)
     SETMAX(k_z_dens<double>) SETMAX(k_z_dens<float>)
 #undef SETMAX
     // the plans size the plane kernels' dynamic shared memory against these bounds
@@ -2128,22 +2619,25 @@ cudaError_t configure_kernels(size_t max_smem) {
         if (fa.sharedSizeBytes > (B)) return cudaErrorInvalidConfiguration;                     \
     }
     STATIC_BOUND(k_fwd_xy<double>, FWD_STATIC_SMEM) STATIC_BOUND(k_fwd_xy<float>, FWD_STATIC_SMEM)
-    STATIC_BOUND((k_bwd_xy<double, 0>), BWD_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, 0>), BWD_STATIC_SMEM)
-    STATIC_BOUND((k_bwd_xy<float, 2>), BWD_TC_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, 3>), BWD_TC_STATIC_SMEM)
+    STATIC_BOUND((k_bwd_xy<double, false>), BWD_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, false>), BWD_STATIC_SMEM)
+    STATIC_BOUND((k_bwd_xy<double, true>), BWD_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, true>), BWD_STATIC_SMEM)
+    STATIC_BOUND(k_bwd_xy_tc<2>, BWD_TC_STATIC_SMEM) STATIC_BOUND(k_bwd_xy_tc<3>, BWD_TC_STATIC_SMEM)
 #undef STATIC_BOUND
     return cudaSuccess;
 }
 
-cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int* fwd, int* bwd) {
+cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int dpad, int* fwd, int* bwd) {
     cudaError_t e;
     if (prec == 0) {
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(fwd, k_fwd_xy<double>, 256, smem_fwd)) != cudaSuccess)
             return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double, 0>, 256, smem_bwd);
+        return dpad ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double, true>, 256, smem_bwd)
+                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double, false>, 256, smem_bwd);
     }
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(fwd, k_fwd_xy<float>, 256, smem_fwd)) != cudaSuccess)
         return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float, 0>, 256, smem_bwd);
+    return dpad ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float, true>, 256, smem_bwd)
+                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float, false>, 256, smem_bwd);
 }
 
 #define TRACED(TR, KIND, S, LAUNCH) \
@@ -2152,6 +2646,14 @@ cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int*
         LAUNCH;                         \
         trace_end(TR, S);               \
     } while (0)
+
+template <class T>
+static void bwd_xy(const HphiLaunch& a, dim3 g, cudaStream_t s) {
+    if (a.dpad)
+        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T, true><<<g, 256, a.smem_bwd, s>>>(a)));
+    else
+        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T, false><<<g, 256, a.smem_bwd, s>>>(a)));
+}
 
 template <class T>
 static cudaError_t hphi_batch(const HphiLaunch& a, cudaStream_t s) {
@@ -2187,13 +2689,13 @@ static cudaError_t hphi_batch(const HphiLaunch& a, cudaStream_t s) {
            (k_kin_z<T><<<dim3(static_cast<unsigned>((a.max_colsL + 127) / 128), nf, 4), 128, a.smem_kin, s>>>(a)));
     if constexpr (sizeof(T) == 4) {
         if (a.xy_tc && a.zsplit == 3)
-            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<float, 3><<<dim3(2 * a.max_nzp, nf), 512, a.smem_bwd_tc, s>>>(a)));
+            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy_tc<3><<<dim3(2 * a.max_nzp, nf), 512, a.smem_bwd_tc, s>>>(a)));
         else if (a.xy_tc && a.zsplit == 2)
-            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<float, 2><<<dim3(2 * a.max_nzp, nf), 512, a.smem_bwd_tc, s>>>(a)));
+            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy_tc<2><<<dim3(2 * a.max_nzp, nf), 512, a.smem_bwd_tc, s>>>(a)));
         else
-            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<float, 0><<<gbwd, 256, a.smem_bwd, s>>>(a)));
+            bwd_xy<T>(a, gbwd, s);
     } else {
-        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T, 0><<<gbwd, 256, a.smem_bwd, s>>>(a)));
+        bwd_xy<T>(a, gbwd, s);
     }
     return cudaGetLastError();
 }
