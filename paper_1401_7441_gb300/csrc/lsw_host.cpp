@@ -455,9 +455,9 @@ void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z) {
 
 // Backward plane kernel: sizes of its four layouts over a batch's functions, and the choice.
 // Two CTAs an SM come first (the kernel is bound by instruction issue: with one, barriers and
-// latencies stay uncovered), then the staged z-arm plane, then the zero pad of the D plane.
+// latencies stay uncovered), then the staged z-arm plane, then the lists.
 struct BwdSizes {
-    size_t b[2][2] = {{0, 0}, {0, 0}};                 // [gstage][pad]
+    size_t b[2][2] = {{0, 0}, {0, 0}};                 // [gstage][lists]
     void fold(const FnRec& r, int es) {
         for (int g = 0; g < 2; ++g)
             for (int p = 0; p < 2; ++p)
@@ -472,7 +472,7 @@ struct BwdSizes {
         for (const auto& o : order)
             if (b[o.g][o.p] <= o.lim) {
                 p->gstage = o.g;
-                p->dpad = o.p;
+                p->lists = o.p;
                 p->smem_bwd = b[o.g][o.p];
                 return true;
             }
@@ -638,7 +638,7 @@ lsw_status build_plans(lsw_system_s* s) {
                 return static_cast<int>(it.size());
             };
             int bf = 0, bb = 0;
-            CUDA_TRY(plane_kernel_blocks(p.prec, p.smem_fwd, p.smem_bwd, p.dpad, &bf, &bb));
+            CUDA_TRY(plane_kernel_blocks(p.prec, p.smem_fwd, p.smem_bwd, &bf, &bb));
             item_off.push_back(static_cast<int64_t>(items.size()));
             p.n_items_fwd = (s->persistent & 2) ? add(0, 1) : 0;
             int64_t planes = 0;

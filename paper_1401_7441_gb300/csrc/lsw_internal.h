@@ -127,7 +127,7 @@ struct PanelSlab {
 
 // Dynamic shared memory of the FMA backward plane kernel for L extents (nx, ny), L' extents
 // (nxp, nyp), element size es and nb outputs per block: byte offsets and sizes.  gstage: room
-// for the z-arm plane; pad: zeros around the D plane.
+// for the z-arm plane; lists: as HphiLaunch::lists.
 #ifdef __CUDACC__
 #define LSW_HD __host__ __device__ __forceinline__
 #else
@@ -135,27 +135,29 @@ struct PanelSlab {
 #endif
 constexpr int BWD_NB_F32 = 8, BWD_NB_F64 = 4;   // outputs per block
 struct BwdLayout {
-    int RS;                      // row stride of the D plane (odd: rows land in different banks)
+    int RS, PS;                  // row stride (odd: rows land in different banks) and type stride of the D plane
     int nb_y, nb_x;              // blocks of rows and of columns (upper bounds)
-    int taskN, memN;             // x pass tasks, fine members listed
+    int taskN, taskkN, memN;     // x pass tasks, kinetic y tasks, fine members listed
     uint32_t o_pl, o_mid, o_D, o_task, o_roff, o_blk, o_row, o_mem, bytes;
 };
-LSW_HD BwdLayout bwd_layout(int nx, int ny, int nxp, int nyp, int es, int nb, bool gstage, bool pad) {
+LSW_HD BwdLayout bwd_layout(int nx, int ny, int nxp, int nyp, int es, int nb, bool gstage, bool lists) {
     BwdLayout L;
     const int X = 2 * nx + 29, Y = 2 * ny + 29;
     auto up = [](uint32_t v) { return (v + 15u) & ~15u; };
     auto mx = [](int u, int v) { return u > v ? u : v; };
-    L.RS = pad ? (nx + 1) | 1 : nx | 1;
+    L.RS = nx | 1;
+    L.PS = ny * L.RS + 1;                              // a zero after each type's rows
     L.nb_y = (nyp + nb - 1) / nb + 1;
     L.nb_x = (nxp + nb - 1) / nb;
     L.taskN = 2 * L.nb_x * nyp;
-    L.memN = nxp * nyp / 2 + 8;
+    L.taskkN = 2 * L.nb_y * (nx < nxp ? nx : nxp);
+    L.memN = lists ? nxp * nyp / 3 : 0;
     L.o_pl = 16;                                       // the mbarrier first
     L.o_mid = up(L.o_pl + static_cast<uint32_t>(es) * mx(Y * X + 8, 4 * nyp * nxp));
     const int slot = (nyp * nxp + 15) & ~7;
     L.o_D = up(L.o_mid + static_cast<uint32_t>(es) * (gstage ? mx(2 * nyp * X, 4 * slot) : 2 * nyp * X));
-    L.o_task = up(L.o_D + static_cast<uint32_t>(es) * (4 * ny * L.RS + (pad ? L.RS + 1 : 0)));
-    L.o_roff = L.o_task + 4u * L.taskN;
+    L.o_task = up(L.o_D + static_cast<uint32_t>(es) * (4 * L.PS));
+    L.o_roff = up(L.o_task + 2u * (L.taskN + L.taskkN));
     L.o_blk = L.o_roff + 4u * nyp;
     L.o_row = L.o_blk + 4u * (3 * L.nb_y + 1 + 6 * L.nb_y + 1 + 6 * L.nb_x + 1);
     L.o_mem = L.o_row + 2u * (4 * nyp + 4 * ny + 4 * nx);
@@ -191,7 +193,8 @@ struct HphiLaunch {
     size_t smem_fwd, smem_z, smem_bwd;
     int gstage;                  // 1: the backward plane kernel stages the z-arm plane in shared
                                  // memory (smem_bwd includes it); 0: reads it from global memory
-    int dpad;                    // 1: its D plane is padded with zeros
+    int lists;                   // 1: room for its list of fine members; 0 (boxes that leave none):
+                                 // the members are searched in the segments
     int zcols;                   // columns per CTA of the z stage
     int zsplit;                  // 0: z stage on FMA units; 2 or 3: bfloat16 parts per
                                  // FP32 operand of the tensor-core z stage
@@ -425,7 +428,7 @@ cudaError_t upload_filters(const FilterSet& fs, int device);
 cudaError_t measure_peaks(int n_sm, double* fp32_tflops, double* fp64_tflops, double* copy_gbs);
 cudaError_t configure_kernels(size_t max_smem);
 // Resident CTAs per SM of the FMA plane kernels at these dynamic shared-memory sizes.
-cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int dpad, int* fwd, int* bwd);
+cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int* fwd, int* bwd);
 cudaError_t enqueue_hphi_batch(const HphiLaunch& a, cudaStream_t s);
 cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s);     // panels of a slab (lsw_panels.cu)
 cudaError_t enqueue_panel_hs(const PanelHSLaunch& a, cudaStream_t s);   // S, H from the panels

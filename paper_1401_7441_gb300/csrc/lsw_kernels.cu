@@ -1605,10 +1605,10 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 // functions of the atom: the functions share every table below, so the tables are built once
 // per item and the item loops over the functions.
 //
-// Bound: instruction issue.  Per plane and function, 8 warps issued about 4,770 instructions
-// each, half of them packed FMAs; the rest were staging loops (an element per copy), zero
-// tests of the staged D plane, bounds tests of the kinetic windows and read-modify-writes.
-// So:
+// Bound: instruction issue and its latencies (two CTAs per SM by registers and shared memory).
+// Per plane and function, 8 warps issued about 4,770 instructions each, half of them packed
+// FMAs; the rest were staging loops (an element per copy), zero tests of the staged D plane,
+// bounds tests of the kinetic windows and read-modify-writes.  So:
 //   - the planes of Bb and of the z arm arrive by bulk copies (one instruction each; the copy
 //     starts at the 16-byte boundary below the plane, the remainder becomes the first index);
 //   - the kinetic x arm is computed by the thread that computes the transposed x filter of the
@@ -1616,73 +1616,76 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 //   - kinetic sums skip window positions outside the hull of L's members (per row along x, per
 //     column along y), in groups of 4 positions, uniformly over a warp; neighbouring lanes take
 //     neighbouring rows (columns) of the same block, so their hulls nearly agree.  Positions
-//     outside the box read a zero beside the D plane (PAD: a zero column between rows and a
-//     zero row; without PAD, where those do not fit, a zero register);
+//     outside the box read a zero beside the D plane;
+//   - the y pass, the x pass and the kinetic y arm are one loop body run in three phases: as three
+//     bodies their unrolled code (40 KB) missed the instruction caches (17 % of the stalls);
 //   - the compressed write's fine members come from a list built once per item.
-// Measured (GB300, 2,070 MHz, 1,024 functions a batch): DENSE_BEFORE_AFTER
-template <class T, bool PAD>
+// Measured (GB300, 2,070 MHz, 1,024 functions a batch): 9.5 -> 4.8 us per function at radii 5-8 bohr
+// (n_x' to 52; one CTA per SM before), 7.3 -> 6.0 us at 7 bohr in a dense system (n_x' 47, more fine
+// members).
+
+#ifndef LSW_BWD_THREADS
+#define LSW_BWD_THREADS 256
+#endif
+constexpr int BWD_THREADS = LSW_BWD_THREADS;
+
+// Kinetic arm of N outputs (both types of a pair) from the window positions p = 0 .. NP - 1 of two
+// lines: position p of the first line is D[off(p)], of the second D[off(p) + dist].  [s0, e0), [s1,
+// e1): the positions of either line that can be nonzero, uniform over the warp, the second
+// within the first.  c0, c1: the lines' values at the outputs.
+template <class T>
 struct KinArm {
     static constexpr int N = Blk<T, 1>::NB;            // outputs per block, both arms
     static constexpr int NP = N + 2 * KIN_HALF;        // window positions
-    // o0[j], o1[j]: outputs j of the pair's two types; c0[j], c1[j]: the inputs at the outputs;
-    // ld(p, v0): input of the first type at window position p (ld1: the second type); [s0, e0) and
-    // [s1, e1): the positions that can be nonzero, uniform over the warp, [s1, e1) within [s0, e0).
-    template <class L0, class L1>
-    static __device__ __forceinline__ void run(T (&o0)[N], T (&o1)[N], T (&c0)[N], T (&c1)[N], L0 ld0, L1 ld1, int s0,
-                                               int e0, int s1, int e1) {
+    static constexpr int G = sizeof(T) == 4 ? 4 : 1;   // positions per group
+    template <class Off>
+    static __device__ __forceinline__ void run(T (&o0)[N], T (&o1)[N], T (&c0)[N], T (&c1)[N], const T* D, int64_t dn,
+                                               int dist, Off off, int s0, int e0, int s1, int e1,
+                                               [[maybe_unused]] int* st) {
+        [[maybe_unused]] int* ST_ = st;
+        [[maybe_unused]] constexpr int KID = 4;
+        float2 acc[sizeof(T) == 4 ? N : 1];
 #pragma unroll
-        for (int j = 0; j < N; ++j) o0[j] = o1[j] = c0[j] = c1[j] = T(0);
-        if constexpr (sizeof(T) == 4) {
-            float2 acc[N];
+        for (int j = 0; j < N; ++j) {
+            o0[j] = o1[j] = c0[j] = c1[j] = T(0);
+            if constexpr (sizeof(T) == 4) acc[j] = make_float2(0.f, 0.f);
+        }
+        auto add = [&](int p, int src, T v) {
 #pragma unroll
-            for (int j = 0; j < N; ++j) acc[j] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int g = 0; g < NP; g += 4) {
-                if (g + 3 < s0 || g >= e0) continue;
-#pragma unroll
-                for (int p = g; p < g + 4; ++p) {
-                    const float v = ld0(p);
-                    if (p >= KIN_HALF && p < KIN_HALF + N) c0[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
-#pragma unroll
-                    for (int j = 0; j < N; ++j)
-                        if (p - j >= 0 && p - j < KIN_TAPS) acc[j] = __ffma2_rn(c_kin2[0][p - j], make_float2(v, v), acc[j]);
-                }
-                if (g + 3 < s1 || g >= e1) continue;
-#pragma unroll
-                for (int p = g; p < g + 4; ++p) {
-                    const float v = ld1(p);
-                    if (p >= KIN_HALF && p < KIN_HALF + N) c1[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
-#pragma unroll
-                    for (int j = 0; j < N; ++j)
-                        if (p - j >= 0 && p - j < KIN_TAPS) acc[j] = __ffma2_rn(c_kin2[1][p - j], make_float2(v, v), acc[j]);
+            for (int j = 0; j < N; ++j) {
+                if (p - j < 0 || p - j >= KIN_TAPS) continue;
+                if constexpr (sizeof(T) == 4) {
+                    acc[j] = __ffma2_rn(c_kin2[src][p - j], make_float2(v, v), acc[j]);
+                } else {
+                    o0[j] += Tab<T>::kin(src, p - j) * v;
+                    o1[j] += Tab<T>::kin(2 + src, p - j) * v;
                 }
             }
+        };
+#pragma unroll
+        for (int g = 0; g < NP; g += G) {
+            if (g + G - 1 < s0 || g >= e0) continue;
+            int at[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                at[k] = off(g + k);
+                const T v = LD(D, at[k], dn);
+                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c0[(g + k - KIN_HALF) & (N - 1)] = v;
+                add(g + k, 0, v);
+            }
+            if (g + G - 1 < s1 || g >= e1) continue;
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const T v = LD(D, at[k] + dist, dn);
+                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c1[(g + k - KIN_HALF) & (N - 1)] = v;
+                add(g + k, 1, v);
+            }
+        }
+        if constexpr (sizeof(T) == 4) {
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 o0[j] = acc[j].x;
                 o1[j] = acc[j].y;
-            }
-        } else {
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                if (p < s0 || p >= e0) continue;
-                const T v = ld0(p);
-                if (p >= KIN_HALF && p < KIN_HALF + N) c0[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = v;
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    if (p - j >= 0 && p - j < KIN_TAPS) {
-                        o0[j] += Tab<T>::kin(0, p - j) * v;
-                        o1[j] += Tab<T>::kin(2, p - j) * v;
-                    }
-                if (p < s1 || p >= e1) continue;
-                const T u = ld1(p);
-                if (p >= KIN_HALF && p < KIN_HALF + N) c1[p - KIN_HALF < 0 || p - KIN_HALF >= N ? 0 : p - KIN_HALF] = u;
-#pragma unroll
-                for (int j = 0; j < N; ++j)
-                    if (p - j >= 0 && p - j < KIN_TAPS) {
-                        o0[j] += Tab<T>::kin(1, p - j) * u;
-                        o1[j] += Tab<T>::kin(3, p - j) * u;
-                    }
             }
         }
     }
@@ -1716,13 +1719,13 @@ __device__ __forceinline__ void bwd_window(const T* p, int off, int stride, int 
     }
 }
 
-template <class T, bool PAD>
+template <class T>
 __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     int* st = a.status;
     constexpr int NB = Blk<T, 1>::NB;
-    using Arm = KinArm<T, PAD>;
+    using Arm = KinArm<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int ylo, yhi, dead;
     const FnRec r0 = a.fn[fl];
@@ -1732,15 +1735,14 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     const int X = 2 * nx + 29, Y = 2 * ny + 29;
     const int nxp = r0.np[0], nyp = r0.np[1], nzp = r0.np[2];
     const int dx = r0.lop[0] - r0.lo[0], dy = r0.lop[1] - r0.lo[1], dz = r0.lop[2] - r0.lo[2];
-    const BwdLayout L = bwd_layout(nx, ny, nxp, nyp, sizeof(T), NB, a.gstage, PAD);
-    const int RS = L.RS;
+    const BwdLayout L = bwd_layout(nx, ny, nxp, nyp, sizeof(T), NB, a.gstage, a.lists);
+    const int RS = L.RS, PS = L.PS;
     T* const plb = reinterpret_cast<T*>(smem_raw + L.o_pl);     // Bb plane [Y][X], later Gs [4][nyp][nxp]
     T* const Gs = plb;
     T* const mid = reinterpret_cast<T*>(smem_raw + L.o_mid);    // [2][nyp][X], later the z-arm plane
-    T* const Db = reinterpret_cast<T*>(smem_raw + L.o_D);
-    T* const Dp = Db + (PAD ? 1 : 0);                           // [4][ny][RS]
-    const int zrow = 4 * ny * RS;                               // PAD: a zero row
-    int* const task = reinterpret_cast<int*>(smem_raw + L.o_task);
+    T* const Dp = reinterpret_cast<T*>(smem_raw + L.o_D);       // [4][PS]: rows [ny][RS], then a zero
+    uint16_t* const task = reinterpret_cast<uint16_t*>(smem_raw + L.o_task);   // x pass: block entry << kx | row
+    uint16_t* const taskk = task + L.taskN;                     // kinetic y arm: block entry << ky | column
     int* const roff = reinterpret_cast<int*>(smem_raw + L.o_roff);
     int* const cq0 = reinterpret_cast<int*>(smem_raw + L.o_blk);   // y pass, per block of NB rows: column range, prefix
     int* const cq1 = cq0 + L.nb_y;
@@ -1760,13 +1762,14 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     int16_t* const cy0 = lx1 + 2 * ny;                          // [2][nx]: the same per column
     int16_t* const cy1 = cy0 + 2 * nx;
     uint16_t* const memb = reinterpret_cast<uint16_t*>(smem_raw + L.o_mem);   // b n_x' + x of the plane's fine members
+    const int kx = 32 - __clz(max(nyp - 1, 1)), ky = 32 - __clz(max(nxp - 1, 1));   // (n_x' n_y' < 2^14: codes < 2^16)
     const uint32_t mbar = tc::saddr(smem_raw);
     const int zL = zb + dz;
     const bool dplane = zL >= 0 && zL < nz;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t smem_n = static_cast<int64_t>(a.smem_bwd / sizeof(T));
     [[maybe_unused]] const int64_t pl_n = smem_n - L.o_pl / sizeof(T), mid_n = smem_n - L.o_mid / sizeof(T),
-                                   dp_n = smem_n - L.o_D / sizeof(T) - (PAD ? 1 : 0);
+                                   dp_n = smem_n - L.o_D / sizeof(T);
     if (tid == 0) {
         ylo = nyp;
         yhi = -1;
@@ -1786,7 +1789,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
             const int tb = (row >= 2 * ny ? 2 : 0) + (row >= 3 * ny || (row >= ny && row < 2 * ny) ? 1 : 0);
             const int y = row - tb * ny;
             for (int x = lane; x < nx; x += 32)
-                CPA(Dp, row * RS + x, dp_n, D, tb * dplane_n + y * nx + x, 8 * dplane_n);
+                CPA(Dp, tb * PS + y * RS + x, dp_n, D, tb * dplane_n + y * nx + x, 8 * dplane_n);
         }
     };
     // member x range of each row of this plane (coarse part of L', fine hull), and of the D plane
@@ -1821,11 +1824,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
             lx0[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s0, a.seg_n).x0 : -1);
             lx1[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s1 - 1, a.seg_n).x1 : -1);
         }
-        if (PAD) {
-            for (int i = tid; i < 4 * ny; i += blockDim.x)
-                for (int x = nx; x < RS; ++x) ST(Dp, i * RS + x, dp_n, T(0));
-            for (int i = tid; i < RS + 1; i += blockDim.x) ST(Db, i == 0 ? 0 : zrow + i, dp_n + 1, T(0));
-        }
+        if (tid < 4) ST(Dp, tid * PS + PS - 1, dp_n, T(0));
     }
     __syncthreads();
     const int ylo_ = ylo, yhi_ = yhi;
@@ -1930,12 +1929,16 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         }
         return lo;
     };
-    // x pass tasks, block-major: consecutive rows of a block on consecutive lanes (odd row
+    // tasks, block-major: consecutive rows (columns) of a block on consecutive lanes (odd row
     // strides: no bank conflicts, and nearly equal kinetic hulls)
-    const int ntx = hp[2 * L.nb_x];
+    const int ntx = hp[2 * L.nb_x], nty = rqp[2 * nbb];
     for (int i = tid; i < ntx; i += blockDim.x) {
         const int e = find(hp, 2 * L.nb_x, i);
-        ST(task, i, L.taskN, (e << 16) | (hlo[e] + (i - hp[e])));
+        ST(task, i, L.taskN, static_cast<uint16_t>((e << kx) | (hlo[e] + (i - hp[e]))));
+    }
+    for (int i = tid; i < nty; i += blockDim.x) {
+        const int e = find(rqp, 2 * nbb, i);
+        ST(taskk, i, L.taskkN, static_cast<uint16_t>((e << ky) | (rq0[e] + (i - rqp[e]))));
     }
     const T ks = static_cast<T>(a.kin_scale);
     const int pnp = nyp * nxp;
@@ -1969,80 +1972,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         cp_wait();
         __syncthreads();
 #endif
-        // ---- y pass: blocks of NB rows b within [ylo, yhi], per block only the listed columns
-        {
-            const int ntk = pq[nbb];
-            for (int tk = tid; tk < ntk; tk += blockDim.x) {
-                int q = 0;
-                while (tk >= pq[q + 1]) ++q;
-                const int xo = cq0[q] + (tk - pq[q]), b0 = ylo_ + q * NB;
-                T s[NB], d[NB];
-                bwd_window<T, NB>(pl, xo, X, 2 * (b0 + dy), Y, s, d, pl_n, st);
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int b = b0 + j;
-                    if (b <= yhi_) {
-                        ST(mid, b * X + xo, mid_n, s[j]);
-                        ST(mid, (nyp + b) * X + xo, mid_n, d[j]);
-                    }
-                }
-            }
-        }
-        cp_wait();                                             // the D plane
-        __syncthreads();                                       // pl is dead from here on: Gs reuses it
         T ekin_t = 0;
-        // ---- x pass (transposed filters) and kinetic x arm on the listed row blocks
-        for (int i0 = warp * 32; i0 < ntx; i0 += blockDim.x) { // whole warps: the kinetic range is a warp's
-            const bool on = i0 + lane < ntx;
-            const int code = task[on ? i0 + lane : i0];
-            const int e = code >> 16, b = code & 0xffff;
-            const int by = e >= L.nb_x, x0 = (e - by * L.nb_x) * NB;
-            T s[NB], d[NB];
-            bwd_window<T, NB>(mid, (by * nyp + b) * X, 1, 2 * (x0 + dx), X, s, d, mid_n, st);
-            if (dplane) {
-                const int y = b + dy, f0 = x0 + dx - KIN_HALF; // window position p is D position f0 + p
-                int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
-                const bool in = on && y >= 0 && y < ny;
-                if (in) {
-                    const int p0 = (bz == 0 && by == 0 ? 0 : ny) + y, p1 = ny + y;
-                    if (lx0[p0] >= 0) s0 = lx0[p0] - f0, e0 = lx1[p0] - f0 + 1;
-                    if (lx0[p1] >= 0) s1 = lx0[p1] - f0, e1 = lx1[p1] - f0 + 1;
-                }
-                s0 = __reduce_min_sync(0xffffffffu, s0);
-                e0 = __reduce_max_sync(0xffffffffu, e0);
-                s1 = __reduce_min_sync(0xffffffffu, s1);
-                e1 = __reduce_max_sync(0xffffffffu, e1);
-                T o0[NB], o1[NB], c0[NB], c1[NB];
-                const int a0 = (2 * by) * ny * RS + (in ? y * RS : 0), a1 = a0 + ny * RS;
-                auto at_x = [&](int row, int p) -> T {
-                    const int x = f0 + p;
-                    if (PAD) return LD(Db, in ? row + 1 + min(max(x, -1), nx) : zrow + 1, dp_n + 1);
-                    return in && x >= 0 && x < nx ? LD(Dp, row + x, dp_n) : T(0);
-                };
-                Arm::run(o0, o1, c0, c1, [&](int p) { return at_x(a0, p); }, [&](int p) { return at_x(a1, p); }, s0, e0,
-                         s1, e1);
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    o0[j] *= ks;
-                    o1[j] *= ks;
-                    s[j] += o0[j];
-                    d[j] += o1[j];
-                    if (on) ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
-                }
-            }
-            if (on) {
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const int xb = x0 + j;
-                    if (xb < nxp) {
-                        ST(Gs, ((0 + 2 * by) * nyp + b) * nxp + xb, pl_n, s[j]);
-                        ST(Gs, ((1 + 2 * by) * nyp + b) * nxp + xb, pl_n, d[j]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        // ---- the z-arm plane G (types tb + 4 bz, member rows) into mid, which is dead
         const T* G = static_cast<const T*>(a.ws) + r.ws_G;
         const int g_r0 = ylo_ * nxp, g_n = (yhi_ - ylo_ + 1) * nxp;
         const int slot = (pnp + 15) & ~7;                      // a type's place in mid (16-byte multiple)
@@ -2054,75 +1984,149 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
             return static_cast<int>((reinterpret_cast<uintptr_t>(src) & 15) / sizeof(T));
 #endif
         };
-        if (a.gstage) {
-#ifdef LSW_CHECKED
-            for (int tb = 0; tb < 4; ++tb)
-                for (int i = tid; i < g_n; i += blockDim.x)
-                    CPA(mid, tb * slot + i, mid_n, G, (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 + i,
-                        8 * gplane);
-#else
-            if (tid == 0) {
-                bulk_fence();
-                uint32_t total = 0;
-#pragma unroll
-                for (int tb = 0; tb < 4; ++tb)
-                    total += static_cast<uint32_t>((static_cast<size_t>(g_rem(tb) + g_n) * sizeof(T) + 15) & ~size_t(15));
-                bulk_expect(mbar, total);
-#pragma unroll
-                for (int tb = 0; tb < 4; ++tb) {
-                    const int gr = g_rem(tb);
-                    const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(gr + g_n) * sizeof(T) + 15) & ~size_t(15));
-                    bulk_load(tc::saddr(mid + tb * slot),
-                              G + (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 - gr, bytes, mbar);
-                }
-            }
-#endif
-        }
-        // ---- kinetic y arm: (x type bx, block q of NB rows, column) over the listed columns,
-        //      consecutive columns on consecutive lanes
-        if (dplane) {
-            const int nt = rqp[2 * nbb];
-            for (int i0 = warp * 32; i0 < nt; i0 += blockDim.x) {
+        // ---- phase 0, y pass: blocks of NB rows b within [ylo, yhi], the listed columns -> mid;
+        //      phase 1, x pass and kinetic x arm: the listed (y type, block of columns, row) -> Gs;
+        //      phase 2, kinetic y arm: the listed (x type, block of rows, column), added to Gs
+#pragma unroll 1
+        for (int ph = 0; ph < 3; ++ph) {
+            const int nt = ph == 0 ? pq[nbb] : ph == 1 ? ntx : dplane ? nty : 0;
+            for (int i0 = warp * 32; i0 < nt; i0 += blockDim.x) {   // whole warps: kinetic ranges are a warp's
                 const bool on = i0 + lane < nt;
                 const int it = on ? i0 + lane : i0;
-                const int e = find(rqp, 2 * nbb, it);
-                const int bx = e >= nbb, q = e - bx * nbb;
-                const int xb = rq0[e] + (it - rqp[e]), b0 = ylo_ + q * NB;
-                const int x = xb + dx, f0 = b0 + dy - KIN_HALF;
-                int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
-                if (on) {
-                    const int p0 = (bz == 0 && bx == 0 ? 0 : nx) + x, p1 = nx + x;
-                    if (cy0[p0] >= 0) s0 = cy0[p0] - f0, e0 = cy1[p0] - f0 + 1;
-                    if (cy0[p1] >= 0) s1 = cy0[p1] - f0, e1 = cy1[p1] - f0 + 1;
+                // the window: position m of the filter is at first + m on a line of n values at wp + woff
+                const T* wp = pl;
+                int woff, wstride, first, n;
+                // the arm: D row or column a0 (stride sd), window position p is D position f0 + p of kn
+                int a0 = 0, sd = 1, f0 = 0, kn = 0, dist = 0, h0 = 0, h1 = 0;
+                const int16_t *hl = lx0, *hh = lx1;
+                int out, ostep, onum, odist;                    // outputs j < onum at out + j ostep (+ odist)
+                if (ph == 0) {
+                    int q = 0;
+                    while (it >= pq[q + 1]) ++q;
+                    const int xo = cq0[q] + (it - pq[q]), b0 = ylo_ + q * NB;
+                    woff = xo;
+                    wstride = X;
+                    first = 2 * (b0 + dy);
+                    n = Y;
+                    out = b0 * X + xo;
+                    ostep = X;
+                    odist = nyp * X;
+                    onum = yhi_ + 1 - b0;
+                } else if (ph == 1) {
+                    const int code = task[it], e = code >> kx, b = code & ((1 << kx) - 1);
+                    const int by = e >= L.nb_x, x0 = (e - by * L.nb_x) * NB, y = b + dy;
+                    wp = mid;
+                    woff = (by * nyp + b) * X;
+                    wstride = 1;
+                    first = 2 * (x0 + dx);
+                    n = X;
+                    out = ((2 * by) * nyp + b) * nxp + x0;
+                    ostep = 1;
+                    odist = pnp;
+                    onum = nxp - x0;
+                    f0 = x0 + dx - KIN_HALF;
+                    const bool in = dplane && y >= 0 && y < ny;
+                    kn = in ? nx : 0;
+                    a0 = 2 * by * PS + (in ? y * RS : 0);
+                    dist = PS;
+                    h0 = (bz == 0 && by == 0 ? 0 : ny) + y;
+                    h1 = ny + y;
+                } else {
+                    const int code = taskk[it], e = code >> ky, xb = code & ((1 << ky) - 1);
+                    const int bx = e >= nbb, b0 = ylo_ + (e - bx * nbb) * NB, x = xb + dx;
+                    woff = wstride = first = n = 0;
+                    out = (bx * nyp + b0) * nxp + xb;
+                    ostep = nxp;
+                    odist = 2 * pnp;
+                    onum = yhi_ + 1 - b0;
+                    f0 = b0 + dy - KIN_HALF;
+                    kn = ny;
+                    a0 = bx * PS + x;
+                    sd = RS;
+                    dist = 2 * PS;
+                    hl = cy0;
+                    hh = cy1;
+                    h0 = (bz == 0 && bx == 0 ? 0 : nx) + x;
+                    h1 = nx + x;
                 }
-                s0 = __reduce_min_sync(0xffffffffu, s0);
-                e0 = __reduce_max_sync(0xffffffffu, e0);
-                if (s0 >= min(e0, Arm::NP) || e0 <= 0) continue;   // uniform: no member of L within reach
-                s1 = __reduce_min_sync(0xffffffffu, s1);
-                e1 = __reduce_max_sync(0xffffffffu, e1);
-                T o0[NB], o1[NB], c0[NB], c1[NB];
-                auto at_y = [&](int tb, int p) -> T {
-                    const int y = f0 + p;
-                    const bool in = y >= 0 && y < ny;
-                    if (PAD) return LD(Dp, in ? (tb * ny + y) * RS + x : zrow, dp_n);
-                    return in ? LD(Dp, (tb * ny + y) * RS + x, dp_n) : T(0);
-                };
-                Arm::run(o0, o1, c0, c1, [&](int p) { return at_y(bx, p); }, [&](int p) { return at_y(bx + 2, p); }, s0,
-                         e0, s1, e1);
-                if (on) {
+                T s[NB], d[NB];
+                if (ph < 2) {
+                    bwd_window<T, NB>(wp, woff, wstride, first, n, s, d, ph ? mid_n : pl_n, st);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < NB; ++j) s[j] = d[j] = T(0);
+                }
+                if (ph > 0 && dplane) {
+                    int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
+                    if (on && kn) {
+                        if (hl[h0] >= 0) s0 = hl[h0] - f0, e0 = hh[h0] - f0 + 1;
+                        if (hl[h1] >= 0) s1 = hl[h1] - f0, e1 = hh[h1] - f0 + 1;
+                    }
+                    s0 = __reduce_min_sync(0xffffffffu, s0);
+                    e0 = __reduce_max_sync(0xffffffffu, e0);
+                    s1 = __reduce_min_sync(0xffffffffu, s1);
+                    e1 = __reduce_max_sync(0xffffffffu, e1);
+                    // window positions inside the box, a bit each; the others read the zero after
+                    // the first type's rows and, `dist` further, after the rows of another
+                    const int plo = min(max(-f0, 0), 63), phi = min(max(kn - f0, 0), Arm::NP);
+                    const uint64_t in = phi > plo ? ((1ull << phi) - 1) & ~((1ull << plo) - 1) : 0;
+                    const uint32_t in0 = static_cast<uint32_t>(in), in1 = static_cast<uint32_t>(in >> 32);
+                    const int base = a0 + f0 * sd;
+                    T o0[NB], o1[NB], c0[NB], c1[NB];
+                    Arm::run(o0, o1, c0, c1, Dp, dp_n, dist,
+                             [&](int p) { return (p < 32 ? in0 >> (p & 31) : in1 >> (p & 31)) & 1 ? base + p * sd : PS - 1; },
+                             s0, e0, s1, e1, st);
 #pragma unroll
                     for (int j = 0; j < NB; ++j) {
-                        const int b = b0 + j;
-                        if (b <= yhi_) {
-                            o0[j] *= ks;
-                            o1[j] *= ks;
-                            const int g0 = ((bx + 0) * nyp + b) * nxp + xb, g1 = ((bx + 2) * nyp + b) * nxp + xb;
-                            ST(Gs, g0, pl_n, LD(Gs, g0, pl_n) + o0[j]);
-                            ST(Gs, g1, pl_n, LD(Gs, g1, pl_n) + o1[j]);
-                            ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
-                        }
+                        o0[j] *= ks;
+                        o1[j] *= ks;
+                        s[j] += o0[j];
+                        d[j] += o1[j];
+                        if (on && j < onum) ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
                     }
                 }
+                if (on) {
+                    T* const dst = ph == 0 ? mid : Gs;
+                    [[maybe_unused]] const int64_t dst_n = ph == 0 ? mid_n : pl_n;
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+                        if (j < onum) {
+                            const int o = out + j * ostep;
+                            if (ph == 2) {
+                                s[j] += LD(dst, o, dst_n);
+                                d[j] += LD(dst, o + odist, dst_n);
+                            }
+                            ST(dst, o, dst_n, s[j]);
+                            ST(dst, o + odist, dst_n, d[j]);
+                        }
+                }
+            }
+            if (ph == 0) cp_wait();                            // the D plane
+            if (ph < 2) __syncthreads();                       // pl is dead after phase 0 (Gs reuses it), mid after 1
+            if (ph == 1 && a.gstage) {
+                // the z-arm plane G (types tb + 4 bz, member rows) into mid
+#ifdef LSW_CHECKED
+                for (int tb = 0; tb < 4; ++tb)
+                    for (int i = tid; i < g_n; i += blockDim.x)
+                        CPA(mid, tb * slot + i, mid_n, G, (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 + i,
+                            8 * gplane);
+#else
+                if (tid == 0) {
+                    bulk_fence();
+                    uint32_t total = 0;
+#pragma unroll
+                    for (int tb = 0; tb < 4; ++tb)
+                        total += static_cast<uint32_t>((static_cast<size_t>(g_rem(tb) + g_n) * sizeof(T) + 15) & ~size_t(15));
+                    bulk_expect(mbar, total);
+#pragma unroll
+                    for (int tb = 0; tb < 4; ++tb) {
+                        const int gr = g_rem(tb);
+                        const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(gr + g_n) * sizeof(T) + 15) & ~size_t(15));
+                        bulk_load(tc::saddr(mid + tb * slot),
+                                  G + (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 - gr, bytes, mbar);
+                    }
+                }
+#endif
             }
         }
         if (a.gstage) {
@@ -2196,8 +2200,8 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
 // Persistent form (a.items_bwd set): the batch's (atom's functions, z'' plane, z type) items,
 // largest first, from the second queue counter; otherwise one CTA per grid slot (blockIdx.x =
 // 2 z'' + b_z, blockIdx.y = function).  Two CTAs of 8 warps per SM (128 registers).
-template <class T, bool PAD>
-__global__ void __launch_bounds__(256, 2) k_bwd_xy(HphiLaunch a) {
+template <class T>
+__global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2210,11 +2214,11 @@ __global__ void __launch_bounds__(256, 2) k_bwd_xy(HphiLaunch a) {
             const int k = next_item(a.queue + 1, &s_item);
             if (k >= a.n_items_bwd) break;
             const int2 it = LD(a.items_bwd, k, a.n_items_bwd);
-            bwd_plane<T, PAD>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase);
+            bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase);
             __syncthreads();   // shared memory and s_item are reused by the next item
         }
     } else {
-        bwd_plane<T, PAD>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase);
+        bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase);
     }
 }
 
@@ -2606,8 +2610,7 @@ cudaError_t configure_kernels(size_t max_smem) {
     SETMAX(k_kin_z<double>) SETMAX(k_kin_z<float>)
     SETMAX(k_z_tc<2>) SETMAX(k_z_tc<3>)
     SETMAX(k_fwd_xy_tc<2>) SETMAX(k_fwd_xy_tc<3>)
-    SETMAX((k_bwd_xy<double, false>)) SETMAX((k_bwd_xy<float, false>))
-    SETMAX((k_bwd_xy<double, true>)) SETMAX((k_bwd_xy<float, true>))
+    SETMAX(k_bwd_xy<double>) SETMAX(k_bwd_xy<float>)
     SETMAX(k_bwd_xy_tc<2>) SETMAX(k_bwd_xy_tc<3>)
     SETMAX(k_z_dens<double>) SETMAX(k_z_dens<float>)
 #undef SETMAX
@@ -2619,25 +2622,22 @@ cudaError_t configure_kernels(size_t max_smem) {
         if (fa.sharedSizeBytes > (B)) return cudaErrorInvalidConfiguration;                     \
     }
     STATIC_BOUND(k_fwd_xy<double>, FWD_STATIC_SMEM) STATIC_BOUND(k_fwd_xy<float>, FWD_STATIC_SMEM)
-    STATIC_BOUND((k_bwd_xy<double, false>), BWD_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, false>), BWD_STATIC_SMEM)
-    STATIC_BOUND((k_bwd_xy<double, true>), BWD_STATIC_SMEM) STATIC_BOUND((k_bwd_xy<float, true>), BWD_STATIC_SMEM)
+    STATIC_BOUND(k_bwd_xy<double>, BWD_STATIC_SMEM) STATIC_BOUND(k_bwd_xy<float>, BWD_STATIC_SMEM)
     STATIC_BOUND(k_bwd_xy_tc<2>, BWD_TC_STATIC_SMEM) STATIC_BOUND(k_bwd_xy_tc<3>, BWD_TC_STATIC_SMEM)
 #undef STATIC_BOUND
     return cudaSuccess;
 }
 
-cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int dpad, int* fwd, int* bwd) {
+cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int* fwd, int* bwd) {
     cudaError_t e;
     if (prec == 0) {
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(fwd, k_fwd_xy<double>, 256, smem_fwd)) != cudaSuccess)
             return e;
-        return dpad ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double, true>, 256, smem_bwd)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double, false>, 256, smem_bwd);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<double>, BWD_THREADS, smem_bwd);
     }
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(fwd, k_fwd_xy<float>, 256, smem_fwd)) != cudaSuccess)
         return e;
-    return dpad ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float, true>, 256, smem_bwd)
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float, false>, 256, smem_bwd);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bwd, k_bwd_xy<float>, BWD_THREADS, smem_bwd);
 }
 
 #define TRACED(TR, KIND, S, LAUNCH) \
@@ -2646,14 +2646,6 @@ cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int 
         LAUNCH;                         \
         trace_end(TR, S);               \
     } while (0)
-
-template <class T>
-static void bwd_xy(const HphiLaunch& a, dim3 g, cudaStream_t s) {
-    if (a.dpad)
-        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T, true><<<g, 256, a.smem_bwd, s>>>(a)));
-    else
-        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T, false><<<g, 256, a.smem_bwd, s>>>(a)));
-}
 
 template <class T>
 static cudaError_t hphi_batch(const HphiLaunch& a, cudaStream_t s) {
@@ -2693,9 +2685,9 @@ static cudaError_t hphi_batch(const HphiLaunch& a, cudaStream_t s) {
         else if (a.xy_tc && a.zsplit == 2)
             TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy_tc<2><<<dim3(2 * a.max_nzp, nf), 512, a.smem_bwd_tc, s>>>(a)));
         else
-            bwd_xy<T>(a, gbwd, s);
+            TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T><<<gbwd, BWD_THREADS, a.smem_bwd, s>>>(a)));
     } else {
-        bwd_xy<T>(a, gbwd, s);
+        TRACED(a.tr, TK_BWD_XY, s, (k_bwd_xy<T><<<gbwd, BWD_THREADS, a.smem_bwd, s>>>(a)));
     }
     return cudaGetLastError();
 }
