@@ -201,8 +201,10 @@ struct lsw_system_s {
     // atoms of each slab and the panel buffers of one slab (reused slab after slab)
     DeviceBuf d_ptiles, d_patoms, d_ttab, d_items, d_citems, d_slab_atoms, d_PA, d_PQ, d_mcoef;
     // Fermi operator expansion: transposed positions, diagonal positions, the identity on
-    // the pattern, work matrices and the dense row scratch of the triple products
-    DeviceBuf d_tpos, d_diag, d_ident, d_foe, d_foe_scratch;
+    // the pattern, work matrices, the dense row scratch of the triple products, row groups
+    DeviceBuf d_tpos, d_diag, d_ident, d_foe, d_foe_scratch, d_foe_grp;
+    int foe_ng = 0;                     // groups of rows (atoms with functions), their neighbour entries
+    int64_t foe_nn = 0;
     // confinement and preconditioning: per-atom tables of the 1D operators X_d^2, X_d^4,
     // the boxes, tables and maps of a batch, and the conjugate-gradient vectors and scalars
     DeviceBuf d_qtab, d_qtab_off, d_cbox, d_cg, d_cgs;
@@ -1717,8 +1719,19 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
     (void)cudaGetLastError();   // an earlier call's error is not this call's
     cudaStream_t st = sys->stream;
     const int triple_ctas = std::max(1, std::min(n, 4 * sys->ctx->n_sm));
+    int max_nsf = 1;
+    for (int a = 0; a < sys->n_atoms; ++a) max_nsf = std::max(max_nsf, sys->nsf[a]);
+    size_t triple_smem = static_cast<size_t>(max_nsf) * n * sizeof(double);
+    if (triple_smem > sys->ctx->max_smem - 1024) triple_smem = 0;
+    // The T_j of the recursion are kept for the sum of K' where they take at most 4 GiB; else the
+    // recursion runs a second time.
+    const bool keep = static_cast<double>(n_pl) * nnz * sizeof(double) <= 4.0 * (1ull << 30);
+    const int64_t slots = keep ? std::max(n_pl, 3) : 3;
+    const size_t need = static_cast<size_t>(std::max<int64_t>(nnz, 1)) * static_cast<size_t>(slots + 4) * sizeof(double) +
+                        static_cast<size_t>(2 * (n_pl + 1) + 1 + FOE_PARTS) * sizeof(double);
     if (sys->d_tpos.bytes == 0) {
-        // transposed and diagonal positions of the pattern, the identity on it
+        // transposed and diagonal positions of the pattern, the identity on it; the groups of
+        // rows (the functions of an atom) and their neighbours
         std::vector<int64_t> tpos(nnz), diag(n, -1);
         std::vector<double> ident(nnz, 0.0);
         for (int a = 0; a < n; ++a)
@@ -1733,19 +1746,41 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
             }
         for (int a = 0; a < n; ++a)
             if (diag[a] < 0) return fail(LSW_ERR_UNSUPPORTED, "lsw_foe: the pattern lacks a diagonal entry");
-        CUDA_TRY(sys->d_tpos.upload(tpos, st));
+        std::vector<int32_t> gfirst, grp(n), nb;       // nb: nptr, then ngrp, then npos
+        for (int f = 0; f < n; ++f) {
+            if (f == 0 || sys->sf_atom[f] != sys->sf_atom[f - 1]) gfirst.push_back(f);
+            grp[f] = static_cast<int32_t>(gfirst.size()) - 1;
+        }
+        const int ng = static_cast<int>(gfirst.size());
+        gfirst.push_back(n);
+        std::vector<int32_t> nptr(1, 0), ngrp, npos;
+        for (int g = 0; g < ng; ++g) {
+            const int64_t r0 = sys->row_ptr[gfirst[g]], r1 = sys->row_ptr[gfirst[g] + 1];
+            for (int64_t k = r0; k < r1; ++k)
+                if (k == r0 || grp[sys->col[k]] != grp[sys->col[k - 1]]) {
+                    ngrp.push_back(grp[sys->col[k]]);
+                    npos.push_back(static_cast<int32_t>(k - r0));
+                }
+            nptr.push_back(static_cast<int32_t>(ngrp.size()));
+        }
+        nb = gfirst;
+        nb.insert(nb.end(), nptr.begin(), nptr.end());
+        nb.insert(nb.end(), ngrp.begin(), ngrp.end());
+        nb.insert(nb.end(), npos.begin(), npos.end());
+        sys->foe_ng = ng;
+        sys->foe_nn = static_cast<int64_t>(ngrp.size());
         CUDA_TRY(sys->d_diag.upload(diag, st));
         CUDA_TRY(sys->d_ident.upload(ident, st));
-        CUDA_TRY(sys->d_foe.alloc(static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 9 * sizeof(double) +
-                                  static_cast<size_t>(n_pl + 1 + 2) * sizeof(double)));
-        CUDA_TRY(sys->d_foe_scratch.alloc(static_cast<size_t>(triple_ctas) * n * sizeof(double)));
-        CUDA_TRY(cudaMemsetAsync(sys->d_foe_scratch.p, 0, sys->d_foe_scratch.bytes, st));
+        CUDA_TRY(sys->d_foe_grp.upload(nb, st));
+        if (!triple_smem) {
+            CUDA_TRY(sys->d_foe_scratch.alloc(static_cast<size_t>(triple_ctas) * n * sizeof(double)));
+            CUDA_TRY(cudaMemsetAsync(sys->d_foe_scratch.p, 0, sys->d_foe_scratch.bytes, st));
+        }
+        CUDA_TRY(sys->d_tpos.upload(tpos, st));        // last: marks the plan as built
     }
-    if (sys->d_foe.bytes < static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 9 * sizeof(double) +
-                               static_cast<size_t>(n_pl + 3) * sizeof(double)) {
+    if (sys->d_foe.bytes < need) {
         CUDA_TRY(cudaStreamSynchronize(st));
-        CUDA_TRY(sys->d_foe.alloc(static_cast<size_t>(std::max<int64_t>(nnz, 1)) * 9 * sizeof(double) +
-                                  static_cast<size_t>(n_pl + 3) * sizeof(double)));
+        CUDA_TRY(sys->d_foe.alloc(need));
     }
     FoeLaunch f;
     f.n = n;
@@ -1754,45 +1789,51 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
     f.col = static_cast<const int32_t*>(sys->d_col.p);
     f.tpos = static_cast<const int64_t*>(sys->d_tpos.p);
     f.diag = static_cast<const int64_t*>(sys->d_diag.p);
+    f.ng = sys->foe_ng;
+    f.nn = sys->foe_nn;
+    f.gfirst = static_cast<const int32_t*>(sys->d_foe_grp.p);
+    f.nptr = f.gfirst + f.ng + 1;
+    f.ngrp = f.nptr + f.ng + 1;
+    f.npos = f.ngrp + f.nn;
+    f.triple_smem = triple_smem;
     f.scratch = static_cast<double*>(sys->d_foe_scratch.p);
     f.triple_ctas = triple_ctas;
-    f.cheb_ctas = std::max(1, std::min(n, 2 * sys->ctx->n_sm));
+    // as many CTAs of the Chebyshev step as the SMs hold (its map takes 4 bytes a function)
+    f.chunk = foe_cheb_smem(n, 256) <= sys->ctx->max_smem ? 256 : 32;
+    const int per_sm = static_cast<int>(std::max<size_t>(1, std::min<size_t>(8, sys->ctx->max_smem / (foe_cheb_smem(n, f.chunk) + 1024))));
+    // a CTA waits on L2 for most of a group's work: small systems spread a group over several
+    f.split = std::max(1, std::min(4, per_sm * sys->ctx->n_sm / std::max(1, f.ng)));
+    f.cheb_ctas = std::max(1, std::min(f.ng * f.split, per_sm * sys->ctx->n_sm));
     f.status = static_cast<int*>(sys->d_status.p);
     double* w = static_cast<double*>(sys->d_foe.p);
     double* Ht = w;
     double* X = w + nnz;
     double* Htp = w + 2 * nnz;
-    double* T[3] = {w + 3 * nnz, w + 4 * nnz, w + 5 * nnz};
-    double* Kc = w + 6 * nnz;
-    double* tmp = w + 7 * nnz;
-    double* tr_d = w + 9 * nnz;          // n_pl + 1 traces, then E_BS
+    double* Kc = w + 3 * nnz;
+    double* T = w + 4 * nnz;             // T_1, T_2, ... (or three slots in turn)
+    double* tr_d = w + (4 + slots) * nnz;   // n_pl + 1 traces, n_pl + 1 coefficients, E_BS, its partial sums
+    double* c_d = tr_d + n_pl + 1;
+    double* ebs_d = c_d + n_pl + 1;
     const double* I = static_cast<const double*>(sys->d_ident.p);
     const double sigma = 2.0 / (e_max - e_min), tau = 0.5 * (e_min + e_max);
     CUDA_TRY(foe_prep(f, H, S, sigma, tau, Ht, X, st));
     CUDA_TRY(foe_triple(f, X, Ht, Htp, st));
-    // the Chebyshev recursion t^{j+1} = 2 H~' t^j - t^{j-1} on every pattern column;
-    // pass 1 keeps the traces (for the search of mu), pass 2 sums K'
+    // the Chebyshev recursion t^{j+1} = 2 H~' t^j - t^{j-1} on every pattern column.  Pass 1
+    // keeps the traces (for the search of mu); K' is summed from the stored T_j or in a pass 2.
+    auto slot = [&](int j) { return T + (keep ? j - 1 : (j - 1) % 3) * nnz; };
     auto recursion = [&](const std::vector<double>* c) -> lsw_status {
-        const double* prev = I;
-        double* cur = T[0];
-        CUDA_TRY(foe_cheb(f, Htp, I, nullptr, 1.0, cur, st));
-        if (c) CUDA_TRY(foe_axpy_t(f, Kc, cur, (*c)[1], st));
-        else CUDA_TRY(foe_trace(f, cur, tr_d + 1, st));
-        int slot = 1;
-        for (int j = 2; j <= n_pl; ++j) {
-            double* next = T[slot];
-            CUDA_TRY(foe_cheb(f, Htp, cur, prev, 2.0, next, st));
-            if (c) CUDA_TRY(foe_axpy_t(f, Kc, next, (*c)[j], st));
-            else CUDA_TRY(foe_trace(f, next, tr_d + j, st));
-            prev = cur;
-            cur = next;
-            slot = (slot + 1) % 3;
-            if (T[slot] == prev) slot = (slot + 1) % 3;
+        for (int j = 1; j <= n_pl; ++j) {
+            const double* cur = j == 1 ? I : slot(j - 1);
+            const double* prev = j == 1 ? nullptr : j == 2 ? I : slot(j - 2);
+            CUDA_TRY(foe_cheb(f, Htp, cur, prev, j == 1 ? 1.0 : 2.0, slot(j), st));
+            if (c) CUDA_TRY(foe_axpy_t(f, Kc, slot(j), (*c)[j], st));
+            else if (!keep) CUDA_TRY(foe_traces(f, slot(j), 1, tr_d + j, st));
         }
         return LSW_OK;
     };
     lsw_status e = recursion(nullptr);
     if (e != LSW_OK) return e;
+    if (keep) CUDA_TRY(foe_traces(f, T, n_pl, tr_d + 1, st));
     std::vector<double> tr(n_pl + 1);
     CUDA_TRY(cudaMemcpyAsync(tr.data() + 1, tr_d + 1, n_pl * sizeof(double), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1824,17 +1865,21 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
         if (trace < n_el) lo = mu;
         else hi = mu;
     }
-    CUDA_TRY(cudaMemsetAsync(Kc, 0, nnz * sizeof(double), st));
-    CUDA_TRY(foe_axpy_t(f, Kc, I, 0.5 * c[0], st));
-    e = recursion(&c);
-    if (e != LSW_OK) return e;
+    if (keep) {
+        CUDA_TRY(cudaMemcpyAsync(c_d, c.data(), Nn * sizeof(double), cudaMemcpyHostToDevice, st));
+        CUDA_TRY(foe_kernel_sum(f, I, T, c_d, n_pl, Kc, st));
+    } else {
+        CUDA_TRY(cudaMemsetAsync(Kc, 0, nnz * sizeof(double), st));
+        CUDA_TRY(foe_axpy_t(f, Kc, I, 0.5 * c[0], st));
+        e = recursion(&c);
+        if (e != LSW_OK) return e;
+    }
     CUDA_TRY(foe_transpose(f, Kc, Kp_out, st));        // K' (columns were kept on the CSR rows)
     CUDA_TRY(foe_triple(f, X, Kp_out, K_out, st));     // K = S^-1/2 K' S^-1/2 on the pattern
-    CUDA_TRY(foe_ebs(f, K_out, Ht, S, sigma, tau, tr_d + n_pl + 1, st));
+    CUDA_TRY(foe_ebs(f, K_out, Ht, S, sigma, tau, ebs_d + 1, ebs_d, st));
     double ebs = 0.0;
-    CUDA_TRY(cudaMemcpyAsync(&ebs, tr_d + n_pl + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaMemcpyAsync(&ebs, ebs_d, sizeof(double), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    (void)tmp;
     if (mu_out) *mu_out = mu;
     if (ebs_out) *ebs_out = ebs;
     if (trace_out) *trace_out = trace;
@@ -2293,7 +2338,7 @@ lsw_status lsw_workspace_bytes(lsw_system sys, int64_t* bytes) {
                                &sys->d_sfatom, &sys->d_rowp, &sys->d_col, &sys->d_tile_fine,
                                &sys->d_listA, &sys->d_listB, &sys->d_ptiles, &sys->d_patoms, &sys->d_ttab,
                                &sys->d_items, &sys->d_citems, &sys->d_slab_atoms, &sys->d_PA, &sys->d_PQ, &sys->d_mcoef,
-                               &sys->d_tpos, &sys->d_diag, &sys->d_ident, &sys->d_foe, &sys->d_foe_scratch,
+                               &sys->d_tpos, &sys->d_diag, &sys->d_ident, &sys->d_foe, &sys->d_foe_scratch, &sys->d_foe_grp,
                                &sys->d_qtab, &sys->d_qtab_off, &sys->d_cbox, &sys->d_cg, &sys->d_cgs,
                                &sys->d_ws, &sys->d_status, &sys->d_plane_items, &sys->d_queue, &sys->d_colz,
                                &sys->d_escratch, &sys->d_phi, &sys->d_hphi, &sys->d_H, &sys->d_S, &sys->d_ek,

@@ -318,21 +318,36 @@ struct FoeLaunch {
     const int32_t* col;
     const int64_t* tpos;         // position of the transposed entry of each entry
     const int64_t* diag;         // position of the diagonal entry of each row
+    // groups: the functions of an atom, which share their pattern row
+    int ng;
+    const int32_t* gfirst;       // first function of each group (ng + 1)
+    const int32_t* nptr;         // neighbours of a group: ngrp, npos [nptr[g] .. nptr[g + 1])
+    const int32_t* ngrp;         // neighbour group
+    const int32_t* npos;         // position of its first function in the group's rows
+    int64_t nn;                  // neighbour entries
+    size_t triple_smem;          // dynamic shared memory of the grouped triple product (0: the rows
+                                 // of w do not fit; scratch is used)
     double* scratch;             // triple_ctas dense rows of n values, zero between uses
     int triple_ctas, cheb_ctas;
+    int split;                   // CTAs that share a group's neighbours in the Chebyshev step
+    int chunk;                   // entries a warp of the Chebyshev step lists at a time (a multiple of 32)
     int* status;
 };
+inline size_t foe_cheb_smem(int n, int chunk) { return (static_cast<size_t>(n) + 8 * static_cast<size_t>(chunk)) * sizeof(int); }
 cudaError_t configure_foe_kernels(size_t max_smem);
 cudaError_t foe_prep(const FoeLaunch& a, const double* H, const double* S, double sigma, double tau, double* Ht,
                      double* X, cudaStream_t s);
 cudaError_t foe_triple(const FoeLaunch& a, const double* X, const double* A, double* Y, cudaStream_t s);
 cudaError_t foe_cheb(const FoeLaunch& a, const double* Htp, const double* Tc, const double* Tp, double alpha, double* Tn,
                      cudaStream_t s);
-cudaError_t foe_trace(const FoeLaunch& a, const double* T, double* out, cudaStream_t s);
+cudaError_t foe_traces(const FoeLaunch& a, const double* T, int count, double* out, cudaStream_t s);
+cudaError_t foe_kernel_sum(const FoeLaunch& a, const double* I, const double* T, const double* c, int m, double* K,
+                           cudaStream_t s);
+constexpr int FOE_PARTS = 1024;  // partial sums of E_BS
 cudaError_t foe_axpy_t(const FoeLaunch& a, double* K, const double* T, double c, cudaStream_t s);
 cudaError_t foe_transpose(const FoeLaunch& a, const double* src, double* dst, cudaStream_t s);
 cudaError_t foe_ebs(const FoeLaunch& a, const double* K, const double* Ht, const double* S, double sigma, double tau,
-                    double* out, cudaStream_t s);
+                    double* part, double* out, cudaStream_t s);
 
 // Quartic confinement and preconditioning (lsw_confine.cu): one batch of functions
 // f0 .. f0 + nfn - 1.  Boxes (FP64, strides s_* in elements per function, x fastest, 8 types
