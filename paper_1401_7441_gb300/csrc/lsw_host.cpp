@@ -851,14 +851,17 @@ lsw_status build_hs_plan(lsw_system_s* s) {
                             it.pad = 0;
                             items.push_back(it);
                         }
+                    // combination: all of a tile's panel entries with one set of coefficients, or 128
+                    // of them where that leaves too few items to fill the GPU
+                    const int cw = static_cast<int64_t>(tiles.size()) >= 8LL * s->ctx->n_sm ? std::max(pt.kp, 1) : 128;
                     for (int a0 = 0; a0 < pt.nA; a0 += 64)
-                        for (int c0 = 0; c0 < pt.kp; c0 += 128) {
+                        for (int c0 = 0; c0 < pt.kp; c0 += cw) {
                             PanelItem it;
                             it.tile = static_cast<int32_t>(w);
                             it.a0 = a0;
                             it.na = std::min(64, pt.nA - a0);
                             it.c0 = c0;
-                            it.nc = std::min(128, pt.kp - c0);
+                            it.nc = std::min(cw, pt.kp - c0);
                             it.pad = 0;
                             citems.push_back(it);
                         }
@@ -1120,6 +1123,7 @@ PanelHSLaunch product_launch(lsw_system_s* s, Tracer* tr, const PanelSlab& sl, b
     p.nitems = combine ? sl.ci1 - sl.ci0 : sl.i1 - sl.i0;
     p.listA = static_cast<const int32_t*>(s->d_listA.p);
     p.listB = static_cast<const int32_t*>(s->d_listB.p);
+    p.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
     p.row_ptr = static_cast<const int64_t*>(s->d_rowp.p);
     p.col = static_cast<const int32_t*>(s->d_col.p);
     p.PA = s->d_PA.p;

@@ -297,6 +297,7 @@ struct PanelHSLaunch {
     int64_t nitems;
     const int32_t* listA;
     const int32_t* listB;
+    const int32_t* sf_atom;
     const int64_t* row_ptr;      // pattern CSR
     const int32_t* col;
     const void* PA;

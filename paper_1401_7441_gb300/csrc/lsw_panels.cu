@@ -12,7 +12,11 @@
 //                of the tile's points, then the 7 wavelet values of each of the tile's
 //                fine points, 0 where the function has no member (A side: phi on L; Q
 //                side: H phi on L').  The region's row tables are staged in shared
-//                memory, so a panel value costs one lookup, one load and one store.
+//                memory.  Bound by instruction issue: a lookup per panel value, with three
+//                divisions by the tile edge, was most of it; a fine point is now looked up
+//                once for its 7 wavelet values and the divisions are multiplications.  3,000
+//                atoms (8,448 functions, tile edge 6) 8.8 -> 6.9 ms; unpack (600 atoms) 0.95
+//                -> 0.41 ms.
 //   k_panel_hs   per work item (tile, up to 64 A rows, up to 128 columns of [A; Q]): the
 //                dense product of the A panel with the [A; Q] panel over the tile's
 //                panel length, 4 x 8 outputs per thread in the system's precision, then
@@ -29,6 +33,13 @@ namespace lsw {
 // ---------------------------------------------------------------- pack
 
 constexpr int PK_THREADS = 512;   // 16 warps: many tiles' loads in flight per CTA
+
+// n / d for 0 <= n < 2^16 and a loop-invariant d, 1 <= d < 2^16, by multiplication: exact there
+struct SmallDiv {
+    uint32_t m;
+    __device__ __forceinline__ explicit SmallDiv(int d) : m(d > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(d) + 1u : 0u) {}
+    __device__ __forceinline__ int div(int n) const { return m ? static_cast<int>(__umulhi(static_cast<uint32_t>(n), m)) : n; }
+};
 
 template <class T, bool Unpack>
 __global__ void __launch_bounds__(PK_THREADS, 2) k_pack(PackLaunch a) {
@@ -95,7 +106,8 @@ __global__ void __launch_bounds__(PK_THREADS, 2) k_pack(PackLaunch a) {
     const int64_t dst_n = side ? a.PQ_n : a.PA_n;
     (void)dst;
     (void)src_n;
-    const int TE = a.tile, T2 = TE * TE, T3 = T2 * TE;
+    const int TE = a.tile, T3 = TE * TE * TE;
+    const SmallDiv fd_T(TE);
     int64_t of4[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) of4[j] = j < pa.nsf ? LD(offs, pa.f0 + j, a.n_sf + 1) : 0;
@@ -111,74 +123,86 @@ __global__ void __launch_bounds__(PK_THREADS, 2) k_pack(PackLaunch a) {
         const PanelTile tl = LD(a.tiles, ent.x, a.n_tiles);
         const int kp = tl.kp;
         const int64_t base = (side ? tl.pQ : tl.pA) + static_cast<int64_t>(ent.y) * kp;
-        // offset of panel entry k inside a compressed function of the atom (-1: not a member)
-        auto rel_of = [&](int k) -> int64_t {
-            int64_t rel = -1;
-            int x = 0, y = 0, z = 0, t = 0;
-            bool coarse = k < T3, valid = false;
-            if (coarse) {
-                x = tl.org[0] + k % TE - lo[0];
-                y = tl.org[1] + (k / TE) % TE - lo[1];
-                z = tl.org[2] + k / T2 - lo[2];
-                valid = true;
-            } else {
-                const int q = (k - T3) / 7;
-                t = (k - T3) - 7 * q;
-                if (q < tl.nfine) {
-                    const int code = LD(a.tile_fine, tl.fine0 + q, a.fine_n);
-                    x = tl.org[0] + (code & 255) - lo[0];
-                    y = tl.org[1] + ((code >> 8) & 255) - lo[1];
-                    z = tl.org[2] + (code >> 16) - lo[2];
-                    valid = true;
-                }
+        // offset, inside a compressed function of the atom, of the coarse (part 0) or the first
+        // wavelet (part 1) coefficient of the tile's point (px, py, pz); -1: not a member
+        auto rel_of = [&](int part, int px, int py, int pz) -> int {
+            const int x = tl.org[0] + px - lo[0], y = tl.org[1] + py - lo[1], z = tl.org[2] + pz - lo[2];
+            if (static_cast<unsigned>(x) >= static_cast<unsigned>(n[0]) || static_cast<unsigned>(y) >= static_cast<unsigned>(n[1]) ||
+                static_cast<unsigned>(z) >= static_cast<unsigned>(n[2]))
+                return -1;
+            const int row = y + n[1] * z;
+            const int32_t* rp = part ? rpf : rpc;
+            const Seg* sg = part ? sgf : sgc;
+            const int s0 = LD(rp, row, rp_n), s1 = LD(rp, row + 1, rp_n);
+            for (int s = s0; s < s1; ++s) {
+                const Seg g = LD(sg, s, part ? sgf_n : sgc_n);
+                if (x < g.x0) break;                       // segments ascend along the row
+                if (x <= g.x1) return (part ? nc : 0) + g.off + (x - g.x0);
             }
-            if (valid && x >= 0 && y >= 0 && z >= 0 && x < n[0] && y < n[1] && z < n[2]) {
-                const int row = y + n[1] * z;
-                const int32_t* rp = coarse ? rpc : rpf;
-                const Seg* sg = coarse ? sgc : sgf;
-                const int s0 = LD(rp, row, rp_n), s1 = LD(rp, row + 1, rp_n);
-                for (int s = s0; s < s1; ++s) {
-                    const Seg g = LD(sg, s, coarse ? sgc_n : sgf_n);
-                    if (x >= g.x0 && x <= g.x1) {
-                        rel = coarse ? g.off + (x - g.x0) : nc + g.off + (x - g.x0) + static_cast<int64_t>(t) * nf;
-                        break;
-                    }
-                }
-            }
-            return rel;
+            return -1;
         };
-        if constexpr (Unpack) {
-            for (int k = lane; k < kp; k += 32) {
-                // combination result: panel row of the A side (in the Q buffer) -> members of L
-                const int64_t rel = rel_of(k);
-                if (rel >= 0)
-                    for (int j = 0; j < pa.nsf; ++j) {
-                        const int64_t o = LD(offs, pa.f0 + j, a.n_sf + 1);
-                        ST(out, o + rel, a.out_n, LD(static_cast<const T*>(a.PQ), base + static_cast<int64_t>(j) * kp + k, a.PQ_n));
-                    }
-            }
-        } else {
-            // 4 entries per lane and 4 functions at a time: 16 loads in flight before the stores
-            for (int kb = lane; kb < kp; kb += 128) {
-                int64_t rel[4];
+        // panel entries k0 + 32 u < end at offsets rel[u] (< 0: no member) and 4 functions at a
+        // time, every load before the stores
+        auto move = [&](int k0, int end, const int (&rel)[4]) {
+            for (int j0 = 0; j0 < pa.nsf; j0 += 4) {
+                T v[4][4];
+                int64_t o[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) rel[u] = kb + 32 * u < kp ? rel_of(kb + 32 * u) : -1;
-                for (int j0 = 0; j0 < pa.nsf; j0 += 4) {
-                    T v[4][4];
+                for (int j = 0; j < 4; ++j) o[j] = j0 + j < pa.nsf ? (j0 == 0 ? of4[j] : LD(offs, pa.f0 + j0 + j, a.n_sf + 1)) : 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const bool have = rel[u] >= 0 && j0 + j < pa.nsf;
+                        if constexpr (Unpack)
+                            v[u][j] = have ? LD(static_cast<const T*>(a.PQ), base + static_cast<int64_t>(j0 + j) * kp + k0 + 32 * u, a.PQ_n) : T(0);
+                        else
+                            v[u][j] = have ? LD(src, o[j] + rel[u], src_n) : T(0);
+                    }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int64_t o = j0 + j < pa.nsf ? (j0 + j < 4 ? of4[j] : LD(offs, pa.f0 + j0 + j, a.n_sf + 1)) : 0;
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            v[u][j] = (rel[u] >= 0 && j0 + j < pa.nsf) ? LD(src, o + rel[u], src_n) : T(0);
+                        if (k0 + 32 * u >= end || j0 + j >= pa.nsf) continue;
+                        if constexpr (Unpack) {            // combination result (A layout, Q buffer) -> members of L
+                            if (rel[u] >= 0) ST(out, o[j] + rel[u], a.out_n, v[u][j]);
+                        } else {
+                            ST(dst, base + static_cast<int64_t>(j0 + j) * kp + k0 + 32 * u, dst_n, v[u][j]);
+                        }
                     }
+            }
+        };
+        // coarse points
+        for (int kb = lane; kb < T3; kb += 128) {
+            int rel[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < 4; ++u) {
+                const int e = kb + 32 * u;
+                const int r = fd_T.div(e), z = fd_T.div(r);
+                rel[u] = e < T3 ? rel_of(0, e - r * TE, r - z * TE, z) : -1;
+            }
+            move(kb, T3, rel);
+        }
+        // fine points: a lane looks one up for its 7 wavelet entries, which the lanes then take
+        // in panel order; the padding after them is zero
+        for (int q0 = 0; T3 + 7 * q0 < kp; q0 += 32) {
+            int mine = -1;
+            if (q0 + lane < tl.nfine) {
+                const int code = LD(a.tile_fine, tl.fine0 + q0 + lane, a.fine_n);
+                mine = rel_of(1, code & 255, (code >> 8) & 255, code >> 16);
+            }
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (kb + 32 * u < kp && j0 + j < pa.nsf)
-                                ST(dst, base + static_cast<int64_t>(j0 + j) * kp + kb + 32 * u, dst_n, v[u][j]);
+            for (int i0 = 0; i0 < 8; i0 += 4) {
+                if (T3 + 7 * q0 + 32 * i0 >= kp) break;    // uniform
+                const int end = min(kp, T3 + 7 * q0 + 224);
+                int rel[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int e = (i0 + u) * 32 + lane, q = e / 7;     // entry of this group of 32 points (224)
+                    const int r = __shfl_sync(0xffffffffu, mine, q & 31);
+                    rel[u] = q < 32 && r >= 0 ? r + (e - 7 * q) * nf : -1;
                 }
+                move(T3 + 7 * q0 + i0 * 32 + lane, end, rel);
             }
         }
     }
@@ -652,18 +676,55 @@ __global__ void __launch_bounds__(256, 2) k_panel_hs_tc(PanelHSLaunch a) {
 // ---------------------------------------------------------------- sparse combination
 
 // (M Phi)_a = P_L(a) sum_b M_ab phi_b (Sec. "Orthogonalization", Eq. gradient): per work
-// item (tile, up to 64 A rows, up to 128 panel entries starting at c0), the A panel's
-// rows combined with the coefficients M_ab of the tile's A functions (looked up in the
+// item (tile, up to 64 A rows, a range of panel entries), the A panel's rows combined with the coefficients M_ab of the tile's A functions (looked up in the
 // pattern CSR, 0 outside it), written to the output panel at the A panel's place in the
 // Q buffer; the unpack then copies each member of L(a) from the tile holding it.
+//
+// The functions of an atom are consecutive in a tile's list and in the pattern, and their
+// pattern rows are equal: the pattern is searched once per pair of atoms (of the item's rows
+// and of a chunk of 32 functions), not once per coefficient, and the coefficients stay in shared
+// memory for all of the tile's panel entries (an item per 128 entries looked them up again).
+// 600 atoms (2,049 functions, tile edge 6): 1.32 -> 0.76 ms.
+constexpr int PC_J = PH_KC;      // functions looked up and combined per chunk
+constexpr int PC_R = 128;        // functions whose coefficients a CTA holds
+
+// Leaders of the runs of equal atoms among fn[0 .. n): ld[i] = first index of i's run, run[i] its
+// number, list[r] the leader of run r.  One warp; n <= 64.  Returns the number of runs.
+__device__ __forceinline__ int comb_runs(const int* fn, int n, const int32_t* __restrict__ sf_atom, int* ld, int* run,
+                                         int* list) {
+    const int lane = threadIdx.x & 31;
+    int runs = 0, lead = 0, last = -1;                     // carried from the first 32 to the next
+    for (int b = 0; b < n; b += 32) {
+        const int i = b + lane;
+        const int at = i < n ? sf_atom[fn[i]] : -2;
+        int before = __shfl_up_sync(0xffffffffu, at, 1);
+        if (lane == 0) before = last;
+        const unsigned m = __ballot_sync(0xffffffffu, i < n && at != before);
+        const unsigned up = m & (0xffffffffu >> (31 - lane));
+        if (i < n) {
+            ld[i] = up ? b + 31 - __clz(up) : lead;
+            run[i] = runs + __popc(up) - 1;
+            if (m >> lane & 1) list[run[i]] = i;
+        }
+        if (m) lead = b + 31 - __clz(m);
+        runs += __popc(m);
+        last = __shfl_sync(0xffffffffu, at, 31);
+    }
+    return runs;
+}
+
 template <class T>
 __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 13;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sM = reinterpret_cast<T*>(smem_raw);            // [KC][LDA]: M[a0 + i][j0 + j] at [j][i]
-    T* sP = sM + PH_KC * PH_LDA;                       // [KC][LDC]: PA[j0 + j][c0 + c] at [j][c]
-    constexpr int SM_N = PH_KC * PH_LDA, SP_N = PH_KC * PH_LDC;
+    T* sM = reinterpret_cast<T*>(smem_raw);            // [PC_R][LDA]: M[a0 + i][jb + j] at [j][i]
+    T* sP = sM + PC_R * PH_LDA;                        // [KC][LDC]: PA[j0 + j][c0 + c] at [j][c]
+    constexpr int SM_N = PC_R * PH_LDA, SP_N = PH_KC * PH_LDC;
+    __shared__ int fa[PH_M], lda[PH_M], runa[PH_M], lista[PH_M], fb[PC_J], ldb[PC_J], runb[PC_J], listb[PC_J], nrun[2];
+    __shared__ int rel[PH_M * PC_J];                   // per pair of runs: position of the leader's column in the row, -1: none
+    __shared__ long long rpa[PH_M];
+    __shared__ int lena[PH_M];
     const PanelItem it = LD(a.items, blockIdx.x, a.nitems);
     const PanelTile tl = LD(a.tiles, it.tile, a.n_tiles);
     const int kp = tl.kp;
@@ -671,86 +732,146 @@ __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
     T* PO = static_cast<T*>(const_cast<void*>(a.PQ));
     const int tid = threadIdx.x;
     const int ti = tid >> 4, tj = tid & 15;
-    const bool wide = it.nc > 64;
-    T acc[4][8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = T(0);
-    for (int j0 = 0; j0 < tl.nA; j0 += PH_KC) {
-        const int nj = min(PH_KC, tl.nA - j0);
-        // coefficients: thread (i = tid & 63, j = tid >> 6 + 4 m)
-        {
-            const int i = tid & 63;
-            int64_t r0 = 0, r1 = 0;
-            if (i < it.na) {
-                const int fa = LD(a.listA, tl.listA + it.a0 + i, a.listA_n);
-                r0 = LD(a.row_ptr, fa, a.n_sf + 1);
-                r1 = LD(a.row_ptr, fa + 1, a.n_sf + 1);
-            }
-            for (int j = tid >> 6; j < PH_KC; j += 4) {
-                T m = T(0);
-                if (i < it.na && j < nj) {
-                    const int fb = LD(a.listA, tl.listA + j0 + j, a.listA_n);
-                    int64_t lo = r0, hi = r1 - 1;
-                    while (lo <= hi) {
-                        const int64_t mid = (lo + hi) >> 1;
-                        const int cm = LD(a.col, mid, a.nnz);
-                        if (cm == fb) {
-                            m = static_cast<T>(LD(a.M, mid, a.nnz));
-                            break;
-                        }
-                        if (cm < fb) lo = mid + 1;
-                        else hi = mid - 1;
-                    }
-                }
-                ST(sM, j * PH_LDA + i, SM_N, m);
-            }
-        }
-        // panel rows j0 .. j0 + nj, entries c0 .. c0 + nc: thread (row j = tid >> 3, quad q = tid & 7 + 8 m)
-        {
-            const int j = tid >> 3;
-            for (int q = tid & 7; q < PH_N / 4; q += 8) {
-                const int c = 4 * q;
-                Quad<T> v;
-                if (j < nj && c < it.nc) ld4(v, PA, tl.pA + static_cast<int64_t>(j0 + j) * kp + it.c0 + c, a.PA_n, ST_, KID);
-                else v.zero();
-#pragma unroll
-                for (int e = 0; e < 4; ++e) ST(sP, j * PH_LDC + c + e, SP_N, v[e]);
-            }
-        }
-        __syncthreads();
-        for (int j = 0; j < nj; ++j) {
-            T av[4], cv[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) av[i] = LD(sM, j * PH_LDA + 4 * ti + i, SM_N);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) cv[c] = LD(sP, j * PH_LDC + 4 * tj + c, SP_N);
-            if (wide) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) cv[4 + c] = LD(sP, j * PH_LDC + 64 + 4 * tj + c, SP_N);
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
-            }
-        }
-        __syncthreads();
+    if (tid < it.na) {
+        const int f = LD(a.listA, tl.listA + it.a0 + tid, a.listA_n);
+        fa[tid] = f;
+        const int64_t r0 = LD(a.row_ptr, f, a.n_sf + 1);
+        rpa[tid] = r0;
+        lena[tid] = static_cast<int>(LD(a.row_ptr, f + 1, a.n_sf + 1) - r0);
     }
+    __syncthreads();
+    if (tid < 32) {
+        const int r = comb_runs(fa, it.na, a.sf_atom, lda, runa, lista);
+        if (tid == 0) nrun[0] = r;
+    }
+    for (int jb = 0; jb < tl.nA; jb += PC_R) {
+        const int nr = min(PC_R, tl.nA - jb);
+        // ---- the coefficients M[a0 ..][jb .. jb + nr), for every panel entry of the item
+        for (int j0 = 0; j0 < nr; j0 += PC_J) {
+            const int nj = min(PC_J, nr - j0);
+            if (tid < nj) fb[tid] = LD(a.listA, tl.listA + jb + j0 + tid, a.listA_n);
+            __syncthreads();
+            if (tid < 32) {
+                const int r = comb_runs(fb, nj, a.sf_atom, ldb, runb, listb);
+                if (tid == 0) nrun[1] = r;
+            }
+            __syncthreads();
+            for (int e = tid; e < nrun[0] * nrun[1]; e += blockDim.x) {
+                const int ra = e / nrun[1], rb = e - ra * nrun[1];
+                const int i = lista[ra], want = fb[listb[rb]];
+                const int64_t r0 = rpa[i];
+                int lo = 0, hi = lena[i] - 1, pos = -1;
+                while (lo <= hi) {
+                    const int mid = (lo + hi) >> 1;
+                    const int cm = LD(a.col, r0 + mid, a.nnz);
+                    if (cm == want) {
+                        pos = mid;
+                        break;
+                    }
+                    if (cm < want) lo = mid + 1;
+                    else hi = mid - 1;
+                }
+                rel[ra * PC_J + rb] = pos;
+            }
+            __syncthreads();
+            const int i = tid & 63;                    // thread (i = tid & 63, j = tid >> 6 + 4 m)
+            for (int j = tid >> 6; j < nj; j += 4) {
+                T m = T(0);
+                if (i < it.na) {
+                    const int r = rel[runa[i] * PC_J + runb[j]];
+                    if (r >= 0) m = static_cast<T>(LD(a.M, rpa[i] + r + (j - ldb[j]), a.nnz));
+                }
+                ST(sM, (j0 + j) * PH_LDA + i, SM_N, m);
+            }
+            __syncthreads();
+        }
+        // ---- their products with the panel rows, 128 entries at a time
+        for (int c0 = it.c0; c0 < it.c0 + it.nc; c0 += PH_N) {
+            const int nc = min(PH_N, it.c0 + it.nc - c0);
+            const bool wide = nc > 64;
+            T acc[4][8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = 4 * ti + i;
-        if (r >= it.na) continue;
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int cc = c < 4 ? 4 * tj + c : 64 + 4 * tj + (c - 4);
-            if (cc >= it.nc) continue;
-            ST(PO, tl.pA + static_cast<int64_t>(it.a0 + r) * kp + it.c0 + cc, a.PQ_n, acc[i][c]);
+                for (int c = 0; c < 8; ++c) {
+                    const int r = 4 * ti + i, cc = c < 4 ? 4 * tj + c : 64 + 4 * tj + (c - 4);
+                    acc[i][c] = jb > 0 && r < it.na && cc < nc      // sums of the earlier functions
+                                    ? LD(PO, tl.pA + static_cast<int64_t>(it.a0 + r) * kp + c0 + cc, a.PQ_n)
+                                    : T(0);
+                }
+            // panel rows of a chunk: thread (row j = tid >> 3, quads (tid & 7) + 8 m), a chunk ahead in registers
+            Quad<T> pre[4];
+            auto fetch = [&](int j0) {
+                const int j = tid >> 3;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int c = 4 * ((tid & 7) + 8 * m);
+                    if (j0 + j < nr && c < nc)
+                        ld4(pre[m], PA, tl.pA + static_cast<int64_t>(jb + j0 + j) * kp + c0 + c, a.PA_n, ST_, KID);
+                    else
+                        pre[m].zero();
+                }
+            };
+            fetch(0);
+            for (int j0 = 0; j0 < nr; j0 += PH_KC) {
+                const int nj = min(PH_KC, nr - j0);
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) ST(sP, (tid >> 3) * PH_LDC + 4 * ((tid & 7) + 8 * m) + e, SP_N, pre[m][e]);
+                __syncthreads();
+                if (j0 + PH_KC < nr) fetch(j0 + PH_KC);
+#ifndef LSW_CHECKED
+                if constexpr (sizeof(T) == 4) {
+                    // 16-byte shared loads and packed two-lane FMAs (the same bits as below)
+#pragma unroll 4
+                    for (int j = 0; j < nj; ++j) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(sM + (j0 + j) * PH_LDA + 4 * ti);
+                        const float4 c4 = *reinterpret_cast<const float4*>(sP + j * PH_LDC + 4 * tj);
+                        const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+                        float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (wide) d4 = *reinterpret_cast<const float4*>(sP + j * PH_LDC + 64 + 4 * tj);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float2 ai = make_float2(av[i], av[i]);
+                            const float2 r0 = __ffma2_rn(ai, make_float2(c4.x, c4.y), make_float2(acc[i][0], acc[i][1]));
+                            const float2 r1 = __ffma2_rn(ai, make_float2(c4.z, c4.w), make_float2(acc[i][2], acc[i][3]));
+                            acc[i][0] = r0.x, acc[i][1] = r0.y, acc[i][2] = r1.x, acc[i][3] = r1.y;
+                            if (wide) {
+                                const float2 r2 = __ffma2_rn(ai, make_float2(d4.x, d4.y), make_float2(acc[i][4], acc[i][5]));
+                                const float2 r3 = __ffma2_rn(ai, make_float2(d4.z, d4.w), make_float2(acc[i][6], acc[i][7]));
+                                acc[i][4] = r2.x, acc[i][5] = r2.y, acc[i][6] = r3.x, acc[i][7] = r3.y;
+                            }
+                        }
+                    }
+                } else
+#endif
+                for (int j = 0; j < nj; ++j) {
+                    T av[4], cv[8];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) av[i] = LD(sM, (j0 + j) * PH_LDA + 4 * ti + i, SM_N);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) cv[c] = LD(sP, j * PH_LDC + 4 * tj + c, SP_N);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) cv[4 + c] = wide ? LD(sP, j * PH_LDC + 64 + 4 * tj + c, SP_N) : T(0);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
+                }
+                __syncthreads();
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = 4 * ti + i;
+                if (r >= it.na) continue;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int cc = c < 4 ? 4 * tj + c : 64 + 4 * tj + (c - 4);
+                    if (cc >= nc) continue;
+                    ST(PO, tl.pA + static_cast<int64_t>(it.a0 + r) * kp + c0 + cc, a.PQ_n, acc[i][c]);
+                }
+            }
         }
     }
 }
@@ -807,7 +928,8 @@ cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s) {
 
 cudaError_t enqueue_panel_combine(const PanelHSLaunch& a, cudaStream_t s) {
     if (a.nitems == 0) return cudaSuccess;
-    const size_t smem = panel_hs_smem(a.prec);
+    const size_t smem = (static_cast<size_t>(PC_R) * PH_LDA + static_cast<size_t>(PH_KC) * PH_LDC) *
+                        (a.prec == 0 ? sizeof(double) : sizeof(float));
     if (a.prec == 0)
         TRACED(a.tr, TK_HS, s, (k_panel_combine<double><<<static_cast<unsigned>(a.nitems), 256, smem, s>>>(a)));
     else
