@@ -447,12 +447,14 @@ lsw_status build_pattern(lsw_system_s* s) {
 
 int64_t align64(int64_t x) { return (x + ALIGN_ELEMS - 1) / ALIGN_ELEMS * ALIGN_ELEMS; }
 
-// Dynamic shared memory of the pass kernels for a function record.
-void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z) {
+// Dynamic shared memory of the pass kernels for a function record.  z_lim: the size that decides
+// whether a box is taken (separate buffers of inputs and products).
+void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z, size_t* z_lim) {
     const int64_t X = 2 * r.n[0] + 29, Z = 2 * r.n[2] + 29;
     const int64_t RS = r.n[0] | 1;
     *fwd = es * static_cast<size_t>(4 * r.n[1] * RS + 2 * r.n[1] * X);
-    *z = es * static_cast<size_t>((2 * r.n[2] + Z) * zcols);
+    *z = es * static_cast<size_t>((2 * r.n[2] + 30) * zcols);
+    *z_lim = es * static_cast<size_t>((2 * r.n[2] + Z) * zcols);
 }
 
 // Backward plane kernel: sizes of its four layouts over a batch's functions, and the choice.
@@ -460,6 +462,7 @@ void pass_smem(const FnRec& r, size_t es, int zcols, size_t* fwd, size_t* z) {
 // latencies stay uncovered), then the staged z-arm plane, then the lists.
 struct BwdSizes {
     size_t b[2][2] = {{0, 0}, {0, 0}};                 // [gstage][lists]
+    size_t z_lim = 0;                                  // (allocation-free path) the z stage's, see pass_smem
     void fold(const FnRec& r, int es) {
         for (int g = 0; g < 2; ++g)
             for (int p = 0; p < 2; ++p)
@@ -557,6 +560,7 @@ lsw_status build_plans(lsw_system_s* s) {
         p.zcols = zcols;
         p.fwd_list = s->fwd_list;
         BwdSizes bwd;
+        size_t smem_z_lim = 0;
         int64_t o = 0;
         for (int64_t f = f0; f < f0 + b.nfn; ++f) {
             recs[f].ws_D = o;
@@ -590,11 +594,12 @@ lsw_status build_plans(lsw_system_s* s) {
             p.max_rowsL = std::max(p.max_rowsL, r.n[1] * r.n[2]);
             p.max_segL = std::max<int>(p.max_segL, static_cast<int>((Lh.c.keys.size() + Lh.f.keys.size()) / 3));
             p.max_segP = std::max<int>(p.max_segP, static_cast<int>((Ph.c.keys.size() + Ph.f.keys.size()) / 3));
-            size_t a1, a2;
-            pass_smem(r, s->esize, zcols, &a1, &a2);
+            size_t a1, a2, a3;
+            pass_smem(r, s->esize, zcols, &a1, &a2, &a3);
+            smem_z_lim = std::max(smem_z_lim, a3);
             p.smem_fwd = std::max(p.smem_fwd, a1);
             p.smem_z = std::max(p.smem_z, a2);
-            p.smem_kin = std::max(p.smem_kin, static_cast<size_t>(2 * r.n[2] * 128) * (p.prec == 0 ? 8 : 4));
+            p.smem_kin = std::max(p.smem_kin, static_cast<size_t>(2 * (r.n[2] + 1) * 128) * (p.prec == 0 ? 8 : 4));
             bwd.fold(r, static_cast<int>(s->esize));
             if (s->zsplit) {
                 if (!ztc_fits(r))
@@ -610,11 +615,11 @@ lsw_status build_plans(lsw_system_s* s) {
         }
         p.zsplit = s->zsplit;
         p.xy_tc = s->zsplit ? s->xy_tc : 0;
-        if (!bwd.choose(s->ctx->max_smem, &p) || p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || p.smem_z > s->ctx->max_smem ||
+        if (!bwd.choose(s->ctx->max_smem, &p) || p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || smem_z_lim > s->ctx->max_smem ||
             p.smem_ztc > s->ctx->max_smem || p.smem_kin > s->ctx->max_smem || p.smem_bwd_tc + BWD_TC_STATIC_SMEM > s->ctx->max_smem ||
             p.smem_fwd_tc > s->ctx->max_smem)
             return fail(LSW_ERR_UNSUPPORTED, "locreg box too large for the on-chip pass tiles (%zu/%zu/%zu/%zu > %zu bytes)",
-                        p.smem_fwd, p.smem_z, bwd.b[0][0], p.smem_ztc, s->ctx->max_smem);
+                        p.smem_fwd, smem_z_lim, bwd.b[0][0], p.smem_ztc, s->ctx->max_smem);
         // persistent FMA plane kernels: the batch's (functions, plane, z type) items, largest
         // first (stable in function and plane order), and as many CTAs as fit.  The backward
         // kernel's items take an atom's functions together (their tables are built once), as
@@ -1363,11 +1368,12 @@ void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* 
     p->max_rowsL = std::max(p->max_rowsL, r.n[1] * r.n[2]);
     p->max_segL = std::max<int>(p->max_segL, static_cast<int>((Lh.c.keys.size() + Lh.f.keys.size()) / 3));
     p->max_segP = std::max<int>(p->max_segP, static_cast<int>((Ph.c.keys.size() + Ph.f.keys.size()) / 3));
-    size_t a1, a2;
-    pass_smem(r, s->esize, zcols, &a1, &a2);
+    size_t a1, a2, a3;
+    pass_smem(r, s->esize, zcols, &a1, &a2, &a3);
+    bwd->z_lim = std::max(bwd->z_lim, a3);
     p->smem_fwd = std::max(p->smem_fwd, a1);
     p->smem_z = std::max(p->smem_z, a2);
-    p->smem_kin = std::max(p->smem_kin, static_cast<size_t>(2 * r.n[2] * 128) * (p->prec == 0 ? 8 : 4));
+    p->smem_kin = std::max(p->smem_kin, static_cast<size_t>(2 * (r.n[2] + 1) * 128) * (p->prec == 0 ? 8 : 4));
     bwd->fold(r, static_cast<int>(s->esize));
     if (s->zsplit) {
         p->smem_ztc = std::max(p->smem_ztc, ztc_smem(r, s->zsplit));
@@ -1381,7 +1387,7 @@ void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* 
 bool noalloc_finish(const lsw_system_s* s, HphiLaunch* p, const BwdSizes& bwd) {
     const size_t mx = s->ctx->max_smem;
     return bwd.choose(mx, p) &&
-           !(p->smem_fwd + FWD_STATIC_SMEM > mx || p->smem_z > mx || p->smem_ztc > mx ||
+           !(p->smem_fwd + FWD_STATIC_SMEM > mx || bwd.z_lim > mx || p->smem_ztc > mx ||
              p->smem_kin > mx || p->smem_bwd_tc + BWD_TC_STATIC_SMEM > mx || p->smem_fwd_tc > mx);
 }
 }  // namespace

@@ -363,6 +363,59 @@ __device__ __forceinline__ void kin_block<float>(const float (&k0)[KW], const fl
 }
 #endif
 
+// FP64 forms (bound by the FP64 pipe, 1/64 of the FP32 rate): products only where the input can
+// be nonzero, decided position by position.  8 outputs of the upsampling block at coarse step
+// q0 + 15 from the inputs ld(b, q), q within [l0, h0] for the first type, [l1, h1] for the second.
+template <class T, class Ld>
+__device__ __forceinline__ void fwd_range(T (&u)[2 * FB], Ld ld, int q0, int l0, int h0, int l1, int h1) {
+#pragma unroll
+    for (int k = 0; k < 2 * FB; ++k) u[k] = T(0);
+#pragma unroll
+    for (int i = 0; i < FW; ++i) {
+        const int q = q0 + i;
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            if (q < (b ? l1 : l0) || q > (b ? h1 : h0)) continue;
+            const T v = ld(b, q);
+#pragma unroll
+            for (int j = 0; j < FB; ++j) {
+                const int k = j + 15 - i;
+                if (k < 0 || k > 15) continue;
+                u[2 * j] += Tab<T>::fwd(b, 2 * k) * v;
+                if (k < 15) u[2 * j + 1] += Tab<T>::fwd(b, 2 * k + 1) * v;
+            }
+        }
+    }
+}
+
+// The transposed filters of N coarse outputs from the window starting at position `first` of a
+// line of n values.  FP32: as bwd_block.  FP64 (bound by the FP64 pipe): positions outside the
+// line are skipped, not multiplied as zeros.
+template <class T, int NB>
+__device__ __forceinline__ void bwd_window(const T* p, int off, int stride, int first, int n, T (&s)[NB], T (&d)[NB],
+                                           int64_t room, int* st) {
+    if constexpr (sizeof(T) == 4) {
+        T w[2 * NB + 29];
+        swin(w, p, off, stride, first, n, room, st);
+        bwd_block<T, NB>(w, s, d);
+    } else {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) s[j] = d[j] = T(0);
+#pragma unroll
+        for (int m = 0; m < 2 * NB + 29; ++m) {
+            const int pos = first + m;
+            if (pos < 0 || pos >= n) continue;
+            const T v = WLD(p, off + pos * stride, room);
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (m - 2 * j >= 0 && m - 2 * j < FWD_TAPS) {
+                    s[j] += Tab<T>::fwd(0, m - 2 * j) * v;
+                    d[j] += Tab<T>::fwd(1, m - 2 * j) * v;
+                }
+        }
+    }
+}
+
 // ---------------------------------------------------------------- forward x, y
 
 template <class T>
@@ -470,15 +523,42 @@ __device__ __forceinline__ void fwd_plane(const HphiLaunch& a, int fl, int z, in
             const int row = by * ny + y;
             const int p0 = blk * FB;
             const int s0 = ((2 * by) * ny + y) * RS, d0 = s0 + ny * RS;
-            T w0[FW], w1[FW], u[2 * FB];
-            swin(w0, in, s0, 1, p0 - 15, nx, smem_n, st);
-            swin(w1, in, d0, 1, p0 - 15, nx, smem_n, st);
-            fwd_block(w0, w1, u);
+            T u[2 * FB];
+            if constexpr (sizeof(T) == 4) {
+                T w0[FW], w1[FW];
+                swin(w0, in, s0, 1, p0 - 15, nx, smem_n, st);
+                swin(w1, in, d0, 1, p0 - 15, nx, smem_n, st);
+                fwd_block(w0, w1, u);
+            } else {
+                // the row's members where they are listed (of both types: the second's are fine)
+                const int l0 = listed ? ix0[by][y] : 0, h0 = listed ? ix1[by][y] : nx - 1;
+                const int l1 = listed ? ix0[1][y] : 0, h1 = listed ? ix1[1][y] : nx - 1;
+                fwd_range<T>(u, [&](int b, int q) { return LD(in, (b ? d0 : s0) + q, smem_n); }, p0 - 15, max(l0, 0),
+                             l0 < 0 ? -1 : h0, max(l1, 0), l1 < 0 ? -1 : h1);
+            }
 #pragma unroll
             for (int k = 0; k < 2 * FB; ++k) {
                 const int xo = 2 * p0 + k;
                 if (xo < X) ST(mid, row * X + xo, mid_n, u[k]);
             }
+        }
+    }
+    // rows with members, per y type (FP64: the y pass sums over them)
+    [[maybe_unused]] __shared__ int yh[4];
+    if constexpr (sizeof(T) == 8) {
+        if (threadIdx.x < 2) {
+            int lo = 0, hi = ny - 1;
+            if (listed) {
+                lo = ny;
+                hi = -1;
+                for (int y = 0; y < ny; ++y)
+                    if (ix0[threadIdx.x][y] >= 0) {
+                        lo = min(lo, y);
+                        hi = y;
+                    }
+            }
+            yh[2 * threadIdx.x] = lo;
+            yh[2 * threadIdx.x + 1] = hi;
         }
     }
     __syncthreads();
@@ -490,10 +570,16 @@ __device__ __forceinline__ void fwd_plane(const HphiLaunch& a, int fl, int z, in
     for (int task = threadIdx.x; task < X * nby; task += blockDim.x) {
         const int blk = fd_X.div(task), xo = task - blk * X;
         const int p0 = blk * FB;
-        T w0[FW], w1[FW], u[2 * FB];
-        swin(w0, mid, xo, X, p0 - 15, ny, mid_n, st);
-        swin(w1, mid, ny * X + xo, X, p0 - 15, ny, mid_n, st);
-        fwd_block(w0, w1, u);
+        T u[2 * FB];
+        if constexpr (sizeof(T) == 4) {
+            T w0[FW], w1[FW];
+            swin(w0, mid, xo, X, p0 - 15, ny, mid_n, st);
+            swin(w1, mid, ny * X + xo, X, p0 - 15, ny, mid_n, st);
+            fwd_block(w0, w1, u);
+        } else {
+            fwd_range<T>(u, [&](int b, int q) { return LD(mid, (b * ny + q) * X + xo, mid_n); }, p0 - 15, yh[0], yh[1], yh[2],
+                         yh[3]);
+        }
 #pragma unroll
         for (int k = 0; k < 2 * FB; ++k) {
             const int yo = 2 * p0 + k;
@@ -534,6 +620,16 @@ __global__ void __launch_bounds__(256) k_fwd_xy(HphiLaunch a) {
 
 // ---------------------------------------------------------------- z stage with V
 
+// One thread per real-space column (x', y'): 8 outputs u of the synthesis + magic filter at a
+// time from the column's coefficients, times V, then the transposed filters back.  The column
+// lives in one shared buffer of 2 n_z + 30 slots per thread: input (b, q) starts in slot
+// 30 + 2 q + b, and the block of outputs 2 p0 .. 2 p0 + 7 overwrites slots that no later block
+// reads (the next one starts at input p0 - 11, slot 2 p0 + 8).  With the inputs and the
+// products in buffers of their own, shared memory held 8 warps per SM and the kernel waited on
+// its own latencies (issue 54 %): 3.0 -> 2.4 us per function at radii 5-8 bohr.  V is fetched a block ahead into registers.
+// FP64 (bound by the FP64 pipe): products run over the hull of the warp's nonzero inputs, per
+// type, and within the column, not over zeros: 82 -> 53 us per function at 6 bohr.
+constexpr int Z_HEAD = 30;            // slots ahead of the inputs
 template <class T>
 __global__ void __launch_bounds__(ZCols<T>::C) k_z(HphiLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
@@ -543,7 +639,7 @@ __global__ void __launch_bounds__(ZCols<T>::C) k_z(HphiLaunch a) {
     constexpr int C = ZCols<T>::C;       // columns per block = threads; a compile-time
                                          // stride turns window offsets into immediates
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sm = reinterpret_cast<T*>(smem_raw);
+    T* sm = reinterpret_cast<T*>(smem_raw);   // [2 nz + 30][C] (each thread owns its column)
     const FnRec r = a.fn[blockIdx.y];
     const int nx = r.n[0], ny = r.n[1], nz = r.n[2];
     const int X = 2 * nx + 29, Y = 2 * ny + 29, Z = 2 * nz + 29;
@@ -552,54 +648,78 @@ __global__ void __launch_bounds__(ZCols<T>::C) k_z(HphiLaunch a) {
     if (blockIdx.x * C >= cols) return;
     const bool valid = c < cols;
     const int t = threadIdx.x;
-    T* cin = sm;                  // [2][nz][C]  (each thread owns its column)
-    T* vs = sm + 2 * nz * C;      // [Z][C]
     [[maybe_unused]] const int64_t smem_n = static_cast<int64_t>(a.smem_z / sizeof(T));
-    [[maybe_unused]] const int64_t vs_n = smem_n - 2 * nz * C;
     const T* Bf = static_cast<const T*>(a.ws) + r.ws_Bf;
     T epot_t = 0;   // per-thread partial in the kernel's precision (no FP64 in FP32 loops)
+    int hl[2] = {0, 0}, hh[2] = {nz - 1, nz - 1};
+    if (valid)
+        for (int q = 0; q < nz; ++q)
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+                CPA(sm, (Z_HEAD + 2 * q + b) * C + t, smem_n, Bf, static_cast<int64_t>(b * nz + q) * cols + c, 2LL * nz * cols);
+    cp_wait();   // each thread reads only its own column: no barrier needed
+    if constexpr (sizeof(T) == 8) {
+        const unsigned all = __ballot_sync(0xffffffffu, valid);
+        if (valid)
+            for (int b = 0; b < 2; ++b) {
+                hl[b] = nz;
+                hh[b] = -1;
+                for (int q = 0; q < nz; ++q)
+                    if (__any_sync(all, (__double_as_longlong(LD(sm, (Z_HEAD + 2 * q + b) * C + t, smem_n)) << 1) != 0)) {
+                        hl[b] = min(hl[b], q);
+                        hh[b] = q;
+                    }
+            }
+    }
     if (valid) {
-        // Stage the column's input and its slice of V first: all loads independent and
-        // in flight together (the multiply below then reads V from shared memory).
         const int xo = c % X, yo = c / X;
         const int64_t jx = 2LL * r.lo[0] - V_REACH + xo - a.vlo[0];
         const int64_t jy = 2LL * r.lo[1] - V_REACH + yo - a.vlo[1];
         const int64_t jz0 = 2LL * r.lo[2] - V_REACH - a.vlo[2];
         const T* V = static_cast<const T*>(a.V);
-        const int64_t vrow = jy * a.vn[0] + jx;
         const int64_t vstride = a.vn[0] * a.vn[1];
-        for (int q = 0; q < 2 * nz; ++q)
-            CPA(cin, q * C + t, smem_n, Bf, static_cast<int64_t>(q) * cols + c, 2LL * nz * cols);
-        for (int zo = 0; zo < Z; ++zo)
-            CPA(vs, zo * C + t, vs_n, V, (jz0 + zo) * vstride + vrow, a.v_n);
-        cp_wait();   // each thread reads only its own column: no barrier needed
+        const int64_t v0 = jz0 * vstride + jy * a.vn[0] + jx;
+        T vn[2 * FB];
+#pragma unroll
+        for (int k = 0; k < 2 * FB; ++k) vn[k] = k < Z ? LD(V, v0 + k * vstride, a.v_n) : T(0);
         for (int p0 = 0; 2 * p0 < Z; p0 += FB) {
-            T w0[FW], w1[FW], u[2 * FB];
+            T u[2 * FB], vv[2 * FB];
             const int q0 = p0 - 15;
-            if (q0 >= 0 && q0 + FW <= nz) {
 #pragma unroll
-                for (int i = 0; i < FW; ++i) {
-                    w0[i] = LD(cin, (q0 + i) * C + t, smem_n);
-                    w1[i] = LD(cin, (nz + q0 + i) * C + t, smem_n);
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < FW; ++i) {
-                    const int q = q0 + i;
-                    const bool ok = q >= 0 && q < nz;
-                    w0[i] = ok ? LD(cin, q * C + t, smem_n) : T(0);
-                    w1[i] = ok ? LD(cin, (nz + q) * C + t, smem_n) : T(0);
-                }
+            for (int k = 0; k < 2 * FB; ++k) {
+                vv[k] = vn[k];
+                const int zo = 2 * (p0 + FB) + k;
+                if (zo < Z) vn[k] = LD(V, v0 + zo * vstride, a.v_n);
             }
-            fwd_block(w0, w1, u);
+            if constexpr (sizeof(T) == 4) {
+                T w0[FW], w1[FW];
+                if (q0 >= 0 && q0 + FW <= nz) {
+#pragma unroll
+                    for (int i = 0; i < FW; ++i) {
+                        w0[i] = LD(sm, (Z_HEAD + 2 * (q0 + i)) * C + t, smem_n);
+                        w1[i] = LD(sm, (Z_HEAD + 2 * (q0 + i) + 1) * C + t, smem_n);
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < FW; ++i) {
+                        const int q = q0 + i;
+                        const bool ok = q >= 0 && q < nz;
+                        w0[i] = ok ? LD(sm, (Z_HEAD + 2 * q) * C + t, smem_n) : T(0);
+                        w1[i] = ok ? LD(sm, (Z_HEAD + 2 * q + 1) * C + t, smem_n) : T(0);
+                    }
+                }
+                fwd_block(w0, w1, u);
+            } else {
+                fwd_range<T>(u, [&](int b, int q) { return LD(sm, (Z_HEAD + 2 * q + b) * C + t, smem_n); }, q0, hl[0], hh[0],
+                             hl[1], hh[1]);
+            }
 #pragma unroll
             for (int k = 0; k < 2 * FB; ++k) {
                 const int zo = 2 * p0 + k;
                 if (zo < Z) {
-                    const T vv = LD(vs, zo * C + t, vs_n);
-                    const T v = vv * u[k];
+                    const T v = vv[k] * u[k];
                     epot_t += v * u[k];
-                    ST(vs, zo * C + t, vs_n, v);
+                    ST(sm, zo * C + t, smem_n, v);
                 }
             }
         }
@@ -607,19 +727,24 @@ __global__ void __launch_bounds__(ZCols<T>::C) k_z(HphiLaunch a) {
         const int dz = r.lop[2] - r.lo[2];
         T* Bb = static_cast<T*>(a.ws) + r.ws_Bb;
         for (int b0 = 0; b0 < nzp; b0 += NB) {
-            T w[W], s[NB], d[NB];
+            T s[NB], d[NB];
             const int z0 = 2 * (b0 + dz);
-            if (z0 >= 0 && z0 + W <= Z) {
+            if constexpr (sizeof(T) == 4) {
+                T w[W];
+                if (z0 >= 0 && z0 + W <= Z) {
 #pragma unroll
-                for (int i = 0; i < W; ++i) w[i] = LD(vs, (z0 + i) * C + t, vs_n);
-            } else {
+                    for (int i = 0; i < W; ++i) w[i] = LD(sm, (z0 + i) * C + t, smem_n);
+                } else {
 #pragma unroll
-                for (int i = 0; i < W; ++i) {
-                    const int zo = z0 + i;
-                    w[i] = (zo >= 0 && zo < Z) ? LD(vs, zo * C + t, vs_n) : T(0);
+                    for (int i = 0; i < W; ++i) {
+                        const int zo = z0 + i;
+                        w[i] = (zo >= 0 && zo < Z) ? LD(sm, zo * C + t, smem_n) : T(0);
+                    }
                 }
+                bwd_block<T, NB>(w, s, d);
+            } else {
+                bwd_window<T, NB>(sm, t, C, z0, Z, s, d, smem_n, a.status);
             }
-            bwd_block<T, NB>(w, s, d);
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
                 const int b = b0 + j;
@@ -1042,13 +1167,78 @@ __global__ void __launch_bounds__(256) k_fwd_xy_tc(HphiLaunch a) {
     if (warp == 0) tc::tmem_free(tmem, 128);
 }
 
+// Kinetic arm of N outputs (both types of a pair) from the window positions p = 0 .. NP - 1 of two
+// lines: position p of the first line is D[off(p)], of the second D[off(p) + dist].  [s0, e0), [s1,
+// e1): the positions of either line that can be nonzero, uniform over the warp, the second
+// within the first.  c0, c1: the lines' values at the outputs.
+template <class T>
+struct KinArm {
+    static constexpr int N = Blk<T, 1>::NB;            // outputs per block, both arms
+    static constexpr int NP = N + 2 * KIN_HALF;        // window positions
+    static constexpr int G = sizeof(T) == 4 ? 4 : 1;   // positions per group
+    template <class Off>
+    static __device__ __forceinline__ void run(T (&o0)[N], T (&o1)[N], T (&c0)[N], T (&c1)[N], const T* D, int64_t dn,
+                                               int dist, Off off, int s0, int e0, int s1, int e1,
+                                               [[maybe_unused]] int* st) {
+        [[maybe_unused]] int* ST_ = st;
+        [[maybe_unused]] constexpr int KID = 4;
+        float2 acc[sizeof(T) == 4 ? N : 1];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            o0[j] = o1[j] = c0[j] = c1[j] = T(0);
+            if constexpr (sizeof(T) == 4) acc[j] = make_float2(0.f, 0.f);
+        }
+        auto add = [&](int p, int src, T v) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                if (p - j < 0 || p - j >= KIN_TAPS) continue;
+                if constexpr (sizeof(T) == 4) {
+                    acc[j] = __ffma2_rn(c_kin2[src][p - j], make_float2(v, v), acc[j]);
+                } else {
+                    o0[j] += Tab<T>::kin(src, p - j) * v;
+                    o1[j] += Tab<T>::kin(2 + src, p - j) * v;
+                }
+            }
+        };
+#pragma unroll
+        for (int g = 0; g < NP; g += G) {
+            if (g + G - 1 < s0 || g >= e0) continue;
+            int at[G];
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                at[k] = off(g + k);
+                const T v = LD(D, at[k], dn);
+                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c0[(g + k - KIN_HALF) & (N - 1)] = v;
+                add(g + k, 0, v);
+            }
+            if (g + G - 1 < s1 || g >= e1) continue;
+#pragma unroll
+            for (int k = 0; k < G; ++k) {
+                const T v = LD(D, at[k] + dist, dn);
+                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c1[(g + k - KIN_HALF) & (N - 1)] = v;
+                add(g + k, 1, v);
+            }
+        }
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                o0[j] = acc[j].x;
+                o1[j] = acc[j].y;
+            }
+        }
+    }
+};
+
 // ---------------------------------------------------------------- kinetic z arm
 
 // Per (x, y) column of the L box and type pair (t, t + 4): the kinetic arm along z,
 // written to G on the L' box column (G holds only this arm; the backward plane kernel
 // adds the rest).  Runs before the backward plane kernel.  The column pair is staged in
 // shared memory; a column pair that is zero (outside the L sphere, or wavelet types off
-// the fine region) only clears its flag, and the plane kernel then skips its G.
+// the fine region) only clears its flag, and the plane kernel then skips its G.  Products run
+// over the hull of a warp's nonzero inputs, 8 planes (FP64: 4) per block: with the whole window,
+// its bounds tests and 4 planes per block it issued about twice the instructions.
+// 0.79 -> 0.61 us per function at radii 5-8 bohr, FP64 27 -> 11 us at 6 bohr.
 template <class T>
 __global__ void __launch_bounds__(128) k_kin_z(HphiLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
@@ -1064,55 +1254,75 @@ __global__ void __launch_bounds__(128) k_kin_z(HphiLaunch a) {
     const int t = threadIdx.x;
     const int c = blockIdx.x * 128 + t;                    // column (x, y) of the L box
     const int tb = blockIdx.z;                             // type pair (tb, tb + 4)
-    T* col = reinterpret_cast<T*>(smem_raw);               // [2][nz][128]: this thread's column pair
+    T* col = reinterpret_cast<T*>(smem_raw);               // [2][nz + 1][128]: this thread's column pair, each with a zero row
+    using Arm = KinArm<T>;
     [[maybe_unused]] const int64_t col_n = static_cast<int64_t>(a.smem_kin / sizeof(T));
     unsigned char* flag = reinterpret_cast<unsigned char*>(static_cast<T*>(a.ws) + r.ws_Gf) + tb * pn;
     T ekin_t = 0;
+    int hl[2] = {nz, nz}, hh[2] = {-1, -1};                // hulls of the pair's nonzero inputs
+    int zlo = nzp, zhi = -1;                               // planes of L' this column writes
+    int64_t gcol = 0;
+    ST(col, nz * 128 + t, col_n, T(0));
+    ST(col, (2 * nz + 1) * 128 + t, col_n, T(0));
     if (c < pn) {
         const T* D = static_cast<const T*>(a.ws) + r.ws_D;
         const int64_t plane = static_cast<int64_t>(nx) * ny * nz;
         for (int q = 0; q < nz; ++q) {
             CPA(col, q * 128 + t, col_n, D, tb * plane + static_cast<int64_t>(q) * pn + c, 8 * plane);
-            CPA(col, (nz + q) * 128 + t, col_n, D, (tb + 4) * plane + static_cast<int64_t>(q) * pn + c, 8 * plane);
+            CPA(col, (nz + 1 + q) * 128 + t, col_n, D, (tb + 4) * plane + static_cast<int64_t>(q) * pn + c, 8 * plane);
         }
         cp_wait();
-        bool nonzero = false;
-        for (int q = 0; q < 2 * nz; ++q) nonzero |= LD(col, q * 128 + t, col_n) != T(0);
+        for (int q = 0; q < nz; ++q)
+#pragma unroll
+            for (int b = 0; b < 2; ++b)
+                if (LD(col, (b * (nz + 1) + q) * 128 + t, col_n) != T(0)) {
+                    hl[b] = min(hl[b], q);
+                    hh[b] = q;
+                }
+        const bool nonzero = max(hh[0], hh[1]) >= 0;
         ST(flag, c, 4LL * pn, nonzero ? 1 : 0);
         const int y = c / nx, x = c - y * nx;
         const int xb = x - dx, yb = y - dy;             // the same column in the L' box
         if (nonzero && xb >= 0 && xb < nxp && yb >= 0 && yb < nyp) {
-            T* G = static_cast<T*>(a.ws) + r.ws_G;
-            const int64_t gplane = static_cast<int64_t>(nxp) * nyp * nzp;
-            const int64_t pnp = static_cast<int64_t>(nxp) * nyp;
-            const int64_t gcol = static_cast<int64_t>(yb) * nxp + xb;
-            const T ks = static_cast<T>(a.kin_scale);
+            gcol = static_cast<int64_t>(yb) * nxp + xb;
             // the planes of this column the compressed H phi reads: the coarse members' z
             // range where the pair holds type 0 (tb = 0), else the fine members' z hull (the
             // D values of the pair are zero off those, so E_kin loses no term)
-            int zlo = 0, zhi = nzp - 1;
+            zlo = 0;
+            zhi = nzp - 1;
             if (a.colz) {
                 const ColZ cz = LD(a.colz, a.atoms[r.atom].colz + gcol, a.colz_n);
                 zlo = tb == 0 ? cz.c0 : cz.f0;
                 zhi = tb == 0 ? cz.c1 : cz.f1;
+                if (zlo < 0) zlo = nzp;
             }
-            for (int b0 = zlo < 0 ? nzp : (zlo / BB) * BB; b0 <= zhi; b0 += BB) {
-                T k0[KW], k1[KW], o0[BB], o1[BB];
-                swin(k0, col, t, 128, b0 + dz - KIN_HALF, nz, col_n, st);
-                swin(k1, col, nz * 128 + t, 128, b0 + dz - KIN_HALF, nz, col_n, st);
-                kin_block(k0, k1, o0, o1);
+        }
+    }
+    // a warp's columns together: the blocks of planes any of them needs, products over the hull
+    // of their nonzero inputs (positions outside the column read the zero row)
+    const int z0 = __reduce_min_sync(0xffffffffu, zlo), z1 = __reduce_max_sync(0xffffffffu, zhi);
+    const int l0 = __reduce_min_sync(0xffffffffu, hl[0]), h0 = __reduce_max_sync(0xffffffffu, hh[0]);
+    const int l1 = __reduce_min_sync(0xffffffffu, hl[1]), h1 = __reduce_max_sync(0xffffffffu, hh[1]);
+    T* G = static_cast<T*>(a.ws) + r.ws_G;
+    const int64_t gplane = static_cast<int64_t>(nxp) * nyp * nzp;
+    const int64_t pnp = static_cast<int64_t>(nxp) * nyp;
+    const T ks = static_cast<T>(a.kin_scale);
+    for (int b0 = (z0 / Arm::N) * Arm::N; b0 <= z1; b0 += Arm::N) {
+        const int f0 = b0 + dz - KIN_HALF;              // window position p is input f0 + p
+        T o0[Arm::N], o1[Arm::N], c0[Arm::N], c1[Arm::N];
+        // both types' ranges within one for the first type (the run's condition)
+        Arm::run(o0, o1, c0, c1, col, col_n, (nz + 1) * 128,
+                 [&](int p) { const int q = f0 + p; return (q >= 0 && q < nz ? q : nz) * 128 + t; },
+                 min(l0, l1) - f0, max(h0, h1) - f0 + 1, l1 - f0, h1 - f0 + 1, st);
 #pragma unroll
-                for (int j = 0; j < BB; ++j) {
-                    const int b = b0 + j;
-                    if (b < nzp) {
-                        o0[j] *= ks;
-                        o1[j] *= ks;
-                        ST(G, tb * gplane + b * pnp + gcol, 8 * gplane, o0[j]);
-                        ST(G, (tb + 4) * gplane + b * pnp + gcol, 8 * gplane, o1[j]);
-                        const int zz = b + dz;
-                        if (zz >= 0 && zz < nz) ekin_t += k0[KIN_HALF + j] * o0[j] + k1[KIN_HALF + j] * o1[j];
-                    }
-                }
+        for (int j = 0; j < Arm::N; ++j) {
+            const int b = b0 + j;
+            if (b >= zlo && b <= zhi) {
+                o0[j] *= ks;
+                o1[j] *= ks;
+                ST(G, tb * gplane + b * pnp + gcol, 8 * gplane, o0[j]);
+                ST(G, (tb + 4) * gplane + b * pnp + gcol, 8 * gplane, o1[j]);
+                ekin_t += c0[j] * o0[j] + c1[j] * o1[j];
             }
         }
     }
@@ -1628,96 +1838,6 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 #define LSW_BWD_THREADS 256
 #endif
 constexpr int BWD_THREADS = LSW_BWD_THREADS;
-
-// Kinetic arm of N outputs (both types of a pair) from the window positions p = 0 .. NP - 1 of two
-// lines: position p of the first line is D[off(p)], of the second D[off(p) + dist].  [s0, e0), [s1,
-// e1): the positions of either line that can be nonzero, uniform over the warp, the second
-// within the first.  c0, c1: the lines' values at the outputs.
-template <class T>
-struct KinArm {
-    static constexpr int N = Blk<T, 1>::NB;            // outputs per block, both arms
-    static constexpr int NP = N + 2 * KIN_HALF;        // window positions
-    static constexpr int G = sizeof(T) == 4 ? 4 : 1;   // positions per group
-    template <class Off>
-    static __device__ __forceinline__ void run(T (&o0)[N], T (&o1)[N], T (&c0)[N], T (&c1)[N], const T* D, int64_t dn,
-                                               int dist, Off off, int s0, int e0, int s1, int e1,
-                                               [[maybe_unused]] int* st) {
-        [[maybe_unused]] int* ST_ = st;
-        [[maybe_unused]] constexpr int KID = 4;
-        float2 acc[sizeof(T) == 4 ? N : 1];
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            o0[j] = o1[j] = c0[j] = c1[j] = T(0);
-            if constexpr (sizeof(T) == 4) acc[j] = make_float2(0.f, 0.f);
-        }
-        auto add = [&](int p, int src, T v) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                if (p - j < 0 || p - j >= KIN_TAPS) continue;
-                if constexpr (sizeof(T) == 4) {
-                    acc[j] = __ffma2_rn(c_kin2[src][p - j], make_float2(v, v), acc[j]);
-                } else {
-                    o0[j] += Tab<T>::kin(src, p - j) * v;
-                    o1[j] += Tab<T>::kin(2 + src, p - j) * v;
-                }
-            }
-        };
-#pragma unroll
-        for (int g = 0; g < NP; g += G) {
-            if (g + G - 1 < s0 || g >= e0) continue;
-            int at[G];
-#pragma unroll
-            for (int k = 0; k < G; ++k) {
-                at[k] = off(g + k);
-                const T v = LD(D, at[k], dn);
-                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c0[(g + k - KIN_HALF) & (N - 1)] = v;
-                add(g + k, 0, v);
-            }
-            if (g + G - 1 < s1 || g >= e1) continue;
-#pragma unroll
-            for (int k = 0; k < G; ++k) {
-                const T v = LD(D, at[k] + dist, dn);
-                if (g + k >= KIN_HALF && g + k < KIN_HALF + N) c1[(g + k - KIN_HALF) & (N - 1)] = v;
-                add(g + k, 1, v);
-            }
-        }
-        if constexpr (sizeof(T) == 4) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                o0[j] = acc[j].x;
-                o1[j] = acc[j].y;
-            }
-        }
-    }
-};
-
-// The transposed filters of N coarse outputs from the window starting at position `first` of a
-// line of n values.  FP32: as bwd_block.  FP64 (bound by the FP64 pipe): positions outside the
-// line are skipped, not multiplied as zeros.
-template <class T, int NB>
-__device__ __forceinline__ void bwd_window(const T* p, int off, int stride, int first, int n, T (&s)[NB], T (&d)[NB],
-                                           int64_t room, int* st) {
-    if constexpr (sizeof(T) == 4) {
-        T w[2 * NB + 29];
-        swin(w, p, off, stride, first, n, room, st);
-        bwd_block<T, NB>(w, s, d);
-    } else {
-#pragma unroll
-        for (int j = 0; j < NB; ++j) s[j] = d[j] = T(0);
-#pragma unroll
-        for (int m = 0; m < 2 * NB + 29; ++m) {
-            const int pos = first + m;
-            if (pos < 0 || pos >= n) continue;
-            const T v = WLD(p, off + pos * stride, room);
-#pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (m - 2 * j >= 0 && m - 2 * j < FWD_TAPS) {
-                    s[j] += Tab<T>::fwd(0, m - 2 * j) * v;
-                    d[j] += Tab<T>::fwd(1, m - 2 * j) * v;
-                }
-        }
-    }
-}
 
 template <class T>
 __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase) {
