@@ -215,6 +215,7 @@ struct lsw_system_s {
     bool dens_ready = false;
     int64_t dens_lo[3] = {0, 0, 0}, dens_n[3] = {0, 0, 0};
     int32_t dens_ntile[3] = {0, 0, 0};
+    int dens_max_m = 0, dens_max_g = 0;
     int64_t U_elems = 0;
     std::vector<Batch> batches;
     int64_t ws_elems = 0;
@@ -1218,6 +1219,16 @@ lsw_status build_density_plan(lsw_system_s* s, const int64_t* lo, const int64_t*
             each_tile(dfn[f], [&](int64_t t) { tfn[fill[t]++] = static_cast<int32_t>(f); });
     }
     s->dens_ready = false;
+    // most functions and atoms of a tile; the products keep their tables in shared memory where
+    // two CTAs an SM still fit (about 100 functions of 100 atoms), else a variant searches them anew
+    s->dens_max_m = s->dens_max_g = 0;
+    for (int64_t t = 0; t < ntiles; ++t) {
+        int g = 0;
+        for (int64_t k = tptr[t]; k < tptr[t + 1]; ++k) g += k == tptr[t] || s->sf_atom[tfn[k]] != s->sf_atom[tfn[k - 1]];
+        s->dens_max_m = std::max(s->dens_max_m, static_cast<int>(tptr[t + 1] - tptr[t]));
+        s->dens_max_g = std::max(s->dens_max_g, g);
+    }
+    if (density_smem(s->prec, s->dens_max_m, s->dens_max_g) > s->ctx->max_smem / 2 - 4096) s->dens_max_m = s->dens_max_g = 0;
     cudaStream_t st = s->stream;
     CUDA_TRY(s->d_dfn.upload(dfn, st));
     CUDA_TRY(s->d_tptr.upload(tptr, st));
@@ -1262,6 +1273,7 @@ lsw_status enqueue_density_all(lsw_system_s* s, Tracer* tr, const void* phi, con
     d.U = s->d_U.p;
     d.tptr = static_cast<const int64_t*>(s->d_tptr.p);
     d.tfn = static_cast<const int32_t*>(s->d_tfn.p);
+    d.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
     d.row_ptr = static_cast<const int64_t*>(s->d_rowp.p);
     d.col = static_cast<const int32_t*>(s->d_col.p);
     d.K = K;
@@ -1270,6 +1282,8 @@ lsw_status enqueue_density_all(lsw_system_s* s, Tracer* tr, const void* phi, con
         d.gn[k] = s->dens_n[k];
         d.ntile[k] = s->dens_ntile[k];
     }
+    d.max_m = s->dens_max_m;
+    d.max_g = s->dens_max_g;
     d.status = static_cast<int*>(s->d_status.p);
     d.U_n = s->U_elems;
     d.tfn_n = static_cast<int64_t>(s->d_tfn.bytes / sizeof(int32_t));

@@ -247,12 +247,14 @@ struct DensLaunch {
     const void* U;               // real-space store
     const int64_t* tptr;         // [ntiles + 1]: functions of tile t are tfn[tptr[t] .. tptr[t+1])
     const int32_t* tfn;          // ascending within a tile
+    const int32_t* sf_atom;
     const int64_t* row_ptr;      // pattern CSR
     const int32_t* col;
     const double* K;             // density kernel on the pattern
     double* rho;                 // [gz][gy][gx]
     int64_t gn[3];               // grid extents
     int32_t ntile[3];
+    int max_m, max_g;            // most functions and atoms of a tile (0: too many for shared memory)
     int* status;
     // extents used by the self-checking build (-DLSW_CHECKED)
     int64_t U_n, tfn_n, nnz, rho_n, fn_n, tptr_n, rowp_n;
@@ -455,6 +457,7 @@ cudaError_t configure_panel_kernels(size_t max_smem);
 size_t panel_hs_smem(int prec);
 cudaError_t enqueue_dens_batch(const HphiLaunch& a, cudaStream_t s);   // real-space values
 cudaError_t enqueue_density(const DensLaunch& a, cudaStream_t s);      // pair products
+size_t density_smem(int prec, int max_m, int max_g);
 
 // Status word bits set by device-side checks.
 enum : int {

@@ -2354,12 +2354,77 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
 // B chunk's values there in registers; the coefficient block sits in shared memory and is
 // read as a broadcast.  Products and the chunk-pair partial sums run in T, the total per
 // point in FP64; every point of the grid is written (0 where no block reaches).
+//
+// The chunks (32 functions of the tile's list in order) fix the sums; what is left out adds exact
+// zeros.  Bound: instruction issue and its latencies at two CTAs an SM (128 registers: a chunk's
+// values at two points are 64 of them).  What took the time, 300 atoms (1,038 functions) in FP32:
+//   - 13.0 ms: a warp's points were rows of 32 x, so nearly every function of the tile counted,
+//     and the pattern was searched 2,048 times per pair of chunks.  One search per pair of atoms
+//     (an atom's functions have equal pattern rows and consecutive columns) and four A functions
+//     at a time: 12.4; the searches once per tile instead of once per pair of chunks: no less;
+//   - a warp takes a block of 8 x 4 x 2 points and forms only the products of A functions with
+//     a value there, with groups of four B functions that have one and are in the pattern: 7.6
+//     (with the pattern searched per pair of chunks 9.2: the tile's tables pay now);
+//   - the next pair's coefficients copied during the products into a second block, one barrier
+//     per pair; what belongs to a lane's B function kept in registers: 7.1;
+//   - a chunk's values are loaded where their boxes meet the warp's block, all loads before the
+//     first test of a value: 5.1.
 
-// K_ab from the pattern CSR (binary search of b in row a), 0 outside the pattern.
-__device__ __forceinline__ double dens_k(const DensLaunch& a, int fa, int fb) {
+struct __align__(16) DensRec {       // one function of a chunk
+    int64_t off;                     // block in the store
+    int o[3], d[3];
+    int64_t rp;                      // first pattern entry
+    int f;
+    int lead, grp;                   // first entry of its atom, number of its atom (in the chunk or tile)
+};
+
+// u_f at the thread's points (x, y, z + i); 0 outside f's block.
+template <class T>
+__device__ __forceinline__ void dens_u(const DensLaunch& a, const DensRec& df, int x, int y, int z, T (&u)[DT_PP]) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 13;
-    int64_t lo = LD(a.row_ptr, fa, a.rowp_n), hi = LD(a.row_ptr, fa + 1, a.rowp_n);
+    const int lx = x - df.o[0], ly = y - df.o[1], lz = z - df.o[2];
+    const bool in = static_cast<unsigned>(lx) < static_cast<unsigned>(df.d[0]) &&
+                    static_cast<unsigned>(ly) < static_cast<unsigned>(df.d[1]);
+    const T* U = static_cast<const T*>(a.U);
+    // 32 bits hold a place in the block (its planes fit in shared memory), and are used only inside it
+    const uint32_t n = static_cast<uint32_t>(df.d[0]) * df.d[1], at = lz * n + static_cast<uint32_t>(ly) * df.d[0] + lx;
+#pragma unroll
+    for (int i = 0; i < DT_PP; ++i)
+        u[i] = in && static_cast<unsigned>(lz + i) < static_cast<unsigned>(df.d[2]) ? LD(U, df.off + static_cast<int64_t>(at + i * n), a.U_n) : T(0);
+}
+
+// Records of the chunk of n functions tfn[at ..] (one warp); returns the number of atoms.
+__device__ __forceinline__ int dens_records(const DensLaunch& a, int64_t at, int n, DensRec* rec, int* leads) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 13;
+    const int lane = threadIdx.x & 31;
+    int atom = -1;
+    if (lane < n) {
+        DensRec& r = rec[lane];
+        r.f = LD(a.tfn, at + lane, a.tfn_n);
+        const DensFn df = LD(a.fn, r.f, a.fn_n);
+        r.off = df.off;
+        r.rp = LD(a.row_ptr, r.f, a.rowp_n);
+        for (int k = 0; k < 3; ++k) r.o[k] = df.o[k], r.d[k] = df.d[k];
+        atom = LD(a.sf_atom, r.f, a.fn_n);
+    }
+    const int before = __shfl_up_sync(0xffffffffu, atom, 1);
+    const unsigned m = __ballot_sync(0xffffffffu, lane < n && (lane == 0 || atom != before));
+    if (lane < n) {
+        const unsigned up = m & (0xffffffffu >> (31 - lane));
+        rec[lane].lead = 31 - __clz(up);
+        rec[lane].grp = __popc(up) - 1;
+        if (m >> lane & 1) leads[__popc(up) - 1] = lane;
+    }
+    return __popc(m);
+}
+
+// Position of column fb in row fa of the pattern, from the row's start; -1 outside the pattern.
+__device__ __forceinline__ int dens_find(const DensLaunch& a, int64_t rp, int fa, int fb) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 13;
+    int64_t lo = rp, hi = LD(a.row_ptr, fa + 1, a.rowp_n);
     const int64_t end = hi;
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
@@ -2368,21 +2433,7 @@ __device__ __forceinline__ double dens_k(const DensLaunch& a, int fa, int fb) {
         else
             hi = mid;
     }
-    return (lo < end && LD(a.col, lo, a.nnz) == fb) ? LD(a.K, lo, a.nnz) : 0.0;
-}
-
-// u_f at grid point (x, y, z); 0 outside f's block.
-template <class T>
-__device__ __forceinline__ T dens_u(const DensLaunch& a, const DensFn& df, int x, int y, int z) {
-    [[maybe_unused]] int* ST_ = a.status;
-    [[maybe_unused]] constexpr int KID = 13;
-    const int lx = x - df.o[0], ly = y - df.o[1], lz = z - df.o[2];
-    if (static_cast<unsigned>(lx) >= static_cast<unsigned>(df.d[0]) ||
-        static_cast<unsigned>(ly) >= static_cast<unsigned>(df.d[1]) ||
-        static_cast<unsigned>(lz) >= static_cast<unsigned>(df.d[2]))
-        return T(0);
-    const T* U = static_cast<const T*>(a.U);
-    return LD(U, df.off + (static_cast<int64_t>(lz) * df.d[1] + ly) * df.d[0] + lx, a.U_n);
+    return (lo < end && LD(a.col, lo, a.nnz) == fb) ? static_cast<int>(lo - rp) : -1;
 }
 
 __device__ __forceinline__ void lds16(const float* p, float (&v)[4]) {
@@ -2394,89 +2445,338 @@ __device__ __forceinline__ void lds16(const double* p, double (&v)[2]) {
     v[0] = t.x, v[1] = t.y;
 }
 
+// The points of a thread and their sums, and the values of the B chunk there.  A warp's points
+// are a block of 8 x 4 x DT_PP.
 template <class T>
-__global__ void __launch_bounds__(DT_THREADS) k_density(DensLaunch a) {
-    [[maybe_unused]] int* ST_ = a.status;
-    [[maybe_unused]] constexpr int KID = 13;
-    constexpr int VW = 16 / sizeof(T);
-    __shared__ __align__(16) T kb[DT_MC * DT_MC];
-    const int tile = blockIdx.x;
-    const int tx = tile % a.ntile[0];
-    const int ty = (tile / a.ntile[0]) % a.ntile[1];
-    const int tz = tile / (a.ntile[0] * a.ntile[1]);
-    const int64_t t0 = LD(a.tptr, tile, a.tptr_n);
-    const int m = static_cast<int>(LD(a.tptr, tile + 1, a.tptr_n) - t0);
-    int px[DT_PP], py[DT_PP], pz[DT_PP];
+struct DensPoints {
+    int x, y, z;
     double acc[DT_PP];
+    T ub[DT_MC][DT_PP];
+    unsigned fmask;            // B functions with a nonzero value at some point of the warp
+    __device__ __forceinline__ void init(const DensLaunch& a) {
+        static_assert(DT_X == 32 && DT_Y == 4 && DT_PP * DT_THREADS == DT_X * DT_Y * DT_Z, "a warp's block of points");
+        const int tile = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const int tx = tile % a.ntile[0];
+        const int ty = (tile / a.ntile[0]) % a.ntile[1];
+        const int tz = tile / (a.ntile[0] * a.ntile[1]);
+        x = tx * DT_X + (warp & 3) * 8 + (lane & 7);
+        y = ty * DT_Y + (lane >> 3);
+        z = tz * DT_Z + (warp >> 2) * DT_PP;
 #pragma unroll
-    for (int i = 0; i < DT_PP; ++i) {
-        const int p = threadIdx.x + i * DT_THREADS;
-        px[i] = tx * DT_X + p % DT_X;
-        py[i] = ty * DT_Y + (p / DT_X) % DT_Y;
-        pz[i] = tz * DT_Z + p / (DT_X * DT_Y);
-        acc[i] = 0.0;
+        for (int i = 0; i < DT_PP; ++i) acc[i] = 0.0;
     }
-    for (int cb = 0; cb < m; cb += DT_MC) {
-        const int nb = min(DT_MC, m - cb);
-        T ub[DT_MC][DT_PP];
+    __device__ __forceinline__ void load_b(const DensLaunch& a, const DensRec* rb, int nb) {
+        const int lane = threadIdx.x & 31;
+        bool meets = false;                        // lane j: the box of function j and the warp's block of points
+        if (lane < nb) {
+            const DensRec& r = rb[lane];
+            const int bx = x - (lane & 7) - r.o[0], by = y - (lane >> 3) - r.o[1], bz = z - r.o[2];
+            meets = bx + 8 > 0 && bx < r.d[0] && by + 4 > 0 && by < r.d[1] && bz + DT_PP > 0 && bz < r.d[2];
+        }
+        const unsigned bmask = __ballot_sync(0xffffffffu, meets);
 #pragma unroll
         for (int j = 0; j < DT_MC; ++j) {
-            if (j < nb) {
-                const DensFn df = LD(a.fn, LD(a.tfn, t0 + cb + j, a.tfn_n), a.fn_n);
-#pragma unroll
-                for (int i = 0; i < DT_PP; ++i) ub[j][i] = dens_u<T>(a, df, px[i], py[i], pz[i]);
+            if (bmask >> j & 1) {
+                dens_u<T>(a, rb[j], x, y, z, ub[j]);
             } else {
 #pragma unroll
                 for (int i = 0; i < DT_PP; ++i) ub[j][i] = T(0);
             }
         }
+        fmask = 0;
+#pragma unroll
+        for (int j = 0; j < DT_MC; ++j) {
+            bool any = false;
+#pragma unroll
+            for (int i = 0; i < DT_PP; ++i) any |= ub[j][i] != T(0);
+            if (__any_sync(0xffffffffu, any)) fmask |= 1u << j;
+        }
+    }
+    // acc += sum over the A chunk of u_a sum_b kb_ab u_b (partial sums of the pair of chunks in T).
+    // amask: the A functions with a nonzero value at some point of the warp; kmask: the B
+    // functions within the pattern, per A function.  RW rows (A functions) at a time, each a chain of
+    // its own: one row's products depend on one another (up to 32 in a row).
+    __device__ __forceinline__ void products(const DensLaunch& a, const DensRec* ra, unsigned amask, const T* kb,
+                                             const unsigned* kmask) {
+        constexpr int VW = 16 / sizeof(T), NG = DT_MC / 4, RW = sizeof(T) == 4 ? 4 : 1;
+        const int lane = threadIdx.x & 31;
+        unsigned rows = __ballot_sync(0xffffffffu, (amask >> lane & 1) && (kmask[lane] & fmask));
+        if (rows == 0) return;                     // every product is an exact zero
+        T part[DT_PP], next[RW][DT_PP];
+        int id[RW];
+        auto take = [&]() {
+#pragma unroll
+            for (int w = 0; w < RW; ++w) {
+                id[w] = __ffs(rows) - 1;
+                rows &= rows - 1;
+                if (id[w] >= 0) {
+                    dens_u<T>(a, ra[id[w]], x, y, z, next[w]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < DT_PP; ++i) next[w][i] = T(0);
+                }
+            }
+        };
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i) part[i] = T(0);
+        take();
+        while (id[0] >= 0) {
+            T ua[RW][DT_PP], zz[RW][DT_PP];
+            const T* row[RW];
+            unsigned on = 0;
+#pragma unroll
+            for (int w = 0; w < RW; ++w) {
+                const int r = id[w] >= 0 ? id[w] : id[0];
+                on |= kmask[r];
+                row[w] = kb + r * DT_MC;
+#pragma unroll
+                for (int i = 0; i < DT_PP; ++i) {
+                    ua[w][i] = next[w][i];
+                    zz[w][i] = T(0);
+                }
+            }
+            take();
+            on &= fmask;
+#pragma unroll
+            for (int g = 0; g < NG; ++g) {
+                if (!(on >> (4 * g) & 15)) continue;
+#pragma unroll
+                for (int q = 4 * g; q < 4 * g + 4; q += VW) {
+                    T k[RW][VW];
+#pragma unroll
+                    for (int w = 0; w < RW; ++w) lds16(row[w] + q, k[w]);
+#pragma unroll
+                    for (int e = 0; e < VW; ++e)
+#pragma unroll
+                        for (int w = 0; w < RW; ++w) {
+                            if constexpr (sizeof(T) == 4 && DT_PP == 2) {   // both points in one packed FMA: the same bits
+                                const float2 t = __ffma2_rn(make_float2(k[w][e], k[w][e]), make_float2(ub[q + e][0], ub[q + e][1]),
+                                                            make_float2(zz[w][0], zz[w][1]));
+                                zz[w][0] = t.x, zz[w][1] = t.y;
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < DT_PP; ++i) zz[w][i] += k[w][e] * ub[q + e][i];
+                            }
+                        }
+                }
+            }
+#pragma unroll
+            for (int w = 0; w < RW; ++w)
+#pragma unroll
+                for (int i = 0; i < DT_PP; ++i) part[i] += ua[w][i] * zz[w][i];
+        }
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i) acc[i] += static_cast<double>(part[i]);
+    }
+    __device__ __forceinline__ void store(const DensLaunch& a) const {
+        [[maybe_unused]] int* ST_ = a.status;
+        [[maybe_unused]] constexpr int KID = 13;
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i)
+            if (x < a.gn[0] && y < a.gn[1] && z + i < a.gn[2])
+                ST(a.rho, ((z + i) * a.gn[1] + y) * a.gn[0] + x, a.rho_n, acc[i]);
+    }
+};
+
+// Row ia of the coefficient block (a warp): the value of lane b, and whether (a, b) is in the pattern.
+template <class T>
+__device__ __forceinline__ void dens_row(T* kb, unsigned* kmask, int ia, double v, bool in) {
+    const int lane = threadIdx.x & 31;
+    kb[ia * DT_MC + lane] = static_cast<T>(v);
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    if (lane == 0) kmask[ia] = m;
+}
+
+constexpr int DENS_MASKS = 64;       // chunks whose masks a warp keeps (the others' functions all count as present)
+
+// The records of all functions of the tile and the pattern positions of all pairs of their
+// atoms in shared memory (a.max_m functions, a.max_g atoms at most), built once per tile; the
+// coefficients of the next pair of chunks are copied during the products of this one.
+template <class T>
+__global__ void __launch_bounds__(DT_THREADS) k_density(DensLaunch a) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 13;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double* kraw = reinterpret_cast<double*>(smem_raw);                  // [2][MC][MC]: K_ab, K_ba
+    T* kb = reinterpret_cast<T*>(kraw + 2 * DT_MC * DT_MC);              // [2][MC][MC], in turn
+    DensRec* rec = reinterpret_cast<DensRec*>(kb + 2 * DT_MC * DT_MC);   // [max_m]
+    int* rel = reinterpret_cast<int*>(rec + a.max_m);                    // [atoms][RS]
+    const int RS = a.max_g | 1;                                          // odd: a column's entries in different banks
+    int* lead = rel + a.max_g * RS;                                 // [max_g]
+    __shared__ unsigned um[DT_THREADS / 32][DENS_MASKS];
+    __shared__ unsigned kmask[2][DT_MC];        // per A function: groups of 4 B functions with a nonzero coefficient
+    __shared__ int s_ng;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t0 = LD(a.tptr, blockIdx.x, a.tptr_n);
+    const int m = static_cast<int>(LD(a.tptr, blockIdx.x + 1, a.tptr_n) - t0);
+    DensPoints<T> P;
+    P.init(a);
+    auto all = [&](int ca) { return 0xffffffffu >> (DT_MC - min(DT_MC, m - ca)); };
+    for (int k = threadIdx.x; k < m; k += DT_THREADS) {
+        DensRec& r = rec[k];
+        r.f = LD(a.tfn, t0 + k, a.tfn_n);
+        const DensFn df = LD(a.fn, r.f, a.fn_n);
+        r.off = df.off;
+        r.rp = LD(a.row_ptr, r.f, a.rowp_n);
+        for (int d = 0; d < 3; ++d) r.o[d] = df.o[d], r.d[d] = df.d[d];
+        r.grp = LD(a.sf_atom, r.f, a.fn_n);    // its atom, renumbered below
+    }
+    __syncthreads();
+    if (warp == 0) {                           // atoms of the list, numbered in order
+        int runs = 0, first = 0, last = -1;
+        for (int b = 0; b < m; b += 32) {
+            const int k = b + lane;
+            const int at = k < m ? rec[k].grp : -2;
+            int before = __shfl_up_sync(0xffffffffu, at, 1);
+            if (lane == 0) before = last;
+            const unsigned mk = __ballot_sync(0xffffffffu, k < m && at != before);
+            const unsigned up = mk & (0xffffffffu >> (31 - lane));
+            if (k < m) {
+                rec[k].lead = up ? b + 31 - __clz(up) : first;
+                rec[k].grp = runs + __popc(up) - 1;
+                if (mk >> lane & 1) lead[rec[k].grp] = k;
+            }
+            if (mk) first = b + 31 - __clz(mk);
+            runs += __popc(mk);
+            last = __shfl_sync(0xffffffffu, at, 31);
+        }
+        if (lane == 0) s_ng = runs;
+    }
+    __syncthreads();
+    const int ng = s_ng;
+    for (int e = threadIdx.x; e < ng * ng; e += DT_THREADS) {
+        const DensRec &A = rec[lead[e / ng]], &B = rec[lead[e % ng]];
+        rel[e / ng * RS + e % ng] = dens_find(a, A.rp, A.f, B.f);
+    }
+    __syncthreads();
+    // coefficients of the pair of chunks (ca, cb): each thread copies its own entries
+    unsigned in = 0;                           // per row of this warp: the lane's pair is in the pattern
+    int ib = -1, gb = 0;                       // the lane's B function and what belongs to it
+    int64_t rb = 0;
+    int ob = 0;
+    auto issue = [&](int ca, int cb) {
+        in = 0;
+        if (ib != cb + lane) {
+            ib = cb + lane;
+            if (ib < m) gb = rec[ib].grp, rb = rec[ib].rp, ob = ib - rec[ib].lead;
+        }
+#pragma unroll
+        for (int k = 0; k < DT_MC * 32 / DT_THREADS; ++k) {
+            const int ia = warp + k * (DT_THREADS / 32);
+            int64_t ab = -1, ba = -1;
+            if (ca + ia < m && ib < m) {
+                const DensRec& A = rec[ca + ia];
+                const int r = rel[A.grp * RS + gb], q = ca != cb ? rel[gb * RS + A.grp] : -1;
+                if (r >= 0) ab = A.rp + (r + ob);
+                if (q >= 0) ba = rb + (q + ca + ia - A.lead);
+                if (r >= 0 || q >= 0) in |= 1u << k;
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int64_t at = s ? ba : ab;
+                const int to = (s * DT_MC + ia) * DT_MC + lane;
+                if (at >= 0) CPA(kraw, to, 2 * DT_MC * DT_MC, a.K, at, a.nnz);
+                else kraw[to] = 0.0;
+            }
+        }
+    };
+    auto finish = [&](int to) {
+        cp_wait();
+#pragma unroll
+        for (int k = 0; k < DT_MC * 32 / DT_THREADS; ++k) {
+            const int ia = warp + k * (DT_THREADS / 32);
+            dens_row(kb + to * DT_MC * DT_MC, kmask[to], ia, kraw[ia * DT_MC + lane] + kraw[(DT_MC + ia) * DT_MC + lane], in >> k & 1);
+        }
+        __syncthreads();
+    };
+    int cur = 0;
+    if (m > 0) {
+        issue(0, 0);
+        finish(0);
+    }
+    for (int cb = 0; cb < m; cb += DT_MC) {
+        P.load_b(a, rec + cb, min(DT_MC, m - cb));
+        if (cb / DT_MC < DENS_MASKS && lane == 0) um[warp][cb / DT_MC] = P.fmask;
+        __syncwarp();
+        for (int ca = 0; ca <= cb; ca += DT_MC) {
+            const bool more = ca < cb || cb + DT_MC < m;
+            if (more) issue(ca < cb ? ca + DT_MC : 0, ca < cb ? cb : cb + DT_MC);
+            P.products(a, rec + ca, ca / DT_MC < DENS_MASKS ? um[warp][ca / DT_MC] : all(ca), kb + cur * DT_MC * DT_MC, kmask[cur]);
+            cur ^= 1;                          // the other block's readers passed the last barrier
+            if (more) finish(cur);
+        }
+    }
+    P.store(a);
+}
+
+// The same for tiles whose records and positions do not fit: a chunk's records at a time, the
+// pattern searched per pair of chunks.
+template <class T>
+__global__ void __launch_bounds__(DT_THREADS) k_density_big(DensLaunch a) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 13;
+    __shared__ __align__(16) T kb[DT_MC * DT_MC];
+    __shared__ DensRec ra[DT_MC], rb[DT_MC];
+    __shared__ int la[DT_MC], lb[DT_MC], rel[2][DT_MC * DT_MC], ng[2];
+    __shared__ unsigned um[DT_THREADS / 32][DENS_MASKS];
+    __shared__ unsigned kmask[DT_MC];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t t0 = LD(a.tptr, blockIdx.x, a.tptr_n);
+    const int m = static_cast<int>(LD(a.tptr, blockIdx.x + 1, a.tptr_n) - t0);
+    DensPoints<T> P;
+    P.init(a);
+    auto all = [&](int ca) { return 0xffffffffu >> (DT_MC - min(DT_MC, m - ca)); };
+    for (int cb = 0; cb < m; cb += DT_MC) {
+        const int nb = min(DT_MC, m - cb);
+        __syncthreads();       // the previous chunk's readers of rb are done
+        if (warp == 0) {
+            const int g = dens_records(a, t0 + cb, nb, rb, lb);
+            if (lane == 0) ng[1] = g;
+        }
+        __syncthreads();
+        P.load_b(a, rb, nb);
+        if (cb / DT_MC < DENS_MASKS && lane == 0) um[warp][cb / DT_MC] = P.fmask;
+        __syncwarp();
         for (int ca = 0; ca <= cb; ca += DT_MC) {
             const int na = min(DT_MC, m - ca);
             __syncthreads();   // the previous block's readers are done
-            for (int e = threadIdx.x; e < DT_MC * DT_MC; e += DT_THREADS) {
-                const int ia = e / DT_MC, ib = e % DT_MC;
-                double v = 0.0;
-                if (ia < na && ib < nb) {
-                    const int fa = LD(a.tfn, t0 + ca + ia, a.tfn_n);
-                    const int fb = LD(a.tfn, t0 + cb + ib, a.tfn_n);
-                    v = dens_k(a, fa, fb);
-                    if (ca != cb) v += dens_k(a, fb, fa);
-                }
-                kb[e] = static_cast<T>(v);
+            if (warp == 0) {
+                const int g = dens_records(a, t0 + ca, na, ra, la);
+                if (lane == 0) ng[0] = g;
             }
             __syncthreads();
-            T part[DT_PP];
-#pragma unroll
-            for (int i = 0; i < DT_PP; ++i) part[i] = T(0);
-            for (int ia = 0; ia < na; ++ia) {
-                const DensFn df = LD(a.fn, LD(a.tfn, t0 + ca + ia, a.tfn_n), a.fn_n);
-                T ua[DT_PP], z[DT_PP];
-#pragma unroll
-                for (int i = 0; i < DT_PP; ++i) {
-                    ua[i] = dens_u<T>(a, df, px[i], py[i], pz[i]);
-                    z[i] = T(0);
-                }
-                const T* row = kb + ia * DT_MC;
-#pragma unroll
-                for (int q = 0; q < DT_MC; q += VW) {
-                    T k[VW];
-                    lds16(row + q, k);
-#pragma unroll
-                    for (int w = 0; w < VW; ++w)
-#pragma unroll
-                        for (int i = 0; i < DT_PP; ++i) z[i] += k[w] * ub[q + w][i];
-                }
-#pragma unroll
-                for (int i = 0; i < DT_PP; ++i) part[i] += ua[i] * z[i];
+            for (int e = threadIdx.x; e < ng[0] * ng[1]; e += DT_THREADS) {
+                const int ga = e / ng[1], gb = e - ga * ng[1];
+                const DensRec &A = ra[la[ga]], &B = rb[lb[gb]];
+                rel[0][ga * DT_MC + gb] = dens_find(a, A.rp, A.f, B.f);
+                if (ca != cb) rel[1][ga * DT_MC + gb] = dens_find(a, B.rp, B.f, A.f);
             }
-#pragma unroll
-            for (int i = 0; i < DT_PP; ++i) acc[i] += static_cast<double>(part[i]);
+            __syncthreads();
+            for (int ia = warp; ia < DT_MC; ia += DT_THREADS / 32) {
+                double v = 0.0;
+                bool in = false;
+                if (ia < na && lane < nb) {
+                    const DensRec &A = ra[ia], &B = rb[lane];
+                    const int r = rel[0][A.grp * DT_MC + B.grp];
+                    if (r >= 0) v = LD(a.K, A.rp + r + (lane - B.lead), a.nnz), in = true;
+                    if (ca != cb) {
+                        const int q = rel[1][A.grp * DT_MC + B.grp];
+                        if (q >= 0) v += LD(a.K, B.rp + q + (ia - A.lead), a.nnz), in = true;
+                    }
+                }
+                dens_row(kb, kmask, ia, v, in);
+            }
+            __syncthreads();
+            P.products(a, ra, ca / DT_MC < DENS_MASKS ? um[warp][ca / DT_MC] : all(ca), kb, kmask);
         }
     }
-#pragma unroll
-    for (int i = 0; i < DT_PP; ++i)
-        if (px[i] < a.gn[0] && py[i] < a.gn[1] && pz[i] < a.gn[2])
-            ST(a.rho, (pz[i] * a.gn[1] + py[i]) * a.gn[0] + px[i], a.rho_n, acc[i]);
+    P.store(a);
+}
+
+// Dynamic shared memory of k_density.
+size_t density_smem(int prec, int max_m, int max_g) {
+    return static_cast<size_t>(DT_MC) * DT_MC * 2 * (sizeof(double) + (prec == 0 ? sizeof(double) : sizeof(float))) +
+           static_cast<size_t>(max_m) * sizeof(DensRec) + (static_cast<size_t>(max_g) * (max_g | 1) + max_g) * sizeof(int);
 }
 
 // ---------------------------------------------------------------- peak probes
@@ -2726,6 +3026,7 @@ cudaError_t configure_kernels(size_t max_smem) {
         if ((e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, m)) != cudaSuccess) \
             return e;                                                                           \
     }
+    SETMAX(k_density<double>) SETMAX(k_density<float>)
     SETMAX(k_fwd_xy<double>) SETMAX(k_fwd_xy<float>)
     SETMAX(k_z<double>) SETMAX(k_z<float>)
     SETMAX(k_kin_z<double>) SETMAX(k_kin_z<float>)
@@ -2839,10 +3140,19 @@ cudaError_t enqueue_dens_batch(const HphiLaunch& a, cudaStream_t s) {
 cudaError_t enqueue_density(const DensLaunch& a, cudaStream_t s) {
     const int64_t nt = static_cast<int64_t>(a.ntile[0]) * a.ntile[1] * a.ntile[2];
     if (nt == 0) return cudaSuccess;
-    if (a.prec == 0)
-        TRACED(a.tr, TK_DENSITY, s, (k_density<double><<<static_cast<unsigned>(nt), DT_THREADS, 0, s>>>(a)));
-    else
-        TRACED(a.tr, TK_DENSITY, s, (k_density<float><<<static_cast<unsigned>(nt), DT_THREADS, 0, s>>>(a)));
+    const unsigned g = static_cast<unsigned>(nt);
+    // tables in shared memory where two CTAs an SM fit with the tile of most functions
+    if (a.max_m > 0) {
+        const size_t smem = density_smem(a.prec, a.max_m, a.max_g);
+        if (a.prec == 0)
+            TRACED(a.tr, TK_DENSITY, s, (k_density<double><<<g, DT_THREADS, smem, s>>>(a)));
+        else
+            TRACED(a.tr, TK_DENSITY, s, (k_density<float><<<g, DT_THREADS, smem, s>>>(a)));
+    } else if (a.prec == 0) {
+        TRACED(a.tr, TK_DENSITY, s, (k_density_big<double><<<g, DT_THREADS, 0, s>>>(a)));
+    } else {
+        TRACED(a.tr, TK_DENSITY, s, (k_density_big<float><<<g, DT_THREADS, 0, s>>>(a)));
+    }
     return cudaGetLastError();
 }
 
