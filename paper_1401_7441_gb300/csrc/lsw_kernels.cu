@@ -1830,9 +1830,14 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 //     outside the box read a zero beside the D plane;
 //   - the y pass, the x pass and the kinetic y arm are one loop body run in three phases: as three
 //     bodies their unrolled code (40 KB) missed the instruction caches (17 % of the stalls);
-//   - the compressed write's fine members come from a list built once per item.
-// Measured (GB300, 2,070 MHz, 1,024 functions a batch): 9.5 -> 4.8 us per function at radii 5-8 bohr
-// (n_x' to 52; one CTA per SM before), 7.3 -> 6.0 us at 7 bohr in a dense system (n_x' 47, more fine
+//   - the compressed write's fine members come from a list built once per item;
+//   - the tables are one chain of loads (a row and part per thread), ranges by atomics, prefix
+//     sums and tasks by warps, while the first function's planes arrive: before that they took
+//     15 % of the time for atoms of several functions, 32 % for single ones (1,052 -> 865 us for
+//     64 atoms, where most items are single functions).  The next item is fetched during the last
+//     write, no earlier: a CTA that holds an item unbegun delays the end (FP64 11.1 -> 10.0 ms).
+// Measured (GB300, 2,070 MHz, 1,024 functions a batch): 9.5 -> 4.4 us per function at radii 5-8 bohr
+// (n_x' to 52; one CTA per SM before), 7.3 -> 5.4 us at 7 bohr in a dense system (n_x' 47, more fine
 // members).
 
 #ifndef LSW_BWD_THREADS
@@ -1841,7 +1846,7 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 constexpr int BWD_THREADS = LSW_BWD_THREADS;
 
 template <class T>
-__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase) {
+__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase, int2* s_next) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     int* st = a.status;
@@ -1878,10 +1883,8 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     int16_t* const rx1 = rx0 + nyp;
     int16_t* const fx0 = rx1 + nyp;                             // hull of the row's fine members, -1: none
     int16_t* const fx1 = fx0 + nyp;
-    int16_t* const lx0 = fx1 + nyp;                             // [2][ny]: hull of L's coarse, fine members per row of the D plane
-    int16_t* const lx1 = lx0 + 2 * ny;
-    int16_t* const cy0 = lx1 + 2 * ny;                          // [2][nx]: the same per column
-    int16_t* const cy1 = cy0 + 2 * nx;
+    int* const lxr = reinterpret_cast<int*>(fx1 + nyp);         // [2][ny]: hull of L's coarse, fine members per row of the D plane
+    int* const cyr = lxr + 2 * ny;                              // [2][nx]: the same per column; first << 16 | last, -1: none
     uint16_t* const memb = reinterpret_cast<uint16_t*>(smem_raw + L.o_mem);   // b n_x' + x of the plane's fine members
     const int kx = 32 - __clz(max(nyp - 1, 1)), ky = 32 - __clz(max(nxp - 1, 1));   // (n_x' n_y' < 2^14: codes < 2^16)
     const uint32_t mbar = tc::saddr(smem_raw);
@@ -1891,16 +1894,6 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     const int64_t smem_n = static_cast<int64_t>(a.smem_bwd / sizeof(T));
     [[maybe_unused]] const int64_t pl_n = smem_n - L.o_pl / sizeof(T), mid_n = smem_n - L.o_mid / sizeof(T),
                                    dp_n = smem_n - L.o_D / sizeof(T);
-    if (tid == 0) {
-        ylo = nyp;
-        yhi = -1;
-        dead = 0;
-    }
-    for (int i = tid; i < 2 * L.nb_x; i += blockDim.x) {
-        hlo[i] = nyp;
-        hhi[i] = -1;
-    }
-    __syncthreads();
     const int pn = nx * ny;
     const int64_t dplane_n = static_cast<int64_t>(pn) * nz;
     // the D plane of function f (types tb + 4 bz), an element per copy into the padded rows
@@ -1913,43 +1906,103 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                 CPA(Dp, tb * PS + y * RS + x, dp_n, D, tb * dplane_n + y * nx + x, 8 * dplane_n);
         }
     };
-    // member x range of each row of this plane (coarse part of L', fine hull), and of the D plane
+    // the copies of the first function's planes are in flight while the tables are built
+    auto load_Bb = [&](const FnRec& r) {                       // one thread
+        const T* Bb = static_cast<const T*>(a.ws) + r.ws_Bb + (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
+        const int rem = static_cast<int>((reinterpret_cast<uintptr_t>(Bb) & 15) / sizeof(T));
+        const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(rem + Y * X) * sizeof(T) + 15) & ~size_t(15));
+        bulk_fence();                                          // Gs was read and written there
+        bulk_expect(mbar, bytes);
+        bulk_load(tc::saddr(plb), Bb - rem, bytes, mbar);
+    };
+    auto wait = [&]() {                                        // for the bulk copies in flight
+#ifndef LSW_CHECKED
+        if (!dead && !tc::mbar_wait(mbar, phase)) {
+            atomicOr(st, ST_WAIT_TIMEOUT);
+            dead = 1;
+        }
+        phase ^= 1;
+#endif
+    };
+#ifndef LSW_CHECKED
+    if (tid == 0) load_Bb(r0);
+#endif
+    // the CTA's next item, by the last thread: taken no earlier than at the end of this one (a CTA
+    // that holds a second item unbegun delays the last ones)
+    const bool fetch = s_next && tid == blockDim.x - 1;
+    auto item = [&](int k) { return k < a.n_items_bwd ? a.items_bwd[k] : make_int2(0, -1); };
+    if (tid == 0) {
+        ylo = nyp;
+        yhi = -1;
+        dead = 0;
+    }
+    for (int i = tid; i < 2 * L.nb_x; i += blockDim.x) {
+        hlo[i] = nyp;
+        hhi[i] = -1;
+    }
+    for (int i = tid; i < 2 * L.nb_y; i += blockDim.x) {
+        if (i < L.nb_y) {
+            cq0[i] = X;
+            cq1[i] = -1;
+        }
+        rq0[i] = nxp;
+        rq1[i] = -1;
+    }
+    if (dplane) stage_D(r0);
     const int64_t crow0 = at.rowPc + static_cast<int64_t>(nyp) * zb, frow0 = at.rowPf + static_cast<int64_t>(nyp) * zb;
-    for (int y = tid; y < nyp; y += blockDim.x) {
-        const int s0 = LD(a.rowptr, crow0 + y, a.rowptr_n), s1 = LD(a.rowptr, crow0 + y + 1, a.rowptr_n);
+    const int q0 = LD(a.rowptr, frow0, a.rowptr_n), q1 = LD(a.rowptr, frow0 + nyp, a.rowptr_n);
+    __syncthreads();
+    // member x range of each row of this plane (coarse part of L', fine hull) and of the D plane
+    // (coarse and fine members of L), a row and part per thread: one chain of loads for all
+    for (int i = tid; i < 2 * nyp + (dplane ? 2 * ny : 0); i += blockDim.x) {
+        const bool inP = i < 2 * nyp;
+        const int part = inP ? i >= nyp : i - 2 * nyp >= ny, y = inP ? i - part * nyp : i - 2 * nyp - part * ny;
+        const int64_t row = inP ? (part ? frow0 : crow0) + y : (part ? at.rowLf : at.rowLc) + y + static_cast<int64_t>(ny) * zL;
+        const int64_t sg = inP ? (part ? at.segPf : at.segPc) : (part ? at.segLf : at.segLc);
+        const int s0 = LD(a.rowptr, row, a.rowptr_n), s1 = LD(a.rowptr, row + 1, a.rowptr_n);
         int lo = -1, hi = -1, off = 0;
         if (s1 > s0) {
-            const Seg sg = LD(a.seg, at.segPc + s0, a.seg_n);
-            lo = sg.x0;
-            off = sg.off;
-            hi = LD(a.seg, at.segPc + s1 - 1, a.seg_n).x1;
+            const Seg first = LD(a.seg, sg + s0, a.seg_n);
+            lo = first.x0;
+            off = first.off;
+            hi = LD(a.seg, sg + s1 - 1, a.seg_n).x1;
         }
-        rx0[y] = static_cast<int16_t>(lo);
-        rx1[y] = static_cast<int16_t>(hi);
-        roff[y] = off;
-        const int q0 = LD(a.rowptr, frow0 + y, a.rowptr_n), q1 = LD(a.rowptr, frow0 + y + 1, a.rowptr_n);
-        const int flo = q1 > q0 ? LD(a.seg, at.segPf + q0, a.seg_n).x0 : -1;
-        fx0[y] = static_cast<int16_t>(flo);
-        fx1[y] = static_cast<int16_t>(q1 > q0 ? LD(a.seg, at.segPf + q1 - 1, a.seg_n).x1 : -1);
-        if ((bz == 0 ? lo : flo) >= 0) {                       // rows that the compressed write reads
+        if (!inP) {
+            lxr[part * ny + y] = lo < 0 ? -1 : lo << 16 | hi;
+            continue;
+        }
+        (part ? fx0 : rx0)[y] = static_cast<int16_t>(lo);
+        (part ? fx1 : rx1)[y] = static_cast<int16_t>(hi);
+        if (!part) roff[y] = off;
+        if (lo >= 0 && part == (bz != 0)) {                    // rows that the compressed write reads
             atomicMin(&ylo, y);
             atomicMax(&yhi, y);
         }
     }
-    if (dplane) {
-        for (int i = tid; i < 2 * ny; i += blockDim.x) {
-            const int part = i >= ny, y = i - part * ny;
-            const int64_t row = (part ? at.rowLf : at.rowLc) + y + static_cast<int64_t>(ny) * zL;
-            const int64_t sg = part ? at.segLf : at.segLc;
-            const int s0 = LD(a.rowptr, row, a.rowptr_n), s1 = LD(a.rowptr, row + 1, a.rowptr_n);
-            lx0[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s0, a.seg_n).x0 : -1);
-            lx1[i] = static_cast<int16_t>(s1 > s0 ? LD(a.seg, sg + s1 - 1, a.seg_n).x1 : -1);
-        }
-        if (tid < 4) ST(Dp, tid * PS + PS - 1, dp_n, T(0));
+    if (dplane && tid < 4) ST(Dp, tid * PS + PS - 1, dp_n, T(0));
+    // the plane's fine members: m0 .. m0 + nm - 1 of each type's block
+    int m0 = 0, nm = 0;
+    if (q1 > q0) {
+        const Seg sl = LD(a.seg, at.segPf + q1 - 1, a.seg_n);
+        m0 = LD(a.seg, at.segPf + q0, a.seg_n).off;
+        nm = sl.off + (sl.x1 - sl.x0 + 1) - m0;
     }
+    const bool listed = nm <= L.memN;
+    if (listed)
+        for (int q = q0 + static_cast<int>(blockDim.x) - 1 - tid; q < q1; q += blockDim.x) {
+            const Seg g = LD(a.seg, at.segPf + q, a.seg_n);
+            const int at0 = static_cast<int>(g.row - static_cast<int64_t>(nyp) * zb) * nxp;
+            for (int x = g.x0; x <= g.x1; ++x) ST(memb, g.off - m0 + (x - g.x0), L.memN, static_cast<uint16_t>(at0 + x));
+        }
     __syncthreads();
     const int ylo_ = ylo, yhi_ = yhi;
-    if (yhi_ < 0) return;                                      // uniform; nothing to write in this plane
+    if (yhi_ < 0) {                                            // uniform; nothing to write in this plane
+        wait();
+        cp_wait();
+        if (fetch) *s_next = item(atomicAdd(a.queue + 1, 1));
+        __syncthreads();
+        return;
+    }
     // The x range of row b whose outputs of the y-type pair `by` (types 2 by, 2 by + 1 of
     // this plane) the compressed write reads: the coarse members where the pair holds the
     // scaling type 0 (bz = 0, by = 0), else the hull of the row's fine members (the wavelet
@@ -1959,43 +2012,22 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         lo = c ? rx0[b] : fx0[b];
         hi = c ? rx1[b] : fx1[b];
     };
-    // ---- ranges, in one phase: the y pass's columns per block of NB rows (for row b and pair by
-    //      its blocks k = lo/NB .. hi/NB of the needed range read x' in [2 (k NB + dx),
+    // ---- ranges: the y pass's columns per block of NB rows (for row b and pair by its blocks
+    //      k = lo/NB .. hi/NB of the needed range read x' in [2 (k NB + dx),
     //      2 (k NB + NB - 1 + dx) + 30]); the kinetic y arm's columns (per x type bx, the pair of
     //      types bx, bx + 2, and block of rows: the hull of the rows' needed ranges); the x pass's
-    //      rows per (pair, block of NB columns); the member hulls of D's columns; the fine members
+    //      rows per (pair, block of NB columns); beside them, on other warps first, the hulls of
+    //      D's columns
     const int nbb = (yhi_ - ylo_ + NB) / NB;
-    for (int q = tid; q < nbb; q += blockDim.x) {
-        int c0 = X, c1 = -1;
-        for (int b = ylo_ + q * NB; b < min(ylo_ + (q + 1) * NB, yhi_ + 1); ++b)
-            for (int by = 0; by < 2; ++by) {
-                int lo, hi;
-                need(by, b, lo, hi);
-                if (lo < 0) continue;
-                c0 = min(c0, 2 * ((lo / NB) * NB + dx));
-                c1 = max(c1, 2 * ((hi / NB) * NB + NB - 1 + dx) + 30);
-            }
-        cq0[q] = max(c0, 0);
-        cq1[q] = min(c1, X - 1);
-    }
-    for (int i = tid - 32; i >= 0 && i < 2 * nbb; i += blockDim.x) {
-        const int bx = i >= nbb, q = i - bx * nbb;
-        int c0 = nxp, c1 = -1;
-        for (int b = ylo_ + q * NB; b < min(ylo_ + (q + 1) * NB, yhi_ + 1); ++b) {
-            int lo, hi;
-            need(bx, b, lo, hi);                               // the same rule with the x type
-            if (lo < 0) continue;
-            c0 = min(c0, lo);
-            c1 = max(c1, hi);
-        }
-        rq0[i] = max(c0, -dx);                                 // columns of the D plane
-        rq1[i] = min(c1, nx - 1 - dx);
-    }
-    for (int i = tid; i < 2 * (yhi_ - ylo_ + 1); i += blockDim.x) {
-        const int by = i & 1, b = ylo_ + (i >> 1);
+    for (int i = static_cast<int>(blockDim.x) - 1 - tid; i < 2 * (yhi_ - ylo_ + 1); i += blockDim.x) {
+        const int by = i & 1, b = ylo_ + (i >> 1), q = (b - ylo_) / NB;
         int lo, hi;
-        need(by, b, lo, hi);
+        need(by, b, lo, hi);                                   // (the same rule for x types)
         if (lo < 0) continue;
+        atomicMin(&cq0[q], 2 * ((lo / NB) * NB + dx));
+        atomicMax(&cq1[q], 2 * ((hi / NB) * NB + NB - 1 + dx) + 30);
+        atomicMin(&rq0[by * nbb + q], lo);
+        atomicMax(&rq1[by * nbb + q], hi);
         for (int k = lo / NB; k <= hi / NB; ++k) {
             atomicMin(&hlo[by * L.nb_x + k], b);
             atomicMax(&hhi[by * L.nb_x + k], b);
@@ -2004,68 +2036,61 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     if (dplane)
         for (int i = tid; i < 2 * nx; i += blockDim.x) {
             const int part = i >= nx, x = i - part * nx;
-            int lo = -1, hi = -1;
-            for (int y = 0; y < ny; ++y)
-                if (lx0[part * ny + y] >= 0 && x >= lx0[part * ny + y] && x <= lx1[part * ny + y]) {
+            const int* rows = lxr + part * ny;
+            int lo = -1, hi = 0;
+#pragma unroll 8
+            for (int y = 0; y < ny; ++y) {
+                const int v = rows[y];
+                if (v >= 0 && x >= v >> 16 && x <= (v & 0xffff)) {
                     if (lo < 0) lo = y;
                     hi = y;
                 }
-            cy0[i] = static_cast<int16_t>(lo);
-            cy1[i] = static_cast<int16_t>(hi);
-        }
-    const int q0 = LD(a.rowptr, frow0, a.rowptr_n), q1 = LD(a.rowptr, frow0 + nyp, a.rowptr_n);
-    int m0 = 0, nm = 0;                                        // fine members m0 .. m0 + nm - 1 of each type's block
-    if (q1 > q0) {
-        const Seg sl = LD(a.seg, at.segPf + q1 - 1, a.seg_n);
-        m0 = LD(a.seg, at.segPf + q0, a.seg_n).off;
-        nm = sl.off + (sl.x1 - sl.x0 + 1) - m0;
-    }
-    const bool listed = nm <= L.memN;
-    if (listed)
-        for (int q = q0 + tid; q < q1; q += blockDim.x) {
-            const Seg g = LD(a.seg, at.segPf + q, a.seg_n);
-            const int at0 = static_cast<int>(g.row - static_cast<int64_t>(nyp) * zb) * nxp;
-            for (int x = g.x0; x <= g.x1; ++x) ST(memb, g.off - m0 + (x - g.x0), L.memN, static_cast<uint16_t>(at0 + x));
+            }
+            cyr[i] = lo < 0 ? -1 : lo << 16 | hi;
         }
     __syncthreads();
-    if (tid == 0) {
-        pq[0] = 0;
-        for (int q = 0; q < nbb; ++q) pq[q + 1] = pq[q] + max(0, cq1[q] - cq0[q] + 1);
-    }
-    if (tid == 32) {
-        rqp[0] = 0;
-        for (int i = 0; i < 2 * nbb; ++i) rqp[i + 1] = rqp[i] + max(0, rq1[i] - rq0[i] + 1);
-    }
-    if (tid == 64) {
-        hp[0] = 0;
-        for (int i = 0; i < 2 * L.nb_x; ++i) hp[i + 1] = hp[i] + max(0, hhi[i] - hlo[i] + 1);
-    }
-    __syncthreads();
-    auto find = [](const int* pre, int n, int i) {             // the entry e with pre[e] <= i < pre[e + 1]
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int m = (lo + hi + 1) >> 1;
-            if (pre[m] <= i) lo = m;
-            else hi = m - 1;
+    // pre[e] = the counts of entries before e (a warp)
+    auto scan = [&](int* pre, int n, auto count) {
+        if (lane == 0) pre[0] = 0;
+        int base = 0;
+        for (int k = 0; k < n; k += 32) {
+            int v = k + lane < n ? count(k + lane) : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            if (k + lane < n) pre[k + lane + 1] = base + v;
+            base += __shfl_sync(0xffffffffu, v, 31);
         }
-        return lo;
     };
+    if (warp == 0)
+        scan(pq, nbb, [&](int q) {
+            cq0[q] = max(cq0[q], 0);
+            cq1[q] = min(cq1[q], X - 1);
+            return max(0, cq1[q] - cq0[q] + 1);
+        });
+    if (warp == 1)
+        scan(rqp, 2 * nbb, [&](int i) {
+            rq0[i] = max(rq0[i], -dx);                         // columns of the D plane
+            rq1[i] = min(rq1[i], nx - 1 - dx);
+            return max(0, rq1[i] - rq0[i] + 1);
+        });
+    if (warp == 2) scan(hp, 2 * L.nb_x, [&](int e) { return max(0, hhi[e] - hlo[e] + 1); });
+    __syncthreads();
     // tasks, block-major: consecutive rows (columns) of a block on consecutive lanes (odd row
-    // strides: no bank conflicts, and nearly equal kinetic hulls)
-    const int ntx = hp[2 * L.nb_x], nty = rqp[2 * nbb];
-    for (int i = tid; i < ntx; i += blockDim.x) {
-        const int e = find(hp, 2 * L.nb_x, i);
-        ST(task, i, L.taskN, static_cast<uint16_t>((e << kx) | (hlo[e] + (i - hp[e]))));
-    }
-    for (int i = tid; i < nty; i += blockDim.x) {
-        const int e = find(rqp, 2 * nbb, i);
-        ST(taskk, i, L.taskkN, static_cast<uint16_t>((e << ky) | (rq0[e] + (i - rqp[e]))));
-    }
+    // strides: no bank conflicts, and nearly equal kinetic hulls); a warp per block
+    const int ntx = hp[2 * L.nb_x], nty = rqp[2 * nbb], nwarp = blockDim.x >> 5;
+    for (int e = warp; e < 2 * L.nb_x; e += nwarp)
+        for (int b = hlo[e] + lane; b <= hhi[e]; b += 32)
+            ST(task, hp[e] + b - hlo[e], L.taskN, static_cast<uint16_t>((e << kx) | b));
+    for (int e = nwarp - 1 - warp; e < 2 * nbb; e += nwarp)
+        for (int x = rq0[e] + lane; x <= rq1[e]; x += 32)
+            ST(taskk, rqp[e] + x - rq0[e], L.taskkN, static_cast<uint16_t>((e << ky) | x));
     const T ks = static_cast<T>(a.kin_scale);
     const int pnp = nyp * nxp;
     const int64_t gplane = static_cast<int64_t>(pnp) * nzp;
     const FastDiv fd_nxp(nxp);
-    if (dplane) stage_D(r0);
     for (int c = 0; c < cnt; ++c) {
         const FnRec r = a.fn[fl + c];
         const T* Bb = static_cast<const T*>(a.ws) + r.ws_Bb + (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
@@ -2077,17 +2102,8 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
 #else
         const int rem = static_cast<int>((reinterpret_cast<uintptr_t>(Bb) & 15) / sizeof(T));
         T* const pl = plb + rem;
-        if (tid == 0) {
-            const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(rem + Y * X) * sizeof(T) + 15) & ~size_t(15));
-            bulk_fence();                                      // Gs was read and written there
-            bulk_expect(mbar, bytes);
-            bulk_load(tc::saddr(plb), Bb - rem, bytes, mbar);
-        }
-        if (!dead && !tc::mbar_wait(mbar, phase)) {
-            atomicOr(st, ST_WAIT_TIMEOUT);
-            dead = 1;
-        }
-        phase ^= 1;
+        if (tid == 0 && c > 0) load_Bb(r);
+        wait();
 #endif
 #ifdef LSW_CHECKED
         cp_wait();
@@ -2119,7 +2135,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                 int woff, wstride, first, n;
                 // the arm: D row or column a0 (stride sd), window position p is D position f0 + p of kn
                 int a0 = 0, sd = 1, f0 = 0, kn = 0, dist = 0, h0 = 0, h1 = 0;
-                const int16_t *hl = lx0, *hh = lx1;
+                const int* hull = lxr;
                 int out, ostep, onum, odist;                    // outputs j < onum at out + j ostep (+ odist)
                 if (ph == 0) {
                     int q = 0;
@@ -2165,8 +2181,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                     a0 = bx * PS + x;
                     sd = RS;
                     dist = 2 * PS;
-                    hl = cy0;
-                    hh = cy1;
+                    hull = cyr;
                     h0 = (bz == 0 && bx == 0 ? 0 : nx) + x;
                     h1 = nx + x;
                 }
@@ -2180,8 +2195,9 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                 if (ph > 0 && dplane) {
                     int s0 = Arm::NP, e0 = 0, s1 = Arm::NP, e1 = 0;
                     if (on && kn) {
-                        if (hl[h0] >= 0) s0 = hl[h0] - f0, e0 = hh[h0] - f0 + 1;
-                        if (hl[h1] >= 0) s1 = hl[h1] - f0, e1 = hh[h1] - f0 + 1;
+                        const int v0 = hull[h0], v1 = hull[h1];
+                        if (v0 >= 0) s0 = (v0 >> 16) - f0, e0 = (v0 & 0xffff) - f0 + 1;
+                        if (v1 >= 0) s1 = (v1 >> 16) - f0, e1 = (v1 & 0xffff) - f0 + 1;
                     }
                     s0 = __reduce_min_sync(0xffffffffu, s0);
                     e0 = __reduce_max_sync(0xffffffffu, e0);
@@ -2253,13 +2269,8 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         if (a.gstage) {
 #ifdef LSW_CHECKED
             cp_wait();
-#else
-            if (!dead && !tc::mbar_wait(mbar, phase)) {
-                atomicOr(st, ST_WAIT_TIMEOUT);
-                dead = 1;
-            }
-            phase ^= 1;
 #endif
+            wait();
         }
         __syncthreads();
         if (c + 1 < cnt && dplane) stage_D(a.fn[fl + c + 1]);  // the D plane is dead; in flight during the write
@@ -2273,6 +2284,9 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
             if (a.gstage) return LD(mid, (t & 3) * slot + g_rem(t & 3) + i - g_r0, mid_n);
             return LD(G, t * gplane + static_cast<int64_t>(zb) * pnp + i, 8 * gplane);
         };
+        int nk = 0;
+        int2 ni = make_int2(0, -1);
+        if (fetch && c + 1 == cnt) nk = atomicAdd(a.queue + 1, 1);
         if (bz == 0) {                                         // scaling part s (type 0) on the coarse members
             for (int b = ylo_ + warp; b <= yhi_; b += (blockDim.x >> 5)) {
                 if (rx0[b] < 0) continue;
@@ -2286,6 +2300,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                 }
             }
         }
+        if (fetch && c + 1 == cnt) ni = item(nk);
         for (int m = tid; m < nm; m += blockDim.x) {
             int i;
             if (listed) {
@@ -2312,6 +2327,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                 ST(out, at.ncP + static_cast<int64_t>(t - 1) * at.nfP + m0 + m, out_room, v);
             }
         }
+        if (fetch && c + 1 == cnt) *s_next = ni;
         const double ekin = warp_sum(static_cast<double>(ekin_t));
         if (lane == 0 && ekin != 0.0) atomicAdd(a.e_kin + r.f, ekin);
         __syncthreads();                                       // Gs and mid are free for the next function
@@ -2330,16 +2346,19 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
     __syncthreads();
     uint32_t phase = 0;
     if (a.items_bwd) {
-        __shared__ int s_item;
+        __shared__ int2 s_item;
+        if (threadIdx.x == 0) {
+            const int k = atomicAdd(a.queue + 1, 1);
+            s_item = k < a.n_items_bwd ? a.items_bwd[k] : make_int2(0, -1);
+        }
+        __syncthreads();
         for (;;) {
-            const int k = next_item(a.queue + 1, &s_item);
-            if (k >= a.n_items_bwd) break;
-            const int2 it = LD(a.items_bwd, k, a.n_items_bwd);
-            bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase);
-            __syncthreads();   // shared memory and s_item are reused by the next item
+            const int2 it = s_item;   // (the next one is written behind the plane's barriers)
+            if (it.y < 0) break;
+            bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase, &s_item);
         }
     } else {
-        bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase);
+        bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase, nullptr);
     }
 }
 
