@@ -434,7 +434,7 @@ lsw_status lsw_load_phi(lsw_system sys, const char* path, void* phi_dev);
  * consecutive tile-z layers are built and consumed slab by slab, default 8192),
  * "persistent" (bit 0: the backward FMA plane kernel of H phi, bit 1: the forward one,
  * runs as a persistent grid, as many CTAs as fit on the GPU, taking the batch's
- * (function, plane) items largest first from a device queue; a clear bit: one CTA per
+ * (functions of an atom, plane) items largest first from a device queue; a clear bit: one CTA per
  * plane slot of a (planes, functions) grid; the default 1, the backward kernel only,
  * measured fastest; the results are the same bits), "fwd_list" (1, the default: the forward plane kernel's x
  * pass computes only the blocks whose input window meets the row's members of L and

@@ -626,7 +626,8 @@ __global__ void __launch_bounds__(256) k_fwd_xy(HphiLaunch a) {
 // 30 + 2 q + b, and the block of outputs 2 p0 .. 2 p0 + 7 overwrites slots that no later block
 // reads (the next one starts at input p0 - 11, slot 2 p0 + 8).  With the inputs and the
 // products in buffers of their own, shared memory held 8 warps per SM and the kernel waited on
-// its own latencies (issue 54 %): 3.0 -> 2.4 us per function at radii 5-8 bohr.  V is fetched a block ahead into registers.
+// its own latencies (issue 54 %): 3.0 -> 2.4 us per function at radii 5-8 bohr.  V is fetched a
+// block ahead into registers.
 // FP64 (bound by the FP64 pipe): products run over the hull of the warp's nonzero inputs, per
 // type, and within the column, not over zeros: 82 -> 53 us per function at 6 bohr.
 constexpr int Z_HEAD = 30;            // slots ahead of the inputs
@@ -2728,8 +2729,8 @@ __global__ void __launch_bounds__(DT_THREADS) k_density(DensLaunch a) {
     P.store(a);
 }
 
-// The same for tiles whose records and positions do not fit: a chunk's records at a time, the
-// pattern searched per pair of chunks.
+// The same for grids with a tile whose tables do not fit: a chunk's records at a time, the pattern
+// searched per pair of chunks (300 atoms: 9.2 ms where the tables give 7.6).
 template <class T>
 __global__ void __launch_bounds__(DT_THREADS) k_density_big(DensLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
