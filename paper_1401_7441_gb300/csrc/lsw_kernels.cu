@@ -110,48 +110,62 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 
 // ---------------------------------------------------------------- uncompress / compress
 
+// Bound: the chain of loads ahead of a row's stores (record, rows, segments, values), then DRAM.  An
+// atom's functions have the same rows: with `group` functions per grid slot the tables are read
+// once for those of one atom (FP32, 6 CTAs an SM): 1.75 -> 1.35 ms for 1,200 atoms of radii 5-8
+// bohr, 4.11 -> 2.92 ms for 3,000 dense ones.
 template <class T>
-__global__ void __launch_bounds__(256) k_uncompress(HphiLaunch a) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4) k_uncompress(HphiLaunch a, int group) {
     // Warp per (y, z) row of the L box: writes all 8 types of the row, the members' values
     // from the compressed phi (one coarse segment per row of the sphere, a few fine
     // segments) and zero elsewhere, so the box needs no separate clearing.
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 1;
-    const FnRec r = a.fn[blockIdx.y];
-    const AtomRec& at = a.atoms[r.atom];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nx = r.n[0], nrows = r.n[1] * r.n[2];
     const int row = blockIdx.x * (blockDim.x >> 5) + warp;
-    if (row >= nrows) return;
-    const int64_t plane = static_cast<int64_t>(nx) * nrows;
-    T* D = static_cast<T*>(a.ws) + r.ws_D + static_cast<int64_t>(row) * nx;
-    const T* phi = static_cast<const T*>(a.phi) + r.off_phi;
-    const int64_t phi_room = a.phi_n - r.off_phi;
-    const int c0 = LD(a.rowptr, at.rowLc + row, a.rowptr_n), c1 = LD(a.rowptr, at.rowLc + row + 1, a.rowptr_n);
-    const int f0 = LD(a.rowptr, at.rowLf + row, a.rowptr_n), f1 = LD(a.rowptr, at.rowLf + row + 1, a.rowptr_n);
-    Seg cs{};
-    cs.x0 = 1;
-    cs.x1 = 0;                                         // empty unless the row has members
-    if (c1 > c0) {
-        cs = LD(a.seg, at.segLc + c0, a.seg_n);
-        if (c1 - c0 > 1 || cs.x0 < 0 || cs.x1 >= nx || cs.row != row) {
-            if (lane == 0) atomicOr(a.status, ST_BAD_SEG);
-            return;
+    const int fe = min(static_cast<int>(blockIdx.y + 1) * group, a.nfn);
+    for (int f = blockIdx.y * group; f < fe;) {
+        const int atom = a.fn[f].atom, first = f;
+        do {
+            ++f;
+        } while (f < fe && a.fn[f].atom == atom);
+        const FnRec& r = a.fn[first];
+        const AtomRec& at = a.atoms[atom];
+        const int nx = r.n[0], nrows = r.n[1] * r.n[2];
+        if (row >= nrows) continue;
+        const int64_t plane = static_cast<int64_t>(nx) * nrows;
+        const int c0 = LD(a.rowptr, at.rowLc + row, a.rowptr_n), c1 = LD(a.rowptr, at.rowLc + row + 1, a.rowptr_n);
+        const int f0 = LD(a.rowptr, at.rowLf + row, a.rowptr_n), f1 = LD(a.rowptr, at.rowLf + row + 1, a.rowptr_n);
+        Seg cs{};
+        cs.x0 = 1;
+        cs.x1 = 0;                                     // empty unless the row has members
+        if (c1 > c0) {
+            cs = LD(a.seg, at.segLc + c0, a.seg_n);
+            if (c1 - c0 > 1 || cs.x0 < 0 || cs.x1 >= nx || cs.row != row) {
+                if (lane == 0) atomicOr(a.status, ST_BAD_SEG);
+                continue;
+            }
         }
-    }
-    for (int x = lane; x < nx; x += 32) {
-        ST(D, x, 8 * plane - static_cast<int64_t>(row) * nx,
-           (x >= cs.x0 && x <= cs.x1) ? LD(phi, cs.off + (x - cs.x0), phi_room) : T(0));
-        // wavelet types: the fine segment of this row holding x, if any
-        int64_t fo = -1;
-        for (int q = f0; q < f1; ++q) {
-            const Seg fs = LD(a.seg, at.segLf + q, a.seg_n);
-            if (x >= fs.x0 && x <= fs.x1) fo = fs.off + (x - fs.x0);
-        }
+        for (int x = lane; x < nx; x += 32) {
+            // wavelet types: the fine segment of this row holding x, if any
+            int64_t fo = -1;
+            for (int q = f0; q < f1; ++q) {
+                const Seg fs = LD(a.seg, at.segLf + q, a.seg_n);
+                if (x >= fs.x0 && x <= fs.x1) fo = fs.off + (x - fs.x0);
+            }
+            for (int k = first; k < f; ++k) {
+                T* D = static_cast<T*>(a.ws) + a.fn[k].ws_D + static_cast<int64_t>(row) * nx;
+                const T* phi = static_cast<const T*>(a.phi) + a.fn[k].off_phi;
+                const int64_t phi_room = a.phi_n - a.fn[k].off_phi;
+                T v[8];
+                v[0] = x >= cs.x0 && x <= cs.x1 ? LD(phi, cs.off + (x - cs.x0), phi_room) : T(0);
 #pragma unroll
-        for (int t = 1; t < 8; ++t)
-            ST(D, t * plane + x, 8 * plane - static_cast<int64_t>(row) * nx,
-               fo >= 0 ? LD(phi, at.ncL + static_cast<int64_t>(t - 1) * at.nfL + fo, phi_room) : T(0));
+                for (int t = 1; t < 8; ++t)
+                    v[t] = fo >= 0 ? LD(phi, at.ncL + static_cast<int64_t>(t - 1) * at.nfL + fo, phi_room) : T(0);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) ST(D, t * plane + x, 8 * plane - static_cast<int64_t>(row) * nx, v[t]);
+            }
+        }
     }
 }
 
@@ -3089,10 +3103,17 @@ cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int*
         trace_end(TR, S);               \
     } while (0)
 
+// Functions per grid slot of k_uncompress: eight where that leaves eight waves of CTAs (six an SM), else
+// four (batches of 32 functions, 64 atoms: 89 us with four, 119 with one or eight).
+static int uncompress_group(const HphiLaunch& a) {
+    return static_cast<int64_t>(a.nfn) * ((a.max_rowsL + 7) / 8) >= 8 * 8 * 6 * 152 ? 8 : 4;
+}
+
 template <class T>
 static cudaError_t hphi_batch(const HphiLaunch& a, cudaStream_t s) {
     const int nf = a.nfn;
-    TRACED(a.tr, TK_UNCOMPRESS, s, (k_uncompress<T><<<dim3((a.max_rowsL + 7) / 8, nf), 256, 0, s>>>(a)));
+    const int ug = uncompress_group(a);
+    TRACED(a.tr, TK_UNCOMPRESS, s, (k_uncompress<T><<<dim3((a.max_rowsL + 7) / 8, (nf + ug - 1) / ug), 256, 0, s>>>(a, ug)));
     const dim3 gfwd = a.items_fwd ? dim3(a.grid_fwd) : dim3(2 * a.max_nz, nf);
     const dim3 gbwd = a.items_bwd ? dim3(a.grid_bwd) : dim3(2 * a.max_nzp, nf);
     if constexpr (sizeof(T) == 4) {
@@ -3143,11 +3164,12 @@ cudaError_t enqueue_hphi_batch(const HphiLaunch& a, cudaStream_t s) {
 template <class T>
 static cudaError_t dens_batch(HphiLaunch a, cudaStream_t s) {
     const int nf = a.nfn;
+    const int ug = uncompress_group(a);
     constexpr int C = ZCols<T>::C;
     a.items_fwd = a.items_bwd = nullptr;       // one CTA per grid slot here
     a.queue = nullptr;
     a.smem_z = sizeof(T) * 2 * static_cast<size_t>(a.max_nz) * C;
-    TRACED(a.tr, TK_UNCOMPRESS, s, (k_uncompress<T><<<dim3((a.max_rowsL + 7) / 8, nf), 256, 0, s>>>(a)));
+    TRACED(a.tr, TK_UNCOMPRESS, s, (k_uncompress<T><<<dim3((a.max_rowsL + 7) / 8, (nf + ug - 1) / ug), 256, 0, s>>>(a, ug)));
     TRACED(a.tr, TK_FWD_XY, s, (k_fwd_xy<T><<<dim3(2 * a.max_nz, nf), 256, a.smem_fwd, s>>>(a)));
     TRACED(a.tr, TK_DENS_U, s, (k_z_dens<T><<<dim3((a.max_cols + C - 1) / C, nf), C, a.smem_z, s>>>(a)));
     return cudaGetLastError();
