@@ -2005,33 +2005,12 @@ lsw_status build_conf_tables(lsw_system_s* s) {
     return LSW_OK;
 }
 
-// Launch arguments of the confinement kernels for a region: box and map strides over every
-// function's atom, the tables (first call), the batch buffer (a budget of 2 GiB) and the
-// functions per batch.
-lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double* acoef, const double* eps, ConfLaunch* out,
-                        int* batch) {
-    if (s->d_qtab.bytes == 0) {
-        lsw_status e = build_conf_tables(s);
-        if (e != LSW_OK) return e;
-    }
+// Box and map strides of the confinement kernels for a region, over every function's atom.
+// Returns the bytes of one function in the batch buffer.
+size_t conf_strides(const lsw_system_s* s, int region, ConfLaunch* out) {
     ConfLaunch& c = *out;
     std::memset(&c, 0, sizeof(c));
-    c.prec = s->prec;
     c.region = region;
-    c.precond = precond ? 1 : 0;
-    c.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
-    c.atoms = static_cast<const AtomRec*>(s->d_atoms.p);
-    c.seg = static_cast<const Seg*>(s->d_seg.p);
-    c.rowptr = static_cast<const int32_t*>(s->d_rowptr.p);
-    c.off_L = static_cast<const int64_t*>(s->d_offL.p);
-    c.off_Lp = static_cast<const int64_t*>(s->d_offLp.p);
-    c.qtab = static_cast<const double*>(s->d_qtab.p);
-    c.qtab_off = static_cast<const int64_t*>(s->d_qtab_off.p);
-    c.acoef = acoef;
-    c.eps = eps;
-    for (int b = 0; b < 4; ++b)
-        for (int l = 0; l < KIN_TAPS; ++l) c.kin[b][l] = s->ctx->filters.kin[b][l];
-    c.kin_scale = -1.0 / (2.0 * s->h * s->h);
     for (int a = 0; a < s->n_atoms; ++a) {
         if (s->nsf[a] == 0) continue;
         const LocregHost& L = s->L[a];
@@ -2062,13 +2041,48 @@ lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double*
     c.s_comb = align64(3LL * 4 * c.max_m * KIN_TAPS);
     c.s_maps = c.s_mem + c.s_xy + c.s_xz + c.s_x + c.s_row + c.s_oxz;
     const int64_t doubles = c.s_P + 2 * c.s_A + 2 * c.s_B + c.s_F + c.s_comb;
-    const size_t per = static_cast<size_t>(doubles) * sizeof(double) + static_cast<size_t>(c.s_maps);
+    return static_cast<size_t>(doubles) * sizeof(double) + static_cast<size_t>(c.s_maps);
+}
+
+// Functions of a batch: a budget of 2 GiB.
+int conf_batch(const lsw_system_s* s, size_t per) {
     const int64_t nf = static_cast<int64_t>(s->sf_atom.size());
-    const int b = static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, nf, static_cast<int64_t>((size_t(2) << 30) / per)})));
-    if (s->d_cbox.bytes < per * b) {
-        CUDA_TRY(cudaStreamSynchronize(s->stream));
-        CUDA_TRY(s->d_cbox.alloc(per * b));
+    return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, nf, static_cast<int64_t>((size_t(2) << 30) / per)})));
+}
+
+// Launch arguments of the confinement kernels for a region, the tables (first call), the batch
+// buffer and the functions per batch.  The buffer is sized for both regions at the first call and
+// stays where it is: a caller's captured graph holds its address.
+lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double* acoef, const double* eps, ConfLaunch* out,
+                        int* batch) {
+    if (s->d_qtab.bytes == 0) {
+        lsw_status e = build_conf_tables(s);
+        if (e != LSW_OK) return e;
     }
+    ConfLaunch& c = *out;
+    ConfLaunch other;
+    const size_t per = conf_strides(s, region, &c), per_other = conf_strides(s, 1 - region, &other);
+    const int b = conf_batch(s, per);
+    const size_t need = std::max(per * b, per_other * conf_batch(s, per_other));
+    if (s->d_cbox.bytes < need) {
+        CUDA_TRY(cudaStreamSynchronize(s->stream));
+        CUDA_TRY(s->d_cbox.alloc(need));
+    }
+    c.prec = s->prec;
+    c.precond = precond ? 1 : 0;
+    c.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
+    c.atoms = static_cast<const AtomRec*>(s->d_atoms.p);
+    c.seg = static_cast<const Seg*>(s->d_seg.p);
+    c.rowptr = static_cast<const int32_t*>(s->d_rowptr.p);
+    c.off_L = static_cast<const int64_t*>(s->d_offL.p);
+    c.off_Lp = static_cast<const int64_t*>(s->d_offLp.p);
+    c.qtab = static_cast<const double*>(s->d_qtab.p);
+    c.qtab_off = static_cast<const int64_t*>(s->d_qtab_off.p);
+    c.acoef = acoef;
+    c.eps = eps;
+    for (int k = 0; k < 4; ++k)
+        for (int l = 0; l < KIN_TAPS; ++l) c.kin[k][l] = s->ctx->filters.kin[k][l];
+    c.kin_scale = -1.0 / (2.0 * s->h * s->h);
     double* p = static_cast<double*>(s->d_cbox.p);
     auto take = [&](int64_t stride) {
         double* q = p;
@@ -2090,7 +2104,7 @@ lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double*
     c.rowptr_n = static_cast<int64_t>(s->d_rowptr.bytes / sizeof(int32_t));
     c.vec_n = s->off_L.back();
     c.dst_n = s->off_Lp.back();
-    c.n_sf = static_cast<int>(nf);
+    c.n_sf = static_cast<int>(s->sf_atom.size());
     c.n_atoms = s->n_atoms;
     *batch = b;
     return LSW_OK;
