@@ -33,6 +33,7 @@
 //   k_conf_load    compressed phi on L -> the L box P (FP64; members only, zero elsewhere)
 //   k_conf_pass    the passes along z, y, x
 //   k_conf_store   result -> compressed members of L or L' (optionally added to the target)
+//   k_conf_energy  <phi|Q phi> of a function from its rows' sums
 //   k_cg_*         the conjugate-gradient updates, a CTA per function
 #include <algorithm>
 #include <cstdint>
@@ -445,10 +446,10 @@ __global__ void __launch_bounds__(256) k_conf_pass(ConfLaunch a) {
 // ---------------------------------------------------------------- store
 
 // F on the members of the region (0: L, 1: L') -> compressed vector; dst (+)= F (- eps_f P for
-// the preconditioning operator).  e[f] += sum of P F over the members of L.  A warp per row.
+// the preconditioning operator).  With `energy`, the row's sum of P F over the members of L is left
+// in B (read for the last time by the x pass) for k_conf_energy.  A warp per row.
 template <class T>
-__global__ void __launch_bounds__(256) k_conf_store(ConfLaunch a, T* __restrict__ dst, int accumulate,
-                                                    double* __restrict__ e) {
+__global__ void __launch_bounds__(256) k_conf_store(ConfLaunch a, T* __restrict__ dst, int accumulate, int energy) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 23;
     const int k = blockIdx.y;
@@ -486,7 +487,7 @@ __global__ void __launch_bounds__(256) k_conf_store(ConfLaunch a, T* __restrict_
                 for (int t = part ? 1 : 0; t < (part ? 8 : 1); ++t) {
                     const int64_t o = off + (part ? nc + rel + static_cast<int64_t>(t - 1) * nf : rel);
                     double v = LD(F, t * vF + pf, a.s_F);
-                    if (in_L && (a.precond || e)) {
+                    if (in_L && (a.precond || energy)) {
                         const double p = LD(P, t * vP + pp, a.s_P);
                         sum = fma(p, v, sum);
                         v = fma(ef, p, v);
@@ -496,10 +497,25 @@ __global__ void __launch_bounds__(256) k_conf_store(ConfLaunch a, T* __restrict_
             }
         }
     }
-    if (e) {
+    if (energy) {
         sum = warp_sum_c(sum);
-        if (lane == 0 && sum != 0.0) atomicAdd(e + f, sum);
+        if (lane == 0) ST(a.B, k * a.s_B + static_cast<int64_t>(z) * g.m[1] + y, (k + 1) * a.s_B, sum);
     }
+}
+
+// e[f] = the sum of the rows' sums that k_conf_store left, in a fixed order (the same bits on every
+// call); a CTA per function
+__global__ void __launch_bounds__(256) k_conf_energy(ConfLaunch a, double* __restrict__ e) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 24;
+    const int f = static_cast<int>(a.f0) + blockIdx.x;
+    const AtomRec at = LD(a.atoms, LD(a.sf_atom, f, a.n_sf), a.n_atoms);
+    const ConfGeo g = conf_geo(at, a.region);
+    const double* rows = a.B + blockIdx.x * a.s_B;
+    double v = 0.0;
+    for (int i = threadIdx.x; i < g.m[1] * g.m[2]; i += blockDim.x) v += LD(rows, i, a.s_B);
+    v = block_sum_c(v);
+    if (threadIdx.x == 0) e[f] = v;
 }
 
 // ---------------------------------------------------------------- conjugate gradients
@@ -603,12 +619,9 @@ static cudaError_t conf_apply_t(const ConfLaunch& a, const void* vin, void* dst,
     conf_pass<2>(a, s);
     conf_pass<1>(a, s);
     conf_pass<0>(a, s);
-    if (energy) {
-        const cudaError_t e = cudaMemsetAsync(energy + a.f0, 0, static_cast<size_t>(a.nfn) * sizeof(double), s);
-        if (e != cudaSuccess) return e;
-    }
     k_conf_store<T><<<dim3(static_cast<unsigned>(((a.region ? a.max_rows_P : a.max_rows_L) + 7) / 8), a.nfn), 256, 0, s>>>(
-        a, static_cast<T*>(dst), accumulate, energy);
+        a, static_cast<T*>(dst), accumulate, energy != nullptr);
+    if (energy) k_conf_energy<<<a.nfn, 256, 0, s>>>(a, energy);
     return cudaGetLastError();
 }
 

@@ -70,3 +70,28 @@ def test_confinement_and_preconditioner_edges(name, prec):
                 assert np.linalg.norm(x[S.off_L[f]:S.off_L[f] + n] - xr) <= 1e-11 * np.linalg.norm(xr), (name, f)
     finally:
         S.close()
+
+
+@pytest.mark.parametrize("prec", [lsw.LSW_FP64, lsw.LSW_FP32])
+def test_confinement_energy_same_bits_on_every_call(prec):
+    # hundreds of rows per function: partial sums added in the order they finish would differ
+    import torch
+    N, n_sf = (41, 39, 40), 6
+    S = lsw.System(N, H, np.array([[9.7, 9.6, 10.1]]), np.array([6.0]), np.array([2.2]), np.array([n_sf]), 4.0, 0, 8.0, 0,
+                   prec, device=0, stream=torch.cuda.current_stream().cuda_stream)
+    try:
+        dt = torch.float64 if prec == lsw.LSW_FP64 else torch.float32
+        rng = np.random.default_rng(7)
+        phi = torch.tensor(rng.standard_normal(S.total_L), dtype=dt, device="cuda")
+        a = torch.tensor(rng.uniform(0.001, 0.01, n_sf), device="cuda")
+        hphi = torch.zeros(S.total_Lp, dtype=dt, device="cuda")
+        runs = []
+        for _ in range(12):
+            e = torch.full((n_sf,), float("nan"), dtype=torch.float64, device="cuda")
+            lsw.lsw_add_confinement(S.sys, a, phi, hphi, e)
+            lsw.lsw_sync(S.sys, 60.0)
+            runs.append(e.cpu().numpy())
+        assert np.all(np.isfinite(runs[0])) and np.all(runs[0] > 0)
+        assert all(np.array_equal(runs[0], r) for r in runs[1:])
+    finally:
+        S.close()
