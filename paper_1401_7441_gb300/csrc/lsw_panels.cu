@@ -41,7 +41,10 @@ struct SmallDiv {
     __device__ __forceinline__ int div(int n) const { return m ? static_cast<int>(__umulhi(static_cast<uint32_t>(n), m)) : n; }
 };
 
-template <class T, bool Unpack>
+// Small: tile edges 2 and 3 (at most 27 points of each part).  With one part after the other, as for
+// larger tiles, most of a lane's four entries are empty there (edge 3, 200 atoms in FP32: 1.05 ms, so
+// 0.72; at edges from 4 on the parts one after the other are the faster form, 5 to 15 %).
+template <class T, bool Unpack, bool Small>
 __global__ void __launch_bounds__(PK_THREADS, 2) k_pack(PackLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = Unpack ? 12 : 10;
@@ -172,6 +175,30 @@ __global__ void __launch_bounds__(PK_THREADS, 2) k_pack(PackLaunch a) {
                     }
             }
         };
+        if constexpr (Small) {
+            // a lane looks up a coarse and a fine point; the entries of both parts follow one
+            // another in panel order, 128 at a time, then the zero padding
+            int mine_c = -1, mine = -1;
+            if (lane < T3) {
+                const int r = fd_T.div(lane), z = fd_T.div(r);
+                mine_c = rel_of(0, lane - r * TE, r - z * TE, z);
+            }
+            if (lane < tl.nfine) {
+                const int code = LD(a.tile_fine, tl.fine0 + lane, a.fine_n);
+                mine = rel_of(1, code & 255, (code >> 8) & 255, code >> 16);
+            }
+            for (int k0 = 0; k0 < kp; k0 += 128) {
+                int rel[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int e = k0 + 32 * u + lane - T3, q = max(e, 0) / 7;
+                    const int r = __shfl_sync(0xffffffffu, mine, q & 31);
+                    rel[u] = e < 0 ? mine_c : q < 32 && r >= 0 ? r + (e - 7 * q) * nf : -1;
+                }
+                move(k0 + lane, kp, rel);
+            }
+            continue;
+        }
         // coarse points
         for (int kb = lane; kb < T3; kb += 128) {
             int rel[4];
@@ -894,10 +921,14 @@ size_t panel_hs_smem(int prec) {
 
 cudaError_t configure_panel_kernels(size_t max_smem) {
     cudaError_t e;
-    const void* ks[] = {reinterpret_cast<const void*>(k_pack<double, false>),
-                        reinterpret_cast<const void*>(k_pack<float, false>),
-                        reinterpret_cast<const void*>(k_pack<double, true>),
-                        reinterpret_cast<const void*>(k_pack<float, true>),
+    const void* ks[] = {reinterpret_cast<const void*>(k_pack<double, false, false>),
+                        reinterpret_cast<const void*>(k_pack<float, false, false>),
+                        reinterpret_cast<const void*>(k_pack<double, true, false>),
+                        reinterpret_cast<const void*>(k_pack<float, true, false>),
+                        reinterpret_cast<const void*>(k_pack<double, false, true>),
+                        reinterpret_cast<const void*>(k_pack<float, false, true>),
+                        reinterpret_cast<const void*>(k_pack<double, true, true>),
+                        reinterpret_cast<const void*>(k_pack<float, true, true>),
                         reinterpret_cast<const void*>(k_panel_hs<double>),
                         reinterpret_cast<const void*>(k_panel_hs<float>),
                         reinterpret_cast<const void*>(k_panel_combine<double>),
@@ -913,18 +944,22 @@ cudaError_t configure_panel_kernels(size_t max_smem) {
     return cudaSuccess;
 }
 
+template <class T, bool Unpack>
+static void pack(const PackLaunch& a, dim3 grid, cudaStream_t s) {
+    if (a.tile <= 3) TRACED(a.tr, TK_PACK, s, (k_pack<T, Unpack, true><<<grid, PK_THREADS, a.smem, s>>>(a)));
+    else TRACED(a.tr, TK_PACK, s, (k_pack<T, Unpack, false><<<grid, PK_THREADS, a.smem, s>>>(a)));
+}
+
 cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s) {
     if (a.n_slab_atoms == 0) return cudaSuccess;
     const dim3 grid(static_cast<unsigned>(a.n_slab_atoms), a.hphi && !a.out ? 2 : 1);
     if (a.out) {
-        if (a.prec == 0)
-            TRACED(a.tr, TK_PACK, s, (k_pack<double, true><<<grid, PK_THREADS, a.smem, s>>>(a)));
-        else
-            TRACED(a.tr, TK_PACK, s, (k_pack<float, true><<<grid, PK_THREADS, a.smem, s>>>(a)));
+        if (a.prec == 0) pack<double, true>(a, grid, s);
+        else pack<float, true>(a, grid, s);
     } else if (a.prec == 0) {
-        TRACED(a.tr, TK_PACK, s, (k_pack<double, false><<<grid, PK_THREADS, a.smem, s>>>(a)));
+        pack<double, false>(a, grid, s);
     } else {
-        TRACED(a.tr, TK_PACK, s, (k_pack<float, false><<<grid, PK_THREADS, a.smem, s>>>(a)));
+        pack<float, false>(a, grid, s);
     }
     return cudaGetLastError();
 }
