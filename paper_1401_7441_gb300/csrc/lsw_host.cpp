@@ -209,6 +209,7 @@ struct lsw_system_s {
     // the boxes, tables and maps of a batch, and the conjugate-gradient vectors and scalars
     DeviceBuf d_qtab, d_qtab_off, d_cbox, d_cg, d_cgs;
     std::vector<PanelSlab> slabs;
+    int max_tile_nA = 0;                // most functions whose L touches one tile
     DeviceBuf d_shift, d_fn_all;   // reformat: per-atom shifts, records of every function
     // density: real-space store, block records, tile lists (built for one grid)
     DeviceBuf d_U, d_dfn, d_tptr, d_tfn;
@@ -910,6 +911,8 @@ lsw_status build_hs_plan(lsw_system_s* s) {
         sl.smem_pack = need <= smem_cap ? need : 0;
     }
     cudaStream_t st = s->stream;
+    s->max_tile_nA = 0;
+    for (const PanelTile& t : tiles) s->max_tile_nA = std::max<int>(s->max_tile_nA, t.nA);
     CUDA_TRY(s->d_ptiles.upload(tiles, st));
     CUDA_TRY(s->d_patoms.upload(patoms, st));
     CUDA_TRY(s->d_ttab.upload(ttab, st));
@@ -1130,6 +1133,7 @@ PanelHSLaunch product_launch(lsw_system_s* s, Tracer* tr, const PanelSlab& sl, b
     p.listA = static_cast<const int32_t*>(s->d_listA.p);
     p.listB = static_cast<const int32_t*>(s->d_listB.p);
     p.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
+    p.coef_rows = combine_rows(s->max_tile_nA);
     p.row_ptr = static_cast<const int64_t*>(s->d_rowp.p);
     p.col = static_cast<const int32_t*>(s->d_col.p);
     p.PA = s->d_PA.p;

@@ -307,6 +307,7 @@ struct PanelHSLaunch {
     double* H;
     double* S;
     const double* M;             // combination: coefficients on the pattern
+    int coef_rows;               // combination: functions whose coefficients a CTA holds at a time (a multiple of 32)
     int tc;                      // 1: FP32 products on the tensor cores (split bfloat16)
     int* status;
     int64_t listA_n, listB_n, nnz, PA_n, PQ_n, n_tiles;
@@ -450,6 +451,7 @@ cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int*
 cudaError_t enqueue_hphi_batch(const HphiLaunch& a, cudaStream_t s);
 cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s);     // panels of a slab (lsw_panels.cu)
 cudaError_t enqueue_panel_hs(const PanelHSLaunch& a, cudaStream_t s);   // S, H from the panels
+int combine_rows(int max_functions);   // PanelHSLaunch::coef_rows for tiles of at most that many functions
 cudaError_t enqueue_panel_combine(const PanelHSLaunch& a, cudaStream_t s);   // M Phi panels
 cudaError_t enqueue_lowdin_coeffs(const int64_t* row_ptr, const int32_t* col, const double* S, double* T, int n_sf,
                                   cudaStream_t s);

@@ -22,6 +22,7 @@
 //                panel length, 4 x 8 outputs per thread in the system's precision, then
 //                each pattern entry (a, b) gets its tile sum added to S_ab (column in A)
 //                or H_ab (column in Q) in FP64.
+#include <algorithm>
 #include <cstdint>
 
 #include "lsw_device.h"
@@ -705,28 +706,31 @@ __global__ void __launch_bounds__(256, 2) k_panel_hs_tc(PanelHSLaunch a) {
 
 // ---------------------------------------------------------------- sparse combination
 
-// (M Phi)_a = P_L(a) sum_b M_ab phi_b (Sec. "Orthogonalization", Eq. gradient): per work
-// item (tile, up to 64 A rows, a range of panel entries), the A panel's rows combined with the coefficients M_ab of the tile's A functions (looked up in the
-// pattern CSR, 0 outside it), written to the output panel at the A panel's place in the
-// Q buffer; the unpack then copies each member of L(a) from the tile holding it.
+// (M Phi)_a = P_L(a) sum_b M_ab phi_b (Sec. "Orthogonalization", Eq. gradient): per work item
+// (tile, up to 64 A rows, a range of panel entries), the A panel's rows combined with the
+// coefficients M_ab of the tile's A functions (looked up in the pattern CSR, 0 outside it),
+// written to the output panel at the A panel's place in the Q buffer; the unpack then copies
+// each member of L(a) from the tile holding it.
 //
 // The functions of an atom are consecutive in a tile's list and in the pattern, and their
 // pattern rows are equal: the pattern is searched once per pair of atoms (of the item's rows
 // and of a chunk of 32 functions), not once per coefficient, and the coefficients stay in shared
-// memory for all of the tile's panel entries (an item per 128 entries looked them up again).
-// 600 atoms (2,049 functions, tile edge 6): 1.32 -> 0.76 ms.
+// memory for all of the item's panel entries.  Items of few coefficients (small tiles) are a
+// chain of loads, which only more CTAs on an SM cover: three in FP32 (two in FP64, whose pipe is
+// the bound), room for no more coefficients than the fullest tile has, the first panel rows
+// fetched ahead of the lookups.  600 atoms (2,049 functions, tile edge 6), FP32: 1.31 -> 0.63 ms;
+// 64 atoms, edge 4, FP64: 0.54 -> 0.25 ms.
 constexpr int PC_J = PH_KC;      // functions looked up and combined per chunk
-constexpr int PC_R = 128;        // functions whose coefficients a CTA holds
+constexpr int PC_R = 128;        // most functions whose coefficients a CTA holds (a.coef_rows: the room taken)
 
-// Leaders of the runs of equal atoms among fn[0 .. n): ld[i] = first index of i's run, run[i] its
+// Leaders of the runs of equal atoms among atom[0 .. n): ld[i] = first index of i's run, run[i] its
 // number, list[r] the leader of run r.  One warp; n <= 64.  Returns the number of runs.
-__device__ __forceinline__ int comb_runs(const int* fn, int n, const int32_t* __restrict__ sf_atom, int* ld, int* run,
-                                         int* list) {
+__device__ __forceinline__ int comb_runs(const int* atom, int n, int* ld, int* run, int* list) {
     const int lane = threadIdx.x & 31;
     int runs = 0, lead = 0, last = -1;                     // carried from the first 32 to the next
     for (int b = 0; b < n; b += 32) {
         const int i = b + lane;
-        const int at = i < n ? sf_atom[fn[i]] : -2;
+        const int at = i < n ? atom[i] : -2;
         int before = __shfl_up_sync(0xffffffffu, at, 1);
         if (lane == 0) before = last;
         const unsigned m = __ballot_sync(0xffffffffu, i < n && at != before);
@@ -744,15 +748,20 @@ __device__ __forceinline__ int comb_runs(const int* fn, int n, const int32_t* __
 }
 
 template <class T>
-__global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_panel_combine(PanelHSLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 13;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* sM = reinterpret_cast<T*>(smem_raw);            // [PC_R][LDA]: M[a0 + i][jb + j] at [j][i]
-    T* sP = sM + PC_R * PH_LDA;                        // [KC][LDC]: PA[j0 + j][c0 + c] at [j][c]
-    constexpr int SM_N = PC_R * PH_LDA, SP_N = PH_KC * PH_LDC;
-    __shared__ int fa[PH_M], lda[PH_M], runa[PH_M], lista[PH_M], fb[PC_J], ldb[PC_J], runb[PC_J], listb[PC_J], nrun[2];
-    __shared__ int rel[PH_M * PC_J];                   // per pair of runs: position of the leader's column in the row, -1: none
+    const int R = a.coef_rows;
+    T* sM = reinterpret_cast<T*>(smem_raw);            // [R][LDA]: M[a0 + i][jb + j] at [j][i]
+    T* sP = sM + R * PH_LDA;                           // [KC][LDC]: PA[j0 + j][c0 + c] at [j][c]
+    [[maybe_unused]] const int SM_N = R * PH_LDA;
+    constexpr int SP_N = PH_KC * PH_LDC;
+    __shared__ int ata[PH_M], lda[PH_M], runa[PH_M], lista[PH_M];                  // the item's rows: atom, run
+    __shared__ int fb[PC_J], atb[PC_J], ldb[PC_J], runb[PC_J], listb[PC_J], nrun[2];   // a chunk's functions
+    // per pair of runs: position of the leader's column in the row, -1: none (in sP, not in use then)
+    int* const rel = reinterpret_cast<int*>(sP);
+    static_assert(PH_M * PC_J * sizeof(int) <= SP_N * sizeof(T), "room for the positions");
     __shared__ long long rpa[PH_M];
     __shared__ int lena[PH_M];
     const PanelItem it = LD(a.items, blockIdx.x, a.nitems);
@@ -762,46 +771,75 @@ __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
     T* PO = static_cast<T*>(const_cast<void*>(a.PQ));
     const int tid = threadIdx.x;
     const int ti = tid >> 4, tj = tid & 15;
-    if (tid < it.na) {
+    // panel rows of a chunk: thread (row j = tid >> 3, quads (tid & 7) + 8 m), a chunk ahead in registers
+    Quad<T> pre[4];
+    auto fetch = [&](int j0, int jend, int c0, int nc) {
+        const int j = tid >> 3;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int c = 4 * ((tid & 7) + 8 * m);
+            if (j0 + j < jend && c < nc)
+                ld4(pre[m], PA, tl.pA + static_cast<int64_t>(j0 + j) * kp + c0 + c, a.PA_n, ST_, KID);
+            else
+                pre[m].zero();
+        }
+    };
+    // position of column f in the row of len entries from r0; -1: none
+    auto find = [&](int64_t r0, int len, int f) -> int {
+        int lo = 0, hi = len - 1;
+        while (lo <= hi) {
+            const int mid = (lo + hi) >> 1;
+            const int cm = LD(a.col, r0 + mid, a.nnz);
+            if (cm == f) return mid;
+            if (cm < f) lo = mid + 1;
+            else hi = mid - 1;
+        }
+        return -1;
+    };
+    // few coefficients (small tiles): each thread looks its own up; a chain of loads is all such an
+    // item takes, and the runs would add two barriers and a load to it
+    const bool few = it.na * tl.nA <= 2 * static_cast<int>(blockDim.x);
+    if (!few && tid < it.na) {
         const int f = LD(a.listA, tl.listA + it.a0 + tid, a.listA_n);
-        fa[tid] = f;
         const int64_t r0 = LD(a.row_ptr, f, a.n_sf + 1);
         rpa[tid] = r0;
         lena[tid] = static_cast<int>(LD(a.row_ptr, f + 1, a.n_sf + 1) - r0);
+        ata[tid] = LD(a.sf_atom, f, a.n_sf);
     }
-    __syncthreads();
-    if (tid < 32) {
-        const int r = comb_runs(fa, it.na, a.sf_atom, lda, runa, lista);
-        if (tid == 0) nrun[0] = r;
-    }
-    for (int jb = 0; jb < tl.nA; jb += PC_R) {
-        const int nr = min(PC_R, tl.nA - jb);
+    for (int jb = 0; jb < tl.nA; jb += R) {
+        const int nr = min(R, tl.nA - jb);
+        fetch(jb, jb + nr, it.c0, min(PH_N, it.nc));   // in flight during the lookups
         // ---- the coefficients M[a0 ..][jb .. jb + nr), for every panel entry of the item
-        for (int j0 = 0; j0 < nr; j0 += PC_J) {
+        if (few) {
+            for (int e = tid; e < it.na * nr; e += blockDim.x) {
+                const int j = e / it.na, i = e - j * it.na;
+                const int fi = LD(a.listA, tl.listA + it.a0 + i, a.listA_n), fj = LD(a.listA, tl.listA + jb + j, a.listA_n);
+                const int64_t r0 = LD(a.row_ptr, fi, a.n_sf + 1);
+                const int r = find(r0, static_cast<int>(LD(a.row_ptr, fi + 1, a.n_sf + 1) - r0), fj);
+                ST(sM, j * PH_LDA + i, SM_N, r >= 0 ? static_cast<T>(LD(a.M, r0 + r, a.nnz)) : T(0));
+            }
+        }
+        for (int j0 = 0; j0 < (few ? 0 : nr); j0 += PC_J) {
             const int nj = min(PC_J, nr - j0);
-            if (tid < nj) fb[tid] = LD(a.listA, tl.listA + jb + j0 + tid, a.listA_n);
+            if (tid >= 128 && tid < 128 + nj) {        // (the rows' loads are other warps')
+                const int f = LD(a.listA, tl.listA + jb + j0 + (tid - 128), a.listA_n);
+                fb[tid - 128] = f;
+                atb[tid - 128] = LD(a.sf_atom, f, a.n_sf);
+            }
             __syncthreads();
-            if (tid < 32) {
-                const int r = comb_runs(fb, nj, a.sf_atom, ldb, runb, listb);
-                if (tid == 0) nrun[1] = r;
+            if (tid < 32 && jb + j0 == 0) {
+                const int r = comb_runs(ata, it.na, lda, runa, lista);
+                if (tid == 0) nrun[0] = r;
+            }
+            if (tid >= 128 && tid < 160) {
+                const int r = comb_runs(atb, nj, ldb, runb, listb);
+                if (tid == 128) nrun[1] = r;
             }
             __syncthreads();
             for (int e = tid; e < nrun[0] * nrun[1]; e += blockDim.x) {
                 const int ra = e / nrun[1], rb = e - ra * nrun[1];
-                const int i = lista[ra], want = fb[listb[rb]];
-                const int64_t r0 = rpa[i];
-                int lo = 0, hi = lena[i] - 1, pos = -1;
-                while (lo <= hi) {
-                    const int mid = (lo + hi) >> 1;
-                    const int cm = LD(a.col, r0 + mid, a.nnz);
-                    if (cm == want) {
-                        pos = mid;
-                        break;
-                    }
-                    if (cm < want) lo = mid + 1;
-                    else hi = mid - 1;
-                }
-                rel[ra * PC_J + rb] = pos;
+                const int i = lista[ra];
+                rel[ra * PC_J + rb] = find(rpa[i], lena[i], fb[listb[rb]]);
             }
             __syncthreads();
             const int i = tid & 63;                    // thread (i = tid & 63, j = tid >> 6 + 4 m)
@@ -829,20 +867,7 @@ __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
                                     ? LD(PO, tl.pA + static_cast<int64_t>(it.a0 + r) * kp + c0 + cc, a.PQ_n)
                                     : T(0);
                 }
-            // panel rows of a chunk: thread (row j = tid >> 3, quads (tid & 7) + 8 m), a chunk ahead in registers
-            Quad<T> pre[4];
-            auto fetch = [&](int j0) {
-                const int j = tid >> 3;
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const int c = 4 * ((tid & 7) + 8 * m);
-                    if (j0 + j < nr && c < nc)
-                        ld4(pre[m], PA, tl.pA + static_cast<int64_t>(jb + j0 + j) * kp + c0 + c, a.PA_n, ST_, KID);
-                    else
-                        pre[m].zero();
-                }
-            };
-            fetch(0);
+            if (c0 > it.c0) fetch(jb, jb + nr, c0, nc);
             for (int j0 = 0; j0 < nr; j0 += PH_KC) {
                 const int nj = 8 * (tid >> 5) < it.na ? min(PH_KC, nr - j0) : 0;   // a warp past the rows: none
 #pragma unroll
@@ -850,7 +875,7 @@ __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
 #pragma unroll
                     for (int e = 0; e < 4; ++e) ST(sP, (tid >> 3) * PH_LDC + 4 * ((tid & 7) + 8 * m) + e, SP_N, pre[m][e]);
                 __syncthreads();
-                if (j0 + PH_KC < nr) fetch(j0 + PH_KC);
+                if (j0 + PH_KC < nr) fetch(jb + j0 + PH_KC, jb + nr, c0, nc);
 #ifndef LSW_CHECKED
                 if constexpr (sizeof(T) == 4) {
                     // 16-byte shared loads and packed two-lane FMAs (the same bits as below)
@@ -883,11 +908,16 @@ __global__ void __launch_bounds__(256) k_panel_combine(PanelHSLaunch a) {
 #pragma unroll
                     for (int c = 0; c < 4; ++c) cv[c] = LD(sP, j * PH_LDC + 4 * tj + c, SP_N);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) cv[4 + c] = wide ? LD(sP, j * PH_LDC + 64 + 4 * tj + c, SP_N) : T(0);
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
+                    if (!wide) continue;               // the second half of the columns holds none
+#pragma unroll
+                    for (int c = 4; c < 8; ++c) cv[c] = LD(sP, j * PH_LDC + 60 + 4 * tj + c, SP_N);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
 #pragma unroll
-                        for (int c = 0; c < 8; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
+                        for (int c = 4; c < 8; ++c) acc[i][c] = fma(av[i], cv[c], acc[i][c]);
                 }
                 __syncthreads();
             }
@@ -964,9 +994,15 @@ cudaError_t enqueue_pack(const PackLaunch& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The chunks of 32 that the fullest tile needs, up to PC_R: small tiles hold few functions, and their
+// items are short chains of lookups that only more CTAs on an SM cover.
+int combine_rows(int max_functions) {
+    return std::min(PC_R, (std::max(max_functions, 1) + PC_J - 1) / PC_J * PC_J);
+}
+
 cudaError_t enqueue_panel_combine(const PanelHSLaunch& a, cudaStream_t s) {
     if (a.nitems == 0) return cudaSuccess;
-    const size_t smem = (static_cast<size_t>(PC_R) * PH_LDA + static_cast<size_t>(PH_KC) * PH_LDC) *
+    const size_t smem = (static_cast<size_t>(a.coef_rows) * PH_LDA + static_cast<size_t>(PH_KC) * PH_LDC) *
                         (a.prec == 0 ? sizeof(double) : sizeof(float));
     if (a.prec == 0)
         TRACED(a.tr, TK_HS, s, (k_panel_combine<double><<<static_cast<unsigned>(a.nitems), 256, smem, s>>>(a)));

@@ -54,3 +54,27 @@ def test_matrices_and_combination_by_tile_edge(name, tile, prec):
     finally:
         S.close()
 
+
+@pytest.mark.parametrize("prec,n_atoms", [(lsw.LSW_FP64, 60), (lsw.LSW_FP32, 250)])
+def test_combination_same_bits_for_every_tile_edge(prec, n_atoms):
+    import torch
+    wl = I.scaled("atoms10k", n_atoms, seed=9)
+    dt = torch.float64 if prec == lsw.LSW_FP64 else torch.float32
+    S = lsw.System(wl.N, wl.h, wl.pos, wl.r_loc, wl.r_fine, wl.nsf, wl.pair_cutoff, wl.pair_mode, wl.lprime_margin, 0,
+                   prec, device=0, stream=torch.cuda.current_stream().cuda_stream)
+    try:
+        gen = torch.Generator(device="cuda").manual_seed(3)
+        phi = torch.randn(S.total_L, generator=gen, dtype=dt, device="cuda")
+        M = torch.rand(len(S.col), generator=gen, dtype=torch.float64, device="cuda") - 0.5
+        outs = []
+        for tile in (8, 3, 6, 5, 2):
+            lsw.lsw_set_option(S.sys, "tile", tile)
+            out = torch.zeros_like(phi)
+            lsw.lsw_combine(S.sys, M, phi, out)
+            lsw.lsw_sync(S.sys, 60.0)
+            outs.append(out)
+        assert float(outs[0].abs().max()) > 0.0
+        for out in outs[1:]:
+            assert torch.equal(out, outs[0])
+    finally:
+        S.close()
