@@ -858,24 +858,36 @@ lsw_status build_hs_plan(lsw_system_s* s) {
                             it.pad = 0;
                             items.push_back(it);
                         }
-                    // combination: all of a tile's panel entries with one set of coefficients, or 128
-                    // of them where that leaves too few items to fill the GPU
-                    const int cw = static_cast<int64_t>(tiles.size()) >= 8LL * s->ctx->n_sm ? std::max(pt.kp, 1) : 128;
-                    for (int a0 = 0; a0 < pt.nA; a0 += 64)
-                        for (int c0 = 0; c0 < pt.kp; c0 += cw) {
-                            PanelItem it;
-                            it.tile = static_cast<int32_t>(w);
-                            it.a0 = a0;
-                            it.na = std::min(64, pt.nA - a0);
-                            it.c0 = c0;
-                            it.nc = std::min(cw, pt.kp - c0);
-                            it.pad = 0;
-                            citems.push_back(it);
-                        }
                 }
                 u = v;
                 if (u < tiles.size()) tz = tiles[u].org[2] / T;
                 else break;
+            }
+            // combination items: up to 64 A rows of a tile and as many blocks of 128 panel entries as
+            // keep the item's products, blocks x functions, under 1/16 of an SM's share of the slab's:
+            // one set of coefficients serves them, and no item outlasts the others.  150 atoms in
+            // FP64, edge 8: 3.1 ms (6.0 with all of a tile's entries in an item, 3.5 and 3.0 with 1/6
+            // and 1/40); 300 atoms in FP32, edge 8: 0.35 ms (1/6: 0.38, 1/40: 0.43).
+            constexpr int64_t SHARES = 16;             // per SM
+            auto blocks = [](int n, int w) { return static_cast<int64_t>((n + w - 1) / w); };
+            int64_t work = 0;
+            for (size_t w = static_cast<size_t>(sl.u0); w < u; ++w)
+                work += blocks(tiles[w].nA, 64) * blocks(tiles[w].kp, 128) * tiles[w].nA;
+            const int64_t share = work / (SHARES * s->ctx->n_sm);
+            for (size_t w = static_cast<size_t>(sl.u0); w < u; ++w) {
+                const PanelTile& pt = tiles[w];
+                const int cw = 128 * static_cast<int>(std::max<int64_t>(1, std::min(blocks(pt.kp, 128), share / std::max(pt.nA, 1))));
+                for (int a0 = 0; a0 < pt.nA; a0 += 64)
+                    for (int c0 = 0; c0 < pt.kp; c0 += cw) {
+                        PanelItem it;
+                        it.tile = static_cast<int32_t>(w);
+                        it.a0 = a0;
+                        it.na = std::min(64, pt.nA - a0);
+                        it.c0 = c0;
+                        it.nc = std::min(cw, pt.kp - c0);
+                        it.pad = 0;
+                        citems.push_back(it);
+                    }
             }
             sl.tz1 = u < tiles.size() ? tiles[u].org[2] / T : nt[2];
             sl.u1 = static_cast<int64_t>(u);
