@@ -2413,8 +2413,8 @@ struct __align__(16) DensRec {       // one function of a chunk
 };
 
 // u_f at the thread's points (x, y, z + i); 0 outside f's block.
-template <class T>
-__device__ __forceinline__ void dens_u(const DensLaunch& a, const DensRec& df, int x, int y, int z, T (&u)[DT_PP]) {
+template <class T, class Rec>
+__device__ __forceinline__ void dens_u(const DensLaunch& a, const Rec& df, int x, int y, int z, T (&u)[DT_PP]) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 13;
     const int lx = x - df.o[0], ly = y - df.o[1], lz = z - df.o[2];
@@ -2807,6 +2807,61 @@ __global__ void __launch_bounds__(DT_THREADS) k_density_big(DensLaunch a) {
     P.store(a);
 }
 
+// Grids whose tiles hold at most M functions: every coefficient looked up by a thread of its own
+// while the threads load the functions' values, one barrier.  There the tables and the masks above
+// are only a longer chain of loads and barriers.  Kernel times with them, with M = 8 and with M = 16:
+// one function on a 31^3 box FP32 33.8, 6.1, 8.1 us, FP64 103, 17, 30; two atoms (8 functions) FP32
+// 47, 15, 23, FP64 194, 111, 209; four atoms (13 functions) FP32 68, -, 30, FP64 343, -, 360: up to
+// 16 in FP32, up to 8 in FP64.  The same sums in the same order as for one chunk.
+template <class T, int M>
+__global__ void __launch_bounds__(DT_THREADS) k_density_few(DensLaunch a) {
+    [[maybe_unused]] int* ST_ = a.status;
+    [[maybe_unused]] constexpr int KID = 13;
+    __shared__ T kb[M * M];
+    const int64_t t0 = LD(a.tptr, blockIdx.x, a.tptr_n);
+    const int m = static_cast<int>(LD(a.tptr, blockIdx.x + 1, a.tptr_n) - t0);
+    DensPoints<T> P;
+    P.init(a);
+    for (int e = threadIdx.x; e < m * m; e += DT_THREADS) {
+        const int ia = e / m, ib = e - ia * m;
+        const int fa = LD(a.tfn, t0 + ia, a.tfn_n), fb = LD(a.tfn, t0 + ib, a.tfn_n);
+        const int64_t rp = LD(a.row_ptr, fa, a.rowp_n);
+        const int r = dens_find(a, rp, fa, fb);
+        kb[ia * M + ib] = r >= 0 ? static_cast<T>(LD(a.K, rp + r, a.nnz)) : T(0);
+    }
+    T u[M][DT_PP];
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i) u[j][i] = T(0);
+        if (j < m) {
+            const DensFn df = LD(a.fn, LD(a.tfn, t0 + j, a.tfn_n), a.fn_n);
+            dens_u<T>(a, df, P.x, P.y, P.z, u[j]);
+        }
+    }
+    __syncthreads();
+    T part[DT_PP];
+#pragma unroll
+    for (int i = 0; i < DT_PP; ++i) part[i] = T(0);
+#pragma unroll
+    for (int ia = 0; ia < M; ++ia) {
+        if (ia >= m) break;
+        T zz[DT_PP];
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i) zz[i] = T(0);
+#pragma unroll
+        for (int ib = 0; ib < M; ++ib)
+            if (ib < m)
+#pragma unroll
+                for (int i = 0; i < DT_PP; ++i) zz[i] += kb[ia * M + ib] * u[ib][i];
+#pragma unroll
+        for (int i = 0; i < DT_PP; ++i) part[i] += u[ia][i] * zz[i];
+    }
+#pragma unroll
+    for (int i = 0; i < DT_PP; ++i) P.acc[i] = static_cast<double>(part[i]);
+    P.store(a);
+}
+
 // Dynamic shared memory of k_density.
 size_t density_smem(int prec, int max_m, int max_g) {
     return static_cast<size_t>(DT_MC) * DT_MC * 2 * (sizeof(double) + (prec == 0 ? sizeof(double) : sizeof(float))) +
@@ -3184,7 +3239,14 @@ cudaError_t enqueue_density(const DensLaunch& a, cudaStream_t s) {
     if (nt == 0) return cudaSuccess;
     const unsigned g = static_cast<unsigned>(nt);
     // tables in shared memory where two CTAs an SM fit with the tile of most functions
-    if (a.max_m > 0) {
+    if (a.max_m > 0 && a.max_m <= (a.prec == 0 ? 8 : 16)) {
+        if (a.prec == 0)
+            TRACED(a.tr, TK_DENSITY, s, (k_density_few<double, 8><<<g, DT_THREADS, 0, s>>>(a)));
+        else if (a.max_m <= 8)
+            TRACED(a.tr, TK_DENSITY, s, (k_density_few<float, 8><<<g, DT_THREADS, 0, s>>>(a)));
+        else
+            TRACED(a.tr, TK_DENSITY, s, (k_density_few<float, 16><<<g, DT_THREADS, 0, s>>>(a)));
+    } else if (a.max_m > 0) {
         const size_t smem = density_smem(a.prec, a.max_m, a.max_g);
         if (a.prec == 0)
             TRACED(a.tr, TK_DENSITY, s, (k_density<double><<<g, DT_THREADS, smem, s>>>(a)));

@@ -61,6 +61,20 @@ def test_density_crowded_tiles(prec, shape):
     assert np.all(got[bound == 0] == 0)
 
 
+# tiles of at most 8 functions (one block of coefficients), 9 to 16 (FP32: another width), 17 (tables)
+@pytest.mark.parametrize("prec", [lsw.LSW_FP64, lsw.LSW_FP32])
+@pytest.mark.parametrize("nsf", [[1], [8], [9], [16], [17], [2, 5]], ids=lambda v: "-".join(map(str, v)))
+def test_density_few_functions(prec, nsf):
+    wl = cluster((8, 9, 7), len(nsf), nsf, [1.6, 1.1], [0.8, 0.5], 0.9 if len(nsf) > 1 else 5.0)
+    gpu = gpu_density(wl, prec, kernel=lambda rp, col, sa: np.random.default_rng(4).uniform(-1.0, 1.0, len(col)))
+    geo = G.build(desc_of(wl))
+    phi = phi_all(wl, geo)
+    rho = Dn.density(geo, phi, gpu["K"], wl.V_lo, wl.V_shape)
+    bound = Dn.density(geo, phi, gpu["K"], wl.V_lo, wl.V_shape, absolute=True)
+    assert np.all(np.abs(gpu["rho"][0] - rho) <= TOL[prec] * bound + FLOOR[prec])
+    assert np.all(gpu["rho"][0][bound == 0] == 0)
+
+
 @pytest.mark.parametrize("prec", [lsw.LSW_FP64, lsw.LSW_FP32])
 @pytest.mark.parametrize("tile", [0, 2, 5])
 def test_matrices_and_combination_many_functions_per_tile(prec, tile):
