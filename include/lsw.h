@@ -260,8 +260,13 @@ lsw_status lsw_lowdin_taylor(lsw_system sys, const double* S_dev, const void* ph
  *   smearing width in the units of H.
  * - Kp_dev, K_dev: FP64 outputs on the pattern (nnz each).  *mu_out, *ebs_out, *trace_out
  *   (host, may be NULL) receive mu, E_BS and the final Tr K'.
- * Synchronous (the search of mu runs on the host from the device traces).  Work buffers
- * are allocated at the first call (lsw_workspace_bytes).
+ * Synchronous (the search of mu runs on the host from the device traces).  Work buffers (seven
+ * matrices of nnz FP64 values) are allocated at the first call (lsw_workspace_bytes).  During a
+ * call the n_pl matrices T_j are kept as well, where they take no more than the option
+ * "foe_keep_mb" and, beyond 256 MiB, a quarter of the free device memory; else the recursion
+ * runs twice.  They come from a memory pool of the context, which holds at most 256 MiB between
+ * calls (not counted by lsw_workspace_bytes) and nothing once another allocation of the library
+ * has failed for lack of memory.
  * Errors: LSW_ERR_ARG (NULL, e_max <= e_min, de <= 0, n_pl < 1), LSW_ERR_STATE (host-only),
  * LSW_ERR_UNSUPPORTED (pattern not symmetric or without the diagonal; more functions than
  * the shared-memory column map holds), LSW_ERR_CUDA. */
@@ -439,6 +444,8 @@ lsw_status lsw_load_phi(lsw_system sys, const char* path, void* phi_dev);
  * measured fastest; the results are the same bits), "fwd_list" (1, the default: the forward plane kernel's x
  * pass computes only the blocks whose input window meets the row's members of L and
  * zeroes the rest; 0: every block; the same bits),
+ * "foe_keep_mb" (lsw_foe: device memory the kept matrices of one call may take, MiB; 0: none
+ * are kept; default 4096),
  * "zsplit" (LSW_FP32_BF16X systems only: 2 or 3 bfloat16 parts per FP32 operand of the
  * tensor-core z stage), "xy_tc" (LSW_FP32_BF16X systems only: 1 runs the x and y passes
  * of the plane kernels as split-bfloat16 tensor-core products as well; 0, the default,

@@ -149,7 +149,15 @@ struct lsw_ctx_s {
     size_t max_smem = 0;
     int n_sm = 0;
     std::atomic<int> live_systems{0};
+    // Fermi operator expansion: the kept T_j of a call come from here and go back at its end; the pool
+    // holds FOE_HELD bytes at most between calls (any thread, any stream of the device)
+    cudaMemPool_t foe_pool = nullptr;
+    ~lsw_ctx_s() {
+        if (foe_pool) cudaMemPoolDestroy(foe_pool);
+    }
 };
+constexpr size_t FOE_HELD = static_cast<size_t>(256) << 20;
+constexpr int64_t FOE_KEEP_MB = 4096;     // default limit of the kept T_j of one call (option "foe_keep_mb")
 
 struct GraphKey {
     const void* a;
@@ -203,6 +211,7 @@ struct lsw_system_s {
     // Fermi operator expansion: transposed positions, diagonal positions, the identity on
     // the pattern, work matrices, the dense row scratch of the triple products, row groups
     DeviceBuf d_tpos, d_diag, d_ident, d_foe, d_foe_scratch, d_foe_grp;
+    int64_t foe_keep_mb = FOE_KEEP_MB;
     int foe_ng = 0;                     // groups of rows (atoms with functions), their neighbour entries
     int64_t foe_nn = 0;
     // confinement and preconditioning: per-atom tables of the 1D operators X_d^2, X_d^4,
@@ -447,6 +456,13 @@ lsw_status build_pattern(lsw_system_s* s) {
     return LSW_OK;
 }
 
+// Allocate; where the memory is short, once more without what the expansion's pool holds.
+cudaError_t alloc_or_trim(lsw_system_s* s, DeviceBuf& b, size_t bytes) {
+    cudaError_t e = b.alloc(bytes);
+    if (e == cudaErrorMemoryAllocation && s->ctx->foe_pool && cudaMemPoolTrimTo(s->ctx->foe_pool, 0) == cudaSuccess) e = b.alloc(bytes);
+    return e;
+}
+
 int64_t align64(int64_t x) { return (x + ALIGN_ELEMS - 1) / ALIGN_ELEMS * ALIGN_ELEMS; }
 
 // Dynamic shared memory of the pass kernels for a function record.  z_lim: the size that decides
@@ -677,7 +693,7 @@ lsw_status build_plans(lsw_system_s* s) {
         p.items_bwd = p.n_items_bwd ? it + p.n_items_fwd : nullptr;
         p.queue = static_cast<int*>(s->d_queue.p);
     }
-    CUDA_TRY(s->d_ws.alloc(static_cast<size_t>(ws_max) * s->esize));
+    CUDA_TRY(alloc_or_trim(s, s->d_ws, static_cast<size_t>(ws_max) * s->esize));
     return LSW_OK;
 }
 
@@ -945,8 +961,8 @@ lsw_status build_hs_plan(lsw_system_s* s) {
 }
 
 lsw_status ensure_panels(lsw_system_s* s) {
-    if (!s->d_PA.p) CUDA_TRY(s->d_PA.alloc(s->panel_bytes_A));
-    if (!s->d_PQ.p) CUDA_TRY(s->d_PQ.alloc(s->panel_bytes_Q));
+    if (!s->d_PA.p) CUDA_TRY(alloc_or_trim(s, s->d_PA, s->panel_bytes_A));
+    if (!s->d_PQ.p) CUDA_TRY(alloc_or_trim(s, s->d_PQ, s->panel_bytes_Q));
     return LSW_OK;
 }
 
@@ -1250,7 +1266,7 @@ lsw_status build_density_plan(lsw_system_s* s, const int64_t* lo, const int64_t*
     CUDA_TRY(s->d_dfn.upload(dfn, st));
     CUDA_TRY(s->d_tptr.upload(tptr, st));
     CUDA_TRY(s->d_tfn.upload(tfn, st));
-    CUDA_TRY(s->d_U.alloc(static_cast<size_t>(off) * s->esize));
+    CUDA_TRY(alloc_or_trim(s, s->d_U, static_cast<size_t>(off) * s->esize));
     s->U_elems = off;
     for (int d = 0; d < 3; ++d) {
         s->dens_lo[d] = lo[d];
@@ -1462,6 +1478,14 @@ lsw_status lsw_ctx_create(int device, void* stream, lsw_ctx* out) {
     CUDA_TRY(configure_panel_kernels(c->max_smem));
     CUDA_TRY(configure_foe_kernels(c->max_smem));
     CUDA_TRY(configure_confine_kernels(c->max_smem));
+    cudaMemPoolProps props;
+    std::memset(&props, 0, sizeof(props));
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    CUDA_TRY(cudaMemPoolCreate(&c->foe_pool, &props));
+    uint64_t held = FOE_HELD;
+    CUDA_TRY(cudaMemPoolSetAttribute(c->foe_pool, cudaMemPoolAttrReleaseThreshold, &held));
     *out = c.release();
     return LSW_OK;
 }
@@ -1736,7 +1760,7 @@ lsw_status lsw_lowdin_taylor(lsw_system sys, const double* S, const void* phi_in
     const int64_t nnz = static_cast<int64_t>(sys->col.size());
     if (sys->d_mcoef.bytes < static_cast<size_t>(std::max<int64_t>(nnz, 1)) * sizeof(double)) {
         CUDA_TRY(cudaStreamSynchronize(sys->stream));
-        CUDA_TRY(sys->d_mcoef.alloc(static_cast<size_t>(std::max<int64_t>(nnz, 1)) * sizeof(double)));
+        CUDA_TRY(alloc_or_trim(sys, sys->d_mcoef, static_cast<size_t>(std::max<int64_t>(nnz, 1)) * sizeof(double)));
     }
     double* T = static_cast<double*>(sys->d_mcoef.p);
     CUDA_TRY(enqueue_lowdin_coeffs(static_cast<const int64_t*>(sys->d_rowp.p), static_cast<const int32_t*>(sys->d_col.p),
@@ -1764,22 +1788,6 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
     for (int a = 0; a < sys->n_atoms; ++a) max_nsf = std::max(max_nsf, sys->nsf[a]);
     size_t triple_smem = static_cast<size_t>(max_nsf) * n * sizeof(double);
     if (triple_smem > sys->ctx->max_smem - 1024) triple_smem = 0;
-    // The T_j of the recursion are kept for the sum of K' where they take at most 4 GiB and a quarter
-    // of the free device memory (the buffer stays with the system); else the recursion runs a
-    // second time over three slots.
-    auto buffer = [&](int64_t slots) {
-        return static_cast<size_t>(std::max<int64_t>(nnz, 1)) * static_cast<size_t>(slots + 4) * sizeof(double) +
-               static_cast<size_t>(2 * (n_pl + 1) + 1 + FOE_PARTS) * sizeof(double);
-    };
-    const int64_t all = std::max(n_pl, 3);
-    bool keep = static_cast<double>(n_pl) * nnz * sizeof(double) <= 4.0 * (1ull << 30);
-    if (keep && sys->d_foe.bytes < buffer(all)) {
-        size_t free_b = 0, total_b = 0;
-        CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-        keep = buffer(all) <= free_b / 4;
-    }
-    const int64_t slots = keep ? all : 3;
-    const size_t need = buffer(slots);
     if (sys->d_tpos.bytes == 0) {
         // transposed and diagonal positions of the pattern, the identity on it; the groups of
         // rows (the functions of an atom) and their neighbours
@@ -1829,9 +1837,34 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
         }
         CUDA_TRY(sys->d_tpos.upload(tpos, st));        // last: marks the plan as built
     }
+    const size_t need = (static_cast<size_t>(nnz) * 7 + static_cast<size_t>(n_pl + 1) * 2 + 1 + FOE_PARTS) * sizeof(double);
     if (sys->d_foe.bytes < need) {
         CUDA_TRY(cudaStreamSynchronize(st));
-        CUDA_TRY(sys->d_foe.alloc(need));
+        CUDA_TRY(alloc_or_trim(sys, sys->d_foe, need));
+    }
+    // The T_j of the recursion are kept for the sum of K' where they fit the option's limit and (beyond
+    // what the pool holds anyway) a quarter of the free device memory; else, or where the memory
+    // cannot be had after all, the recursion runs a second time over three slots.
+    struct KeptT {
+        cudaStream_t st;
+        double* p = nullptr;
+        ~KeptT() { give_back(); }
+        void give_back() {
+            if (p) cudaFreeAsync(p, st);
+            p = nullptr;
+        }
+    } kept{st};
+    const size_t t_bytes = static_cast<size_t>(n_pl) * static_cast<size_t>(nnz) * sizeof(double);
+    bool keep = t_bytes <= static_cast<size_t>(sys->foe_keep_mb) << 20;
+    if (keep && t_bytes > FOE_HELD) {
+        size_t free_b = 0, total_b = 0;
+        CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+        keep = t_bytes <= free_b / 4;
+    }
+    if (keep && cudaMallocFromPoolAsync(reinterpret_cast<void**>(&kept.p), t_bytes, sys->ctx->foe_pool, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        kept.p = nullptr;
+        keep = false;
     }
     FoeLaunch f;
     f.n = n;
@@ -1861,8 +1894,8 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
     double* X = w + nnz;
     double* Htp = w + 2 * nnz;
     double* Kc = w + 3 * nnz;
-    double* T = w + 4 * nnz;             // T_1, T_2, ... (or three slots in turn)
-    double* tr_d = w + (4 + slots) * nnz;   // n_pl + 1 traces, n_pl + 1 coefficients, E_BS, its partial sums
+    double* T = keep ? kept.p : w + 4 * nnz;   // T_1, T_2, ... (or three slots in turn)
+    double* tr_d = w + 7 * nnz;          // n_pl + 1 traces, n_pl + 1 coefficients, E_BS, its partial sums
     double* c_d = tr_d + n_pl + 1;
     double* ebs_d = c_d + n_pl + 1;
     const double* I = static_cast<const double*>(sys->d_ident.p);
@@ -1919,6 +1952,7 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
     if (keep) {
         CUDA_TRY(cudaMemcpyAsync(c_d, c.data(), Nn * sizeof(double), cudaMemcpyHostToDevice, st));
         CUDA_TRY(foe_kernel_sum(f, I, T, c_d, n_pl, Kc, st));
+        kept.give_back();
     } else {
         CUDA_TRY(cudaMemsetAsync(Kc, 0, nnz * sizeof(double), st));
         CUDA_TRY(foe_axpy_t(f, Kc, I, 0.5 * c[0], st));
@@ -2082,7 +2116,7 @@ lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double*
     const size_t need = std::max(per * b, per_other * conf_batch(s, per_other));
     if (s->d_cbox.bytes < need) {
         CUDA_TRY(cudaStreamSynchronize(s->stream));
-        CUDA_TRY(s->d_cbox.alloc(need));
+        CUDA_TRY(alloc_or_trim(s, s->d_cbox, need));
     }
     c.prec = s->prec;
     c.precond = precond ? 1 : 0;
@@ -2175,7 +2209,7 @@ lsw_status lsw_precondition(lsw_system sys, const double* a_dev, const double* e
     const size_t vb = static_cast<size_t>(std::max<int64_t>(nv, 1)) * sys->esize;
     if (sys->d_cg.bytes < 3 * vb || sys->d_cgs.bytes < nf * sizeof(double)) {
         CUDA_TRY(cudaStreamSynchronize(sys->stream));
-        CUDA_TRY(sys->d_cg.alloc(3 * vb));
+        CUDA_TRY(alloc_or_trim(sys, sys->d_cg, 3 * vb));
         CUDA_TRY(sys->d_cgs.alloc(static_cast<size_t>(std::max<int64_t>(nf, 1)) * sizeof(double)));
     }
     unsigned char* V = static_cast<unsigned char*>(sys->d_cg.p);
@@ -2458,8 +2492,8 @@ lsw_status lsw_step_host(lsw_system sys, const void* phi_host, void* hphi_host, 
     const size_t bhphi = static_cast<size_t>(sys->off_Lp.back()) * sys->esize;
     const size_t bnnz = sys->col.size() * sizeof(double);
     if (!sys->d_phi.p) {
-        CUDA_TRY(sys->d_phi.alloc(bphi));
-        CUDA_TRY(sys->d_hphi.alloc(bhphi));
+        CUDA_TRY(alloc_or_trim(sys, sys->d_phi, bphi));
+        CUDA_TRY(alloc_or_trim(sys, sys->d_hphi, bhphi));
         CUDA_TRY(sys->d_H.alloc(std::max<size_t>(bnnz, 8)));
         CUDA_TRY(sys->d_S.alloc(std::max<size_t>(bnnz, 8)));
         CUDA_TRY(sys->d_ek.alloc(nf * sizeof(double)));
@@ -2641,6 +2675,11 @@ lsw_status lsw_set_option(lsw_system sys, const char* name, int64_t value) {
         drop_graphs(sys);
         sys->persistent = static_cast<int>(value);
         return build_plans(sys);
+    }
+    if (std::strcmp(name, "foe_keep_mb") == 0) {
+        if (value < 0 || value > (int64_t(1) << 22)) return fail(LSW_ERR_ARG, "lsw_set_option: foe_keep_mb %lld", static_cast<long long>(value));
+        sys->foe_keep_mb = value;
+        return LSW_OK;
     }
     if (std::strcmp(name, "graph") == 0) {
         if (value != 0 && value != 1) return fail(LSW_ERR_ARG, "lsw_set_option: graph %lld", static_cast<long long>(value));
