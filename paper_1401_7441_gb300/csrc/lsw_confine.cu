@@ -447,9 +447,11 @@ __global__ void __launch_bounds__(256) k_conf_pass(ConfLaunch a) {
 
 // F on the members of the region (0: L, 1: L') -> compressed vector; dst (+)= F (- eps_f P for
 // the preconditioning operator).  With `energy`, the row's sum of P F over the members of L is left
-// in B (read for the last time by the x pass) for k_conf_energy.  A warp per row.
+// in B (read for the last time by the x pass) for k_conf_energy.  A warp per row, a chain of loads each:
+// bound by the warps in flight (20 atoms in FP32, four calls: 176 us with four CTAs an SM, 211 with
+// three, 297 with two).
 template <class T>
-__global__ void __launch_bounds__(256) k_conf_store(ConfLaunch a, T* __restrict__ dst, int accumulate, int energy) {
+__global__ void __launch_bounds__(256, 4) k_conf_store(ConfLaunch a, T* __restrict__ dst, int accumulate, int energy) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 23;
     const int k = blockIdx.y;
