@@ -286,8 +286,10 @@ lsw_status lsw_foe(lsw_system sys, const double* H_dev, const double* S_dev, dou
  * the same manner as the kinetic energy").  Call after lsw_apply_hamiltonian on the same
  * buffers to get H_alpha phi_alpha.  a_dev: n_sf FP64 prefactors (device); phi_dev on L,
  * hphi_dev on L' (layouts of lsw_system_layout, system precision); e_conf_dev: n_sf FP64
- * or NULL.  The first call builds the operator tables of every atom (host, then
- * uploaded; lsw_workspace_bytes) and the batch boxes.  Asynchronous.
+ * or NULL.  The first call (of this or of lsw_precondition) builds the operator tables of every
+ * atom on the device and allocates the boxes of a batch of functions, for both calls: up to 256
+ * functions within 2 GiB, fewer where the memory is short (counted by lsw_workspace_bytes).
+ * e_conf is the same bits on every call.  Asynchronous.
  * Errors: LSW_ERR_ARG (NULL), LSW_ERR_STATE (host-only), LSW_ERR_CUDA. */
 lsw_status lsw_add_confinement(lsw_system sys, const double* a_dev, const void* phi_dev, void* hphi_dev,
                                double* e_conf_dev);

@@ -2094,7 +2094,8 @@ size_t conf_strides(const lsw_system_s* s, int region, ConfLaunch* out) {
     return static_cast<size_t>(doubles) * sizeof(double) + static_cast<size_t>(c.s_maps);
 }
 
-// Functions of a batch: a budget of 2 GiB.
+// Functions of a batch: a budget of 2 GiB.  (64 functions would take half of it in FP32, but their
+// passes end in uneven waves: 150 atoms in FP32, six iterations 195 ms; 128: 168; 256: 158.)
 int conf_batch(const lsw_system_s* s, size_t per) {
     const int64_t nf = static_cast<int64_t>(s->sf_atom.size());
     return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>({256, nf, static_cast<int64_t>((size_t(2) << 30) / per)})));
@@ -2112,12 +2113,18 @@ lsw_status conf_prepare(lsw_system_s* s, int region, bool precond, const double*
     ConfLaunch& c = *out;
     ConfLaunch other;
     const size_t per = conf_strides(s, region, &c), per_other = conf_strides(s, 1 - region, &other);
-    const int b = conf_batch(s, per);
-    const size_t need = std::max(per * b, per_other * conf_batch(s, per_other));
-    if (s->d_cbox.bytes < need) {
+    if (s->d_cbox.bytes == 0) {
+        // smaller batches where the memory is short
+        size_t need = std::max(per * conf_batch(s, per), per_other * conf_batch(s, per_other));
         CUDA_TRY(cudaStreamSynchronize(s->stream));
-        CUDA_TRY(alloc_or_trim(s, s->d_cbox, need));
+        cudaError_t e = alloc_or_trim(s, s->d_cbox, need);
+        while (e == cudaErrorMemoryAllocation && need > std::max(per, per_other)) {
+            need = std::max(need / 2, std::max(per, per_other));
+            e = s->d_cbox.alloc(need);
+        }
+        CUDA_TRY(e);
     }
+    const int b = std::min(conf_batch(s, per), static_cast<int>(s->d_cbox.bytes / per));
     c.prec = s->prec;
     c.precond = precond ? 1 : 0;
     c.sf_atom = static_cast<const int32_t*>(s->d_sfatom.p);
