@@ -448,6 +448,9 @@ lsw_status lsw_load_phi(lsw_system sys, const char* path, void* phi_dev);
  * zeroes the rest; 0: every block; the same bits),
  * "foe_keep_mb" (lsw_foe: device memory the kept matrices of one call may take, MiB; 0: none
  * are kept; default 4096),
+ * "wait_out" (0, the default; 1, for tests of the failure path: the backward FMA plane kernel
+ * takes its waits for its own copies as run out, sets the status bit and ends; lsw_sync then
+ * returns LSW_ERR_STATE and the outputs of H phi are not valid),
  * "zsplit" (LSW_FP32_BF16X systems only: 2 or 3 bfloat16 parts per FP32 operand of the
  * tensor-core z stage), "xy_tc" (LSW_FP32_BF16X systems only: 1 runs the x and y passes
  * of the plane kernels as split-bfloat16 tensor-core products as well; 0, the default,

@@ -238,6 +238,7 @@ struct lsw_system_s {
     int persistent = 1;              // option "persistent": bit 0 the backward, bit 1 the forward
                                      // FMA plane kernel over item queues
     int fwd_list = 1;                // option "fwd_list": forward x pass over member blocks only
+    int wait_out = 0;                // option "wait_out" (tests)
     int use_graph = 1;
     // potential
     const void* V = nullptr;
@@ -577,6 +578,7 @@ lsw_status build_plans(lsw_system_s* s) {
         p.nfn = static_cast<int>(b.nfn);
         p.zcols = zcols;
         p.fwd_list = s->fwd_list;
+        p.wait_out = s->wait_out;
         BwdSizes bwd;
         size_t smem_z_lim = 0;
         int64_t o = 0;
@@ -2681,6 +2683,13 @@ lsw_status lsw_set_option(lsw_system sys, const char* name, int64_t value) {
         CUDA_TRY(cudaStreamSynchronize(sys->stream));
         drop_graphs(sys);
         sys->persistent = static_cast<int>(value);
+        return build_plans(sys);
+    }
+    if (std::strcmp(name, "wait_out") == 0) {
+        if (value != 0 && value != 1) return fail(LSW_ERR_ARG, "lsw_set_option: wait_out %lld", static_cast<long long>(value));
+        CUDA_TRY(cudaStreamSynchronize(sys->stream));
+        drop_graphs(sys);
+        sys->wait_out = static_cast<int>(value);
         return build_plans(sys);
     }
     if (std::strcmp(name, "foe_keep_mb") == 0) {

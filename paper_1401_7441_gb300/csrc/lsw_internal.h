@@ -215,6 +215,7 @@ struct HphiLaunch {
     int* queue;
     int fwd_list;                // 1: the forward x pass computes only the blocks whose input
                                  // window meets the row's members (the rest of its plane is 0)
+    int wait_out;                // 1: the backward kernel's waits count as run out (tests of the failure path)
     const AtomRec* atoms;
     const Seg* seg;
     const int32_t* rowptr;

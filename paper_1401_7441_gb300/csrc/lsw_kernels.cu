@@ -1861,14 +1861,15 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 constexpr int BWD_THREADS = LSW_BWD_THREADS;
 
 template <class T>
-__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase, int2* s_next) {
+__device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase, int& dead,
+                                          int2* s_next) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     int* st = a.status;
     constexpr int NB = Blk<T, 1>::NB;
     using Arm = KinArm<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int ylo, yhi, dead;
+    __shared__ int ylo, yhi;
     const FnRec r0 = a.fn[fl];
     if (zb >= r0.np[2]) return;
     const AtomRec& at = a.atoms[r0.atom];
@@ -1926,15 +1927,19 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         const T* Bb = static_cast<const T*>(a.ws) + r.ws_Bb + (static_cast<int64_t>(bz) * nzp + zb) * Y * X;
         const int rem = static_cast<int>((reinterpret_cast<uintptr_t>(Bb) & 15) / sizeof(T));
         const uint32_t bytes = static_cast<uint32_t>((static_cast<size_t>(rem + Y * X) * sizeof(T) + 15) & ~size_t(15));
+        if (dead) return;
         bulk_fence();                                          // Gs was read and written there
         bulk_expect(mbar, bytes);
         bulk_load(tc::saddr(plb), Bb - rem, bytes, mbar);
     };
-    auto wait = [&]() {                                        // for the bulk copies in flight
+    // For the bulk copies in flight.  Once a wait has run out no more copies are announced or waited
+    // for (the barrier's phase is still open: `dead` keeps it, behind the next barrier of the CTA
+    // every thread sees it), and the CTA ends with this item.
+    auto wait = [&]() {
 #ifndef LSW_CHECKED
-        if (!dead && !tc::mbar_wait(mbar, phase)) {
+        if (!dead && (a.wait_out || !tc::mbar_wait(mbar, phase))) {
             atomicOr(st, ST_WAIT_TIMEOUT);
-            dead = 1;
+            dead = 1 + static_cast<int>(phase);
         }
         phase ^= 1;
 #endif
@@ -1949,7 +1954,6 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
     if (tid == 0) {
         ylo = nyp;
         yhi = -1;
-        dead = 0;
     }
     for (int i = tid; i < 2 * L.nb_x; i += blockDim.x) {
         hlo[i] = nyp;
@@ -2263,7 +2267,7 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
                         CPA(mid, tb * slot + i, mid_n, G, (tb + 4 * bz) * gplane + static_cast<int64_t>(zb) * pnp + g_r0 + i,
                             8 * gplane);
 #else
-                if (tid == 0) {
+                if (tid == 0 && !dead) {
                     bulk_fence();
                     uint32_t total = 0;
 #pragma unroll
@@ -2357,7 +2361,11 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (threadIdx.x == 0) tc::mbar_init(tc::saddr(smem_raw));
+    __shared__ int dead;                       // 1 + the phase of the copies that a wait ran out on, 0: none did
+    if (threadIdx.x == 0) {
+        tc::mbar_init(tc::saddr(smem_raw));
+        dead = 0;
+    }
     __syncthreads();
     uint32_t phase = 0;
     if (a.items_bwd) {
@@ -2369,12 +2377,14 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
         __syncthreads();
         for (;;) {
             const int2 it = s_item;   // (the next one is written behind the plane's barriers)
-            if (it.y < 0) break;
-            bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase, &s_item);
+            if (it.y < 0 || dead) break;
+            bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase, dead, &s_item);
         }
     } else {
-        bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase, nullptr);
+        bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase, dead, nullptr);
     }
+    // the copies still in flight write to this CTA's shared memory: end behind them (or the limit)
+    if (threadIdx.x == 0 && dead) (void)tc::mbar_wait(tc::saddr(smem_raw), dead - 1);
 }
 
 // ---------------------------------------------------------------- density: pair products

@@ -51,3 +51,38 @@ def test_sync_timeout_then_normal_sync():
         assert np.abs(out[0][2]).max() > 0
     finally:
         S.close()
+
+
+@pytest.mark.parametrize("prec,persistent", [(lsw.LSW_FP64, 1), (lsw.LSW_FP32, 1), (lsw.LSW_FP32, 0)])
+def test_waits_that_run_out_end_the_kernel_and_leave_the_system_usable(prec, persistent):
+    # the copies do arrive (the kernel ends behind them): only the waits are taken as run out
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ensure_built()
+    wl = I.scaled("atoms64", 12, seed=3)
+    st = torch.cuda.Stream()
+    S = lsw.System(wl.N, wl.h, wl.pos, wl.r_loc, wl.r_fine, wl.nsf, wl.pair_cutoff, wl.pair_mode, precision=prec,
+                   device=0, stream=st.cuda_stream)
+    try:
+        dt = torch.float64 if prec == lsw.LSW_FP64 else torch.float32
+        phi = torch.randn(S.total_L, generator=torch.Generator(device="cuda").manual_seed(1), dtype=dt, device="cuda")
+        V = torch.tensor(I.potential(wl), dtype=dt, device="cuda")
+        lsw.lsw_set_option(S.sys, "persistent", persistent)
+        lsw.lsw_set_potential(S.sys, V, wl.V_lo, wl.V_shape)
+        out = []
+        for wait_out in (0, 1, 0):
+            lsw.lsw_set_option(S.sys, "wait_out", wait_out)
+            hphi = torch.zeros(S.total_Lp, dtype=dt, device="cuda")
+            torch.cuda.synchronize()
+            lsw.lsw_apply_hamiltonian(S.sys, phi, hphi)
+            if wait_out:
+                with pytest.raises(lsw.LswError) as e:
+                    lsw.lsw_sync(S.sys, 60.0)
+                assert e.value.status == lsw.LSW_ERR_STATE and "status bits 0x10" in str(e.value)
+            else:
+                lsw.lsw_sync(S.sys, 60.0)
+                out.append(hphi.cpu())
+        assert torch.equal(out[0], out[1]) and float(out[0].abs().max()) > 0.0
+    finally:
+        S.close()
