@@ -448,6 +448,12 @@ lsw_status lsw_load_phi(lsw_system sys, const char* path, void* phi_dev);
  * zeroes the rest; 0: every block; the same bits),
  * "foe_keep_mb" (lsw_foe: device memory the kept matrices of one call may take, MiB; 0: none
  * are kept; default 4096),
+ * "bwd_group" (functions of an atom that an item of the persistent backward plane kernel
+ * takes together, 1..64; 0, the default: as many as leave eight items for every CTA) and
+ * "bwd_layout" (its shared memory: 3 room for the kinetic z arm's plane and the list of
+ * fine members, 2 for the list, 0 for neither; -1, the default: the first of them that leaves
+ * room for two CTAs on an SM, else the first that fits; LSW_ERR_UNSUPPORTED if the layout does
+ * not fit) -- the same bits in all of them,
  * "wait_out" (0, the default; 1, for tests of the failure path: the backward FMA plane kernel
  * takes its waits for its own copies as run out, sets the status bit and ends; lsw_sync then
  * returns LSW_ERR_STATE and the outputs of H phi are not valid),

@@ -239,6 +239,8 @@ struct lsw_system_s {
                                      // FMA plane kernel over item queues
     int fwd_list = 1;                // option "fwd_list": forward x pass over member blocks only
     int wait_out = 0;                // option "wait_out" (tests)
+    int bwd_layout = -1;             // options "bwd_layout", "bwd_group": the backward kernel's shared-memory
+    int bwd_group = 0;               // layout and functions per item (-1, 0: by the rules)
     int use_graph = 1;
     // potential
     const void* V = nullptr;
@@ -489,12 +491,13 @@ struct BwdSizes {
                                                                es == 4 ? BWD_NB_F32 : BWD_NB_F64, g != 0, p != 0)
                                                         .bytes);
     }
-    bool choose(size_t max_smem, HphiLaunch* p) const {
+    // forced: option "bwd_layout" (-1: the first that fits)
+    bool choose(size_t max_smem, int forced, HphiLaunch* p) const {
         // an SM holds the largest CTA's shared memory and 1 KiB reserved per CTA
         const size_t half = (max_smem + 1024) / 2 - 1024 - BWD_STATIC_SMEM, all = max_smem - BWD_STATIC_SMEM;
         const struct { int g, p; size_t lim; } order[] = {{1, 1, half}, {0, 1, half}, {1, 1, all}, {0, 1, all}, {0, 0, all}};
         for (const auto& o : order)
-            if (b[o.g][o.p] <= o.lim) {
+            if (b[o.g][o.p] <= o.lim && (forced < 0 || forced == (o.g | o.p << 1))) {
                 p->gstage = o.g;
                 p->lists = o.p;
                 p->smem_bwd = b[o.g][o.p];
@@ -635,7 +638,7 @@ lsw_status build_plans(lsw_system_s* s) {
         }
         p.zsplit = s->zsplit;
         p.xy_tc = s->zsplit ? s->xy_tc : 0;
-        if (!bwd.choose(s->ctx->max_smem, &p) || p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || smem_z_lim > s->ctx->max_smem ||
+        if (!bwd.choose(s->ctx->max_smem, s->bwd_layout, &p) || p.smem_fwd + FWD_STATIC_SMEM > s->ctx->max_smem || smem_z_lim > s->ctx->max_smem ||
             p.smem_ztc > s->ctx->max_smem || p.smem_kin > s->ctx->max_smem || p.smem_bwd_tc + BWD_TC_STATIC_SMEM > s->ctx->max_smem ||
             p.smem_fwd_tc > s->ctx->max_smem)
             return fail(LSW_ERR_UNSUPPORTED, "locreg box too large for the on-chip pass tiles (%zu/%zu/%zu/%zu > %zu bytes)",
@@ -671,7 +674,8 @@ lsw_status build_plans(lsw_system_s* s) {
             int64_t planes = 0;
             for (int64_t f = f0; f < f0 + b.nfn; ++f) planes += 2LL * recs[f].np[2];
             const int64_t fill = 8LL * std::max(1, bb) * s->ctx->n_sm;
-            p.n_items_bwd = (s->persistent & 1) ? add(1, static_cast<int>(std::min<int64_t>(64, std::max<int64_t>(1, planes / fill)))) : 0;
+            const int group = s->bwd_group ? s->bwd_group : static_cast<int>(std::min<int64_t>(64, std::max<int64_t>(1, planes / fill)));
+            p.n_items_bwd = (s->persistent & 1) ? add(1, group) : 0;
             p.grid_fwd = std::max(1, std::min(p.n_items_fwd, std::max(1, bf) * s->ctx->n_sm));
             p.grid_bwd = std::max(1, std::min(p.n_items_bwd, std::max(1, bb) * s->ctx->n_sm));
         } else {
@@ -1435,7 +1439,7 @@ void noalloc_fold(const lsw_system_s* s, const FnRec& r, int zcols, HphiLaunch* 
 // Choose the backward plane kernel's layout and check the tiles against the shared memory.
 bool noalloc_finish(const lsw_system_s* s, HphiLaunch* p, const BwdSizes& bwd) {
     const size_t mx = s->ctx->max_smem;
-    return bwd.choose(mx, p) &&
+    return bwd.choose(mx, s->bwd_layout, p) &&
            !(p->smem_fwd + FWD_STATIC_SMEM > mx || bwd.z_lim > mx || p->smem_ztc > mx ||
              p->smem_kin > mx || p->smem_bwd_tc + BWD_TC_STATIC_SMEM > mx || p->smem_fwd_tc > mx);
 }
@@ -2684,6 +2688,29 @@ lsw_status lsw_set_option(lsw_system sys, const char* name, int64_t value) {
         drop_graphs(sys);
         sys->persistent = static_cast<int>(value);
         return build_plans(sys);
+    }
+    if (std::strcmp(name, "bwd_group") == 0) {
+        if (value < 0 || value > 64) return fail(LSW_ERR_ARG, "lsw_set_option: bwd_group %lld", static_cast<long long>(value));
+        CUDA_TRY(cudaStreamSynchronize(sys->stream));
+        drop_graphs(sys);
+        sys->bwd_group = static_cast<int>(value);
+        return build_plans(sys);
+    }
+    if (std::strcmp(name, "bwd_layout") == 0) {
+        if (value != -1 && value != 0 && value != 2 && value != 3)
+            return fail(LSW_ERR_ARG, "lsw_set_option: bwd_layout %lld", static_cast<long long>(value));
+        CUDA_TRY(cudaStreamSynchronize(sys->stream));
+        drop_graphs(sys);
+        const int old = sys->bwd_layout;
+        sys->bwd_layout = static_cast<int>(value);
+        lsw_status e = build_plans(sys);
+        if (e != LSW_OK) {
+            const std::string msg = g_err;
+            sys->bwd_layout = old;
+            if (build_plans(sys) != LSW_OK) return fail(LSW_ERR_STATE, "lsw_set_option: bwd_layout: cannot restore plans");
+            return fail(e, "%s", msg.c_str());
+        }
+        return LSW_OK;
     }
     if (std::strcmp(name, "wait_out") == 0) {
         if (value != 0 && value != 1) return fail(LSW_ERR_ARG, "lsw_set_option: wait_out %lld", static_cast<long long>(value));
