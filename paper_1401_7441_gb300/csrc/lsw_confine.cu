@@ -82,10 +82,9 @@ __device__ __forceinline__ ConfGeo conf_geo(const AtomRec& at, int region) {
 
 // ---------------------------------------------------------------- tables
 
-// Tables [dim][m = 2, 4][b b'][i over the L box widened by 14][l + 14] of one atom (blockIdx.x):
-//   <chi^b_i|(x - R)^m|chi^b'_{i+l}> = (h/2)^m sum_p C(m,p) sum_k X_k (2i + k - 2R/h)^(m-p) G^p_Y(l, k),
-// G[y][p][l + 14][k] = sum_k' Y_k' F^p(2l + k' - k) from the host.  A thread per entry: on the
-// device because the host loop took about 25 ms per atom, this about 25 us.
+// Tables [dim][m = 2, 4][b b'][i over the L box widened by 14][l + 14] of one atom (blockIdx.x), the
+// entries by conf_entry.  A thread per entry: on the device because the host loop took about 25 ms per
+// atom, this about 25 us.
 __global__ void __launch_bounds__(256) k_conf_table(const AtomRec* __restrict__ atoms, const double* __restrict__ pos,
                                                     const double* __restrict__ G, const double* __restrict__ XY, double h,
                                                     const int64_t* __restrict__ off, double* __restrict__ tab) {
@@ -97,22 +96,7 @@ __global__ void __launch_bounds__(256) k_conf_table(const AtomRec* __restrict__ 
         for (int e = threadIdx.x; e < 8 * E * KIN_TAPS; e += blockDim.x) {
             const int l = e % KIN_TAPS, i = (e / KIN_TAPS) % E, blk = e / (KIN_TAPS * E);
             const int m = blk < 4 ? 2 : 4, b = (blk >> 1) & 1, bp = blk & 1;
-            const double z0 = 2.0 * static_cast<double>(at.lo[d] - KIN_HALF + i) - 2.0 * c;
-            double acc = 0.0, cp = 1.0;
-            for (int p = 0; p <= m; ++p) {
-                if (p > 0) cp = cp * (m - p + 1) / p;
-                const double* Gp = G + ((bp * MOVL_P + p) * KIN_TAPS + l) * D16;
-                double sk = 0.0;
-                for (int k = 0; k < D16; ++k) {
-                    const double z = z0 + (k + H_LO);
-                    double zp = 1.0;
-                    for (int r = 0; r < m - p; ++r) zp *= z;
-                    sk += XY[b * D16 + k] * zp * Gp[k];
-                }
-                acc += cp * sk;
-            }
-            const double h2 = 0.5 * h;
-            out[e] = (m == 2 ? h2 * h2 : h2 * h2 * h2 * h2) * acc;
+            out[e] = conf_entry(G, XY, m, b, bp, l, static_cast<double>(at.lo[d] - KIN_HALF + i), c, h);
         }
         out += 8 * E * KIN_TAPS;
     }

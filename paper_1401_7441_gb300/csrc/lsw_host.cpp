@@ -1982,11 +1982,9 @@ lsw_status lsw_foe(lsw_system sys, const double* H, const double* S, double e_mi
 namespace {
 // Tables of the 1D operators (x - R_d)^m, m = 2, 4, between the scaling (b = 0) and
 // wavelet (b = 1) functions of coarse points i, j = i + l (|l| <= 14) along each
-// dimension of every atom's widened box (i over [lo_d - 14, lo_d + n_d + 13]):
-//   <chi^b_i|(x - R)^m|chi^b'_j> = (h/2)^m sum_p C(m,p) sum_k X_k (2i + k - 2c)^(m-p) G^p_Y(l, k),
-//   G^p_Y(l, k) = sum_k' Y_k' F^p(2l + k' - k),   c = R_d / h,  X, Y = h or g by b, b',
-// F^p the moment overlaps of the filter set (the Galerkin matrix of the multiplication
-// operator x^m in the two-level basis, expanded by the refinement equation).
+// dimension of every atom's widened box (i over [lo_d - 14, lo_d + n_d + 13]): conf_entry, F^p the
+// moment overlaps of the filter set (the Galerkin matrix of the multiplication operator x^m in
+// the two-level basis, expanded by the refinement equation).
 // G[y][p][l + 14][k] = sum_k' Y_k' F^p(2l + k' - k)
 std::vector<double> conf_G(const FilterSet& F) {
     const double* XY[2] = {F.h, F.g};
@@ -2006,28 +2004,11 @@ std::vector<double> conf_G(const FilterSet& F) {
     return G;
 }
 
-// out[l + 14] = <chi^b_i|(x - R)^m|chi^b'_{i+l}>, l = -14..14, c = R / h
-void conf_row(const FilterSet& F, const std::vector<double>& G, int m, int b, int bp, double gi, double c, double h,
-              double* out) {
-    const double* XY[2] = {F.h, F.g};
-    const double hm = std::pow(h / 2.0, m);
-    for (int l = -KIN_HALF; l <= KIN_HALF; ++l) {
-        double acc = 0.0;
-        double cp = 1.0;   // C(m, p)
-        for (int p = 0; p <= m; ++p) {
-            if (p > 0) cp = cp * (m - p + 1) / p;
-            const double* Gp = &G[((bp * MOVL_P + p) * KIN_TAPS + (l + KIN_HALF)) * D16];
-            double sk = 0.0;
-            for (int k = 0; k < D16; ++k) {
-                const double z = 2.0 * gi + (k + H_LO) - 2.0 * c;
-                double zp = 1.0;
-                for (int r = 0; r < m - p; ++r) zp *= z;
-                sk += XY[b][k] * zp * Gp[k];
-            }
-            acc += cp * sk;
-        }
-        out[l + KIN_HALF] = hm * acc;
-    }
+// h, g: the X and Y of conf_entry.
+std::vector<double> conf_XY(const FilterSet& F) {
+    std::vector<double> XY(F.h, F.h + D16);
+    XY.insert(XY.end(), F.g, F.g + D16);
+    return XY;
 }
 
 // The tables of every atom, computed on the device from G and the filters.
@@ -2035,8 +2016,8 @@ lsw_status build_conf_tables(lsw_system_s* s) {
     const FilterSet& F = s->ctx->filters;
     std::vector<double> in = conf_G(F);                // then h, g, the positions
     const size_t nG = in.size();
-    in.insert(in.end(), F.h, F.h + D16);
-    in.insert(in.end(), F.g, F.g + D16);
+    const std::vector<double> XY = conf_XY(F);
+    in.insert(in.end(), XY.begin(), XY.end());
     in.insert(in.end(), s->pos.begin(), s->pos.end());
     const int na = s->n_atoms;
     std::vector<int64_t> off(na + 1, 0);
@@ -2181,7 +2162,9 @@ lsw_status lsw_confinement_row(lsw_system sys, int32_t atom, int32_t dim, int32_
     if (atom < 0 || atom >= sys->n_atoms || dim < 0 || dim > 2 || (m != 2 && m != 4) || b < 0 || b > 1 || bp < 0 || bp > 1)
         return fail(LSW_ERR_ARG, "lsw_confinement_row: argument out of range");
     const std::vector<double> G = conf_G(sys->ctx->filters);
-    conf_row(sys->ctx->filters, G, m, b, bp, static_cast<double>(i), sys->pos[3 * atom + dim] / sys->h, sys->h, out);
+    const std::vector<double> XY = conf_XY(sys->ctx->filters);
+    for (int l = 0; l < KIN_TAPS; ++l)
+        out[l] = conf_entry(G.data(), XY.data(), m, b, bp, l, static_cast<double>(i), sys->pos[3 * atom + dim] / sys->h, sys->h);
     return LSW_OK;
 }
 

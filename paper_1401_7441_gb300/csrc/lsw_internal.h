@@ -165,6 +165,28 @@ LSW_HD BwdLayout bwd_layout(int nx, int ny, int nxp, int nyp, int es, int nb, bo
     return L;
 }
 
+// <chi^b_i|(x - R)^m|chi^b'_{i+l}> = (h/2)^m sum_p C(m,p) sum_k X_k (2i + k - 2c)^(m-p) G^p_Y(l, k),
+// c = R / h, X, Y = XY[b], XY[b'] (h, g), G[y][p][l + 14][k] = sum_k' Y_k' F^p(2l + k' - k); lt = l + 14.
+LSW_HD double conf_entry(const double* G, const double* XY, int m, int b, int bp, int lt, double i, double c, double h) {
+    double acc = 0.0, cp = 1.0;                        // cp = C(m, p)
+    for (int p = 0; p <= m; ++p) {
+        if (p > 0) cp = cp * (m - p + 1) / p;
+        const double* Gp = G + ((bp * MOVL_P + p) * KIN_TAPS + lt) * D16;
+        double sk = 0.0;
+        for (int k = 0; k < D16; ++k) {
+            const double z = 2.0 * i + (k + H_LO) - 2.0 * c;
+            double zp = 1.0;
+            for (int r = 0; r < m - p; ++r) zp *= z;
+            sk += XY[b * D16 + k] * zp * Gp[k];
+        }
+        acc += cp * sk;
+    }
+    const double h2 = 0.5 * h;
+    double hm = 1.0;
+    for (int r = 0; r < m; ++r) hm *= h2;
+    return hm * acc;
+}
+
 // Kernel kinds of the per-launch device trace (lsw_profile / lsw_profile_read).
 enum TraceKind : int {
     TK_MEMSET = 0, TK_UNCOMPRESS, TK_FWD_XY, TK_Z, TK_BWD_XY, TK_KINETIC, TK_PACK, TK_HS,

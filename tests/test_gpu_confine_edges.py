@@ -95,3 +95,54 @@ def test_confinement_energy_same_bits_on_every_call(prec):
         assert all(np.array_equal(runs[0], r) for r in runs[1:])
     finally:
         S.close()
+
+
+def test_confinement_of_one_coefficient_is_the_tables_entry_by_entry():
+    # phi = one coefficient at the end of L along a dimension, a = 1: H phi on the line through it
+    # holds X^4 and the two cross terms' X^2 entries of that dimension, over the whole band
+    import torch
+    N, h = (44, 43, 45), 0.5
+    pos = np.array([[10.37, 10.81, 11.13]])
+    S = lsw.System(N, h, pos, np.array([2.6]), np.array([50.0]), np.array([1]), 4.0, 0, 17.0, 0, lsw.LSW_FP64, device=0,
+                   stream=torch.cuda.current_stream().cuda_stream)
+    try:
+        def members(region, part):
+            k = S.keys(0, region, part)
+            return np.concatenate([np.arange(s, e + 1) for s, e, _ in k])
+
+        Lc, Lf = members(lsw.LSW_REGION_L, lsw.LSW_PART_COARSE), members(lsw.LSW_REGION_L, lsw.LSW_PART_FINE)
+        Pc, Pf = members(lsw.LSW_REGION_LP, lsw.LSW_PART_COARSE), members(lsw.LSW_REGION_LP, lsw.LSW_PART_FINE)
+        assert np.array_equal(Lc, Lf) and np.array_equal(Pc, Pf)          # fine everywhere
+        row = lambda d, m, b, bp, i: lsw.lsw_confinement_row(S.sys, 0, d, m, b, bp, int(i))
+        stride = (1, N[0], N[0] * N[1])
+        ijk = np.stack([Lc % N[0], Lc // N[0] % N[1], Lc // (N[0] * N[1])], 1)
+        mid = np.round(pos[0] / h).astype(int)
+        a = torch.ones(1, dtype=torch.float64, device="cuda")
+        for d in range(3):
+            o = [e for e in range(3) if e != d]
+            line = ijk[(ijk[:, o[0]] == mid[o[0]]) & (ijk[:, o[1]] == mid[o[1]])][:, d]
+            diag = sum(row(e, 2, 0, 0, mid[e])[14] for e in o)            # <s|X_e^2|s> of the other dimensions
+            for j in (line.min(), line.max()):
+                g = int(mid[o[0]] * stride[o[0]] + mid[o[1]] * stride[o[1]] + j * stride[d])
+                for bp in (0, 1):
+                    phi = torch.zeros(S.total_L, dtype=torch.float64, device="cuda")
+                    at = int(np.searchsorted(Lc, g))
+                    phi[at if bp == 0 else len(Lc) + ((1 << d) - 1) * len(Lf) + at] = 1.0
+                    hphi = torch.zeros(S.total_Lp, dtype=torch.float64, device="cuda")
+                    lsw.lsw_add_confinement(S.sys, a, phi, hphi, None)
+                    lsw.lsw_sync(S.sys, 60.0)
+                    out = hphi.cpu().numpy()
+                    for b in (0, 1):
+                        got, want = [], []
+                        for i in range(j - 14, j + 15):
+                            p = int(np.searchsorted(Pc, g + (i - j) * stride[d]))
+                            assert Pc[p] == g + (i - j) * stride[d]
+                            got.append(out[p if b == 0 else len(Pc) + ((1 << d) - 1) * len(Pf) + p])
+                            want.append(row(d, 4, b, bp, i)[14 + j - i] + 2.0 * diag * row(d, 2, b, bp, i)[14 + j - i]
+                                        + (sum(row(e, 4, 0, 0, mid[e])[14] for e in o)
+                                           + 2.0 * row(o[0], 2, 0, 0, mid[o[0]])[14] * row(o[1], 2, 0, 0, mid[o[1]])[14])
+                                        * (i == j and b == bp))
+                        got, want = np.array(got), np.array(want)
+                        assert np.all(np.abs(got - want) <= 1e-13 * np.max(np.abs(want))), (d, j, bp, b)
+    finally:
+        S.close()
