@@ -579,6 +579,7 @@ lsw_status build_plans(lsw_system_s* s) {
         std::memset(&p, 0, sizeof(p));
         p.prec = s->prec;
         p.nfn = static_cast<int>(b.nfn);
+        p.n_sm = s->ctx->n_sm;
         p.zcols = zcols;
         p.fwd_list = s->fwd_list;
         p.wait_out = s->wait_out;
@@ -2322,6 +2323,7 @@ lsw_status lsw_apply_hamiltonian_noalloc(lsw_system sys, const void* phi, void* 
         if (nb == 0 || !noalloc_finish(sys, &p, bwd))   // excluded by the checks above
             return fail(LSW_ERR_STATE, "lsw_apply_hamiltonian_noalloc: inconsistent batch plan");
         p.nfn = nb;
+        p.n_sm = sys->ctx->n_sm;
         p.zsplit = sys->zsplit;
         p.xy_tc = sys->zsplit ? sys->xy_tc : 0;
         CUDA_TRY(enqueue_noalloc_records(static_cast<const FnRec*>(sys->d_fn.p), f, nb,

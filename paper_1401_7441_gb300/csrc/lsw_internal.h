@@ -203,6 +203,7 @@ struct HphiLaunch {
     int prec;                    // 0 FP64, 1 FP32
     const FnRec* fn;             // device records of this batch
     int nfn;
+    int n_sm;                    // of the device
     int max_nz, max_nzp;         // largest L / L' z extents in the batch
     int max_cols;                // largest (2ny+29)(2nx+29) in the batch
     int max_rowsP;               // largest ny'*nz' of L'

@@ -3171,7 +3171,7 @@ cudaError_t plane_kernel_blocks(int prec, size_t smem_fwd, size_t smem_bwd, int*
 // Functions per grid slot of k_uncompress: eight where that leaves eight waves of CTAs (six an SM), else
 // four (batches of 32 functions, 64 atoms: 89 us with four, 119 with one or eight).
 static int uncompress_group(const HphiLaunch& a) {
-    return static_cast<int64_t>(a.nfn) * ((a.max_rowsL + 7) / 8) >= 8 * 8 * 6 * 152 ? 8 : 4;
+    return static_cast<int64_t>(a.nfn) * ((a.max_rowsL + 7) / 8) >= 8LL * 8 * 6 * a.n_sm ? 8 : 4;
 }
 
 template <class T>
