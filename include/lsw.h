@@ -455,7 +455,7 @@ lsw_status lsw_load_phi(lsw_system sys, const char* path, void* phi_dev);
  * room for two CTAs on an SM, else the first that fits; LSW_ERR_UNSUPPORTED if the layout does
  * not fit) -- the same bits in all of them,
  * "wait_out" (0, the default; 1, for tests of the failure path: the backward FMA plane kernel
- * takes its waits for its own copies as run out, sets the status bit and ends; lsw_sync then
+ * takes its waits for its own copies as run out and sets the status bit; lsw_sync then
  * returns LSW_ERR_STATE and the outputs of H phi are not valid),
  * "zsplit" (LSW_FP32_BF16X systems only: 2 or 3 bfloat16 parts per FP32 operand of the
  * tensor-core z stage), "xy_tc" (LSW_FP32_BF16X systems only: 1 runs the x and y passes

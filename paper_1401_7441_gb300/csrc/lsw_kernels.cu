@@ -1860,6 +1860,9 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 #endif
 constexpr int BWD_THREADS = LSW_BWD_THREADS;
 
+// (out of line: the kernel's time depends on what its loops share the instruction caches with)
+static __device__ __noinline__ void bwd_last_wait(uint32_t mbar, uint32_t parity) { (void)tc::mbar_wait(mbar, parity); }
+
 template <class T>
 __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, int zb, int bz, uint32_t& phase, int& dead,
                                           int2* s_next) {
@@ -1932,9 +1935,9 @@ __device__ __forceinline__ void bwd_plane(const HphiLaunch& a, int fl, int cnt, 
         bulk_expect(mbar, bytes);
         bulk_load(tc::saddr(plb), Bb - rem, bytes, mbar);
     };
-    // For the bulk copies in flight.  Once a wait has run out no more copies are announced or waited
-    // for (the barrier's phase is still open: `dead` keeps it, behind the next barrier of the CTA
-    // every thread sees it), and the CTA ends with this item.
+    // For the bulk copies in flight.  Once a wait has run out (dead: 1 + the phase that is still open) no
+    // thread waits any more and the first one, behind the CTA's next barrier, announces no more
+    // copies: a phase may be opened again only once it is complete.
     auto wait = [&]() {
 #ifndef LSW_CHECKED
         if (!dead && (a.wait_out || !tc::mbar_wait(mbar, phase))) {
@@ -2361,7 +2364,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;
     [[maybe_unused]] constexpr int KID = 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int dead;                       // 1 + the phase of the copies that a wait ran out on, 0: none did
+    __shared__ int dead;                       // 1 + the phase that a wait ran out on; 0: none did
     if (threadIdx.x == 0) {
         tc::mbar_init(tc::saddr(smem_raw));
         dead = 0;
@@ -2377,14 +2380,14 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
         __syncthreads();
         for (;;) {
             const int2 it = s_item;   // (the next one is written behind the plane's barriers)
-            if (it.y < 0 || dead) break;
+            if (it.y < 0) break;
             bwd_plane<T>(a, it.x, it.y >> 11, (it.y >> 1) & 1023, it.y & 1, phase, dead, &s_item);
         }
     } else {
         bwd_plane<T>(a, blockIdx.y, 1, blockIdx.x >> 1, blockIdx.x & 1, phase, dead, nullptr);
     }
     // the copies still in flight write to this CTA's shared memory: end behind them (or the limit)
-    if (threadIdx.x == 0 && dead) (void)tc::mbar_wait(tc::saddr(smem_raw), dead - 1);
+    if (threadIdx.x == 0 && dead) bwd_last_wait(tc::saddr(smem_raw), dead - 1);
 }
 
 // ---------------------------------------------------------------- density: pair products
