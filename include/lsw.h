@@ -400,7 +400,7 @@ lsw_status lsw_profile(lsw_system sys, int32_t enable);
 
 /* Summed device milliseconds and launch counts per kernel kind since the last read,
  * kinds in this order: 0 memset, 1 uncompress, 2 forward xy, 3 z stage with V,
- * 4 backward xy (with the compressed write), 5 kinetic z arm, 6 (unused), 7 H/S tiles,
+ * 4 backward xy (with the compressed write), 5 kinetic z arm, 6 H/S pack, 7 H/S tiles,
  * 8 density real-space values, 9 density pair products.  Waits for the stream.  Writes
  * min(max_kinds, *n_kinds) entries of ms[] and launches[]; resets the totals. */
 lsw_status lsw_profile_read(lsw_system sys, int32_t max_kinds, int32_t* n_kinds, double* ms,

@@ -172,9 +172,9 @@ __global__ void __launch_bounds__(256) k_triple(FoeLaunch a, const double* __res
 // the group's rows.  A warp takes a neighbour I of L: it lists, a.chunk entries of I's rows at a
 // time, the columns that both have (position in I's row, position in L's row), and sums the
 // outputs (i, l) over the list, a lane each (several lanes where there are fewer than 32).
-// 400 atoms (1,348 functions, 161 k entries): 62 us a step (86 with a CTA per group: too few
-// warps to cover its loads), 181 with a warp per entry (i, l) that looked every column up for
-// itself and added its lanes.
+// A group is split over several CTAs where there are few (one each: too few warps to cover its
+// loads).  400 atoms (1,348 functions, 161 k entries): 62 us a step, 86 unsplit, 181 with a warp per
+// entry (i, l) that looks every column up for itself.
 __global__ void __launch_bounds__(32 * FOE_WARPS) k_cheb(FoeLaunch a, const double* __restrict__ Htp,
                                                          const double* __restrict__ Tc, const double* __restrict__ Tp,
                                                          double alpha, double* __restrict__ Tn) {

@@ -1260,7 +1260,7 @@ lsw_status build_density_plan(lsw_system_s* s, const int64_t* lo, const int64_t*
     s->dens_ready = false;
     // most functions and atoms of a tile; the products keep their tables in shared memory where
     // two CTAs an SM still fit (about 140 atoms on a tile), else a variant searches the pattern per
-    // pair of chunks (9.2 ms for 300 atoms where the tables gave 7.6)
+    // pair of chunks (6.9 ms for 300 atoms where the tables give 5.1)
     s->dens_max_m = s->dens_max_g = 0;
     for (int64_t t = 0; t < ntiles; ++t) {
         int g = 0;

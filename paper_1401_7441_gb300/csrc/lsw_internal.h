@@ -228,9 +228,10 @@ struct HphiLaunch {
     size_t smem_fwd_tc;          // dynamic shared memory of the tensor-core forward plane kernel
     size_t smem_kin;             // dynamic shared memory of the kinetic z-arm kernel
     // persistent FMA plane kernels: the batch's items (first function, functions << 11 |
-    // plane << 1 | z type; the forward kernel's hold one function), largest first, taken from queue[0] (forward) and queue[1] (backward), which
-    // are zeroed before the batch; grid_* CTAs (as many as fit on the GPU).  NULL items:
-    // one CTA per (2 planes + z type, function) grid slot.
+    // plane << 1 | z type; the forward kernel's hold one function), largest first, taken
+    // from queue[0] (forward) and queue[1] (backward), which are zeroed before the batch;
+    // grid_* CTAs (as many as fit on the GPU).  NULL items: one CTA per (2 planes + z type,
+    // function) grid slot.
     const int2* items_fwd;
     const int2* items_bwd;
     int n_items_fwd, n_items_bwd;

@@ -1832,13 +1832,11 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 // per item and the item loops over the functions.
 //
 // Bound: instruction issue and its latencies (two CTAs per SM by registers and shared memory).
-// Per plane and function, 8 warps issued about 4,770 instructions each, half of them packed
-// FMAs; the rest were staging loops (an element per copy), zero tests of the staged D plane,
-// bounds tests of the kinetic windows and read-modify-writes.  So:
+// What is not arithmetic is kept small:
 //   - the planes of Bb and of the z arm arrive by bulk copies (one instruction each; the copy
 //     starts at the 16-byte boundary below the plane, the remainder becomes the first index);
 //   - the kinetic x arm is computed by the thread that computes the transposed x filter of the
-//     same outputs: one store instead of a store and a read-modify-write, one barrier less;
+//     same outputs: one store, and one barrier for both;
 //   - kinetic sums skip window positions outside the hull of L's members (per row along x, per
 //     column along y), in groups of 12 positions, uniformly over a warp; neighbouring lanes take
 //     neighbouring rows (columns) of the same block, so their hulls nearly agree.  Positions
@@ -1847,13 +1845,13 @@ __global__ void __launch_bounds__(512, 1) k_bwd_xy_tc(HphiLaunch a) {
 //     bodies their unrolled code (40 KB) missed the instruction caches (17 % of the stalls);
 //   - the compressed write's fine members come from a list built once per item;
 //   - the tables are one chain of loads (a row and part per thread), ranges by atomics, prefix
-//     sums and tasks by warps, while the first function's planes arrive: before that they took
-//     15 % of the time for atoms of several functions, 32 % for single ones (1,052 -> 865 us for
-//     64 atoms, where most items are single functions).  The next item is fetched during the last
-//     write, no earlier: a CTA that holds an item unbegun delays the end (FP64 11.1 -> 10.0 ms).
-// Measured (GB300, 2,070 MHz, 1,024 functions a batch): 9.5 -> 4.4 us per function at radii 5-8 bohr
-// (n_x' to 52; one CTA per SM before), 7.3 -> 5.4 us at 7 bohr in a dense system (n_x' 47, more fine
-// members).
+//     sums and tasks by warps, while the first function's planes arrive (built ahead of them by one
+//     thread per table they took 15 % of an item, 32 % of one with a single function).  The next
+//     item is fetched during the last write, no earlier: a CTA that holds an item unbegun delays
+//     the end (64 atoms in FP64: 11.1 ms a step, so 10.0).
+// Measured (GB300, 2,070 MHz, 1,024 functions a batch): 4.4 us per function at radii 5-8 bohr (n_x' to
+// 52), 5.4 us at 7 bohr in a dense system (n_x' 47, more fine members); with an element per copy, an
+// item per function and the arms apart: 9.5 and 7.3.
 
 #ifndef LSW_BWD_THREADS
 #define LSW_BWD_THREADS 256
@@ -2404,18 +2402,17 @@ __global__ void __launch_bounds__(BWD_THREADS, 2) k_bwd_xy(HphiLaunch a) {
 //
 // The chunks (32 functions of the tile's list in order) fix the sums; what is left out adds exact
 // zeros.  Bound: instruction issue and its latencies at two CTAs an SM (128 registers: a chunk's
-// values at two points are 64 of them).  What took the time, 300 atoms (1,038 functions) in FP32:
-//   - 13.0 ms: a warp's points were rows of 32 x, so nearly every function of the tile counted,
-//     and the pattern was searched 2,048 times per pair of chunks.  One search per pair of atoms
-//     (an atom's functions have equal pattern rows and consecutive columns) and four A functions
-//     at a time: 12.4; the searches once per tile instead of once per pair of chunks: no less;
-//   - a warp takes a block of 8 x 4 x 2 points and forms only the products of A functions with
-//     a value there, with groups of four B functions that have one and are in the pattern: 7.6
-//     (with the pattern searched per pair of chunks 9.2: the tile's tables pay now);
-//   - the next pair's coefficients copied during the products into a second block, one barrier
-//     per pair; what belongs to a lane's B function kept in registers: 7.1;
+// values at two points are 64 of them).  So:
+//   - a warp takes a block of 8 x 4 x 2 points (a row of 32 meets nearly every function of the tile)
+//     and forms only the products of A functions with a value there, with groups of four B
+//     functions that have one and are in the pattern;
+//   - the pattern is searched once per pair of atoms of a tile (an atom's functions have equal
+//     pattern rows and consecutive columns), the next pair's coefficients are copied during the
+//     products into a second block, one barrier per pair, four A functions at a time;
 //   - a chunk's values are loaded where their boxes meet the warp's block, all loads before the
-//     first test of a value: 5.1.
+//     first test of a value (7.1 ms with each tested as it arrives).
+// 300 atoms (1,038 functions) in FP32: 5.1 ms; every function of the tile at rows of 32 points, a
+// search per coefficient: 13.0.
 
 struct __align__(16) DensRec {       // one function of a chunk
     int64_t off;                     // block in the store
@@ -2651,7 +2648,7 @@ __global__ void __launch_bounds__(DT_THREADS) k_density(DensLaunch a) {
     const int RS = a.max_g | 1;                                          // odd: a column's entries in different banks
     int* lead = rel + a.max_g * RS;                                 // [max_g]
     __shared__ unsigned um[DT_THREADS / 32][DENS_MASKS];
-    __shared__ unsigned kmask[2][DT_MC];        // per A function: groups of 4 B functions with a nonzero coefficient
+    __shared__ unsigned kmask[2][DT_MC];        // per A function, a bit per B function: the pair is in the pattern
     __shared__ int s_ng;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t t0 = LD(a.tptr, blockIdx.x, a.tptr_n);
@@ -2757,7 +2754,7 @@ __global__ void __launch_bounds__(DT_THREADS) k_density(DensLaunch a) {
 }
 
 // The same for grids with a tile whose tables do not fit: a chunk's records at a time, the pattern
-// searched per pair of chunks (300 atoms: 9.2 ms where the tables give 7.6).
+// searched per pair of chunks (300 atoms in FP32: 6.9 ms where the tables give 5.1; 60 atoms 1.18, 0.93).
 template <class T>
 __global__ void __launch_bounds__(DT_THREADS) k_density_big(DensLaunch a) {
     [[maybe_unused]] int* ST_ = a.status;

@@ -12,11 +12,10 @@
 //                of the tile's points, then the 7 wavelet values of each of the tile's
 //                fine points, 0 where the function has no member (A side: phi on L; Q
 //                side: H phi on L').  The region's row tables are staged in shared
-//                memory.  Bound by instruction issue: a lookup per panel value, with three
-//                divisions by the tile edge, was most of it; a fine point is now looked up
-//                once for its 7 wavelet values and the divisions are multiplications.  3,000
-//                atoms (8,448 functions, tile edge 6) 8.8 -> 6.9 ms; unpack (600 atoms) 0.95
-//                -> 0.41 ms.
+//                memory.  Bound by instruction issue: one lookup per coarse point and one
+//                per fine point (for its 7 wavelet values), divisions by the tile edge as
+//                multiplications.  3,000 atoms (8,448 functions, tile edge 6): 6.9 ms (8.8
+//                with a lookup and three divisions per value); unpack (600 atoms) 0.41 ms.
 //   k_panel_hs   per work item (tile, up to 64 A rows, up to 128 columns of [A; Q]): the
 //                dense product of the A panel with the [A; Q] panel over the tile's
 //                panel length, 4 x 8 outputs per thread in the system's precision, then
